@@ -37,13 +37,16 @@ size_t layout(sgc_state* st, unsigned char* base) {
     st->sel_val = carve<float>(base, off, s);
     st->y64 = carve<double>(base, off, 2 * k);
     st->r64 = carve<double>(base, off, 2 * k);
-    st->r32 = carve<float2>(base, off, k);
+    st->r32 = carve<float2>(base, off, k + 2);                      // read in pairs of rows
     st->sel_cand = carve<unsigned long long>(base, off, sgc::kSelCap);
     st->sel_hist = carve<unsigned int>(base, off, sgc::kSelBins);
-    st->corr_cand = carve<sgc::Cand>(base, off, 2 * (size_t)(st->corr_grid > 32 ? st->corr_grid : 32) * sgc::kCorrTop);
-    st->zsel = carve<uint16_t>(base, off, 2 * s * k);
+    st->corr_cand = carve<sgc::Cand>(base, off, 2 * (size_t)sgc::kCorrBlocks * sgc::kCorrTop);
+    st->zsel = carve<uint16_t>(base, off, sgc::chunk_sized(st) ? 2 * s * k : 1);
+    st->q_basis = carve<double>(base, off, 2 * s * k);
     st->lam = carve<uint32_t>(base, off, 2 * s);
     st->F = carve<double>(base, off, 2 * s * s);
+    st->ccol = carve<double>(base, off, 2 * s * s);
+    st->gam = carve<double>(base, off, 2 * s);
     st->acoef = carve<double>(base, off, 2 * s);
     st->x = carve<double>(base, off, 2 * s);
     st->rnorm = carve<double>(base, off, 2 * s);
@@ -59,10 +62,10 @@ size_t layout(sgc_state* st, unsigned char* base) {
 // for the others, so that thousands of small chunk states do not carry 50 MB each that they never touch
 size_t layout_spec(sgc_state* st, unsigned char* base) {
     size_t off = 0;
-    const size_t k = (size_t)st->k, s = (size_t)st->s;
+    const size_t k = (size_t)st->k, s = (size_t)st->s, kp = (size_t)st->kp;
     {
         const size_t n = (size_t)sgc::kPassMaxN;          // room for a whole batch of same-A states (sgc_step_group)
-        st->rt = carve<uint16_t>(base, off, n * k);
+        st->rt = carve<uint16_t>(base, off, n * kp);
         st->tau = carve<float>(base, off, n);
         st->inv_scale = carve<float>(base, off, n);
         st->rep_count = carve<unsigned int>(base, off, n);
@@ -70,13 +73,13 @@ size_t layout_spec(sgc_state* st, unsigned char* base) {
         st->pick_score = carve<double>(base, off, 2 * s);
         st->cand_list = carve<uint32_t>(base, off, sgc::kCandCap);
         st->cand_bits = carve<unsigned int>(base, off, ((size_t)st->d + 31) / 32);
-        st->rtmp = carve<double>(base, off, k);
         st->rhist = carve<double>(base, off, (size_t)st->pass_n * k);
         st->inv_norm = carve<uint16_t>(base, off, (size_t)st->d);
-        st->zlist = carve<uint16_t>(base, off, (size_t)sgc::kGramList * k);
+        st->zlist = carve<uint16_t>(base, off, (size_t)sgc::kGramList * kp);
         st->gram = carve<double>(base, off, (size_t)sgc::kGramList * sgc::kGramList);
         st->p0 = carve<double>(base, off, 2 * (size_t)sgc::kGramList);
-        st->pick_li = carve<int>(base, off, 2 * s);
+        st->wgram = carve<double>(base, off, 2 * (size_t)sgc::kGramList * s);
+        st->pnorm = carve<double>(base, off, 2 * ((k + 31) / 32) * (sgc::kGramList + 1));
         st->hist_slots = sgc::kHistColumns / (int)s < sgc::kHistSteps ? sgc::kHistColumns / (int)s : sgc::kHistSteps;
         if (st->hist_slots < 1) st->hist_slots = 1;
         st->kept_ring = carve<uint32_t>(base, off, (size_t)st->hist_slots * s);
@@ -91,7 +94,7 @@ size_t layout_spec(sgc_state* st, unsigned char* base) {
 bool finite_f(float v) { return isfinite(v); }
 
 cudaError_t ensure_spec(sgc_state* st) {
-    if (!st->spec_ok || st->spec_ready) return cudaSuccess;
+    if (st->spec_ready) return cudaSuccess;
     {
         sgc_state probe = *st;                                       // measuring must not leave pointers behind
         st->spec_bytes = layout_spec(&probe, nullptr);
@@ -104,6 +107,16 @@ cudaError_t ensure_spec(sgc_state* st) {
     if (e != cudaSuccess) { cudaFree(st->spec_base); st->spec_base = nullptr; return e; }
     st->spec_ready = true;
     return cudaSuccess;
+}
+
+// buffers of the speculative recovery for a state that was created without them and now wants them (k no multiple of 64,
+// d large enough).  Not while the stream is being captured (an allocation is not allowed there), and a state that cannot get
+// them recovers in lock-step.
+void prepare_spec(sgc_state* st, cudaStream_t stream) {
+    if (st->spec_ready || st->spec_refused || st->mode != SGC_MODE_AUTO || st->d < sgc::kSpecMinD) return;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) { cudaGetLastError(); return; }
+    if (ensure_spec(st) != cudaSuccess) { st->spec_refused = true; cudaGetLastError(); }
 }
 
 }  // namespace
@@ -139,7 +152,9 @@ SGC_API int sgc_create(sgc_state** out, int64_t d, int32_t k, int32_t s, uint64_
         layout(st, static_cast<unsigned char*>(st->base));
         e = cudaMemset(st->base, 0, st->bytes);        // M_0 = V_0 = 0, counters, histogram, empty candidate list
     }
-    if (e == cudaSuccess && st->d >= ((int64_t)1 << 16)) e = ensure_spec(st);      // SGC_MODE_AUTO speculates from this size on
+    // SGC_MODE_AUTO speculates from d = 65536 on.  States whose k is no multiple of 64 are mostly chunks of MESGC, which do not
+    // need these buffers: they get them at their first sgc_step instead.
+    if (e == cudaSuccess && st->d >= sgc::kSpecMinD && st->k % 64 == 0) e = ensure_spec(st);
     if (e == cudaSuccess) {
         e = cudaHostAlloc(reinterpret_cast<void**>(&st->h_rounds), sizeof(int), cudaHostAllocMapped);
         if (e == cudaSuccess) { st->h_rounds[0] = 0; e = cudaHostGetDevicePointer(reinterpret_cast<void**>(&st->d_rounds), st->h_rounds, 0); }
@@ -161,6 +176,7 @@ SGC_API int sgc_step(sgc_state* st, const float* grad, float* weight, void* stre
     if (((uintptr_t)grad & 15u) || ((uintptr_t)weight & 15u)) return SGC_ERR_ALIGN;
     if (!on_own_device(st)) return SGC_ERR_DEVICE;
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
+    prepare_spec(st, cs);
     int launches = 0;
     // t counts the steps whose gradient has entered M and V: it moves once the kernel that updates them is enqueued
     st->t += 1;
@@ -172,7 +188,7 @@ SGC_API int sgc_step(sgc_state* st, const float* grad, float* weight, void* stre
     return (int)e;
 }
 
-SGC_API int sgc_step_group(sgc_state* const* states, const float* const* grads, float* const* weights, int32_t n, void* stream) {
+static int step_group(sgc_state* const* states, const float* const* grads, float* const* weights, int32_t n, void* stream, bool own_states) {
     if (!states || !grads || !weights) return SGC_ERR_NULL;
     if (n < 1) return SGC_ERR_DIM;
     for (int32_t i = 0; i < n; ++i) {
@@ -185,6 +201,7 @@ SGC_API int sgc_step_group(sgc_state* const* states, const float* const* grads, 
         if (!on_own_device(states[i])) return SGC_ERR_DEVICE;
     }
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
+    if (own_states) for (int32_t i = 0; i < n; ++i) prepare_spec(states[i], cs);
     std::vector<int> launches((size_t)n, 0);
     cudaError_t e = cudaSuccess;
     for (int32_t i = 0; i < n && e == cudaSuccess; ++i) {           // a1-a3 per state
@@ -202,6 +219,10 @@ SGC_API int sgc_step_group(sgc_state* const* states, const float* const* grads, 
         st->last_launches = launches[i] + (i == 0 ? shared : 0);     // the shared launches are booked on the first state
     }
     return (int)e;
+}
+
+SGC_API int sgc_step_group(sgc_state* const* states, const float* const* grads, float* const* weights, int32_t n, void* stream) {
+    return step_group(states, grads, weights, n, stream, true);
 }
 
 SGC_API int sgc_step_chunked(sgc_state* const* states, int32_t c, const float* grad, float* weight, void* stream) {
@@ -237,7 +258,7 @@ SGC_API int sgc_step_chunked(sgc_state* const* states, int32_t c, const float* g
     std::vector<const float*> gs((size_t)c);
     std::vector<float*> ws((size_t)c);
     for (int32_t i = 0; i < c; ++i) { gs[i] = grad + (size_t)i * dc; ws[i] = weight + (size_t)i * dc; }
-    return sgc_step_group(states, gs.data(), ws.data(), c, stream);
+    return step_group(states, gs.data(), ws.data(), c, stream, false);
 }
 
 SGC_API int sgc_cesgc_step(sgc_state* const* states, int32_t c, const float* B, int32_t r, int32_t m, int32_t n,
@@ -294,7 +315,7 @@ SGC_API int sgc_reproject(sgc_state* st, uint64_t new_seed, void* stream) {
 SGC_API int sgc_set_mode(sgc_state* st, int32_t mode) {
     if (!st) return SGC_ERR_NULL;
     if (mode < SGC_MODE_AUTO || mode > SGC_MODE_SPECULATIVE) return SGC_ERR_WHAT;
-    if (mode == SGC_MODE_SPECULATIVE && !st->spec_ok) return SGC_ERR_DIM;
+    if (mode == SGC_MODE_SPECULATIVE && st->k % 64 != 0) return SGC_ERR_DIM;
     if (mode == SGC_MODE_SPECULATIVE) {
         const cudaError_t e = ensure_spec(st);                       // small states get their speculative buffers here
         if (e != cudaSuccess) return (int)e;

@@ -852,9 +852,11 @@ void free_chunk_ws(sgc_state* st) {
 
 // The batched path serves chunk lists whose states are alike in everything but their moments: same shape, matrix, step
 // count and hyper-parameters, Algorithm 2 as printed, small s and k, and no request for the speculative recovery.
+bool chunk_sized(const sgc_state* st) { return st->s <= kChunkMaxS && st->k <= kChunkMaxK; }
+
 bool chunked_batch_eligible(sgc_state* const* sts, int c) {
     const sgc_state* a = sts[0];
-    if (a->s > kChunkMaxS || a->k > kChunkMaxK || (a->d & 3) || a->d >= (1ll << 31) || c > (1 << 20)) return false;
+    if (!chunk_sized(a) || (a->d & 3) || a->d >= (1ll << 31) || c > (1 << 20)) return false;
     for (int i = 0; i < c; ++i) {
         const sgc_state* b = sts[i];
         if (b->mode == SGC_MODE_SPECULATIVE || b->shared_support || b->residual_tol > 0.0 || b->profile) return false;

@@ -104,15 +104,12 @@ constexpr int kPassMaxK = 65536;       // rows of A of the stand-alone screening
 constexpr int kMaxS = 1024;
 constexpr int kSelCap = 32768;          // candidate slots of the top-s filter
 constexpr int kSelBins = 4096;          // 12-bit magnitude histogram of the sample
-constexpr int kCorrThreads = 512;       // threads per block of the correlation pass
-constexpr int kCorrCols = 2;            // columns per thread and tile
 constexpr int kCorrTop = 3;             // slots per block and residual: its best two columns, and the score of its third best
+constexpr int kCorrBlocks = 256;        // blocks that correlate, at most
 constexpr int kRescoreCap = 16;         // candidates rescored in fp64 per iteration and residual
-constexpr int kBookThreads = 1024;
-constexpr int kOmpThreads = 1024;       // threads per block of the cooperative OMP kernel
+constexpr int kOmpThreads = 1024;       // threads per block of the resolve and finish kernels
 constexpr int kCandCap = 32768;         // candidate columns kept for the restricted (speculative) OMP
 constexpr int kCandKeep = 24576;        // the list is rebuilt from the supports once it grows beyond this
-constexpr int kSmallList = 768;         // lists up to this length are correlated inside the bookkeeping block
 constexpr int kHistSteps = 64;          // steps whose kept indices (Sparsify_s) stay candidates ...
 constexpr int kHistColumns = 8192;      // ... as long as they are at most this many columns
 constexpr int kLookAhead = 12;          // after a refuted pick, every kLookAhead-th later residual is harvested too
@@ -126,6 +123,7 @@ constexpr int kGramList = 256;          // lists up to this length run OMP on th
 constexpr int kRepCap = 8192;           // report slots per residual of one screening pass
 constexpr int kPassMaxN = 256;          // residuals per screening pass (UMMA N)
 constexpr int kPassMaxBatch = 8;        // states whose residuals one screening pass can serve (kPassMaxN / 32)
+constexpr int64_t kSpecMinD = 65536;    // SGC_MODE_AUTO speculates from this many columns on
 constexpr int kMaxRounds = 24;          // speculate / screen / resolve rounds enqueued per step
 constexpr int kTensorMapBytes = 128;    // sizeof(CUtensorMap)
 // |score computed by the screening pass - exact score| <= (kScreenMargin + k * kScreenAccMargin) * ||r|| + kScreenNormMargin * score:
@@ -178,8 +176,6 @@ struct SpecCtl {
     int list_exact[2];      // 1: the last speculation of residual m compared every list member exactly
     int list_version;       // bumped whenever the candidate list changes
     int gram_version;       // list version the stored Gram matrix belongs to
-    int gram_pending;       // list version seen by the round in flight
-    int gram_todo;          // 1: the Gram matrix must be recomputed in this round
     int gram_ok;            // 0: the Gram path gave up in this step (a pick is missing from the list)
     int tv[2];              // tentative picks: confirmed against the wide lists only (tv >= v)
     uint32_t tforced[2];    // column imposed as pick tv[m] by a list pass, or kNoColumn
@@ -249,11 +245,13 @@ struct sgc_state {
     cudaStream_t last_stream; bool has_stream;
     int32_t last_launches; bool stepped;
     bool sel_warm;              // a top-s threshold from the previous step is on the device (one-kernel selection)
-    int corr_grid, corr_smem;
+    int omp_grid2, omp_grid8;   // blocks of the recovery kernel in clusters of 2 and of 8
+    int omp_one;                // 1: a cluster of 16 can be resident
+    int kp;                     // k rounded up to a multiple of 64: row stride of rt and zlist
     int mode;                   // 0 auto, 1 lock-step only, 2 speculative whenever k allows it
     int shared_support;         // 1: OMP(M^) alone selects, V^ is fitted on its support (sgc_set_recovery)
     double residual_tol;        // > 0: recoveries are cut at the first pick that leaves ||r|| <= residual_tol ||y||
-    bool spec_ok;               // speculative recovery usable for this (d, k)
+    bool spec_refused;          // its buffers could not be allocated at a step
     bool spec_ready;            // its buffers exist (second allocation: at creation for d >= 65536, else at sgc_set_mode)
     void* spec_base; size_t spec_bytes;
     int pass_n;                 // residuals per screening pass (multiple of 32, <= 256); pass_n / 2 per residual stream
@@ -271,18 +269,19 @@ struct sgc_state {
     void* base; size_t bytes;
     float *M, *V; double *p, *q;
     uint32_t* sel_idx; float* sel_val;
-    double *y64, *r64;          // [2][k]
+    double *y64, *r64;          // [2][k]; r64: chunk path only
     float2* r32;                // [k] (M^ residual, V^ residual)
     unsigned long long* sel_cand; unsigned int* sel_hist;
-    sgc::Cand* corr_cand;       // [2][corr_grid][kCorrTop]
-    uint16_t* zsel;             // [2][s][k] selected columns of Z as binary16 bits
+    sgc::Cand* corr_cand;       // [2][kCorrBlocks][kCorrTop]
+    uint16_t* zsel;             // [2][s][k] selected columns of Z as binary16 bits (chunk path only)
     uint32_t* lam;              // [2][s]
-    double *F, *acoef, *x, *gvec, *cvec, *rnorm;   // [2][s*s], [2][s] ...
+    double* q_basis;            // [2][s][k] orthogonal basis of the picked columns
+    double *F, *ccol, *acoef, *gam, *x, *rnorm;   // [2][s*s] (coefficients c by pick and by row; the chunk path keeps its F there), [2][s]
     uint32_t* upd_idx; double* upd_val;
     sgc::Counters* cnt;
     // speculative recovery
     sgc::SpecCtl* ctl;
-    uint16_t* rt;               // R^T [pass_n][k] binary16 bits: the residuals screened by one pass, each row scaled
+    uint16_t* rt;               // R^T [pass_n][kp] binary16 bits: the residuals screened by one pass, each row scaled
     float* tau;                 // [pass_n] thresholds (in the scaled units of the row)
     float* inv_scale;           // [pass_n] 1 / (power-of-two scale of the row)
     unsigned int* rep_count;    // [pass_n]
@@ -290,13 +289,13 @@ struct sgc_state {
     double* pick_score;         // [2][s] exact score |<Z_i, r>| / ||Z_i|| of every speculative pick
     uint32_t* cand_list;        // [kCandCap]
     unsigned int* cand_bits;    // bitmap over [0, d): membership in cand_list
-    double* rtmp;               // [k] scratch residual of the resolve kernel
     double* rhist;              // [pass_n][k] the screened residuals of this state in fp64 (row = stream * rows per stream + position)
     uint16_t* inv_norm;         // [d] 1 / ||Z_i|| as binary16, filled once at creation (the screening pass reads it)
-    uint16_t* zlist;            // [kGramList][k] the candidate columns as binary16 (Gram path)
+    uint16_t* zlist;            // [kGramList][kp] the candidate columns as binary16 (Gram path)
     double* gram;               // [kGramList][kGramList] Z_C^T Z_C
     double* p0;                 // [2][kGramList] Z_C^T y per residual
-    int* pick_li;               // [2][s] list position of every pick (Gram path)
+    double* wgram;              // [2][s][kGramList] products of the list with the orthogonal basis (lists that outgrow shared memory)
+    double* pnorm;              // [2][k / 32][kGramList + 1] partial squared residual norms
     uint32_t* kept_ring;         // [hist_slots][s] kept indices of the last steps (all of them are columns M^ and V^ are made of)
     int hist_slots;
     sgc::ChunkWs* chunk_ws;     // batched chunk path: workspace built for the chunk list that starts with this state
@@ -345,6 +344,7 @@ cudaError_t launch_recover_group(sgc_state* const* sts, float* const* weights, i
 cudaError_t launch_z_block(uint64_t seed, int64_t row0, int64_t nrows, int64_t col0, int64_t ncols, float* out,
                            cudaStream_t stream);
 // MESGC with small per-chunk problems (s <= 32, k <= 256): the whole step of all chunks in 2 + 2s launches
+bool chunk_sized(const sgc_state* st);          // small enough in s and k
 bool chunked_batch_eligible(sgc_state* const* sts, int c);
 cudaError_t launch_chunked_batch(sgc_state* const* sts, int c, const float* grad, float* weight, cudaStream_t stream,
                                  int* launches);

@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
     unsigned int list_n0 = 0, list_n = 0, num_super = a.num_super;
     if (WIDE && a.list_ctl != nullptr) {
         const volatile SpecCtl* lc = a.list_ctl;
-        if (!lc->round_active || lc->fallback || lc->mini_done || lc->n_cand <= kSmallList) return;
+        if (!lc->round_active || lc->fallback || lc->mini_done || lc->n_cand <= kGramList) return;
         list_n0 = min(a.big_count[0], (unsigned int)a.big_cap);
         // the half-width pass serves the first stream alone: its own list is all it needs
         list_n = list_n0 + ((a.sel != nullptr && a.sel_value == 1) ? 0u : min(a.big_count[1], (unsigned int)a.big_cap));
