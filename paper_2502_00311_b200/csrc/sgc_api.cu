@@ -83,7 +83,7 @@ size_t layout_spec(sgc_state* st, unsigned char* base) {
         st->hist_slots = sgc::kHistColumns / (int)s < sgc::kHistSteps ? sgc::kHistColumns / (int)s : sgc::kHistSteps;
         if (st->hist_slots < 1) st->hist_slots = 1;
         st->kept_ring = carve<uint32_t>(base, off, (size_t)st->hist_slots * s);
-        st->wide_tau = carve<float>(base, off, sgc::kPassMaxN / 8);
+        st->wide_tau = carve<float>(base, off, sgc::kPassMaxN);
         st->wide_list = carve<uint32_t>(base, off, 2 * (size_t)sgc::kWideCap);
         st->wide_count = carve<unsigned int>(base, off, 2);
         st->wide_bits = carve<unsigned int>(base, off, 2 * (((size_t)st->d + 31) / 32));

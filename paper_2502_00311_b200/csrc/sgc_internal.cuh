@@ -300,7 +300,8 @@ struct sgc_state {
     int hist_slots;
     sgc::ChunkWs* chunk_ws;     // batched chunk path: workspace built for the chunk list that starts with this state
     bool two_level;             // host: wide lists and list passes are in use (steps that need several full passes)
-    float* wide_tau;            // [kPassMaxN / 8] thresholds of the wide lists, one per 8th screened residual
+    float* wide_tau;            // [kPassMaxN] thresholds of the wide lists, +inf for residuals that do not feed them
+    int wide_every;             // every so many screened residuals of a stream feed its wide list
     uint32_t* wide_list;        // [2][kWideCap]
     unsigned int* wide_count;   // [2]
     unsigned int* wide_bits;    // [2] bitmaps over [0, d): the column is in the stream's wide list
@@ -359,7 +360,7 @@ cudaError_t finish_recover_setup(sgc_state* st); // after the workspace exists: 
 
 // wide lists of the two-level screening (sgc_pass.cu): a full pass fills them, a list pass screens only their columns
 struct PassWide {
-    const float* tau;            // [n / 8] thresholds of the wide lists (scaled units of rows 0, 8, 16, ...)
+    const float* tau;            // [n] thresholds of the wide lists (scaled units of the rows; +inf: the row feeds none)
     uint32_t* list;              // [2][cap]
     unsigned int* count;         // [2]
     unsigned int* bits;          // [2] bitmaps over [0, d), one per stream: a column enters a list once

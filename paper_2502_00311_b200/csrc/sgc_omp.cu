@@ -1020,7 +1020,7 @@ __global__ void __launch_bounds__(kT, 1) k_omp(OmpArgs a, int mode) {
                 a.rep_count[m * a.half_n + c] = 0u;
                 if (c >= keep) {
                     a.tau[m * a.half_n + c] = __int_as_float(0x7f800000);
-                    if ((c & 7) == 0) a.wide_tau[(m * a.half_n + c) >> 3] = __int_as_float(0x7f800000);
+                    a.wide_tau[m * a.half_n + c] = __int_as_float(0x7f800000);
                 }
             }
         }
@@ -1117,7 +1117,7 @@ __global__ void __launch_bounds__(kT, 1) k_omp(OmpArgs a, int mode) {
                     const double psc = fabs(dot) / sqrt(n2);
                     a.pick_score[(size_t)m * s + j] = psc;
                     a.tau[m * a.half_n + c] = (float)(report_threshold(a, cur_rnorm, psc) * residual_scale(cur_rnorm));
-                    if ((c & 7) == 0) a.wide_tau[(m * a.half_n + c) >> 3] = wide_threshold(a, cur_rnorm);
+                    a.wide_tau[m * a.half_n + c] = wide_threshold(a, c, cur_rnorm);
                     a.lam[(size_t)m * s + j] = col;
                 }
                 if (!(piv > kPivot * n2)) rc = 2;
@@ -1188,7 +1188,7 @@ __global__ void __launch_bounds__(kT, 1) k_omp(OmpArgs a, int mode) {
                         extra = 1;
                         if (g == 0 && t == 0) {
                             a.tau[m * a.half_n + c] = (float)(a.z_harvest * cur_rnorm / sqrt((double)k) * residual_scale(cur_rnorm));
-                            if ((c & 7) == 0) a.wide_tau[(m * a.half_n + c) >> 3] = wide_threshold(a, cur_rnorm);
+                            a.wide_tau[m * a.half_n + c] = wide_threshold(a, c, cur_rnorm);
                         }
                     } else { dep = 1; hi = j + 1; }
                     if (g == 0 && t == 0) a.ctl->stop[m] = 1;

@@ -26,7 +26,7 @@ struct OmpArgs {
     uint16_t* rt; float* tau; float* inv_scale; unsigned int* rep_count; double* pick_score;
     double* rhist;                     // fp64 copies of the screened residuals (row = m * half_n + position), for the resolve kernel
     // two-level screening
-    float* wide_tau; double z_wide; unsigned int* wide_count; unsigned int* wide_bits;
+    float* wide_tau; double z_wide; int wide_every; unsigned int* wide_count; unsigned int* wide_bits;
     int mini;                          // 1: speculation ahead of a list pass (at most `depth` picks)
     int depth;
     const uint32_t* cand_list;
@@ -46,8 +46,9 @@ __device__ __forceinline__ double warp_sum(double v) {
 }
 
 // threshold of a wide list: every column scoring at least z_wide noise deviations against a screened residual (norm rn)
-// whose row index is a multiple of 8, in the scaled units of that row
-__device__ __forceinline__ float wide_threshold(const OmpArgs& a, double rn) {
+// in place c of its stream, in the scaled units of that row; +inf where the place feeds no list
+__device__ __forceinline__ float wide_threshold(const OmpArgs& a, int c, double rn) {
+    if (c % a.wide_every != 0) return __int_as_float(0x7f800000);
     return (float)(a.z_wide * rn / sqrt((double)a.k) * residual_scale(rn));
 }
 

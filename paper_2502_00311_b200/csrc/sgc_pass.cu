@@ -55,11 +55,11 @@ struct PassArgs {
     unsigned int* rep_count;     // [n]
     uint2* rep;                  // [n][rep_cap]  (column, score bits)
     int rep_cap;
-    // Two-level screening (single state only).  A full pass also collects, for every 8th residual of each stream,
-    // every column scoring at least big_tau[row / 8] into the stream's "wide list" (some 10^5 columns; the bitmap lets a
+    // Two-level screening (single state only).  A full pass also collects, for some residuals of each stream,
+    // every column scoring at least big_tau[row] into the stream's "wide list" (some 10^5 columns; the bitmap lets a
     // column in once).  A list pass (list_ctl != nullptr) then screens only the columns of the two wide lists: a few
     // percent of the work of a full pass.
-    const float* big_tau;        // [n / 8] or nullptr
+    const float* big_tau;        // [n] (+inf: the residual feeds no list) or nullptr
     uint32_t* big_list;          // [2][big_cap]
     unsigned int* big_count;     // [2]
     unsigned int* big_bits;      // [2] bitmaps over [0, d), one per stream
@@ -175,7 +175,7 @@ __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t
 // dynamic shared memory (after alignment to 1024 bytes):
 //   stages x { A tile 0 (16 KB) | A tile 1 (16 KB) | R^T chunk (n x 128 B) }
 //   norms  float[kNormRing][256][2]      partial ||Z_i||^2 of the two generator threads of each column
-//   tau    float[256], 1 / tau float[256]
+//   tau    float[256], 1 / tau float[256], 1 / wide-list threshold float[256]
 //   mbarriers: full[stages], empty[stages], acc_full[2], acc_empty[2], drain;  tensor-memory base;  abort flag
 // WIDE: the two-level screening code (wide-list harvest, list passes) is compiled in
 // SUB: 64-row chunks of A per slot of the ring, i.e. per hand-off between generators, TMA and MMA issuer (2 when the
@@ -215,7 +215,8 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
     float* norms = reinterpret_cast<float*>(gen_base + norms_off);
     float* tau_s = norms + kNormRing * kSuperCols * 2;
     float* itau_s = tau_s + 256;                                     // 1 / tau: a group of 16 residuals is skipped on one compare
-    uint64_t* bars = reinterpret_cast<uint64_t*>(itau_s + 256);
+    float* iwide_s = itau_s + 256;                                   // 1 / threshold of the wide lists
+    uint64_t* bars = reinterpret_cast<uint64_t*>(iwide_s + 256);
     const uint32_t bar_full = smem_u32(bars), bar_empty = bar_full + 8u * a.stages;
     const uint32_t bar_accf = bar_empty + 8u * a.stages, bar_acce = bar_accf + 16u, bar_drain = bar_acce + 16u;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * a.stages + 5);
@@ -242,6 +243,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
         const float tv = i < a.n ? a.tau[i] : __int_as_float(0x7f800000);
         tau_s[i] = tv;
         itau_s[i] = tv > 0.0f ? 1.0f / tv : 3.0e38f;                 // tau = +inf (unused residual) -> 0
+        if (WIDE) iwide_s[i] = i < a.n && a.big_tau != nullptr ? 1.0f / a.big_tau[i] : 0.0f;
     }
     if (warp == 1) {           // tensor memory: all 512 columns (the only CTA on this SM)
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512u)
@@ -340,9 +342,9 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
                     inv_w[q * 32 + lane] = col < a.d ? half_bits_to_float(a.inv_norm[col]) : 0.0f;
                 }
                 __syncwarp();
-                // every 8th residual feeds the wide list of its stream (full passes of the two-level screening)
-                const bool feeds = WIDE && a.big_tau != nullptr && !listed && (n_res & 7) == 0;
-                const float wide_tau_n = feeds ? a.big_tau[n_res >> 3] : 0.0f;
+                // some residuals feed the wide list of their stream (full passes of the two-level screening)
+                const float wide_tau_n = WIDE && a.big_tau != nullptr && !listed ? a.big_tau[n_res] : __int_as_float(0x7f800000);
+                const bool feeds = WIDE && wide_tau_n < __int_as_float(0x7f800000);
                 // wide-list hits of this warp are queued in shared memory and appended after the sweep, all at once: the two
                 // dependent global atomics of an append then cost the warp two round trips per sweep instead of two per hit
                 // (the warp's 32 residuals belong to one stream whenever the streams' blocks are multiples of 32 rows)
@@ -440,10 +442,18 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
                     uint32_t v[16];
                     tmem_ld16(tmem_base + ((uint32_t)(quad * 32) << 16) + buf * acc_cols + t * a.n + c0, v);
                     if (WIDE && a.big_tau != nullptr && !listed && inv > 0.0f) {
-                        // every 8th residual feeds the wide list of its stream
-                        const bool w0 = fabsf(__uint_as_float(v[0])) * inv >= a.big_tau[c0 >> 3];
-                        const bool w8 = fabsf(__uint_as_float(v[8])) * inv >= a.big_tau[(c0 >> 3) + 1];
-                        if (w0 || w8) {
+                        // some residuals feed the wide list of their stream (16 neighbouring residuals belong to one)
+                        float peak = 0.0f;
+                        const float4* iw4 = reinterpret_cast<const float4*>(iwide_s + c0);
+#pragma unroll
+                        for (int i4 = 0; i4 < 4; ++i4) {
+                            const float4 w = iw4[i4];
+                            peak = fmaxf(peak, fabsf(__uint_as_float(v[4 * i4])) * w.x);
+                            peak = fmaxf(peak, fabsf(__uint_as_float(v[4 * i4 + 1])) * w.y);
+                            peak = fmaxf(peak, fabsf(__uint_as_float(v[4 * i4 + 2])) * w.z);
+                            peak = fmaxf(peak, fabsf(__uint_as_float(v[4 * i4 + 3])) * w.w);
+                        }
+                        if (peak * inv >= 1.0f) {
                             const unsigned int bit = 1u << ((unsigned int)col & 31u);
                             const int m = c0 >= a.big_half ? 1 : 0;
                             if (!(atomicOr(&a.big_bits[(size_t)m * ((a.d + 31) >> 5) + (col >> 5)], bit) & bit)) {
@@ -603,7 +613,7 @@ cudaError_t get_encoder(EncodeTiledFn* out) {
 }
 
 size_t pass_smem_bytes(int n, int slots, int sub) {
-    return 1024 + (size_t)slots * sub * (2 * kTileBytes + (size_t)n * 128) + sizeof(float) * (kNormRing * kSuperCols * 2 + 512) +
+    return 1024 + (size_t)slots * sub * (2 * kTileBytes + (size_t)n * 128) + sizeof(float) * (kNormRing * kSuperCols * 2 + 768) +
            8 * (2 * (size_t)slots + 5) + 16;
 }
 

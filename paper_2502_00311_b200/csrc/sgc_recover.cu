@@ -417,7 +417,7 @@ k_begin(SpecCtl* ctl, int speculate, float* wide_tau, int shared, const uint32_t
     __shared__ int n_s;
     const int t = threadIdx.x;
     // no wide list unless a long-list speculation asks for one
-    if (wide_tau != nullptr && t < kPassMaxN / 8) wide_tau[t] = __int_as_float(0x7f800000);
+    if (wide_tau != nullptr && t < kPassMaxN) wide_tau[t] = __int_as_float(0x7f800000);
     if (t < kMaxRounds) ctl->trace[t][0] = ctl->trace[t][1] = ctl->trace[t][2] = 0;
     const int n0 = ctl->n_cand, version = ctl->list_version;
     const int slot = speculate ? ctl->hist_next % hist_slots : 0;
@@ -661,7 +661,7 @@ OmpArgs make_args(const sgc_state* st) {
     a.rhist = st->rhist;
     a.cand_list = st->cand_list;
     a.zlist = st->zlist; a.gram = st->gram; a.p0 = st->p0; a.wgram = st->wgram; a.pnorm = st->pnorm;
-    a.wide_tau = st->wide_tau; a.z_wide = st->z_wide; a.wide_count = nullptr; a.wide_bits = st->wide_bits; a.mini = 0;
+    a.wide_tau = st->wide_tau; a.z_wide = st->z_wide; a.wide_every = st->wide_every; a.wide_count = nullptr; a.wide_bits = st->wide_bits; a.mini = 0;
     a.depth = 1 << 30;
     return a;
 }
@@ -688,6 +688,11 @@ cudaError_t configure_recover(sgc_state* st) {
     st->z_harvest = normal_tail_threshold_impl((double)st->d, 3072.0);
     st->z_floor = normal_tail_threshold_impl((double)st->d, 6144.0);
     st->z_wide = normal_tail_threshold_impl((double)st->d, 100000.0);
+    // How often a screened residual feeds the wide lists: a pick takes 25-30 / k of the residual's energy, so the scores of the
+    // columns drift the faster the smaller k is.  Mean step (full passes per step) at every 8th / 4th / 2nd residual, 4096 x 11008:
+    // k = 256, s = 16: 16.2 (2.80) / 14.7 (2.45) / 14.1 ms (2.25); k = 2048, s = 128: 125 (3.50) / 117 (3.19) / 119 ms (3.19);
+    // k = 4096, s = 256: 247 (2.55) / 259 (2.60) / 263 ms (2.60): denser feeding makes the lists longer.
+    st->wide_every = st->k < 512 ? 2 : st->k <= 2048 ? 4 : 8;
     return pass_configure(kPassMaxN);
 }
 
