@@ -40,7 +40,7 @@ size_t layout(sgc_state* st, unsigned char* base) {
     st->r32 = carve<float2>(base, off, k + 2);                      // read in pairs of rows
     st->sel_cand = carve<unsigned long long>(base, off, sgc::kSelCap);
     st->sel_hist = carve<unsigned int>(base, off, sgc::kSelBins);
-    st->corr_cand = carve<sgc::Cand>(base, off, 2 * (size_t)sgc::kCorrBlocks * sgc::kCorrTop);
+    st->corr_cand = carve<float4>(base, off, 2 * (size_t)sgc::kCorrBlocks);
     st->zsel = carve<uint16_t>(base, off, sgc::chunk_sized(st) ? 2 * s * k : 1);
     st->q_basis = carve<double>(base, off, 2 * s * k);
     st->lam = carve<uint32_t>(base, off, 2 * s);
@@ -113,7 +113,7 @@ cudaError_t ensure_spec(sgc_state* st) {
 // d large enough).  Not while the stream is being captured (an allocation is not allowed there), and a state that cannot get
 // them recovers in lock-step.
 void prepare_spec(sgc_state* st, cudaStream_t stream) {
-    if (st->spec_ready || st->spec_refused || st->mode != SGC_MODE_AUTO || st->d < sgc::kSpecMinD) return;
+    if (st->spec_ready || st->spec_refused || !sgc::will_speculate(st)) return;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) { cudaGetLastError(); return; }
     if (ensure_spec(st) != cudaSuccess) { st->spec_refused = true; cudaGetLastError(); }

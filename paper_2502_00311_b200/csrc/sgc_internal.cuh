@@ -104,8 +104,7 @@ constexpr int kPassMaxK = 65536;       // rows of A of the stand-alone screening
 constexpr int kMaxS = 1024;
 constexpr int kSelCap = 32768;          // candidate slots of the top-s filter
 constexpr int kSelBins = 4096;          // 12-bit magnitude histogram of the sample
-constexpr int kCorrTop = 3;             // slots per block and residual: its best two columns, and the score of its third best
-constexpr int kCorrBlocks = 256;        // blocks that correlate, at most
+constexpr int kCorrBlocks = 160;        // blocks that correlate, at most (a multiple of 32)
 constexpr int kRescoreCap = 16;         // candidates rescored in fp64 per iteration and residual
 constexpr int kOmpThreads = 1024;       // threads per block of the resolve and finish kernels
 constexpr int kCandCap = 32768;         // candidate columns kept for the restricted (speculative) OMP
@@ -190,6 +189,7 @@ struct SpecCtl {
     int hist_count, hist_next;  // ring of the kept index sets of the last steps: valid slots, slot of the next step
     int trace[kMaxRounds][3];   // per round: confirmed picks of both streams and the list length after it
     double ynorm[2];        // ||y|| per residual
+    int inexact_streak;     // speculating steps in a row that needed more than one confirming pass
 };
 
 // device-resident counters of one state
@@ -256,6 +256,7 @@ struct sgc_state {
     void* spec_base; size_t spec_bytes;
     int pass_n;                 // residuals per screening pass (multiple of 32, <= 256); pass_n / 2 per residual stream
     double z_harvest, z_floor;  // thresholds of the screening pass in units of ||r|| / sqrt(k)
+    double z_harvest_few;       // the same for states whose picks are confirmed without contest
     double z_wide;              // threshold of the wide lists, same units
     unsigned char tmap[8][128]; // CUtensorMaps of the residual matrix R^T, one per number of states batched into a pass
     unsigned char tmap_half[128]; // the same for a pass over the first stream's residuals alone (shared-support variant)
@@ -272,7 +273,7 @@ struct sgc_state {
     double *y64, *r64;          // [2][k]; r64: chunk path only
     float2* r32;                // [k] (M^ residual, V^ residual)
     unsigned long long* sel_cand; unsigned int* sel_hist;
-    sgc::Cand* corr_cand;       // [2][kCorrBlocks][kCorrTop]
+    float4* corr_cand;          // [2][kCorrBlocks]
     uint16_t* zsel;             // [2][s][k] selected columns of Z as binary16 bits (chunk path only)
     uint32_t* lam;              // [2][s]
     double* q_basis;            // [2][s][k] orthogonal basis of the picked columns
@@ -299,6 +300,7 @@ struct sgc_state {
     uint32_t* kept_ring;         // [hist_slots][s] kept indices of the last steps (all of them are columns M^ and V^ are made of)
     int hist_slots;
     sgc::ChunkWs* chunk_ws;     // batched chunk path: workspace built for the chunk list that starts with this state
+    int lock_steps;             // host: lock-step steps since the last speculating one (states that have speculated)
     bool two_level;             // host: wide lists and list passes are in use (steps that need several full passes)
     float* wide_tau;            // [kPassMaxN] thresholds of the wide lists, +inf for residuals that do not feed them
     int wide_every;             // every so many screened residuals of a stream feed its wide list
@@ -339,6 +341,7 @@ struct PhaseTimer {
 // launchers (each returns the cudaError_t of its launches); defined in the .cu files
 cudaError_t launch_select(sgc_state* st, const float* grad, cudaStream_t stream, int* launches);
 cudaError_t launch_project_adam(sgc_state* st, cudaStream_t stream, int* launches);
+bool will_speculate(const sgc_state* st);       // the next step of this state speculates, its buffers permitting
 cudaError_t launch_recover(sgc_state* st, float* weight, cudaStream_t stream, int* launches);
 cudaError_t launch_reproject(sgc_state* st, uint64_t new_seed, cudaStream_t stream);
 cudaError_t launch_recover_group(sgc_state* const* sts, float* const* weights, int n, cudaStream_t stream, int* launches);

@@ -29,40 +29,33 @@ namespace {
 
 constexpr int kT = 512;                               // threads per block of k_omp
 constexpr int kWarps = kT / 32;
-constexpr size_t kOmpDynBytes = 204 * 1024;           // dynamic shared memory of every launch (one block per SM)
+constexpr size_t kOmpDynBytes = 196 * 1024;           // dynamic shared memory of every launch (one block per SM)
 constexpr int kRescanCap = 64;
 constexpr double kOmpOneWork = 1.2e6;                  // k * d up to which one cluster of 16 serves the lock-step recovery
 constexpr double kOmpPairWork = 2.0e8;                 // k * d from which pairs do
 constexpr double kPivot = 1e-10;                      // a new column whose orthogonal part is below this share is dependent
 
-// the best two columns seen, and the largest score among all others (what is dropped: the caller can tell whether a
-// dropped column could still have mattered)
-struct Top2 {
-    float s1, s2, s3; uint32_t i1, i2;
-    __device__ __forceinline__ void init() { s1 = s2 = s3 = -1.0f; i1 = i2 = kNoColumn; }
+// the best column seen (lowest index on ties), and the largest score among all others (what is dropped: the caller can tell
+// whether a dropped column could still have mattered)
+struct Top {
+    float s1, s2; uint32_t i1;
+    __device__ __forceinline__ void init() { s1 = s2 = -1.0f; i1 = kNoColumn; }
     __device__ __forceinline__ void push(float s, uint32_t i) {
-        if (better(s, i, s1, i1)) { s3 = fmaxf(s3, s2); s2 = s1; i2 = i1; s1 = s; i1 = i; }
-        else if (better(s, i, s2, i2)) { s3 = fmaxf(s3, s2); s2 = s; i2 = i; }
-        else s3 = fmaxf(s3, s);
+        if (better(s, i, s1, i1)) { s2 = s1; s1 = s; i1 = i; }
+        else s2 = fmaxf(s2, s);
     }
 };
 
 __device__ __forceinline__ unsigned int score_key(float s) { return s >= 0.0f ? __float_as_uint(s) + 1u : 0u; }
 __device__ __forceinline__ float key_score(unsigned int k) { return k ? __uint_as_float(k - 1u) : -1.0f; }
 
-// best two and third-best score over the lanes of a warp (every lane returns the result); columns of different lanes differ
-__device__ __forceinline__ void warp_merge(Top2& t) {
-    Top2 r;
-    r.init();
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-        const unsigned int best = __reduce_max_sync(0xffffffffu, score_key(t.s1));
-        const uint32_t idx = __reduce_min_sync(0xffffffffu, (best != 0u && score_key(t.s1) == best) ? t.i1 : kNoColumn);
-        if (u == 0) { r.s1 = key_score(best); r.i1 = idx; } else { r.s2 = key_score(best); r.i2 = idx; }
-        if (best != 0u && t.i1 == idx && score_key(t.s1) == best) { t.s1 = t.s2; t.i1 = t.i2; t.s2 = t.s3; t.s3 = -1.0f; t.i2 = kNoColumn; }
-    }
-    r.s3 = key_score(__reduce_max_sync(0xffffffffu, score_key(t.s1)));
-    t = r;
+// best column and second-best score over the lanes of a warp (every lane returns the result); columns of different lanes differ
+__device__ __forceinline__ void warp_merge(Top& t) {
+    const unsigned int mine = score_key(t.s1), best = __reduce_max_sync(0xffffffffu, mine);
+    const uint32_t idx = __reduce_min_sync(0xffffffffu, (best != 0u && mine == best) ? t.i1 : kNoColumn);
+    const bool holder = best != 0u && mine == best && t.i1 == idx;
+    const unsigned int second = __reduce_max_sync(0xffffffffu, holder ? score_key(t.s2) : mine);
+    t.s1 = key_score(best); t.i1 = idx; t.s2 = key_score(second);
 }
 
 __device__ __forceinline__ bool in_list(const uint32_t* lam, int n, uint32_t col) {
@@ -74,13 +67,12 @@ __device__ __forceinline__ bool in_list(const uint32_t* lam, int n, uint32_t col
 struct OmpSmem {
     unsigned int wkey[kWarps], wkey2[kWarps];
     float npart[64][16];
-    int wcnt[kWarps];
     double wsum[kWarps];
-    Top2 wtop[2][kWarps];
-    uint32_t cidx[kRescoreCap]; float csc[kRescoreCap];
+    Top wtop[2][kWarps];
+    uint32_t cidx[kRescoreCap];
     uint32_t rbuf[kRescanCap];
-    int rescan_blk[8];
-    int nc, rescan_n, rbuf_n;
+    int rescan_blk[8]; uint32_t rescan_col[8];
+    int nc, peer_nc, rescan_n, rbuf_n;
     __align__(16) uint32_t sup[2][kMaxS];
 };
 
@@ -95,7 +87,7 @@ struct OmpSmem {
 // anyway.  A tile's rows are split over several warps when the block has fewer tiles than warps.  When the generated entries
 // of the block's columns fit its shared memory they are kept from the first iteration on, as operand registers: an iteration
 // then reads 16 bytes per lane and 16 rows instead of regenerating them.  The norms are summed in the first iteration.
-struct CorrPlan { int e0, cnt, tiles, ks, kblocks; bool cached, norms; size_t part_off, inv_off, z_off; };
+struct CorrPlan { int e0, cnt, tiles, ks, kblocks; bool cached, norms; size_t part_off, inv_off, col_off, z_off; };
 
 __host__ __device__ inline size_t frag_bytes(int k) { return (size_t)((k + 15) / 16) * 128; }
 
@@ -118,8 +110,9 @@ __device__ CorrPlan corr_plan(const OmpArgs& a, unsigned int n, int blk, int nbl
     // word offsets in the correlation's part of shared memory: partial sums of split tiles, norms, generated entries
     c.part_off = 0;
     c.inv_off = best > 1 ? (size_t)tiles * best * 32 : 0;
-    c.norms = c.inv_off + (size_t)tiles * 16 <= (size_t)a.z_words;
-    c.z_off = (c.inv_off + (c.norms ? (size_t)tiles * 16 : 0) + 3) & ~(size_t)3;
+    c.norms = c.inv_off + (size_t)tiles * 32 <= (size_t)a.z_words;      // norms, and the columns themselves (lists)
+    c.col_off = c.inv_off + (size_t)tiles * 16;
+    c.z_off = (c.inv_off + (c.norms ? (size_t)tiles * 32 : 0) + 3) & ~(size_t)3;
     c.cached = c.norms && c.z_off + (size_t)tiles * c.kblocks * 128 <= (size_t)a.z_words;
     return c;
 }
@@ -134,9 +127,9 @@ __device__ __forceinline__ bool in_support4(const uint32_t* sup, int n, uint32_t
     return hit;
 }
 
-// (a column of the support scores rounding noise: the look-up is needed only for what would enter the best three)
-__device__ __forceinline__ void offer(const OmpSmem& sh, Top2& best, const int* picks, int m, float score, uint32_t col) {
-    if (score > best.s3 && !in_support4(sh.sup[m], picks[m], col)) best.push(score, col);
+// (a column of the support scores rounding noise: the look-up is needed only for what would enter the best two)
+__device__ __forceinline__ void offer(const OmpSmem& sh, Top& best, const int* picks, int m, float score, uint32_t col) {
+    if (score > best.s2 && !in_support4(sh.sup[m], picks[m], col)) best.push(score, col);
 }
 
 __device__ __forceinline__ void mma_16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
@@ -152,13 +145,34 @@ __device__ __forceinline__ uint32_t pack_half(float lo, float hi) {
 // The residuals as B operands: for each 16 rows, lane (g, t) with g < 4 holds rows 2t, 2t + 1 and 2t + 8, 2t + 9 of column g: 0 and
 // 1 value and remainder of the M^ residual, 2 and 3 of V^'s.  Each residual is scaled by a power of two (largest entry in
 // [2^10, 2^11)); a score is homogeneous in it, and back[m] undoes it.
-__device__ void stage_residuals(const OmpArgs& a, OmpSmem& sh, uint2* frag, float* back) {
+__device__ void stage_residuals(const OmpArgs& a, OmpSmem& sh, uint2* frag, float* back, const int* picks) {
+    constexpr int kHold = 4;                                          // row pairs per thread fetched once (k <= 4096)
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5, k = a.k;
-    const float2* r = reinterpret_cast<const float2*>(a.r32);
+    const float4* r = reinterpret_cast<const float4*>(a.r32);         // (padded by two rows: a pair may be read whole)
+    const int items = (k + 15) / 16 * 8;                              // row pairs: (16-row block, which half, t)
+    auto fetch = [&](int it) -> float4 {
+        const int pair = (it >> 3) * 8 + (it & 1) * 4 + ((it >> 1) & 3);
+        float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (2 * pair < k) v = __ldcg(r + pair);
+        if (2 * pair + 1 >= k) v.z = v.w = 0.0f;
+        return v;
+    };
+    float4 v[kHold];
+#pragma unroll
+    for (int u = 0; u < kHold; ++u) v[u] = t + u * kT < items ? fetch(t + u * kT) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    const uint32_t l0 = t < picks[0] ? __ldcg(a.lam + t) : kNoColumn, l1 = t < picks[1] ? __ldcg(a.lam + a.s + t) : kNoColumn;
     unsigned int m0 = 0u, m1 = 0u;
-    for (int row = t; row < k; row += kT) {
-        const float2 v = __ldcg(r + row);
-        m0 = max(m0, __float_as_uint(v.x) & 0x7FFFFFFFu); m1 = max(m1, __float_as_uint(v.y) & 0x7FFFFFFFu);
+    auto widest = [&](const float4& f) {
+        m0 = max(m0, max(__float_as_uint(f.x) & 0x7FFFFFFFu, __float_as_uint(f.z) & 0x7FFFFFFFu));
+        m1 = max(m1, max(__float_as_uint(f.y) & 0x7FFFFFFFu, __float_as_uint(f.w) & 0x7FFFFFFFu));
+    };
+#pragma unroll
+    for (int u = 0; u < kHold; ++u) widest(v[u]);
+    for (int it = t + kHold * kT; it < items; it += kT) widest(fetch(it));
+    sh.sup[0][t] = l0; sh.sup[1][t] = l1;
+    for (int e = kT + t; e < kMaxS; e += kT) {
+        if (e < ((picks[0] + 3) & ~3)) sh.sup[0][e] = e < picks[0] ? __ldcg(a.lam + e) : kNoColumn;
+        if (e < ((picks[1] + 3) & ~3)) sh.sup[1][e] = e < picks[1] ? __ldcg(a.lam + a.s + e) : kNoColumn;
     }
     m0 = __reduce_max_sync(0xffffffffu, m0); m1 = __reduce_max_sync(0xffffffffu, m1);
     if (lane == 0) { sh.wkey[warp] = m0; sh.wkey2[warp] = m1; }
@@ -170,14 +184,9 @@ __device__ void stage_residuals(const OmpArgs& a, OmpSmem& sh, uint2* frag, floa
     e0 = e0 < 20 ? 20 : (e0 > 250 ? 250 : e0); e1 = e1 < 20 ? 20 : (e1 > 250 ? 250 : e1);
     const float s0 = __uint_as_float((unsigned int)(264 - e0) << 23), s1 = __uint_as_float((unsigned int)(264 - e1) << 23);
     back[0] = __uint_as_float((unsigned int)(e0 - 10) << 23); back[1] = __uint_as_float((unsigned int)(e1 - 10) << 23);
-    const int items = (k + 15) / 16 * 8;                              // (16-row block, t): two row pairs of both residuals
-    for (int it = t; it < items; it += kT) {
+    auto put = [&](int it, const float4& f) {
         const int kb = it >> 3, q = (it >> 1) & 3, which = it & 1;    // which: rows 2q.. or 2q + 8..
-        const int row = kb * 16 + 2 * q + 8 * which;
-        float2 v0 = make_float2(0.0f, 0.0f), v1 = v0;
-        if (row < k) v0 = __ldcg(r + row);
-        if (row + 1 < k) v1 = __ldcg(r + row + 1);
-        const float a0 = v0.x * s0, a1 = v1.x * s0, b0 = v0.y * s1, b1 = v1.y * s1;
+        const float a0 = f.x * s0, a1 = f.z * s0, b0 = f.y * s1, b1 = f.w * s1;
         const uint32_t ah = pack_half(a0, a1), bh = pack_half(b0, b1);
         const float2 af = half2_bits_to_float2(ah), bf = half2_bits_to_float2(bh);
         uint32_t* w = reinterpret_cast<uint32_t*>(frag + (size_t)kb * 16) + which;
@@ -185,23 +194,24 @@ __device__ void stage_residuals(const OmpArgs& a, OmpSmem& sh, uint2* frag, floa
         w[2 * (1 * 4 + q)] = pack_half(a0 - af.x, a1 - af.y);
         w[2 * (2 * 4 + q)] = bh;
         w[2 * (3 * 4 + q)] = pack_half(b0 - bf.x, b1 - bf.y);
-    }
+    };
+#pragma unroll
+    for (int u = 0; u < kHold; ++u) if (t + u * kT < items) put(t + u * kT, v[u]);
+    for (int it = t + kHold * kT; it < items; it += kT) put(it, fetch(it));
 }
 
 __device__ void correlate(const OmpArgs& a, OmpSmem& sh, const CorrPlan& c, const uint32_t* col_list, uint2* frag, float* mem,
                           bool filled, const int* picks, int blk, int nblk) {
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5, g = lane >> 2, q = lane & 3;
-#pragma unroll
-    for (int m = 0; m < 2; ++m)
-        for (int e = t; e < ((picks[m] + 3) & ~3); e += kT) sh.sup[m][e] = e < picks[m] ? __ldcg(a.lam + (size_t)m * a.s + e) : kNoColumn;
     float back[2];
-    stage_residuals(a, sh, frag, back);
+    stage_residuals(a, sh, frag, back, picks);
     __syncthreads();
     float* part = mem + c.part_off;
     float* inv_s = mem + c.inv_off;
+    uint32_t* col_s = reinterpret_cast<uint32_t*>(mem + c.col_off);
     uint4* zc = reinterpret_cast<uint4*>(mem + c.z_off);
     const bool have = filled && c.norms, read = filled && c.cached;
-    Top2 best;                                                        // of residual q & 1
+    Top best;                                                         // of residual q & 1
     best.init();
     const int units = c.tiles * c.ks, kper = (c.kblocks + c.ks - 1) / c.ks;
     for (int u = warp; u < units; u += kWarps) {
@@ -212,8 +222,9 @@ __device__ void correlate(const OmpArgs& a, OmpSmem& sh, const CorrPlan& c, cons
         float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
         float n0 = 0.0f, n1 = 0.0f;
         uint32_t col0 = kNoColumn, col1 = kNoColumn;
-        if (ok0) col0 = col_list ? col_list[c.e0 + i0] : (uint32_t)(c.e0 + i0);
-        if (ok1) col1 = col_list ? col_list[c.e0 + i1] : (uint32_t)(c.e0 + i1);
+        if (ok0) col0 = col_list ? (have ? col_s[i0] : col_list[c.e0 + i0]) : (uint32_t)(c.e0 + i0);
+        if (ok1) col1 = col_list ? (have ? col_s[i1] : col_list[c.e0 + i1]) : (uint32_t)(c.e0 + i1);
+        if (c.norms && !have && part_k == 0 && q == 0) { col_s[i0] = col0; col_s[i1] = col1; }
         const uint2* fb = frag + lane;
         uint4* zt = zc + (size_t)tile * c.kblocks * 32 + lane;
         if (read) {
@@ -299,13 +310,13 @@ __device__ void correlate(const OmpArgs& a, OmpSmem& sh, const CorrPlan& c, cons
             else { inv = n2 > 0.0f ? 1.0f / n2 : 0.0f; if (c.norms && m == 0) inv_s[idx] = inv; }
             if (idx < c.cnt) {
                 const float f = d * (m == 0 ? back[0] : back[1]);
-                offer(sh, best, picks, m, f * f * inv, col_list ? col_list[c.e0 + idx] : (uint32_t)(c.e0 + idx));
+                offer(sh, best, picks, m, f * f * inv, col_list ? (c.norms ? col_s[idx] : col_list[c.e0 + idx]) : (uint32_t)(c.e0 + idx));
             }
         }
         // (kT is even: a thread has met one residual only, that of its own parity)
     }
     const int mine = c.ks > 1 ? (t & 1) : (q < 2 ? q : -1);
-    Top2 none, m0 = best, m1 = best;
+    Top none, m0 = best, m1 = best;
     none.init();
     if (mine != 0) m0 = none;
     if (mine != 1) m1 = none;
@@ -314,14 +325,12 @@ __device__ void correlate(const OmpArgs& a, OmpSmem& sh, const CorrPlan& c, cons
     if (lane == 0) { sh.wtop[0][warp] = m0; sh.wtop[1][warp] = m1; }
     __syncthreads();
     if (warp < 2) {
-        Top2 m = none;
+        Top m = none;
         if (lane < kWarps) m = sh.wtop[warp][lane];
         warp_merge(m);
         if (lane == 0) {
-            Cand* o = a.corr_cand + ((size_t)warp * nblk + blk) * kCorrTop;
-            o[0].score = m.s1; o[0].idx = m.i1;
-            o[1].score = m.s2; o[1].idx = m.i2;
-            o[2].score = m.s3; o[2].idx = kNoColumn;        // score of the best column this block did not forward
+            // best column, its score, and the best score that this block did not forward
+            a.corr_cand[(size_t)warp * nblk + blk] = make_float4(m.s1, __uint_as_float(m.i1), m.s2, 0.0f);
         }
     }
 }
@@ -334,14 +343,17 @@ template <int CL> struct Group { static constexpr int GS = CL == 16 ? 8 : CL; };
 // row slices: an even number of rows per block (a generated word holds two rows)
 __host__ __device__ inline int slice_rows(int k, int gs) { return 2 * ((k + 2 * gs - 1) / (2 * gs)); }
 
-// dynamic shared memory of a bookkeeping block, in doubles, after the residual pairs of the correlation
+// dynamic shared memory of a bookkeeping block, in doubles: residual slice | partial sums | exchanged sums | exchange slots | q
 struct BookMem {
-    double *an, *rr, *alt, *cs, *x0, *x1, *xrn, *qs;
+    double *rr, *part, *cs, *x0, *x1, *xrn, *qs;
     int R, P, row0, rows;                                  // slice length, parts per row in the update, first row, rows owned
 };
+__host__ __device__ inline int even(int n) { return (n + 1) & ~1; }
+// a slot of the exchange: products with q_l and the residual (by l), then ||a||^2, ||r||^2, and two values per further candidate
+__host__ __device__ inline int exchange_stride(int s) { return even(s + 2 + 2 * kRescoreCap); }
 __host__ __device__ inline size_t book_doubles(int k, int s, int gs, bool two) {
     const int R = slice_rows(k, gs);
-    return (size_t)2 * R + (R > kT ? R : kT) + (s + 2) + (size_t)(two ? 2 : 1) * gs * (s + 2 + 2 * kRescoreCap) + 2 * gs;
+    return (size_t)R + (R > kT ? R : kT) + even(s + 4) + (size_t)(two ? 2 : 1) * gs * exchange_stride(s) + 2 * gs;
 }
 
 __device__ BookMem book_mem(const OmpArgs& a, double* base, int gs, int g, bool two) {
@@ -350,81 +362,143 @@ __device__ BookMem book_mem(const OmpArgs& a, double* base, int gs, int g, bool 
     b.row0 = g * b.R;
     b.rows = b.row0 >= a.k ? 0 : (a.k - b.row0 < b.R ? a.k - b.row0 : b.R);
     b.P = b.R >= kT ? 1 : kT / b.R;
-    b.an = base; b.rr = b.an + b.R; b.alt = b.rr + b.R;
-    b.cs = b.alt + (b.R > kT ? b.R : kT);
-    b.x0 = b.cs + (a.s + 2);
-    b.x1 = two ? b.x0 + (size_t)gs * (a.s + 2 + 2 * kRescoreCap) : b.x0;
-    b.xrn = b.x1 + (size_t)gs * (a.s + 2 + 2 * kRescoreCap);
+    b.rr = base; b.part = b.rr + b.R;
+    b.cs = b.part + (b.R > kT ? b.R : kT);
+    b.x0 = b.cs + even(a.s + 4);
+    b.x1 = two ? b.x0 + (size_t)gs * exchange_stride(a.s) : b.x0;
+    b.xrn = b.x1 + (size_t)gs * exchange_stride(a.s);
     b.qs = b.xrn + 2 * gs;
     return b;
 }
 
-// rows of one column in this slice, scaled by sigma (rows beyond k are zero)
-__device__ __forceinline__ void make_column(const OmpArgs& a, const BookMem& b, uint32_t col, double* out) {
-    const ColKey key = column_key(a.seed_lo, a.seed_hi, col);
-    for (int p = threadIdx.x; p < b.R / 2; p += kT) {
-        const int row = b.row0 + 2 * p;
-        const float2 z = half2_bits_to_float2(z_pair_from_word(key.ck + (uint32_t)(row >> 1) * key.mk));
-        out[2 * p] = row < a.k ? a.sigma * (double)z.x : 0.0;
-        out[2 * p + 1] = row + 1 < a.k ? a.sigma * (double)z.y : 0.0;
-    }
+// rows 2 p, 2 p + 1 of a column in this slice, scaled by sigma (rows beyond k are zero)
+__device__ __forceinline__ double2 column_rows(const OmpArgs& a, const BookMem& b, const ColKey& key, int p) {
+    const int row = b.row0 + 2 * p;
+    const float2 z = half2_bits_to_float2(z_pair_from_word(key.ck + (uint32_t)(row >> 1) * key.mk));
+    return make_double2(row < a.k ? a.sigma * (double)z.x : 0.0, row + 1 < a.k ? a.sigma * (double)z.y : 0.0);
 }
 
-// vector l of the products with a new column: q_l (l < j), then the residual, then the column itself
-__device__ __forceinline__ const double* dot_vector(const OmpArgs& a, const BookMem& b, int m, int j, int l, const double* an) {
-    if (l == j) return b.rr;
-    if (l == j + 1) return an;
+// q_l of this slice: in shared memory for the first q_cols, in global memory beyond
+__device__ __forceinline__ const double* q_slice(const OmpArgs& a, const BookMem& b, int m, int l) {
     return l < a.q_cols ? b.qs + (size_t)l * b.R : a.q + ((size_t)m * a.s + l) * a.k + b.row0;
 }
 
-// partial products of `an` with the vectors lo .. hi of dot_vector over this slice, sent to slot g of the exchange buffer of
-// every block of the group: warp = four vectors at a time
+template <int N>
+__device__ __forceinline__ void warp_sums(double (&v)[N]) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+        for (int u = 0; u < N; ++u) v[u] += __shfl_xor_sync(0xffffffffu, v[u], o);
+    }
+}
+
+constexpr int kLanePairs = 4;                              // row pairs of a column that a lane generates at a time (256 rows per warp)
+
+// Partial products of column `col` over this slice with q_0 .. q_(j-1) and the residual, and (full) its squared norm and the
+// residual's, sent to slot g of the exchange buffer of every block of the group.  Warp = four vectors at a time; every warp
+// generates the slice of the column for itself (a few words per lane), which saves a barrier.
 template <int GS>
-__device__ void send_products(cg::cluster_group& cluster, const OmpArgs& a, const BookMem& b, int m, int j, int lo, int hi,
-                              const double* an, double* xbuf, int xstride, int off, int rank0, int g) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int l0 = lo + warp; l0 < hi; l0 += 4 * kWarps) {
+__device__ void send_products(cg::cluster_group& cluster, const OmpArgs& a, const BookMem& b, int m, int j, uint32_t col, bool full,
+                              double* xbuf, int rank0, int g) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, pairs = b.R / 2, xstride = exchange_stride(a.s);
+    const ColKey key = column_key(a.seed_lo, a.seed_hi, col);
+    const bool vec = (a.k & 1) == 0 || j <= a.q_cols;
+    for (int l0 = warp; l0 <= j; l0 += 4 * kWarps) {
         double acc[4] = {0.0, 0.0, 0.0, 0.0};
         const double* v[4];
+        bool live[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) { const int l = l0 + u * kWarps; v[u] = dot_vector(a, b, m, j, l < hi ? l : l0, an); }
-        for (int r = lane; r < b.rows; r += 32) {
-            const double x = an[r];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) acc[u] = fma(v[u][r], x, acc[u]);
+        for (int u = 0; u < 4; ++u) {
+            const int l = l0 + u * kWarps;
+            live[u] = l <= j;
+            v[u] = l < j ? q_slice(a, b, m, l) : b.rr;
         }
+        for (int p0 = lane; p0 < pairs; p0 += 32 * kLanePairs) {
+            double2 x[kLanePairs];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
+            for (int i = 0; i < kLanePairs; ++i) x[i] = p0 + 32 * i < pairs ? column_rows(a, b, key, p0 + 32 * i) : make_double2(0.0, 0.0);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], o);
+            for (int u = 0; u < 4; ++u) {
+                if (!live[u]) continue;
+#pragma unroll
+                for (int i = 0; i < kLanePairs; ++i) {
+                    const int r = 2 * (p0 + 32 * i);
+                    if (r >= b.rows) continue;
+                    if (vec) {
+                        const double2 y = *reinterpret_cast<const double2*>(v[u] + r);       // (an odd last row: shared memory, zero beyond)
+                        acc[u] = fma(y.x, x[i].x, acc[u]); acc[u] = fma(y.y, x[i].y, acc[u]);
+                    } else {
+                        acc[u] = fma(v[u][r], x[i].x, acc[u]);
+                        if (r + 1 < b.rows) acc[u] = fma(v[u][r + 1], x[i].y, acc[u]);
+                    }
+                }
+            }
         }
+        warp_sums(acc);
         if (lane < GS) {
             double* dst = cluster.map_shared_rank(xbuf, rank0 + lane) + (size_t)g * xstride;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) { const int l = l0 + u * kWarps; if (l < hi) dst[l - lo + off] = acc[u]; }
+            for (int u = 0; u < 4; ++u) if (live[u]) dst[l0 + u * kWarps] = acc[u];
+        }
+    }
+    if (full && warp == kWarps - 1) {
+        double acc[2] = {0.0, 0.0};
+        for (int p = lane; p < pairs; p += 32) {
+            const double2 x = column_rows(a, b, key, p), y = *reinterpret_cast<const double2*>(b.rr + 2 * p);
+            acc[0] = fma(x.x, x.x, acc[0]); acc[0] = fma(x.y, x.y, acc[0]);
+            acc[1] = fma(y.x, y.x, acc[1]); acc[1] = fma(y.y, y.y, acc[1]);
+        }
+        warp_sums(acc);
+        if (lane < GS) {
+            double* dst = cluster.map_shared_rank(xbuf, rank0 + lane) + (size_t)g * xstride;
+            dst[a.s] = acc[0]; dst[a.s + 1] = acc[1];
         }
     }
 }
 
-// sum of two block-wide partial values, sent to slot g of xrn of every block of the group
+// a further candidate: its product with the residual and its squared norm (warp = one candidate)
 template <int GS>
-__device__ void send_norm(cg::cluster_group& cluster, OmpSmem& sh, const BookMem& b, double v, int rank0, int g) {
-    v = warp_sum(v);
-    if ((threadIdx.x & 31) == 0) sh.wsum[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x < GS) {
-        double s = 0.0;
-        for (int w = 0; w < kWarps; ++w) s += sh.wsum[w];
-        cluster.map_shared_rank(b.xrn, rank0 + threadIdx.x)[g] = s;
+__device__ void send_candidate(cg::cluster_group& cluster, const OmpArgs& a, const BookMem& b, uint32_t col, int e, double* xbuf, int rank0, int g) {
+    const int lane = threadIdx.x & 31, pairs = b.R / 2;
+    const ColKey key = column_key(a.seed_lo, a.seed_hi, col);
+    double acc[2] = {0.0, 0.0};
+    for (int p = lane; p < pairs; p += 32) {
+        const double2 x = column_rows(a, b, key, p), y = *reinterpret_cast<const double2*>(b.rr + 2 * p);
+        acc[0] = fma(x.x, y.x, acc[0]); acc[0] = fma(x.y, y.y, acc[0]);
+        acc[1] = fma(x.x, x.x, acc[1]); acc[1] = fma(x.y, x.y, acc[1]);
+    }
+    warp_sums(acc);
+    if (lane < GS) {
+        double* dst = cluster.map_shared_rank(xbuf, rank0 + lane) + (size_t)g * exchange_stride(a.s) + a.s + 2 + 2 * (e - 1);
+        dst[0] = acc[0]; dst[1] = acc[1];
     }
 }
 
-// Lock-step only.  Block `blk` of the screen forwarded its best two columns for residual m, but a third scored inside the
+// squared norm of the residual slice, sent to slot g of xrn of every block of the group (one warp)
+template <int GS>
+__device__ void send_norm(cg::cluster_group& cluster, const BookMem& b, int rank0, int g) {
+    if (threadIdx.x >= 32) return;
+    double acc[1] = {0.0};
+    for (int r = threadIdx.x; r < b.R; r += 32) acc[0] = fma(b.rr[r], b.rr[r], acc[0]);
+    warp_sums(acc);
+    if (threadIdx.x < GS) cluster.map_shared_rank(b.xrn, rank0 + threadIdx.x)[g] = acc[0];
+}
+
+// the residual of this slice as row n of the screened batch (scaled binary16, and fp64 for the resolve kernel)
+__device__ void emit_row(const OmpArgs& a, const BookMem& b, size_t n, double rn, int g) {
+    const double sc = residual_scale(rn);
+    for (int r = threadIdx.x; r < b.rows; r += kT) {
+        a.rt[n * a.kp + b.row0 + r] = half_rn_bits(b.rr[r] * sc);
+        a.rhist[n * a.k + b.row0 + r] = b.rr[r];
+    }
+    if (g == 0 && threadIdx.x == 0) a.inv_scale[n] = (float)(1.0 / sc);
+}
+
+// Lock-step only.  Block `blk` of the screen forwarded its best column for residual m, but another scored inside the
 // rescoring window as well.  Its columns are screened again here and every free one inside the window (with a little slack:
 // the sums run in another order) that was not forwarded is noted, so that all of them reach the fp64 decision.
-__device__ void rescan_block(const OmpArgs& a, OmpSmem& sh, int m, int j, int blk, int nblk, float thr, const Cand* fwd) {
+__device__ void rescan_block(const OmpArgs& a, OmpSmem& sh, int m, int j, int blk, int nblk, float thr, uint32_t forwarded) {
     const CorrPlan c = corr_plan(a, (unsigned int)a.d, blk, nblk);
-    const uint32_t f0 = fwd[0].idx, f1 = fwd[1].idx;
     const float2* r = reinterpret_cast<const float2*>(a.r32);
     for (int idx = threadIdx.x; idx < c.cnt; idx += kT) {
         const uint32_t col = (uint32_t)(c.e0 + idx);
@@ -439,7 +513,7 @@ __device__ void rescan_block(const OmpArgs& a, OmpSmem& sh, int m, int j, int bl
             if (row + 1 < a.k) { acc = __fmaf_rn(z.y, m ? r1.y : r1.x, acc); n2 = __fmaf_rn(z.y, z.y, n2); }
         }
         const float sc = n2 > 0.0f ? acc * acc / n2 : 0.0f;
-        if (sc >= thr * 0.9999f && col != f0 && col != f1 && !in_list(a.lam + (size_t)m * a.s, j, col)) {
+        if (sc >= thr * 0.9999f && col != forwarded && !in_list(a.lam + (size_t)m * a.s, j, col)) {
             const int slot = atomicAdd(&sh.rbuf_n, 1);
             if (slot < kRescanCap) sh.rbuf[slot] = col;
         }
@@ -448,64 +522,80 @@ __device__ void rescan_block(const OmpArgs& a, OmpSmem& sh, int m, int j, int bl
 }
 
 // The screened candidates of pick j: everything within 2e-3 (relative, squared scores) of the best fp32 score, the best one
-// first; every block of a group finds the same list.  Returns their number; *inexact: a column inside the window was not
-// forwarded (list mode only: the screening pass judges it).
-__device__ int gather_candidates(const OmpArgs& a, OmpSmem& sh, int m, int j, int nblk, bool lock, bool* inexact) {
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const Cand* cc = a.corr_cand + (size_t)m * nblk * kCorrTop;
-    Cand c[3];
-    c[0].score = c[1].score = c[2].score = -1.0f; c[0].idx = c[1].idx = c[2].idx = kNoColumn;
-    if (t < nblk) {
+// first; every block of a group finds the same list.  Returns their number; *first: the best one (a list of more than one is in
+// sh.cidx); *inexact: a column inside the window was not forwarded (list mode only: the screening pass judges it).  Every warp
+// reads all blocks' entries: the usual case of one candidate needs no barrier.
+__device__ int gather_candidates(const OmpArgs& a, OmpSmem& sh, int m, int j, int nblk, bool lock, uint32_t* first, bool* inexact) {
+    constexpr int kPer = kCorrBlocks / 32;
+    const int t = threadIdx.x, lane = t & 31;
+    const float4* cc = a.corr_cand + (size_t)m * nblk;
+    float4 c[kPer];
 #pragma unroll
-        for (int u = 0; u < 3; ++u) {
-            const float2 f = __ldcg(reinterpret_cast<const float2*>(cc + (size_t)t * kCorrTop + u));
-            c[u].score = f.x; c[u].idx = __float_as_uint(f.y);
-        }
+    for (int u = 0; u < kPer; ++u) {
+        const int e = u * 32 + lane;
+        c[u] = e < nblk ? __ldcg(cc + e) : make_float4(-1.0f, __uint_as_float(kNoColumn), -1.0f, 0.0f);
     }
-    unsigned int key = __reduce_max_sync(0xffffffffu, c[0].idx != kNoColumn ? score_key(c[0].score) : 0u);
-    if (t == 0) { sh.rescan_n = 0; sh.rbuf_n = 0; }
-    if (lane == 0) sh.wkey[warp] = key;
-    __syncthreads();
-    key = __reduce_max_sync(0xffffffffu, lane < kWarps ? sh.wkey[lane] : 0u);
+    unsigned int key = 0u;
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) if (__float_as_uint(c[u].y) != kNoColumn) key = max(key, score_key(c[u].x));
+    key = __reduce_max_sync(0xffffffffu, key);
     if (key == 0u) return 0;
     const float mx = key_score(key);
     const float thr = mx - 2e-3f * fabsf(mx);
-    const bool f0 = c[0].idx != kNoColumn && c[0].score >= thr, f1 = c[1].idx != kNoColumn && c[1].score >= thr;
-    const bool f2 = c[2].score >= 0.0f && c[2].score >= thr;
-    const unsigned int b0 = __ballot_sync(0xffffffffu, f0), b1 = __ballot_sync(0xffffffffu, f1);
-    if (lane == 0) sh.wcnt[warp] = __popc(b0) + __popc(b1);
-    const bool any2 = __syncthreads_or(f2 ? 1 : 0) != 0;
-    int slot = 0, total = 0;
+    int total = 0;
+    bool kept = false;
+    uint32_t best = kNoColumn;
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) { const int n = sh.wcnt[w]; if (w < warp) slot += n; total += n; }
-    const unsigned int below = (1u << lane) - 1u;
-    slot += __popc(b0 & below) + __popc(b1 & below);
-    if (f0 && slot < kRescoreCap) { sh.cidx[slot] = c[0].idx; sh.csc[slot] = c[0].score; }
-    if (f0) ++slot;
-    if (f1 && slot < kRescoreCap) { sh.cidx[slot] = c[1].idx; sh.csc[slot] = c[1].score; }
-    if (any2) {
-        if (!lock) *inexact = true;
-        else {
-            if (f2) { const int q = atomicAdd(&sh.rescan_n, 1); if (q < 8) sh.rescan_blk[q] = t; }
-            __syncthreads();
-            const int n_blk = sh.rescan_n < 8 ? sh.rescan_n : 8;
-            for (int q = 0; q < n_blk; ++q)
-                rescan_block(a, sh, m, j, sh.rescan_blk[q], nblk, thr, cc + (size_t)sh.rescan_blk[q] * kCorrTop);
-            const bool over = sh.rescan_n > 8 || sh.rbuf_n > kRescanCap || total + sh.rbuf_n > kRescoreCap;
-            if (t == 0) {
-                if (over) atomicOr(&a.cnt->status, (unsigned int)SGC_STATUS_CANDIDATE_OVERFLOW);
-                else {
-                    // ascending order, so that every block of the group has the same list whatever order the atomics gave
-                    for (int e = 0; e < sh.rbuf_n; ++e) {
-                        int lo = e;
-                        for (int q = e + 1; q < sh.rbuf_n; ++q) if (sh.rbuf[q] < sh.rbuf[lo]) lo = q;
-                        const uint32_t v = sh.rbuf[lo]; sh.rbuf[lo] = sh.rbuf[e]; sh.rbuf[e] = v;
-                        sh.cidx[total + e] = v; sh.csc[total + e] = 0.0f;
-                    }
-                }
+    for (int u = 0; u < kPer; ++u) {
+        const bool in = __float_as_uint(c[u].y) != kNoColumn && c[u].x >= thr;
+        total += __popc(__ballot_sync(0xffffffffu, in));
+        if (in && score_key(c[u].x) == key) best = min(best, __float_as_uint(c[u].y));
+        kept = kept || (c[u].z >= 0.0f && c[u].z >= thr);
+    }
+    best = __reduce_min_sync(0xffffffffu, best);
+    kept = __any_sync(0xffffffffu, kept);
+    *first = best;
+    if (kept && !lock) *inexact = true;
+    if (total == 1 && !(kept && lock)) return 1;
+    // several candidates, or columns that a block of the lock-step screen kept to itself
+    __syncthreads();
+    if (t == 0) { sh.nc = 0; sh.rescan_n = 0; sh.rbuf_n = 0; }
+    __syncthreads();
+    if (t < 32) {
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+            const uint32_t idx = __float_as_uint(c[u].y);
+            const bool in = idx != kNoColumn && c[u].x >= thr && idx != best;
+            const unsigned int b = __ballot_sync(0xffffffffu, in);
+            const int slot = 1 + sh.nc + __popc(b & ((1u << lane) - 1u));
+            if (in && slot < kRescoreCap) sh.cidx[slot] = idx;
+            __syncwarp();
+            if (lane == 0) sh.nc += __popc(b);
+            __syncwarp();
+            if (c[u].z >= 0.0f && c[u].z >= thr) {
+                const int q = atomicAdd(&sh.rescan_n, 1);
+                if (q < 8) { sh.rescan_blk[q] = u * 32 + lane; sh.rescan_col[q] = idx; }
             }
-            if (!over) total += sh.rbuf_n;
         }
+        if (lane == 0) sh.cidx[0] = best;
+    }
+    __syncthreads();
+    if (kept && lock) {
+        const int n_blk = sh.rescan_n < 8 ? sh.rescan_n : 8;
+        for (int q = 0; q < n_blk; ++q) rescan_block(a, sh, m, j, sh.rescan_blk[q], nblk, thr, sh.rescan_col[q]);
+        const bool over = sh.rescan_n > 8 || sh.rbuf_n > kRescanCap || total + sh.rbuf_n > kRescoreCap;
+        if (t == 0) {
+            if (over) atomicOr(&a.cnt->status, (unsigned int)SGC_STATUS_CANDIDATE_OVERFLOW);
+            else
+                // ascending order, so that every block of the group has the same list whatever order the atomics gave
+                for (int e = 0; e < sh.rbuf_n; ++e) {
+                    int lo = e;
+                    for (int q = e + 1; q < sh.rbuf_n; ++q) if (sh.rbuf[q] < sh.rbuf[lo]) lo = q;
+                    const uint32_t v = sh.rbuf[lo]; sh.rbuf[lo] = sh.rbuf[e]; sh.rbuf[e] = v;
+                    sh.cidx[total + e] = v;
+                }
+        }
+        if (!over) total += sh.rbuf_n;
     }
     if (total > kRescoreCap) {
         if (t == 0) atomicOr(&a.cnt->status, (unsigned int)SGC_STATUS_CANDIDATE_OVERFLOW);
@@ -513,14 +603,6 @@ __device__ int gather_candidates(const OmpArgs& a, OmpSmem& sh, int m, int j, in
         *inexact = true;
     }
     __syncthreads();
-    if (total > 1) {                                                  // the best fp32 score goes first
-        if (t == 0) {
-            int at = 0;
-            for (int q = 1; q < total; ++q) if (sh.csc[q] > sh.csc[at]) at = q;
-            const uint32_t v = sh.cidx[at]; sh.cidx[at] = sh.cidx[0]; sh.cidx[0] = v;
-        }
-        __syncthreads();
-    }
     return total;
 }
 
@@ -652,17 +734,20 @@ __device__ void gram_picks(const OmpArgs& a, int m, int n, double* dyn) {
     if (ctl->finished[m]) return;
     const double inv_g = my_g > 0.0 ? 1.0 / my_g : 0.0;
     int hi = base, extra = 0, dep = 0;
+    const int nw = (n + 31) >> 5;                                     // the warps that hold members go on by themselves
+    if (warp >= nw) return;
+    auto meet = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(nw * 32) : "memory"); };
     for (int j = 0; j < end; ++j) {
         const int par = j & 1;
         const bool given = j < base;                                  // a confirmed pick (j < v0) or the prescribed one
         if (member) ps[par][t] = p;
         int q;
         if (given) {
-            __syncthreads();
+            meet();
             q = li[j];
         } else {
             // "Select": argmax of p_i^2 / g_ii over the free list members, lowest column index on ties
-            if (warp < 8) {
+            {
                 const double sc = (member && !taken && my_g > 0.0) ? p * p * inv_g : -1.0;
                 const unsigned long long bits = sc >= 0.0 ? (unsigned long long)__double_as_longlong(sc) + 1ull : 0ull;
                 const unsigned int h = __reduce_max_sync(0xffffffffu, (unsigned int)(bits >> 32));
@@ -673,9 +758,9 @@ __device__ void gram_picks(const OmpArgs& a, int m, int n, double* dyn) {
                 const unsigned int who = __ballot_sync(0xffffffffu, e2 && my_col == c);
                 if (lane == 0) { khi[par][warp] = h; klo[par][warp] = l; kcol[par][warp] = c; kidx[par][warp] = who ? warp * 32 + __ffs(who) - 1 : -1; }
             }
-            __syncthreads();
-            const unsigned int h0 = lane < 8 ? khi[par][lane] : 0u, l0 = lane < 8 ? klo[par][lane] : 0u;
-            const uint32_t c0 = lane < 8 ? kcol[par][lane] : kNoColumn;
+            meet();
+            const unsigned int h0 = lane < nw ? khi[par][lane] : 0u, l0 = lane < nw ? klo[par][lane] : 0u;
+            const uint32_t c0 = lane < nw ? kcol[par][lane] : kNoColumn;
             const unsigned int h = __reduce_max_sync(0xffffffffu, h0);
             const unsigned int l = __reduce_max_sync(0xffffffffu, h0 == h ? l0 : 0u);
             const bool e = h0 == h && l0 == l && c0 != kNoColumn;
@@ -724,7 +809,7 @@ __device__ void gram_picks(const OmpArgs& a, int m, int n, double* dyn) {
             p -= aj * w;
             if (t == q) taken = true;
         }
-        for (int l = t; l < j; l += kT) {
+        for (int l = t; l < j; l += nw * 32) {
             const double c = sigma * W[(size_t)l * n + q];
             crow[(size_t)j * s + l] = c; ccol[(size_t)l * s + j] = c;
         }
@@ -963,7 +1048,7 @@ __global__ void __launch_bounds__(kT, 1) k_omp(OmpArgs a, int mode) {
     uint2* frag = reinterpret_cast<uint2*>(dyn_raw);
     const BookMem bk = book_mem(a, reinterpret_cast<double*>(dyn_raw + pb), GS, g, kOneCluster);
     float* corr_mem = reinterpret_cast<float*>(dyn_raw + ((pb + bb + 15) & ~(size_t)15));
-    const int xstride = s + 2 + 2 * kRescoreCap;
+    const int xstride = exchange_stride(s);
     // the first full pass of a step starts the wide lists afresh; later ones add what their residuals bring (the lists then
     // cover the whole path of this step, which is where the next step's path runs, too)
     if (restart_wide) {
@@ -974,10 +1059,10 @@ __global__ void __launch_bounds__(kT, 1) k_omp(OmpArgs a, int mode) {
     // ---- the books at the first pick: r = y - sum a_l q_l over the picks made so far
     double cur_rnorm = 0.0;                                              // ||r|| of the residual the next pick is made from
     int hi = 0, extra = 0, dep = 0;
-    bool inexact = false, my_stop = false;
+    bool inexact = false;
+    int pend = -1;                                                       // pick whose residual's norm is still spread over the group
     if (book) {
         const int m = mb;
-        double rn2 = 0.0;
         if (!fin[m]) {
             const double* y = a.y64 + (size_t)m * k + bk.row0;
             for (int r = t; r < bk.R; r += kT) {
@@ -989,10 +1074,11 @@ __global__ void __launch_bounds__(kT, 1) k_omp(OmpArgs a, int mode) {
                         v -= __ldcg(a.acoef + (size_t)m * s + l) * q;
                     }
                 bk.rr[r] = v;
-                rn2 += v * v;
                 if (r < bk.rows) a.r32[2 * (bk.row0 + r) + m] = (float)v;
             }
-            send_norm<GS>(cluster, sh, bk, rn2, rank0, g);
+            if ((k & 1) && bk.rows < bk.R) for (int l = t; l < a.q_cols; l += kT) bk.qs[(size_t)l * bk.R + bk.rows] = 0.0;
+            __syncthreads();
+            send_norm<GS>(cluster, bk, rank0, g);
         }
         cluster.sync();
         if (!fin[m]) {
@@ -1004,15 +1090,7 @@ __global__ void __launch_bounds__(kT, 1) k_omp(OmpArgs a, int mode) {
                 a.ctl->stop[m] = 0;
             }
             const int c0 = v0[m] - base[m];
-            if (mode == 0 && !first_final[m] && c0 >= 0 && c0 < a.half_n) {
-                const size_t n = (size_t)m * a.half_n + c0;
-                const double sc = residual_scale(cur_rnorm);
-                for (int r = t; r < bk.rows; r += kT) {
-                    a.rt[n * a.kp + bk.row0 + r] = half_rn_bits(bk.rr[r] * sc);
-                    a.rhist[n * k + bk.row0 + r] = bk.rr[r];
-                }
-                if (g == 0 && t == 0) a.inv_scale[n] = (float)(1.0 / sc);
-            }
+            if (mode == 0 && !first_final[m] && c0 >= 0 && c0 < a.half_n) emit_row(a, bk, (size_t)m * a.half_n + c0, cur_rnorm, g);
         } else if (g == 0 && t == 0) a.ctl->stop[m] = 1;
         if (mode == 0 && g == 0) {
             const int keep = fin[m] ? 0 : (v0[m] - base[m] > 0 ? v0[m] - base[m] : 0);   // rows of earlier tentative picks stay
@@ -1047,123 +1125,119 @@ __global__ void __launch_bounds__(kT, 1) k_omp(OmpArgs a, int mode) {
         barrier();
         const bool active = book && act[mb];
         const int m = mb, j = active ? jm[mb] : 0;
-        const bool first = i == 0 && active && first_col[mb] != kNoColumn;
         const bool speculative = mode == 0 && !(i == 0 && active && first_final[mb]);
         const int c = active ? j - base[mb] : 0;                      // -1 for a confirmed prescribed pick
         int nc = 0;
-        // ---- 1. candidates, their exact scores, the products of the best one with the q_l
+        uint32_t col = kNoColumn;
+        // ---- 1. candidates, their exact scores, the products of the best one with the q_l, ||r||
         if (active) {
-            if (first) {
-                __syncthreads();
-                if (t == 0) sh.cidx[0] = first_col[mb];
-                nc = 1;
-                __syncthreads();
-            } else nc = gather_candidates(a, sh, m, j, nblk, mode == 1, &inexact);
+            if (i == 0 && first_col[mb] != kNoColumn) { col = first_col[mb]; nc = 1; }
+            else nc = gather_candidates(a, sh, m, j, nblk, mode == 1, &col, &inexact);
             if (nc > 0) {
-                make_column(a, bk, sh.cidx[0], bk.an);
-                __syncthreads();
-                send_products<GS>(cluster, a, bk, m, j, 0, j + 2, bk.an, bk.x0, xstride, 0, rank0, g);
-                for (int e = 1; e < nc; ++e) {
-                    __syncthreads();
-                    make_column(a, bk, sh.cidx[e], bk.alt);
-                    __syncthreads();
-                    send_products<GS>(cluster, a, bk, m, j, j, j + 2, bk.alt, bk.x0, xstride, s + 2 + 2 * (e - 1), rank0, g);
-                }
-            }
+                send_products<GS>(cluster, a, bk, m, j, col, true, bk.x0, rank0, g);
+                for (int e = 1 + (t >> 5); e < nc; e += kWarps) send_candidate<GS>(cluster, a, bk, sh.cidx[e], e, bk.x0, rank0, g);
+            } else if (pend >= 0) send_norm<GS>(cluster, bk, rank0, g);
         }
+        if (kOneCluster && t == 0) *cluster.map_shared_rank(&sh.peer_nc, rank ^ GS) = nc;
         if (book) cluster.sync();
         // ---- 2. the winner: largest <a, r>^2 / ||a||^2, lowest index on ties
-        int win = 0;
-        double dot = 0.0, n2 = 1.0;
-        if (active && nc > 0) {
-            double best = -1.0; uint32_t bi = kNoColumn;
-            for (int e = 0; e < nc; ++e) {
-                const int at = e == 0 ? j : s + 2 + 2 * (e - 1);
-                double ed = 0.0, en = 0.0;
-                for (int p = 0; p < GS; ++p) { ed += bk.x0[(size_t)p * xstride + at]; en += bk.x0[(size_t)p * xstride + at + 1]; }
-                const double sc = en > 0.0 ? ed * ed / en : 0.0;
-                const uint32_t idx = sh.cidx[e];
-                if (sc > best || (sc == best && idx < bi)) { best = sc; bi = idx; win = e; dot = ed; n2 = en; }
-            }
-        }
-        const bool again = active && nc > 0 && win != 0;               // the same in every block of the group
-        if (!kOneCluster && again) cluster.sync();                      // everybody has read the exchange buffer
-        if (again) {
-            make_column(a, bk, sh.cidx[win], bk.an);
-            __syncthreads();
-            send_products<GS>(cluster, a, bk, m, j, 0, j, bk.an, bk.x1, xstride, 0, rank0, g);
-        }
-        if (kOneCluster || again) cluster.sync();
-        // ---- 3. c, gamma, a_j; q_j and the new residual of this slice
-        int rc = 0;
-        uint32_t col = kNoColumn;
-        double rn2 = 0.0;
+        bool again = false;
         if (active) {
-            if (nc == 0) rc = 1;
-            else {
-                col = sh.cidx[win];
-                const double* x = again ? bk.x1 : bk.x0;
-                for (int l = t; l < j; l += kT) {
+            if (nc > 0) {
+                for (int l = t; l < j + 3; l += kT) {
+                    const int at = l <= j ? l : s + (l - j - 1);
                     double v = 0.0;
-                    for (int p = 0; p < GS; ++p) v += x[(size_t)p * xstride + l];
+#pragma unroll
+                    for (int p = 0; p < GS; ++p) v += bk.x0[(size_t)p * xstride + at];
                     bk.cs[l] = v;
                 }
                 __syncthreads();
+            }
+            if (pend >= 0) {
+                double rn2 = 0.0;
+                if (nc > 0) rn2 = bk.cs[j + 2];
+                else for (int p = 0; p < GS; ++p) rn2 += bk.xrn[p];
+                cur_rnorm = sqrt(rn2);
+            }
+        }
+        double dot = 0.0, n2 = 1.0;
+        if (active && nc > 0) {
+            dot = bk.cs[j]; n2 = bk.cs[j + 1];
+            if (nc > 1) {
+                double best = n2 > 0.0 ? dot * dot / n2 : 0.0;
+                uint32_t bi = col;
+                int win = 0;
+                for (int e = 1; e < nc; ++e) {
+                    double ed = 0.0, en = 0.0;
+                    for (int p = 0; p < GS; ++p) {
+                        ed += bk.x0[(size_t)p * xstride + s + 2 + 2 * (e - 1)];
+                        en += bk.x0[(size_t)p * xstride + s + 3 + 2 * (e - 1)];
+                    }
+                    const double sc = en > 0.0 ? ed * ed / en : 0.0;
+                    const uint32_t idx = sh.cidx[e];
+                    if (sc > best || (sc == best && idx < bi)) { best = sc; bi = idx; win = e; dot = ed; n2 = en; }
+                }
+                again = win != 0;                                      // the same in every block of the group
+                col = bi;
+            }
+        }
+        const bool more = kOneCluster ? (nc > 1 || sh.peer_nc > 1) : nc > 1;     // the same in every block of the cluster
+        if (more) {
+            if (!kOneCluster) cluster.sync();                           // everybody has read the exchange buffer
+            if (again) send_products<GS>(cluster, a, bk, m, j, col, false, bk.x1, rank0, g);
+            cluster.sync();
+            if (again) {
+                for (int l = t; l < j; l += kT) {
+                    double v = 0.0;
+                    for (int p = 0; p < GS; ++p) v += bk.x1[(size_t)p * xstride + l];
+                    bk.cs[l] = v;
+                }
+                __syncthreads();
+            }
+        }
+        // ---- 3. gamma, a_j; q_j and the new residual of this slice
+        if (active) {
+            int rc = nc == 0 ? 1 : 0;
+            // the residual of the previous pick, whose norm has just come together, is a row of the screened batch
+            if (pend >= 0) {
+                if (g == 0 && t == 0) a.rnorm[(size_t)m * s + pend] = cur_rnorm;
+                if (mode == 0 && c >= 0 && c < a.half_n) emit_row(a, bk, (size_t)m * a.half_n + c, cur_rnorm, g);
+                pend = -1;
+            }
+            if (nc > 0) {
                 double csq = 0.0;
                 for (int l = t & 31; l < j; l += 32) csq = fma(bk.cs[l], bk.cs[l], csq);
                 csq = warp_sum(csq);
                 const double piv = n2 - csq;
-                if (speculative && g == 0 && t == 0) {
-                    const double psc = fabs(dot) / sqrt(n2);
-                    a.pick_score[(size_t)m * s + j] = psc;
-                    a.tau[m * a.half_n + c] = (float)(report_threshold(a, cur_rnorm, psc) * residual_scale(cur_rnorm));
-                    a.wide_tau[m * a.half_n + c] = wide_threshold(a, c, cur_rnorm);
-                    a.lam[(size_t)m * s + j] = col;
-                }
                 if (!(piv > kPivot * n2)) rc = 2;
                 else {
-                    const double gamma = 1.0 / sqrt(piv), aj = gamma * dot;
+                    const double gamma = rsqrt(piv), aj = gamma * dot;
                     const int R = bk.R, P = bk.P;
-                    double* part = bk.alt;
-                    if (P == 1) {
-                        for (int r = t; r < R; r += kT) {
-                            double v0_ = 0.0, v1_ = 0.0;
-                            int l = 0;
-#pragma unroll 4
-                            for (; l + 1 < j; l += 2) {
-                                v0_ = fma(bk.cs[l], r < bk.rows ? dot_vector(a, bk, m, j, l, bk.an)[r] : 0.0, v0_);
-                                v1_ = fma(bk.cs[l + 1], r < bk.rows ? dot_vector(a, bk, m, j, l + 1, bk.an)[r] : 0.0, v1_);
-                            }
-                            if (l < j) v0_ = fma(bk.cs[l], r < bk.rows ? dot_vector(a, bk, m, j, l, bk.an)[r] : 0.0, v0_);
-                            part[r] = v0_ + v1_;
-                        }
-                    } else {
-                        const int r = t % R, h = t / R;
-                        if (h < P) {
-                            double v0_ = 0.0, v1_ = 0.0;
+                    const int r0 = P == 1 ? t : t % R, h = P == 1 ? 0 : t / R;
+                    if (h < P)
+                        for (int r = r0; r < bk.rows; r += P == 1 ? kT : R) {
+                            double va = 0.0, vb = 0.0;
                             int l = h;
 #pragma unroll 4
                             for (; l + P < j; l += 2 * P) {
-                                v0_ = fma(bk.cs[l], r < bk.rows ? dot_vector(a, bk, m, j, l, bk.an)[r] : 0.0, v0_);
-                                v1_ = fma(bk.cs[l + P], r < bk.rows ? dot_vector(a, bk, m, j, l + P, bk.an)[r] : 0.0, v1_);
+                                va = fma(bk.cs[l], q_slice(a, bk, m, l)[r], va);
+                                vb = fma(bk.cs[l + P], q_slice(a, bk, m, l + P)[r], vb);
                             }
-                            if (l < j) v0_ = fma(bk.cs[l], r < bk.rows ? dot_vector(a, bk, m, j, l, bk.an)[r] : 0.0, v0_);
-                            part[h * R + r] = v0_ + v1_;
+                            if (l < j) va = fma(bk.cs[l], q_slice(a, bk, m, l)[r], va);
+                            bk.part[h * R + r] = va + vb;
                         }
-                    }
                     __syncthreads();
+                    const ColKey key = column_key(a.seed_lo, a.seed_hi, col);
                     for (int r = t; r < bk.rows; r += kT) {
                         double v = 0.0;
-                        for (int h = 0; h < P; ++h) v += part[h * R + r];
-                        const double q = gamma * (bk.an[r] - v);
+                        for (int e = 0; e < P; ++e) v += bk.part[e * R + r];
+                        const double q = gamma * (a.sigma * (double)z_at(key, (uint32_t)(bk.row0 + r)) - v);
                         a.q[((size_t)m * s + j) * k + bk.row0 + r] = q;
                         if (j < a.q_cols) bk.qs[(size_t)j * R + r] = q;
                         const double rv = bk.rr[r] - aj * q;
                         bk.rr[r] = rv;
                         a.r32[2 * (bk.row0 + r) + m] = (float)rv;
-                        rn2 += rv * rv;
                     }
-                    send_norm<GS>(cluster, sh, bk, rn2, rank0, g);
                     if (g == 0) {
                         for (int l = t; l < j; l += kT) {
                             a.crow[((size_t)m * s + j) * s + l] = bk.cs[l];
@@ -1175,55 +1249,51 @@ __global__ void __launch_bounds__(kT, 1) k_omp(OmpArgs a, int mode) {
                             if (!speculative) { a.cnt->done[m] = j + 1; a.ctl->v[m] = j + 1; a.ctl->forced[m] = kNoColumn; }
                         }
                     }
+                    pend = j;
                 }
+            }
+            if (nc > 0 && speculative && g == 0 && t == kT - 32) {         // (a warp with little else to do)
+                const double psc = fabs(dot) * rsqrt(n2);
+                a.pick_score[(size_t)m * s + j] = psc;
+                a.tau[m * a.half_n + c] = (float)(report_threshold(a, cur_rnorm, psc) * residual_scale(cur_rnorm));
+                a.wide_tau[m * a.half_n + c] = wide_threshold(a, c, cur_rnorm);
+                a.lam[(size_t)m * s + j] = col;
             }
             // what ends this recovery's run of picks
             if (rc == 0) hi = j + 1;
-            else {
-                my_stop = true;
-                if (speculative) {
-                    // no candidate left: the current residual is screened without a pick; dependent column: the
-                    // pick is screened, and the recovery stops there if the pick is confirmed
-                    if (rc == 1) {
-                        extra = 1;
-                        if (g == 0 && t == 0) {
-                            a.tau[m * a.half_n + c] = (float)(a.z_harvest * cur_rnorm / sqrt((double)k) * residual_scale(cur_rnorm));
-                            a.wide_tau[m * a.half_n + c] = wide_threshold(a, c, cur_rnorm);
-                        }
-                    } else { dep = 1; hi = j + 1; }
-                    if (g == 0 && t == 0) a.ctl->stop[m] = 1;
-                } else if (g == 0 && t == 0) {
-                    // a confirmed pick cannot be made: this recovery ends with j picks
-                    a.cnt->stopped[m] = 1;
-                    atomicOr(&a.cnt->status, (unsigned int)SGC_STATUS_DEPENDENT_COLUMN);
-                    a.cnt->done[m] = j;
-                    a.ctl->v[m] = j;
-                    a.ctl->finished[m] = 1;
-                    a.ctl->stop[m] = 1;
-                }
+            else if (speculative) {
+                // no candidate left: the current residual is screened without a pick; dependent column: the
+                // pick is screened, and the recovery stops there if the pick is confirmed
+                if (rc == 1) {
+                    extra = 1;
+                    if (g == 0 && t == 0) {
+                        a.tau[m * a.half_n + c] = (float)(a.z_harvest * cur_rnorm / sqrt((double)k) * residual_scale(cur_rnorm));
+                        a.wide_tau[m * a.half_n + c] = wide_threshold(a, c, cur_rnorm);
+                    }
+                } else { dep = 1; hi = j + 1; }
+                if (g == 0 && t == 0) a.ctl->stop[m] = 1;
+            } else if (g == 0 && t == 0) {
+                // a confirmed pick cannot be made: this recovery ends with j picks
+                a.cnt->stopped[m] = 1;
+                atomicOr(&a.cnt->status, (unsigned int)SGC_STATUS_DEPENDENT_COLUMN);
+                a.cnt->done[m] = j;
+                a.ctl->v[m] = j;
+                a.ctl->finished[m] = 1;
+                a.ctl->stop[m] = 1;
             }
         }
-        // ---- 4. the new residual becomes a row of the screened batch while the others start on the next correlation
-        if (book) cluster.sync();
-        if (active && rc == 0) {
-            double rn = 0.0;
-            for (int p = 0; p < GS; ++p) rn += bk.xrn[p];
-            rn = sqrt(rn);
-            cur_rnorm = rn;
-            if (g == 0 && t == 0) a.rnorm[(size_t)m * s + j] = rn;
-            if (mode == 0 && c + 1 < a.half_n && j + 1 < s) {
-                const size_t n = (size_t)m * a.half_n + c + 1;
-                const double sc = residual_scale(rn);
-                for (int r = t; r < bk.rows; r += kT) {
-                    a.rt[n * a.kp + bk.row0 + r] = half_rn_bits(bk.rr[r] * sc);
-                    a.rhist[n * k + bk.row0 + r] = bk.rr[r];
-                }
-                if (g == 0 && t == 0) a.inv_scale[n] = (float)(1.0 / sc);
-            }
-        }
-        if (!kOneCluster) grid.sync();
+        barrier();
     }
-    if (kOneCluster) cluster.sync();                                   // nobody leaves while a peer may still write to its memory
+    // the norm of the last residual
+    if (book) {
+        if (pend >= 0) send_norm<GS>(cluster, bk, rank0, g);
+        cluster.sync();
+        if (pend >= 0 && g == 0 && t == 0) {
+            double rn2 = 0.0;
+            for (int p = 0; p < GS; ++p) rn2 += bk.xrn[p];
+            a.rnorm[(size_t)mb * s + pend] = sqrt(rn2);
+        }
+    }
     if (book && g == 0 && t == 0 && !fin[mb]) {
         const int m = mb;
         if (mode == 0) {
@@ -1237,7 +1307,6 @@ __global__ void __launch_bounds__(kT, 1) k_omp(OmpArgs a, int mode) {
             a.ctl->finished[m] = 1;
         }
     }
-    (void)my_stop;
 }
 
 }  // namespace
@@ -1307,6 +1376,8 @@ cudaError_t omp_configure(sgc_state* st) {
     if (e == cudaSuccess) e = resident_clusters<8>(&n8);
     if (e != cudaSuccess) return e;
     if (omp_opt_in<16>() != cudaSuccess || resident_clusters<16>(&n16) != cudaSuccess) { n16 = 0; cudaGetLastError(); }
+    if (2 * n2 > kCorrBlocks) n2 = kCorrBlocks / 2;
+    if (8 * n8 > kCorrBlocks) n8 = kCorrBlocks / 8;
     st->omp_grid2 = 2 * n2; st->omp_grid8 = 8 * n8; st->omp_one = n16 >= 1 ? 1 : 0;
     if (n8 < 3 || n2 < 2) return cudaErrorInvalidConfiguration;
     return cudaSuccess;

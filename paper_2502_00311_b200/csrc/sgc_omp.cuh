@@ -14,7 +14,7 @@ struct OmpArgs {
     int half_n;                        // residuals per stream in one screening pass
     int rows_wide, rows_narrow;        // rows of the pass that serves both streams / the first stream alone
     double z_harvest, z_floor;         // screening thresholds in units of ||r|| / sqrt(k)
-    Cand* corr_cand;                   // [2][blocks][kCorrTop]
+    float4* corr_cand;                 // [2][blocks] (score, column, best score not forwarded, -)
     const double* y64; float* r32;     // r32 viewed as float[2k] (interleaved pairs)
     uint32_t* lam;                     // [2][s]
     // Orthogonal form of Algorithm 3's recurrences, one record per pick j: q_j (unit vector, the new column made orthogonal

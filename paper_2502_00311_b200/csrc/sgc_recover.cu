@@ -22,6 +22,7 @@
 // Several states that share A are recovered together (launch_recover_group): their residuals sit side by
 // side in one screened batch, so one pass serves them all.
 #include <cuda_fp16.h>
+#include <math.h>
 
 #include "sgc_omp.cuh"
 
@@ -408,11 +409,11 @@ __global__ void __launch_bounds__(kOmpThreads, 1) k_resolve(ResolveArgs ra) {
         if (r >= 0 && r < kMaxRounds) { ctl->trace[r][0] = ctl->v[0]; ctl->trace[r][1] = ctl->v[1]; ctl->trace[r][2] = ctl->n_cand; }
     }
 }
-// start of the recovery of one step.  When the step speculates: after Sparsify_s, M^ and V^ are combinations of the columns
+// start of the recovery of one step.  keep_list (a state that speculates, in this step or in others): after Sparsify_s, M^ and V^ are combinations of the columns
 // kept in this and in earlier steps (Eq. 4, 5), so the indices just kept are candidates, and they enter the ring of recent
 // index sets.
 __global__ void __launch_bounds__(kOmpThreads, 1)
-k_begin(SpecCtl* ctl, int speculate, float* wide_tau, int shared, const uint32_t* sel_idx, int s, uint32_t* kept_ring, int hist_slots,
+k_begin(SpecCtl* ctl, int speculate, int keep_list, float* wide_tau, int shared, const uint32_t* sel_idx, int s, uint32_t* kept_ring, int hist_slots,
         uint32_t* cand_list, unsigned int* cand_bits) {
     __shared__ int n_s;
     const int t = threadIdx.x;
@@ -420,10 +421,10 @@ k_begin(SpecCtl* ctl, int speculate, float* wide_tau, int shared, const uint32_t
     if (wide_tau != nullptr && t < kPassMaxN) wide_tau[t] = __int_as_float(0x7f800000);
     if (t < kMaxRounds) ctl->trace[t][0] = ctl->trace[t][1] = ctl->trace[t][2] = 0;
     const int n0 = ctl->n_cand, version = ctl->list_version;
-    const int slot = speculate ? ctl->hist_next % hist_slots : 0;
+    const int slot = keep_list ? ctl->hist_next % hist_slots : 0;
     if (t == 0) n_s = n0;
     __syncthreads();
-    if (speculate) {
+    if (keep_list) {
         for (int e = t; e < s; e += kOmpThreads) kept_ring[(size_t)slot * s + e] = sel_idx[e];
         cand_append(sel_idx, s, &n_s, cand_list, cand_bits);
     }
@@ -441,7 +442,7 @@ k_begin(SpecCtl* ctl, int speculate, float* wide_tau, int shared, const uint32_t
         ctl->stop[0] = ctl->stop[1] = 0;
         ctl->rounds = 0; ctl->pass_error = 0; ctl->pass_rows = 0;
         ctl->gram_ok = 1;
-        if (speculate) {
+        if (keep_list) {
             const int n_new = n_s < kCandCap ? n_s : kCandCap;
             // a version of 0 means a fresh state: no Gram matrix yet
             if (n_new != n0) { ctl->n_cand = n_new; ctl->list_version = version + 1; }
@@ -459,7 +460,7 @@ struct FinishArgs {
     OmpArgs o;
     double* x; float* W; uint32_t* upd_idx; double* upd_val;
     double alpha, eps, lr, tol;
-    int shared, speculate;
+    int shared, speculate, keep_list;
     uint32_t* cand_list; unsigned int* cand_bits; const uint32_t* kept_ring; int* rounds_out;
 };
 constexpr size_t kFinishDynBytes = 160 * 1024;
@@ -599,13 +600,19 @@ __global__ void __launch_bounds__(kOmpThreads, 1) k_finish(FinishArgs f) {
         if (n_neg > 0) bits |= (unsigned int)SGC_STATUS_NEGATIVE_V;
         if (bits) atomicOr(&cnt->status, bits);
     }
-    if (!f.speculate) return;
+    if (!f.keep_list) return;
     // ---- the supports found stay (or become) candidates of the next step
     SpecCtl* ctl = a.ctl;
     // how many rounds this step took (the enqueued rounds if even they were not enough): sizes the next step's launches
-    // bit 8: a list pass refuted a pick (the wide lists earned their keep); bit 9: a full pass refuted a pick
-    if (t == 0)
-        *f.rounds_out = (ctl->fallback ? kMaxRounds : ctl->rounds) | (ctl->list_refuted > 0 ? 256 : 0) | (ctl->refuted > 0 ? 512 : 0);
+    // bit 8: a list pass refuted a pick (the wide lists earned their keep); bit 9: a full pass refuted a pick; bits 10, 11: how
+    // many speculating steps in a row needed more than one confirming pass (at most 3)
+    if (t == 0 && f.speculate) {
+        const bool one = !ctl->fallback && ctl->rounds <= 1 && ctl->list_rounds == 0;
+        const int streak = one ? 0 : (ctl->inexact_streak < 3 ? ctl->inexact_streak + 1 : 3);
+        ctl->inexact_streak = streak;
+        *f.rounds_out = (ctl->fallback ? kMaxRounds : ctl->rounds) | (ctl->list_refuted > 0 ? 256 : 0) | (ctl->refuted > 0 ? 512 : 0) |
+                        (streak << 10);
+    }
     int nl = ctl->n_cand;
     // rebuild from the supports and the ring of kept index sets when the list has outgrown its bound, or when it holds
     // far more than those although a single round confirmed every pick (harvested columns of an earlier cold start)
@@ -686,6 +693,7 @@ cudaError_t configure_recover(sgc_state* st) {
     // shared-support variant: only the first stream has residuals to screen, a pass half as wide does
     st->pass_n_half = ((st->pass_n / 2 + 31) / 32) * 32;
     st->z_harvest = normal_tail_threshold_impl((double)st->d, 3072.0);
+    st->z_harvest_few = normal_tail_threshold_impl((double)st->d, 256.0);
     st->z_floor = normal_tail_threshold_impl((double)st->d, 6144.0);
     st->z_wide = normal_tail_threshold_impl((double)st->d, 100000.0);
     // How often a screened residual feeds the wide lists: a pick takes 25-30 / k of the residual's energy, so the scores of the
@@ -708,6 +716,47 @@ cudaError_t finish_recover_setup(sgc_state* st) {
     return cudaDeviceSynchronize();
 }
 
+// Whether the next step of a state speculates.  Requested modes are obeyed.  SGC_MODE_AUTO compares estimates (us, from the
+// timings below): in lock-step every pick costs its bookkeeping and barriers and one correlation of all columns; a
+// speculation that one pass confirms costs that pass and little per pick; one that is refuted every few picks costs list
+// correlations, list passes and resolving.  Which of the two a state meets is known once it has speculated for two steps; before,
+// the sizes tell: steps of d = 129344, k = 512, s = 33 (k = 1.32 s ln d) are confirmed by one pass, those of 1721085, 384, 26
+// (1.03) and 2^24, 1024, 64 (0.96) are not.
+//   lock-step, us per pick:  d = 50304, k = 128: 15.9;  31820, 1024: 28;  200000, 512: 60      (11 + k d / 2.0e6)
+//   refuted speculation:     d = 151700, k = 320, s = 37: 100;  117656, 832, 102: 81;  1876582, 960, 123: 168;  3001000, 700, 100: 270
+//                                                                                             (100 + k d / 2.0e7)
+//   confirmed speculation, us per step: d = 143488, k = 1600, s = 25: 370 (with the launches; 140 + 1.2 s + k d / 3.3e6)
+// A state that has come to prefer lock-step tries a speculating step now and then: its gradients may have changed.
+constexpr int kRetrySteps = 32;
+constexpr double kFewRoundsWork = 3.0e8;              // k * d up to which a pick in lock-step costs at most 160 us
+constexpr double kTwoLevelWork = 1.0e8;               // k * d from which list passes can be cheaper than full ones
+
+static bool prefers_speculation(const sgc_state* st) {
+    const double kd = (double)st->k * (double)st->d, s = (double)st->s;
+    const double lock = s * (11.0 + kd / 2.0e6);
+    const int seen = *reinterpret_cast<volatile int*>(st->h_rounds);
+    const bool refuted = (seen & 255) != 0 ? ((seen >> 10) & 3) >= 2 : (double)st->k < 1.2 * s * log((double)st->d);
+    const double spec = refuted ? s * (100.0 + kd / 2.0e7) : 140.0 + 1.2 * s + kd / 3.3e6;
+    return spec < lock;
+}
+
+bool will_speculate(const sgc_state* st) {
+    if (st->mode != SGC_MODE_AUTO) return st->mode == SGC_MODE_SPECULATIVE;
+    return st->d >= kSpecMinD && (prefers_speculation(st) || st->lock_steps >= kRetrySteps);
+}
+
+// the same, and counts the lock-step steps since the last speculating one (only a state that has speculated and turned away
+// tries again)
+static bool wants_speculation(sgc_state* st) {
+    const bool yes = will_speculate(st);
+    if (yes) st->lock_steps = 0;
+    else if ((*reinterpret_cast<volatile int*>(st->h_rounds) & 255) != 0) st->lock_steps += 1;
+    return yes;
+}
+
+// the candidate list is kept up in lock-step steps as well, so that a later speculation does not start cold
+static bool keeps_list(const sgc_state* st) { return st->spec_ready && st->mode != SGC_MODE_LOCKSTEP; }
+
 // Recovery (a4 + a5) of n states that share (d, k, s, seed), hence A.  The states' screened residuals are laid out side by
 // side in the screening buffers of the first state of each batch (a batch = as many states as fit kPassMaxN columns), so
 // one pass over A serves a whole batch; everything else runs per state.  n = 1 is the plain sgc_step.
@@ -715,8 +764,7 @@ static cudaError_t recover_batches(sgc_state* const* sts, float* const* weights,
     sgc_state* st0 = sts[0];
     bool speculate = true;
     for (int i = 0; i < n; ++i)
-        speculate = speculate && sts[i]->spec_ready &&
-                    (sts[i]->mode == 2 || (sts[i]->mode == 0 && sts[i]->d >= kSpecMinD));
+        speculate = wants_speculation(sts[i]) && sts[i]->spec_ready && speculate;
     const int per_batch = speculate ? kPassMaxN / st0->pass_n : 1;
     std::vector<OmpArgs> args((size_t)n);
     cudaError_t e = cudaSuccess;
@@ -732,10 +780,14 @@ static cudaError_t recover_batches(sgc_state* const* sts, float* const* weights,
         a.tau = lead->tau + slot * st->pass_n;
         a.inv_scale = lead->inv_scale + slot * st->pass_n;
         a.rep_count = lead->rep_count + slot * st->pass_n;
+        // a state whose picks one pass confirms, step after step, needs no candidates from it: fewer columns are reported
+        // and swept by the resolve kernel
+        const int seen = *reinterpret_cast<volatile int*>(st->h_rounds);
+        if (st->mode == SGC_MODE_AUTO && (seen & 255) == 1 && (seen >> 10) == 0) a.z_harvest = st->z_harvest_few;
         args[i] = a;
         {
             PhaseTimer timer(st, stream, kPhaseBook, 1);
-            k_begin<<<1, kOmpThreads, 0, stream>>>(st->ctl, speculate ? 1 : 0, st->wide_tau, st->shared_support, st->sel_idx, st->s,
+            k_begin<<<1, kOmpThreads, 0, stream>>>(st->ctl, speculate ? 1 : 0, keeps_list(st) ? 1 : 0, st->wide_tau, st->shared_support, st->sel_idx, st->s,
                                                    st->kept_ring, st->hist_slots, st->cand_list, st->cand_bits);
             *launches += 1;
         }
@@ -744,13 +796,17 @@ static cudaError_t recover_batches(sgc_state* const* sts, float* const* weights,
         const int hint = speculate ? *reinterpret_cast<volatile int*>(st->h_rounds) : 0;
         const int last = hint & 255;
         int want = last <= 0 ? 8 : 2 * last + 3;
+        // a state whose steps one pass confirms, and for which finishing in lock-step would cost little: one spare round (each
+        // costs three launches, 12 us, of a step of 300)
+        const bool smooth = st->mode == SGC_MODE_AUTO && last == 1 && (hint >> 10) == 0;
+        if (smooth && (double)st->k * (double)st->d <= kFewRoundsWork) want = 2;
         if (last > 0 && last + 2 > mini_rounds) mini_rounds = last + 2;
         if (last <= 0) mini_rounds = kMaxRounds;
         if (st->max_rounds > 0 && want > st->max_rounds) want = st->max_rounds;
         if (want > n_rounds) n_rounds = want;
         // two-level screening pays where steps need several full passes (recovery picks columns outside the kept sets);
         // it is dropped again when a step needed one pass and its list passes refuted nothing
-        if (last >= 3) st->two_level = true;
+        if (last >= 3 && (double)st->k * (double)st->d >= kTwoLevelWork) st->two_level = true;
         else if (last == 1 && !(hint & 256)) st->two_level = false;
     }
     if (n_rounds > kMaxRounds) n_rounds = kMaxRounds;
@@ -887,7 +943,7 @@ static cudaError_t recover_batches(sgc_state* const* sts, float* const* weights,
         f.o = args[i];
         f.x = st->x; f.W = weights[i]; f.upd_idx = st->upd_idx; f.upd_val = st->upd_val;
         f.alpha = (double)st->alpha; f.eps = (double)st->eps; f.lr = (double)st->lr; f.tol = st->residual_tol;
-        f.shared = st->shared_support; f.speculate = speculate ? 1 : 0;
+        f.shared = st->shared_support; f.speculate = speculate ? 1 : 0; f.keep_list = keeps_list(st) ? 1 : 0;
         f.cand_list = st->cand_list; f.cand_bits = st->cand_bits; f.kept_ring = st->kept_ring; f.rounds_out = st->d_rounds;
         k_finish<<<1, kOmpThreads, kFinishDynBytes, stream>>>(f);
         *launches += 1;
@@ -907,9 +963,9 @@ cudaError_t launch_recover_group(sgc_state* const* sts, float* const* weights, i
     cudaError_t e = cudaSuccess;
     for (int i = 0; i < n && e == cudaSuccess; ++i) {
         sgc_state* st = sts[i];
-        const bool speculates = st->spec_ready && (st->mode == 2 || (st->mode == 0 && st->d >= kSpecMinD));
+        const bool speculates = st->spec_ready && will_speculate(st);
         const int last = speculates ? (*reinterpret_cast<volatile int*>(st->h_rounds) & 255) : 0;
-        const bool alone = speculates && (kPassMaxN / st->pass_n < 2 || st->two_level || last >= 3);
+        const bool alone = !speculates || (kPassMaxN / st->pass_n < 2 || st->two_level || last >= 3);
         if (alone) e = recover_batches(&sts[i], &weights[i], 1, stream, launches);
         else { together.push_back(st); together_w.push_back(weights[i]); }
     }
