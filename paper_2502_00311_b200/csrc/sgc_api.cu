@@ -41,7 +41,6 @@ size_t layout(sgc_state* st, unsigned char* base) {
     st->sel_cand = carve<unsigned long long>(base, off, sgc::kSelCap);
     st->sel_hist = carve<unsigned int>(base, off, sgc::kSelBins);
     st->corr_cand = carve<float4>(base, off, 2 * (size_t)sgc::kCorrBlocks);
-    st->zsel = carve<uint16_t>(base, off, sgc::chunk_sized(st) ? 2 * s * k : 1);
     st->q_basis = carve<double>(base, off, 2 * s * k);
     st->lam = carve<uint32_t>(base, off, 2 * s);
     st->F = carve<double>(base, off, 2 * s * s);

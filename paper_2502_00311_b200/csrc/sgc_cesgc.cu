@@ -2,16 +2,13 @@
 // its update goes back through B^T:  W <- W - eta B^T SGC(B G).  B (r x m, the first r left-singular vectors of a
 // gradient, refreshed by the caller every few hundred steps) is an input here; the two projections around the SGC core
 // are the kernels of this file.
-//   k_cesgc_project   P = B G.  Thread = one column j of G and four rows of B; G is read row by row (coalesced over j),
-//                     the rows of B come from shared memory as broadcasts.  Sums are carried as pairs of floats (error-free
-//                     product through one FMA, error-free two-term sum: some 44 bits in all; fp64 arithmetic runs at a
-//                     64th of the fp32 rate on this part and made this kernel 1.1 ms), and rounded to fp32 once at the
-//                     end.  The top-s selection that follows decides on those values; a reference that forms B G in fp64
-//                     gets the same fp32 numbers but for a few elements in ten thousand (entries much smaller than
-//                     their terms), which differ by one ulp.  Slabs of B and G are staged in shared memory; the next ones travel
-//                     through registers while the current ones are worked on.  The rows of G are split over the CTAs of
-//                     a thread-block cluster (n / 32 column blocks alone would not fill the SMs); their partial sums
-//                     meet in the first CTA through distributed shared memory, added in rank order.
+//   k_cesgc_project   P = B G in fp64, rounded to fp32 once, so that the top-s selection that follows decides on the exactly
+//                     projected gradient.  64 fp64 multiply-adds per cycle and SM bound it (30 us for a 4096 x 4096 gradient at
+//                     r = 32); conversions from fp32, a quarter as fast, are kept out of the way: a thread owns four columns and
+//                     eight rows, converts each element of G once for its eight products and reads B as fp64 from a slab that
+//                     the block has converted on the way in.  (An error-free two-float form took 276 us, fp64 with both operands
+//                     converted per product 1.1 ms.)  The rows of G are split over the CTAs of a thread-block cluster; their
+//                     partial sums meet through distributed shared memory, added in rank order.
 //   k_cesgc_back      W += B^T U for the r x n matrix U that the SGC core left (U = -eta N has at most s non-zeros):
 //                     block = one column of U; columns without a non-zero cost one read of r values.
 #include "sgc_internal.cuh"
@@ -23,112 +20,123 @@ namespace cg = cooperative_groups;
 namespace sgc {
 namespace {
 
-constexpr int kProjCols = 32;            // columns of G per block
-constexpr int kProjRows = 4;             // rows of B per thread
-constexpr int kProjChunk = 64;           // rows of G per staged slab of B
 constexpr int kCesgcMaxR = 64;
-
-constexpr int kProjStage = 8;            // floats of each slab that one thread moves (at 256 threads: 64 x 32 floats)
+constexpr int kProjCols = 128;           // columns of G per block: 32 lanes of four
+constexpr int kProjRows = 8;             // rows of B per thread
+constexpr int kProjPer = 4;              // rows of a slab of G per thread
 constexpr int kProjMaxSplit = 8;         // CTAs of a cluster (the portable limit), each with a range of G's rows
-constexpr int kProjResident = 4 * 148;   // CTAs of this kernel that the SMs hold at once (64 registers, 256 threads)
+constexpr int kProjResident = 148;       // one wave
 
-__global__ void __launch_bounds__(kProjCols * (kCesgcMaxR / kProjRows), 2)   // 64 registers: four blocks of 256 threads per SM
+// groups of 8 rows of B (warps of a part), parts (each with every parts-th row of G) that make up 16 warps at most, rows of G per slab
+__host__ __device__ constexpr int proj_groups(int r) { return (r + kProjRows - 1) / kProjRows; }
+__host__ __device__ constexpr int proj_parts(int r) { return proj_groups(r) > 4 ? 2 : proj_groups(r) > 2 ? 4 : 8; }
+__host__ __device__ constexpr int proj_slab(int r) { return kProjPer * proj_parts(r); }
+// slabs of B (two, fp64) and, at the end, the partial sums of the parts
+__host__ __device__ constexpr size_t proj_smem(int r) {
+    const size_t slab = 2 * (size_t)proj_groups(r) * kProjRows * proj_slab(r) * sizeof(double);
+    const size_t part = (size_t)proj_groups(r) * kProjRows * kProjCols * sizeof(double);
+    return slab > part ? slab : part;
+}
+constexpr size_t proj_smem_max() {
+    size_t v = 0;
+    for (int r = 1; r <= kCesgcMaxR; ++r) if (proj_smem(r) > v) v = proj_smem(r);
+    return v;
+}
+
+template <bool VEC>
+__global__ void __launch_bounds__(512, 1)
 k_cesgc_project(const float* __restrict__ B, const float* __restrict__ G, float* __restrict__ P, int r, int m, int n) {
-    __shared__ __align__(16) float bs[kCesgcMaxR][kProjChunk];       // B[:, row0 .. row0 + 64)
-    __shared__ float gs[kProjChunk][kProjCols];                       // G[row0 .. row0 + 64, the block's columns]
+    extern __shared__ double smem[];
     cg::cluster_group cluster = cg::this_cluster();
-    const int groups = (r + kProjRows - 1) / kProjRows;
-    const int jl = threadIdx.x % kProjCols, ig = threadIdx.x / kProjCols;
-    const int j = blockIdx.x * kProjCols + jl;
-    const bool work = ig < groups && j < n;
+    const int groups = proj_groups(r), rows8 = groups * kProjRows, parts = proj_parts(r), slab_rows = proj_slab(r);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int ig = warp % groups, part = warp / groups;
+    const int j0 = blockIdx.x * kProjCols + 4 * lane;                 // this thread's four columns
     // this CTA's rows of G: whole slabs, the same number for every CTA of the cluster (the last ranges may be empty)
-    const int slabs = (m + kProjChunk - 1) / kProjChunk;
-    const int part_rows = (slabs + (int)gridDim.y - 1) / (int)gridDim.y * kProjChunk;
+    const int slabs = (m + slab_rows - 1) / slab_rows;
+    const int part_rows = (slabs + (int)gridDim.y - 1) / (int)gridDim.y * slab_rows;
     const int m_begin = (int)blockIdx.y * part_rows;
     const int m_end = m_begin + part_rows < m ? m_begin + part_rows : m;
-    const int nb = r * kProjChunk, ng = kProjChunk * kProjCols;       // slab sizes
-    const int per_b = (nb + blockDim.x - 1) / blockDim.x, per_g = (ng + blockDim.x - 1) / blockDim.x;   // <= kProjStage
-    float pb[kProjStage], pg[kProjStage];                             // the next slabs, on their way through registers
-    auto fetch = [&](int row0) {
+    double acc[kProjRows][4];
 #pragma unroll
-        for (int u = 0; u < kProjStage; ++u) {
-            const int eb = threadIdx.x + u * blockDim.x, eg = eb;
-            pb[u] = 0.0f; pg[u] = 0.0f;
-            if (u < per_b && eb < nb) {
-                const int i = eb / kProjChunk, q = eb % kProjChunk;
-                if (row0 + q < m_end) pb[u] = B[(size_t)i * m + row0 + q];
-            }
-            if (u < per_g && eg < ng) {
-                const int q = eg / kProjCols, c = eg % kProjCols;
-                const int col = blockIdx.x * kProjCols + c;
-                if (row0 + q < m_end && col < n) pg[u] = G[(size_t)(row0 + q) * n + col];
-            }
+    for (int u = 0; u < kProjRows; ++u)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[u][c] = 0.0;
+    // slab of B as [row of G][row of B]: a thread reads its eight values of a row of G in four 16-byte broadcasts
+    auto stage = [&](double* dst, int row0) {
+        for (int e = threadIdx.x; e < rows8 * slab_rows; e += blockDim.x) {
+            const int i = e / slab_rows, q = e % slab_rows;
+            dst[q * rows8 + i] = (i < r && row0 + q < m_end) ? (double)B[(size_t)i * m + row0 + q] : 0.0;
         }
     };
-    float hi[kProjRows], lo[kProjRows];
-#pragma unroll
-    for (int u = 0; u < kProjRows; ++u) hi[u] = lo[u] = 0.0f;
-    fetch(m_begin);
-    for (int row0 = m_begin; row0 < m_end; row0 += kProjChunk) {
-        __syncthreads();                                              // the previous slabs have been used up
-#pragma unroll
-        for (int u = 0; u < kProjStage; ++u) {
-            const int e = threadIdx.x + u * blockDim.x;
-            if (u < per_b && e < nb) bs[e / kProjChunk][e % kProjChunk] = pb[u];
-            if (u < per_g && e < ng) gs[e / kProjCols][e % kProjCols] = pg[u];
+    auto load = [&](int row) -> float4 {
+        float4 f = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (row < m_end) {
+            const float* src = G + (size_t)row * n + j0;
+            if (VEC) { if (j0 < n) f = __ldcs(reinterpret_cast<const float4*>(src)); }        // n is a multiple of 4
+            else {
+                if (j0 < n) f.x = src[0];
+                if (j0 + 1 < n) f.y = src[1];
+                if (j0 + 2 < n) f.z = src[2];
+                if (j0 + 3 < n) f.w = src[3];
+            }
         }
-        __syncthreads();
-        if (row0 + kProjChunk < m_end) fetch(row0 + kProjChunk);          // in flight while this slab is worked on
-        if (!work) continue;
-        // rows of this slab, rounded up to four: what lies beyond m_end was staged as zeros and adds nothing
-        const int rows = ((m_end - row0 < kProjChunk ? m_end - row0 : kProjChunk) + 3) & ~3;
-        for (int q = 0; q < rows; q += 4) {
-            const float g4[4] = {gs[q][jl], gs[q + 1][jl], gs[q + 2][jl], gs[q + 3][jl]};
+        return f;
+    };
+    double* bufs[2] = {smem, smem + (size_t)rows8 * slab_rows};
+    float4 next[kProjPer];
+    if (m_begin < m_end) {
+        stage(bufs[0], m_begin);
 #pragma unroll
-            for (int u = 0; u < kProjRows; ++u) {
-                const float4 b4 = *reinterpret_cast<const float4*>(&bs[ig * kProjRows + u][q]);   // one address per warp
-                const float bq[4] = {b4.x, b4.y, b4.z, b4.w};
+        for (int q = 0; q < kProjPer; ++q) next[q] = load(m_begin + q * parts + part);
+    }
+    int b = 0;
+    for (int row0 = m_begin; row0 < m_end; row0 += slab_rows, b ^= 1) {
+        __syncthreads();                                              // this slab is staged, the other one used up
+        float4 g[kProjPer];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {                         // ascending rows of G: the order of the sums is fixed
-                    const float p = __fmul_rn(bq[e], g4[e]);
-                    const float pe = __fmaf_rn(bq[e], g4[e], -p);     // b g = p + pe exactly
-                    const float t = __fadd_rn(hi[u], p);
-                    const float v = __fsub_rn(t, hi[u]);
-                    const float te = __fadd_rn(__fsub_rn(hi[u], __fsub_rn(t, v)), __fsub_rn(p, v));   // hi + p = t + te exactly
-                    hi[u] = t;
-                    lo[u] = __fadd_rn(lo[u], __fadd_rn(te, pe));
-                }
+        for (int q = 0; q < kProjPer; ++q) g[q] = next[q];
+        if (row0 + slab_rows < m_end) {
+#pragma unroll
+            for (int q = 0; q < kProjPer; ++q) next[q] = load(row0 + slab_rows + q * parts + part);
+            stage(bufs[b ^ 1], row0 + slab_rows);
+        }
+        const double* slab = bufs[b] + ig * kProjRows;
+#pragma unroll
+        for (int q = 0; q < kProjPer; ++q) {
+            const double2* bq = reinterpret_cast<const double2*>(slab + (size_t)(q * parts + part) * rows8);
+            const double gx = (double)g[q].x, gy = (double)g[q].y, gz = (double)g[q].z, gw = (double)g[q].w;
+#pragma unroll
+            for (int u = 0; u < kProjRows / 2; ++u) {
+                const double2 v = bq[u];
+                acc[2 * u][0] = fma(v.x, gx, acc[2 * u][0]); acc[2 * u][1] = fma(v.x, gy, acc[2 * u][1]);
+                acc[2 * u][2] = fma(v.x, gz, acc[2 * u][2]); acc[2 * u][3] = fma(v.x, gw, acc[2 * u][3]);
+                acc[2 * u + 1][0] = fma(v.y, gx, acc[2 * u + 1][0]); acc[2 * u + 1][1] = fma(v.y, gy, acc[2 * u + 1][1]);
+                acc[2 * u + 1][2] = fma(v.y, gz, acc[2 * u + 1][2]); acc[2 * u + 1][3] = fma(v.y, gw, acc[2 * u + 1][3]);
             }
         }
     }
-    // the partial sums of the cluster's CTAs, left in each one's shared memory (the slab of B is done with)
-    __syncthreads();
-    float* part_hi = &bs[0][0];
-    float* part_lo = part_hi + kCesgcMaxR * kProjCols;
-    static_assert(2 * kProjCols <= kProjChunk, "two 64 x 32 arrays in the slab of B");
-    if (work) {
+    // the parts of this CTA, one after the other (a fixed order), into shared memory; then the CTAs of the cluster
+    double* sums = smem;                                              // [rows8][kProjCols]
+    for (int p = 0; p < parts; ++p) {
+        __syncthreads();
+        if (part != p) continue;
 #pragma unroll
-        for (int u = 0; u < kProjRows; ++u) {
-            part_hi[(ig * kProjRows + u) * kProjCols + jl] = hi[u];
-            part_lo[(ig * kProjRows + u) * kProjCols + jl] = lo[u];
-        }
+        for (int u = 0; u < kProjRows; ++u)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                double* d = sums + (size_t)(ig * kProjRows + u) * kProjCols + 32 * c + lane;      // (column 4 lane + c at 32 c + lane)
+                *d = p == 0 ? acc[u][c] : *d + acc[u][c];
+            }
     }
     cluster.sync();
-    if (cluster.block_rank() == 0 && work) {
-        const unsigned split = cluster.num_blocks();
-#pragma unroll
-        for (int u = 0; u < kProjRows; ++u) {
-            const int i = ig * kProjRows + u;
-            if (i >= r) continue;
-            double acc = 0.0;
-            for (unsigned y = 0; y < split; ++y) {                    // rank order: the result does not depend on the schedule
-                const float* h = cluster.map_shared_rank(part_hi, y);
-                const float* l = cluster.map_shared_rank(part_lo, y);
-                acc += (double)h[i * kProjCols + jl];
-                acc += (double)l[i * kProjCols + jl];
-            }
-            P[(size_t)i * n + j] = (float)acc;
-        }
+    const unsigned split = cluster.num_blocks(), rank = cluster.block_rank();
+    // the CTAs share the additions: rank order, whoever adds, so the result does not depend on the schedule
+    for (int e = (int)(rank * blockDim.x + threadIdx.x); e < r * kProjCols; e += (int)(split * blockDim.x)) {
+        const int i = e / kProjCols, x = e % kProjCols, col = blockIdx.x * kProjCols + 4 * (x & 31) + (x >> 5);
+        double v = 0.0;
+        for (unsigned y = 0; y < split; ++y) v += cluster.map_shared_rank(sums, y)[(size_t)i * kProjCols + x];
+        if (col < n) P[(size_t)i * n + col] = (float)v;
     }
     cluster.sync();                                                   // nobody leaves while its sums may still be read
 }
@@ -171,23 +179,27 @@ k_cesgc_back(const float* __restrict__ B, const float* __restrict__ U, float* __
 bool cesgc_shape_ok(int r, int m, int n) { return r >= 1 && r <= kCesgcMaxR && m >= 1 && n >= 1; }
 
 cudaError_t launch_cesgc_project(const float* B, const float* G, float* P, int r, int m, int n, cudaStream_t stream) {
-    const int groups = (r + kProjRows - 1) / kProjRows;
-    const int threads = kProjCols * groups < 256 ? 256 : kProjCols * groups;      // at least 256: the slabs are staged 8 floats per thread
     const int col_blocks = (n + kProjCols - 1) / kProjCols;
-    const int slabs = (m + kProjChunk - 1) / kProjChunk;
+    const int slabs = (m + proj_slab(r) - 1) / proj_slab(r);
     int split = kProjResident / col_blocks;                                         // one wave; a function of the shape alone
     if (split > kProjMaxSplit) split = kProjMaxSplit;
     if (split > slabs / 2) split = slabs / 2;                                       // at least two slabs per CTA
     if (split < 1) split = 1;
+    const bool vec = n % 4 == 0 && ((uintptr_t)G & 15u) == 0;
+    const void* fn = vec ? (const void*)k_cesgc_project<true> : (const void*)k_cesgc_project<false>;
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)proj_smem_max());
+    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)col_blocks, (unsigned)split, 1);
-    cfg.blockDim = dim3((unsigned)threads, 1, 1);
+    cfg.blockDim = dim3((unsigned)(32 * proj_groups(r) * proj_parts(r)), 1, 1);
+    cfg.dynamicSmemBytes = proj_smem(r);
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = (unsigned)split; attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_cesgc_project, B, G, P, r, m, n);
+    return vec ? cudaLaunchKernelEx(&cfg, k_cesgc_project<true>, B, G, P, r, m, n)
+               : cudaLaunchKernelEx(&cfg, k_cesgc_project<false>, B, G, P, r, m, n);
 }
 
 cudaError_t launch_cesgc_back(const float* B, const float* U, float* W, int r, int m, int n, cudaStream_t stream) {

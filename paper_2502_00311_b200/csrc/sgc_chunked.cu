@@ -1,27 +1,31 @@
 // MESGC (Section 4.4) with small per-chunk problems: c chunks of one flat vector, each an SGC problem of its own
 // (own M, V; s_c <= 32 kept entries, k_c <= 256 rows), all sharing the matrix A (k_c x d/c) named by one seed.
 // Run chunk by chunk this costs ~25 launches per chunk; here the whole step of all chunks takes 2 + 2 s_c launches:
-//   k_chunk_front    block = chunk: exact top-s_c of the chunk (a1), p = A g~, q = A g~^2 and the k-space Adam moments
-//                    (a2 + a3), residuals r = y for both moments
+//   k_chunk_front    block (or cluster) = chunk: exact top-s_c of the chunk (a1), p = A g~, q = A g~^2 and the k-space Adam
+//                    moments (a2 + a3), residuals r = y for both moments
 //   per OMP iteration (Algorithm 3, all 2c recoveries in lock-step, which is where the shared A pays: a column of A is
 //   generated once and meets the residuals of every chunk):
-//     k_chunk_corr   thread = one residual, block = 256 residuals x a range of columns: fp32 scores |<A_i,r>| / ||A_i||,
-//                    best two columns of the range per residual
-//     k_chunk_pick   block of 128 threads = one recovery: fp64 rescoring of the columns within 2e-3 of the best fp32 score, lowest
-//                    index on ties, then the inverse-Cholesky recurrences of Algorithm 3, x, r
-//   k_chunk_scatter  warp = chunk: Eq. (8) on the common support, weight update (a5)
+//     k_chunk_corr   columns of A as the A operand of mma.m16n8k16, four residuals as two binary16 numbers each as the B
+//                    operand: scores |<A_i,r>| / ||A_i||, best two columns of the block's range per residual
+//     k_chunk_pick   block = one recovery: fp64 rescoring of the columns within 2e-3 of the best score, lowest
+//                    index on ties, then Algorithm 3 in the orthogonal form of sgc_omp.cu: c_l = <q_l, a>, q, a_j, r
+//   k_chunk_scatter  block = chunk: coefficients, Eq. (8) on the common support, weight update (a5)
 // Every record lands in the chunk's own state, so sgc_get works per chunk exactly as after sgc_step.
 #include <algorithm>
 #include <new>
 #include <vector>
 
+#include <cooperative_groups.h>
+
 #include "sgc_internal.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace sgc {
 namespace {
 
 constexpr int kFrontThreads = 512;
-constexpr int kCorrBlock = 256;          // residuals per block of k_chunk_corr
+constexpr int kCorrBlock = 256;          // threads per block of k_chunk_corr
 constexpr int kChunkMaxS = 32;
 constexpr int kChunkMaxK = 256;
 
@@ -33,6 +37,7 @@ struct ChunkArgs {
     double sigma;
     float* r32;                          // [2c][kp]
     Cand* cand;                          // [2c][splits][2]
+    uint32_t* lam;                       // [2c][s] the supports once more, side by side (a state's own copy is an allocation of its own)
     int splits, cols_per_split;
     int early;                           // the iteration's kernels let their successor's blocks in at once (see after_previous_kernel)
     // tensor-core route (see ChunkWs)
@@ -48,75 +53,149 @@ __device__ __forceinline__ double warp_sum_d(double v) {
     return v;
 }
 
-// ---- a1 + a2 + a3, one block per chunk -------------------------------------------------------------------
-// Top-s of the chunk by the key (|g| bits << 32) | ~index (unique; lowest index wins equal magnitudes): every thread
-// keeps the CAP largest keys of its strided share in registers (the s largest of the chunk are among them), then s
-// rounds of "largest head of any thread" pop them in descending order.
-template <int CAP>
-__global__ void __launch_bounds__(kFrontThreads)
+// ---- a1 + a2 + a3, one block or cluster of blocks per chunk -----------------------------------------------
+// Top-s of the chunk by the key (|g| bits << 32) | ~index (unique; lowest index wins equal magnitudes).  One read of the
+// chunk gives every thread the largest magnitude of its strided share; with e = ceil(s / warps), the smallest over the warps of
+// a warp's e-th largest thread maximum is a bound that at least s elements reach.  Only the shares whose maximum
+// reaches it are read again (from L2, a share per warp and trip), and the few elements that do are ranked.  Registers hold one
+// word per thread whatever s is (keeping the s largest of every share in registers and sorting in one thread took 146 us for
+// 256 chunks of 65536 floats at s = 16).  More survivors than can be ranked at once (many equal magnitudes) send the block
+// through s sweeps of "largest key below the last one" instead.  Long chunks in small number are split over a cluster, so
+// that the SMs are all reading.
+constexpr int kFrontCap = 2048;
+constexpr int kFrontRank = 256;                  // survivors ranked all against all
+constexpr int kFrontMaxSplit = 8;
+
+__device__ __forceinline__ unsigned long long front_key(float g, uint32_t i) {
+    return ((unsigned long long)(__float_as_uint(g) & 0x7FFFFFFFu) << 32) | (uint32_t)(~i);
+}
+__device__ __forceinline__ unsigned int mag4(const float4& f) {
+    return max(max(__float_as_uint(f.x) & 0x7FFFFFFFu, __float_as_uint(f.y) & 0x7FFFFFFFu),
+               max(__float_as_uint(f.z) & 0x7FFFFFFFu, __float_as_uint(f.w) & 0x7FFFFFFFu));
+}
+
+// largest 64-bit value over the block (kFrontThreads threads); part: one word per warp
+__device__ unsigned long long front_max(unsigned long long v, unsigned long long* part) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int o = 16; o > 0; o >>= 1) { const unsigned long long t = __shfl_xor_sync(0xffffffffu, v, o); v = t > v ? t : v; }
+    __syncthreads();
+    if (lane == 0) part[warp] = v;
+    __syncthreads();
+    v = 0ull;
+#pragma unroll
+    for (int w = 0; w < kFrontThreads / 32; ++w) v = part[w] > v ? part[w] : v;
+    return v;
+}
+
+__global__ void __launch_bounds__(kFrontThreads, 2)
 k_chunk_front(ChunkArgs a, const float* __restrict__ grad, double b1, double b2, double c1, double c2) {
-    __shared__ unsigned long long wmax[kFrontThreads / 32];
+    __shared__ unsigned long long list[kFrontCap];
+    __shared__ unsigned long long part[kFrontThreads / 32];
+    __shared__ unsigned int wtau[kFrontMaxSplit * kFrontThreads / 32];
     __shared__ unsigned long long sel_key[kChunkMaxS];
     __shared__ ColKey keys[kChunkMaxS];
     __shared__ float vals[kChunkMaxS];
-    const int ch = blockIdx.x, s = a.s, k = a.k;
+    __shared__ int n_list;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int split = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();      // split: a power of two
+    const int ch = blockIdx.x / split, s = a.s, k = a.k, t = threadIdx.x;
     const ChunkRef ref = a.table[ch];
     const float* g = grad + (size_t)ch * a.dc;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned long long top[CAP];
+    const float4* g4 = reinterpret_cast<const float4*>(g);
+    const int lane = t & 31, warp = t >> 5, stride = split * kFrontThreads;
+    const int nvec = (int)(a.dc >> 2);                               // chunks start on 16-byte boundaries, dc % 4 == 0
+    const int v_first = rank * kFrontThreads + t;
+    unsigned int top = 0u;
+    {
+        int v = v_first;
+        for (; v + 7 * stride < nvec; v += 8 * stride) {
+            float4 f[8];
 #pragma unroll
-    for (int q = 0; q < CAP; ++q) top[q] = 0ull;                    // no real key is 0
-    const long long nvec = a.dc >> 2;                                // chunks start on 16-byte boundaries, dc % 4 == 0
-    for (long long v = threadIdx.x; v < nvec; v += kFrontThreads) {
-        const float4 f = __ldcs(reinterpret_cast<const float4*>(g) + v);
-        const float e[4] = {f.x, f.y, f.z, f.w};
+            for (int u = 0; u < 8; ++u) f[u] = g4[v + u * stride];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const uint32_t i = (uint32_t)(4 * v + u);
-            const unsigned long long key = ((unsigned long long)(__float_as_uint(e[u]) & 0x7FFFFFFFu) << 32) | (uint32_t)(~i);
-            if (key > top[CAP - 1]) {
+            for (int u = 0; u < 8; ++u) top = max(top, mag4(f[u]));
+        }
+        for (; v < nvec; v += stride) top = max(top, mag4(g4[v]));
+    }
+    const int warps = split * (kFrontThreads / 32);
+    if (t == 0) n_list = 0;
+    {
+        // the warp's e-th largest thread maximum (equal ones count one by one), told to every block of the cluster
+        const int e = (s + warps - 1) / warps;
+        unsigned int m = 0u;
+        bool out = false;
+        for (int q = 0; q < e; ++q) {
+            m = __reduce_max_sync(0xffffffffu, out ? 0u : top);
+            const unsigned int who = __ballot_sync(0xffffffffu, !out && top == m);
+            if (who != 0u && lane == __ffs(who) - 1) out = true;
+        }
+        if (lane < split) *cluster.map_shared_rank(&wtau[rank * (kFrontThreads / 32) + warp], lane) = m;
+    }
+    if (split > 1) cluster.sync(); else __syncthreads();
+    unsigned int tau = 0xFFFFFFFFu;
+    for (int w = lane; w < warps; w += 32) tau = min(tau, wtau[w]);
+    tau = __reduce_min_sync(0xffffffffu, tau);
+    int* count = cluster.map_shared_rank(&n_list, 0);
+    unsigned long long* dst = cluster.map_shared_rank(list, 0);
+    unsigned int redo = __ballot_sync(0xffffffffu, top >= tau);
+    while (redo) {
+        const int owner = __ffs(redo) - 1;
+        redo &= redo - 1u;
+        for (int v0 = rank * kFrontThreads + warp * 32 + owner; v0 < nvec; v0 += 32 * stride) {
+            const long long v = (long long)v0 + (long long)lane * stride;
+            if (v >= nvec) continue;
+            const float4 f = g4[v];
+            if (mag4(f) < tau) continue;
+            const float x[4] = {f.x, f.y, f.z, f.w};
 #pragma unroll
-                for (int q = CAP - 1; q >= 0; --q) {
-                    const unsigned long long up = q > 0 ? top[q - 1] : ~0ull;
-                    if (key > top[q]) top[q] = key > up ? up : key;
+            for (int u = 0; u < 4; ++u)
+                if ((__float_as_uint(x[u]) & 0x7FFFFFFFu) >= tau) {
+                    const int slot = atomicAdd(count, 1);
+                    if (slot < kFrontCap) dst[slot] = front_key(x[u], (uint32_t)(4 * v + u));
                 }
-            }
         }
     }
-    for (int r = 0; r < s; ++r) {
-        unsigned long long m = top[0];
-        for (int o = 16; o > 0; o >>= 1) { const unsigned long long t = __shfl_xor_sync(0xffffffffu, m, o); m = t > m ? t : m; }
-        if (lane == 0) wmax[warp] = m;
-        __syncthreads();
-        unsigned long long best = 0ull;
-#pragma unroll
-        for (int w = 0; w < kFrontThreads / 32; ++w) best = wmax[w] > best ? wmax[w] : best;
-        if (top[0] == best && best != 0ull) {                        // keys are unique: exactly one thread pops
-#pragma unroll
-            for (int q = 0; q + 1 < CAP; ++q) top[q] = top[q + 1];
-            top[CAP - 1] = 0ull;
-            sel_key[r] = best;
+    if (split > 1) { cluster.sync(); if (rank != 0) return; }          // (nobody reads this block's memory after this)
+    __syncthreads();
+    const int n = n_list;
+    if (n <= kFrontRank) {
+        // rank of every survivor among the others: the s largest
+        if (t < n) {
+            const unsigned long long mine = list[t];
+            int r = 0;
+            for (int q = 0; q < n; ++q) r += list[q] > mine ? 1 : 0;
+            if (r < s) sel_key[r] = mine;
         }
-        __syncthreads();
+    } else {
+        unsigned long long last = ~0ull;
+        for (int r = 0; r < s; ++r) {
+            unsigned long long m = 0ull;                              // no real key is 0
+            if (n <= kFrontCap) { for (int q = t; q < n; q += kFrontThreads) { const unsigned long long v = list[q]; if (v < last && v > m) m = v; } }
+            else
+                for (int v = t; v < nvec; v += kFrontThreads) {
+                    const float4 f = g4[v];
+                    const float x[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) { const unsigned long long key = front_key(x[u], (uint32_t)(4 * v + u)); if (key < last && key > m) m = key; }
+                }
+            last = front_max(m, part);
+            if (t == 0) sel_key[r] = last;
+        }
     }
-    if (threadIdx.x == 0) {
+    __syncthreads();
+    if (t < s) {
         // ascending index order, as the records of sgc_step have it
-        for (int i = 1; i < s; ++i) {
-            const unsigned long long kv = sel_key[i];
-            int j = i - 1;
-            while (j >= 0 && (uint32_t)(~(uint32_t)sel_key[j]) > (uint32_t)(~(uint32_t)kv)) { sel_key[j + 1] = sel_key[j]; --j; }
-            sel_key[j + 1] = kv;
-        }
-        unsigned int bits = 0u;
-        for (int i = 0; i < s; ++i) {
-            const uint32_t idx = ~(uint32_t)sel_key[i];
-            if ((sel_key[i] >> 32) >= 0x7F800000ull) bits |= (unsigned int)SGC_STATUS_NONFINITE_INPUT;
-            const float val = g[idx];
-            ref.sel_idx[i] = idx; ref.sel_val[i] = val;
-            keys[i] = column_key(a.seed_lo, a.seed_hi, idx);
-            vals[i] = val;
-        }
-        if (bits) atomicOr(&ref.cnt->status, bits);
+        const unsigned long long mine = sel_key[t];
+        const uint32_t idx = ~(uint32_t)mine;
+        int r = 0;
+        for (int q = 0; q < s; ++q) r += (uint32_t)(~(uint32_t)sel_key[q]) < idx ? 1 : 0;
+        const float val = g[idx];
+        ref.sel_idx[r] = idx; ref.sel_val[r] = val;
+        keys[r] = column_key(a.seed_lo, a.seed_hi, idx);
+        vals[r] = val;
+        if ((mine >> 32) >= 0x7F800000ull) atomicOr(&ref.cnt->status, (unsigned int)SGC_STATUS_NONFINITE_INPUT);
+    }
+    if (t == 0) {
         ref.cnt->done[0] = ref.cnt->done[1] = 0;
         ref.cnt->stopped[0] = ref.cnt->stopped[1] = 0;
         ref.cnt->n_upd = ref.cnt->mismatch = ref.cnt->negv = 0;
@@ -124,7 +203,7 @@ k_chunk_front(ChunkArgs a, const float* __restrict__ grad, double b1, double b2,
     }
     __syncthreads();
     // a2 + a3: thread = row; fp64 sums in ascending column order (the arithmetic of the one-state kernel, term by term)
-    for (int row = threadIdx.x; row < k; row += kFrontThreads) {
+    for (int row = t; row < k; row += kFrontThreads) {
         double accp = 0.0, accq = 0.0;
         for (int i = 0; i < s; ++i) {
             const double av = a.sigma * (double)z_at(keys[i], (uint32_t)row);
@@ -147,14 +226,19 @@ k_chunk_front(ChunkArgs a, const float* __restrict__ grad, double b1, double b2,
 }
 
 // ---- phase A of one OMP iteration: every column of A against the residuals of all recoveries ------------------
-// grid = (column splits, groups of 256 recoveries).  The block walks its columns in tiles: thread t generates column
-// t of the tile into shared memory (fp32, with 1 / ||Z_i||), then every thread, which holds the residual of one
-// recovery in registers, scores all columns of the tile in ascending order (a strict ">" keeps the lowest index).
-// Only the best two columns per recovery leave the block; columns already in the support are skipped when they show up
-// as a new best.
-__host__ __device__ constexpr int corr_ks(int kp) { return kp > 64 ? kp / 64 : 1; }   // threads that share the rows of a residual: 64 rows each
-__host__ __device__ constexpr int corr_tile(int kp) { return kp <= 64 ? 256 : (kp <= 128 ? 128 : 32); }   // columns per tile
-__host__ __device__ constexpr int corr_group(int kp) { return kCorrBlock / corr_ks(kp); }   // recoveries per block
+// grid = (column splits, groups of recoveries).  The block walks its columns a tile at a time: its warps generate the tile in the
+// register layout of mma.m16n8k16's A operand (a row pair of a column is one register) into shared memory, with 1 / ||Z_i||,
+// and every warp multiplies it with the residuals it holds as B operands: NT tiles of four recoveries, each residual as two
+// binary16 numbers (value and remainder, 22 bits, scaled by a power of two), sums in fp32.  A lane ends up with the scores of
+// one recovery for two columns of every 16; only the best two columns per recovery leave the block; columns already in the
+// support are skipped when they show up as a new best.  (The legacy matrix instruction on purpose: with 2c residuals of k_c
+// rows the tensor work is small, what bounds the kernel is generating, comparing and the launch itself, and an operand in
+// registers needs no hand-off.  With one multiply-add per instruction it took 37 us at k_c = 8, 512 recoveries, 65536
+// columns, and 22 us per iteration at k_c = 217, 128 recoveries, 2048 columns.)
+__host__ __device__ constexpr int corr_kb(int kp) { return kp / 16 > 0 ? kp / 16 : 1; }              // 16-row blocks
+__host__ __device__ constexpr int corr_nt(int kp) { return kp <= 64 ? 8 : (kp <= 128 ? 4 : 2); }     // tiles of four recoveries per warp
+__host__ __device__ constexpr int corr_group(int kp) { return kCorrBlock / 32 * 4 * corr_nt(kp); }   // recoveries per block
+__host__ __device__ constexpr int corr_tile(int kp) { return kp <= 64 ? 64 : 32; }                   // columns generated at a time
 
 // The two kernels of an iteration are launched with programmatic stream serialization: the blocks of the next kernel may
 // become resident while this one is still running, and wait here until it has completed and its writes are visible.
@@ -179,364 +263,381 @@ struct ChainedLaunch {
     }
 };
 
+__device__ __forceinline__ void mma_16816(float (&c)[4], const uint4& x, uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(x.x), "r"(x.y), "r"(x.z), "r"(x.w), "r"(b0), "r"(b1));
+}
+
+// two binary16 numbers of a residual pair: the values (part 0) or what they leave (part 1)
+__device__ __forceinline__ uint32_t residual_part(float x, float y, int part) {
+    const __half2 h = __floats2half2_rn(x, y);
+    if (part == 0) return *reinterpret_cast<const uint32_t*>(&h);
+    const float2 f = __half22float2(h);
+    const __half2 l = __floats2half2_rn(x - f.x, y - f.y);
+    return *reinterpret_cast<const uint32_t*>(&l);
+}
+
+// the two best columns of a recovery
+struct Best2 {
+    float s1, s2; uint32_t i1, i2;
+    __device__ __forceinline__ void push(float s, uint32_t i) {      // i != i1, i2; lower index first on ties
+        if (s > s1 || (s == s1 && i < i1)) { s2 = s1; i2 = i1; s1 = s; i1 = i; }
+        else if (s > s2 || (s == s2 && i < i2)) { s2 = s; i2 = i; }
+    }
+};
+
 // gate != nullptr: the launch is a fallback of the tensor-core route and returns at once unless *gate names this
 // iteration (a.epoch): the word holds the epoch of the last iteration that left a recovery unresolved.
 template <int KP>
 __global__ void __launch_bounds__(kCorrBlock) k_chunk_corr(ChunkArgs a, int iter, const int* gate) {
-    after_previous_kernel(a.early);
-    if (gate != nullptr && *gate != a.epoch0 + iter) return;
-    constexpr int TC = corr_tile(KP);
-    constexpr int KS = corr_ks(KP), KL = KP / KS;                    // KS threads hold KL rows of a residual each
-    constexpr int ZS = KP + 4 * KS;                                  // stride of a tile column: every row part is followed by four
-                                                                     // floats, so that the KS parts a warp reads at once sit in different banks
-    extern __shared__ float smem[];
-    float* zt = smem;                                                // [TC][ZS]
-    float* inv = smem + TC * ZS;                                     // [TC]
-    float* n2p = inv + TC;                                           // [GPC][TC] partial ||Z_i||^2
-    constexpr int GPC = kCorrBlock / TC, RG = KP / GPC;              // generating threads per column, rows each
-    const int h = threadIdx.x % KS;
-    const int res = blockIdx.y * (kCorrBlock / KS) + threadIdx.x / KS;     // recovery = 2 * chunk + moment
-    const bool have = res < 2 * a.c;
-    bool active = false;
-    const uint32_t* sup = nullptr;
-    float rr[KL];
-#pragma unroll
-    for (int q = 0; q < KL; ++q) rr[q] = 0.0f;
-    if (have) {
-        const ChunkRef& ref = a.table[res >> 1];
-        active = ref.cnt->stopped[res & 1] == 0;
-        sup = ref.lam + (size_t)(res & 1) * a.s;
-        const float4* src = reinterpret_cast<const float4*>(a.r32 + (size_t)res * KP + h * KL);
-#pragma unroll
-        for (int q = 0; q < KL / 4; ++q) { const float4 f = src[q]; rr[4 * q] = f.x; rr[4 * q + 1] = f.y; rr[4 * q + 2] = f.z; rr[4 * q + 3] = f.w; }
-    }
-    float s1 = -1.0f, s2 = -1.0f;
-    uint32_t i1 = kNoColumn, i2 = kNoColumn;
+    constexpr int KB = corr_kb(KP), NT = corr_nt(KP), TC = corr_tile(KP), TILES = TC / 16, WARPS = kCorrBlock / 32;
+    constexpr int UNITS = TILES * KB;                                 // (16 columns, 16 rows): one warp's share of the generating
+    extern __shared__ uint4 smem4[];
+    uint4* zt = smem4;                                                // [TILES][KB][32] A operands
+    float* inv = reinterpret_cast<float*>(zt + TILES * KB * 32);      // [TC]
+    float* n2p = inv + TC;                                            // [KB][TC] partial ||Z_i||^2
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, q = lane & 3;
     const long long col0 = (long long)blockIdx.x * a.cols_per_split;
     long long col1 = col0 + a.cols_per_split;
     if (col1 > a.dc) col1 = a.dc;
-    for (long long tile = col0; tile < col1; tile += TC) {
-        __syncthreads();
-        {
-            // every thread generates: GPC threads share a column of the tile, RG rows each
-            const int t = threadIdx.x % TC, part = threadIdx.x / TC;
-            const long long col = tile + t;
-            float n2 = 0.0f;
-            float* dst = zt + t * ZS;
-            if (col < col1) {
-                const ColKey key = column_key(a.seed_lo, a.seed_hi, (uint32_t)col);
-                uint32_t hw = key.ck + (uint32_t)(part * RG / 2) * key.mk;
-#pragma unroll 4
-                for (int q = 0; q < RG; q += 2) {
-                    const int row = part * RG + q;
-                    float2 z = half2_bits_to_float2(z_pair_from_word(hw));
-                    hw += key.mk;
-                    if (row >= a.k) z.x = 0.0f;
-                    if (row + 1 >= a.k) z.y = 0.0f;
-                    const int at = row + 4 * (row / KL);
-                    dst[at] = z.x; dst[at + 1] = z.y;
-                    n2 = __fmaf_rn(z.x, z.x, n2);
-                    n2 = __fmaf_rn(z.y, z.y, n2);
-                }
-            } else {
-                for (int q = 0; q < RG; ++q) { const int row = part * RG + q; dst[row + 4 * (row / KL)] = 0.0f; }
+    auto generate = [&](long long tile0) {
+        for (int u = warp; u < UNITS; u += WARPS) {
+            const int tl = u / KB, kb = u % KB;
+            const uint32_t c0 = (uint32_t)(tile0 + tl * 16 + g), c1 = c0 + 8u;
+            const ColKey k0 = column_key(a.seed_lo, a.seed_hi, c0), k1 = column_key(a.seed_lo, a.seed_hi, c1);
+            const uint32_t h0 = k0.ck + (uint32_t)(kb * 8 + q) * k0.mk, h1 = k1.ck + (uint32_t)(kb * 8 + q) * k1.mk;
+            uint32_t z[4] = {z_pair_from_word(h0), z_pair_from_word(h1), z_pair_from_word(h0 + 4u * k0.mk), z_pair_from_word(h1 + 4u * k1.mk)};
+            float n[2] = {0.0f, 0.0f};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {                             // rows beyond k do not count
+                const int row = kb * 16 + 2 * q + (e & 2 ? 8 : 0);
+                if (row >= a.k) z[e] = 0u;
+                else if (row + 1 >= a.k) z[e] &= 0xFFFFu;
+                const float2 f = half2_bits_to_float2(z[e]);
+                n[e & 1] = __fmaf_rn(f.x, f.x, n[e & 1]); n[e & 1] = __fmaf_rn(f.y, f.y, n[e & 1]);
             }
-            n2p[part * TC + t] = n2;
+            zt[(size_t)u * 32 + lane] = make_uint4(z[0], z[1], z[2], z[3]);
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                n[e] += __shfl_xor_sync(0xffffffffu, n[e], 1); n[e] += __shfl_xor_sync(0xffffffffu, n[e], 2);
+                if (q == 0) n2p[kb * TC + tl * 16 + g + 8 * e] = n[e];
+            }
         }
+    };
+    if (gate == nullptr) generate(col0);                              // the first tile needs nothing of the kernels before
+    after_previous_kernel(a.early);
+    if (gate != nullptr) {
+        if (*gate != a.epoch0 + iter) return;
+        generate(col0);
+    }
+    // residuals as B operands: n = g of a tile is value (g even) or remainder (g odd) of recovery 4 tile + g / 2.  (Recoveries
+    // that have stopped are scored like the others; k_chunk_pick does not look at them.)
+    const int res0 = blockIdx.y * corr_group(KP) + warp * NT * 4;
+    uint32_t bf[NT][KB][2];
+    float back[NT];                                                   // of recovery 4 tile + q, whose scores this lane gets
+    {
+        constexpr int HB = KB * NT <= 8 ? NT : (KB >= 8 ? 1 : 8 / KB);       // tiles whose loads are in flight together
+#pragma unroll
+        for (int i0 = 0; i0 < NT; i0 += HB) {
+            float2 lo[HB][KB], hi[HB][KB];
+#pragma unroll
+            for (int i = 0; i < HB; ++i) {
+                const int res = res0 + 4 * (i0 + i) + (g >> 1);
+                const float* src = a.r32 + (size_t)(res < 2 * a.c ? res : 0) * KP + 2 * q;
+#pragma unroll
+                for (int kb = 0; kb < KB; ++kb) {
+                    lo[i][kb] = *reinterpret_cast<const float2*>(src + 16 * kb);
+                    hi[i][kb] = KP >= 16 ? *reinterpret_cast<const float2*>(src + 16 * kb + 8) : make_float2(0.0f, 0.0f);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < HB; ++i) {
+                unsigned int m = 0u;
+#pragma unroll
+                for (int kb = 0; kb < KB; ++kb) {
+                    m = max(m, max(__float_as_uint(lo[i][kb].x) & 0x7FFFFFFFu, __float_as_uint(lo[i][kb].y) & 0x7FFFFFFFu));
+                    m = max(m, max(__float_as_uint(hi[i][kb].x) & 0x7FFFFFFFu, __float_as_uint(hi[i][kb].y) & 0x7FFFFFFFu));
+                }
+                m = max(m, __shfl_xor_sync(0xffffffffu, m, 1)); m = max(m, __shfl_xor_sync(0xffffffffu, m, 2));
+                int e = (int)(m >> 23);                               // largest entry scaled into [2^10, 2^11)
+                e = e < 20 ? 20 : (e > 250 ? 250 : e);
+                const float sc = __uint_as_float((unsigned int)(264 - e) << 23);
+#pragma unroll
+                for (int kb = 0; kb < KB; ++kb) {
+                    bf[i0 + i][kb][0] = residual_part(lo[i][kb].x * sc, lo[i][kb].y * sc, g & 1);
+                    bf[i0 + i][kb][1] = residual_part(hi[i][kb].x * sc, hi[i][kb].y * sc, g & 1);
+                }
+                back[i0 + i] = __uint_as_float((unsigned int)(__shfl_sync(0xffffffffu, e, 8 * q) - 10) << 23);
+            }
+        }
+    }
+    Best2 best[NT];
+    float least[NT];                                                  // no column at or below this can be among the best two
+#pragma unroll
+    for (int i = 0; i < NT; ++i) {
+        best[i].s1 = best[i].s2 = -1.0f; best[i].i1 = best[i].i2 = kNoColumn;
+        least[i] = res0 + 4 * i + q < 2 * a.c ? -1.0f : 3.0e38f;
+    }
+    for (long long tile0 = col0; tile0 < col1; tile0 += TC) {
+        if (tile0 != col0) { __syncthreads(); generate(tile0); }
         __syncthreads();
         if (threadIdx.x < TC) {
             float n2 = 0.0f;
 #pragma unroll
-            for (int g = 0; g < GPC; ++g) n2 += n2p[g * TC + threadIdx.x];
-            inv[threadIdx.x] = n2 > 0.0f ? 1.0f / sqrtf(n2) : 0.0f;
+            for (int kb = 0; kb < KB; ++kb) n2 += n2p[kb * TC + threadIdx.x];
+            // (-infinity: no column of this block; its score is -infinity or not a number, and passes no comparison)
+            inv[threadIdx.x] = tile0 + threadIdx.x < col1 ? (n2 > 0.0f ? 1.0f / sqrtf(n2) : 0.0f) : __int_as_float(0xff800000);
         }
         __syncthreads();
-        if (KS == 1 && !active) continue;                            // (with KS > 1 the shuffles below need every lane)
-        const int n_here = (int)((col1 - tile) < TC ? (col1 - tile) : TC);
-        // the score of tile column t for this thread's recovery (with KS > 1: every lane of the warp calls it)
-        auto score = [&](int t) -> float {
-            const float4* zc = reinterpret_cast<const float4*>(zt + t * ZS + h * (KL + 4));
-            float acc0 = 0.0f, acc1 = 0.0f;
+        unsigned int moved = 0u;
+#pragma unroll 1
+        for (int tl = 0; tl < TILES; ++tl) {
+            if (tile0 + tl * 16 >= col1) break;
+            float acc[NT][4];
 #pragma unroll
-            for (int q = 0; q < KL / 4; ++q) {
-                const float4 z = zc[q];                              // one address per row part: a broadcast
-                acc0 = __fmaf_rn(z.x, rr[4 * q], acc0);
-                acc1 = __fmaf_rn(z.y, rr[4 * q + 1], acc1);
-                acc0 = __fmaf_rn(z.z, rr[4 * q + 2], acc0);
-                acc1 = __fmaf_rn(z.w, rr[4 * q + 3], acc1);
+            for (int i = 0; i < NT; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.0f;
+#pragma unroll
+            for (int kb = 0; kb < KB; ++kb) {
+                const uint4 x = zt[(size_t)(tl * KB + kb) * 32 + lane];
+#pragma unroll
+                for (int i = 0; i < NT; ++i) mma_16816(acc[i], x, bf[i][kb][0], bf[i][kb][1]);
             }
-            float dot = acc0 + acc1;
+            const float v0 = inv[tl * 16 + g], v1 = inv[tl * 16 + g + 8];
 #pragma unroll
-            for (int o = 1; o < KS; o <<= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);   // the other parts of the rows
-            return fabsf(dot);
-        };
-        auto offer = [&](float sc, int t) {                          // columns are offered in ascending order
-            if (!(sc > s2)) return;
-            const uint32_t col = (uint32_t)(tile + t);
-            bool taken = false;
-            for (int q = 0; q < iter; ++q) taken |= (sup[q] == col);
-            if (taken) return;
-            if (sc > s1) { s2 = s1; i2 = i1; s1 = sc; i1 = col; }
-            else { s2 = sc; i2 = col; }
-        };
-        // from 64 rows on, four columns at a time: four independent chains of multiply-adds, and one compare decides
-        // for all four whether any of them can enter the best two (with few rows the sweep is short, some lane of the
-        // warp nearly always has a new best, and the grouped form only adds work: 63 -> 67 us per step at k_c = 8)
-        int t = 0;
-        for (; KP >= 64 && t + 4 <= n_here; t += 4) {
-            const float4 iv = *reinterpret_cast<const float4*>(inv + t);
-            const float sc0 = score(t) * iv.x, sc1 = score(t + 1) * iv.y, sc2 = score(t + 2) * iv.z, sc3 = score(t + 3) * iv.w;
-            if (active && fmaxf(fmaxf(sc0, sc1), fmaxf(sc2, sc3)) > s2) {
-                offer(sc0, t); offer(sc1, t + 1); offer(sc2, t + 2); offer(sc3, t + 3);
+            for (int i = 0; i < NT; ++i) {
+                const float s0 = fabsf(acc[i][0] + acc[i][1]) * v0, s1 = fabsf(acc[i][2] + acc[i][3]) * v1;
+                if (fmaxf(s0, s1) > least[i]) {
+                    const uint32_t* sup = a.lam + (size_t)(res0 + 4 * i + q) * a.s;
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const float sc = e ? s1 : s0;
+                        if (!(sc > least[i])) continue;
+                        const uint32_t col = (uint32_t)(tile0 + tl * 16 + g + 8 * e);
+                        bool taken = false;
+                        for (int l = 0; l < iter; ++l) taken |= (sup[l] == col);
+                        if (!taken) { best[i].push(sc, col); least[i] = fmaxf(least[i], best[i].s2); moved |= 1u << i; }
+                    }
+                }
             }
         }
-        for (; t < n_here; ++t) {
-            const float sc = score(t) * inv[t];
-            if (active) offer(sc, t);
+        // the eight lanes of a recovery tell one another their second best (a lower bound of the block's): later columns rarely pass it
+        if (tile0 + TC < col1 && __any_sync(0xffffffffu, moved != 0u)) {
+#pragma unroll
+            for (int i = 0; i < NT; ++i) {
+                // second best among the lanes' best two: at least the largest s2, and at least the second largest s1
+                float hi1 = best[i].s1, hi2 = best[i].s2;
+#pragma unroll
+                for (int o = 4; o < 32; o <<= 1) {
+                    const float t1 = __shfl_xor_sync(0xffffffffu, hi1, o), t2 = __shfl_xor_sync(0xffffffffu, hi2, o);
+                    hi2 = fmaxf(fmaxf(hi2, t2), fminf(hi1, t1));
+                    hi1 = fmaxf(hi1, t1);
+                }
+                least[i] = fmaxf(least[i], hi2);
+            }
         }
     }
-    if (have && h == 0) {
-        Cand* out = a.cand + ((size_t)res * a.splits + blockIdx.x) * 2;
-        out[0].score = s1; out[0].idx = i1;
-        out[1].score = s2; out[1].idx = i2;
+    // the eight lanes of a recovery (same q) join their best two
+#pragma unroll
+    for (int i = 0; i < NT; ++i) {
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) {
+            const float t1 = __shfl_xor_sync(0xffffffffu, best[i].s1, o), t2 = __shfl_xor_sync(0xffffffffu, best[i].s2, o);
+            const uint32_t j1 = __shfl_xor_sync(0xffffffffu, best[i].i1, o), j2 = __shfl_xor_sync(0xffffffffu, best[i].i2, o);
+            if (j1 != kNoColumn) best[i].push(t1, j1);
+            if (j2 != kNoColumn) best[i].push(t2, j2);
+        }
+        const int mine = res0 + 4 * i + q;
+        if (g == 0 && mine < 2 * a.c) {
+            float4* out = reinterpret_cast<float4*>(a.cand + ((size_t)mine * a.splits + blockIdx.x) * 2);
+            *out = make_float4(best[i].s1 * back[i], __uint_as_float(best[i].i1), best[i].s2 * back[i], __uint_as_float(best[i].i2));
+        }
     }
 }
 
-// ---- phase B of one OMP iteration: one block of kPickThreads threads per recovery ---------------------------------------------------
-// Argmax among the columns that phase A left within 2e-3 (relative) of the best fp32 score, decided on fp64 scores
-// <Z_i, r>^2 / ||Z_i||^2 with the lowest index winning ties; then Algorithm 3 (Appendix B) for the new column:
-// g = A_Lambda^T a_new, c = F^T g, gamma = 1 / sqrt(g_ll - c^T c) (a pivot below 1e-10 g_ll ends this recovery),
-// new column [-gamma F c; gamma] of F, a_j = gamma <a_new, r>, x = F a, r = y - A_Lambda x.
-constexpr int kPickThreads = 128;        // one block per recovery
+// ---- phase B of one OMP iteration: one block per recovery ---------------------------------------------------------
+// Argmax among the columns that phase A left within 2e-3 (relative) of the best score, decided on fp64 scores
+// <Z_i, r>^2 / ||Z_i||^2 with the lowest index winning ties; then Algorithm 3 (Appendix B) in its orthogonal form for the new
+// column a: c_l = <q_l, a>, gamma = 1 / ||a - sum c_l q_l|| (a squared norm below 1e-10 ||a||^2 ends this recovery),
+// q = gamma (a - sum c_l q_l), a_j = gamma <a, r>, r <- r - a_j q.  The coefficients x follow once, at the end of the step.
+// The orthogonal vectors q_l of the earlier picks are fetched into shared memory in one trip, before anything else; a pick is
+// then four block barriers and j + 1 multiply-adds per row, all fp64, with no conversion in a loop (the inverse-Cholesky form
+// on the stored binary16 columns took 10 to 24 us per pick at k_c = 217).
+constexpr int kPickMaxThreads = 256;
 
 struct PickSmem {
-    double gv[kChunkMaxS], cv[kChunkMaxS], xs[kChunkMaxS];
-    double red[2][kPickThreads / 32];
-    double csq;
+    double cs[kChunkMaxS];
+    double cdot[kRescoreCap], cn2[kRescoreCap];
+    double red[kPickMaxThreads / 32];
+    float fred[kPickMaxThreads / 32];
     uint32_t cidx[kRescoreCap];
     int n_c;
-    float fred[kPickThreads / 32];
 };
 
-// What the update of a pick reads of the recovery's state, fetched in one round trip (pick_stage), lives in dynamic
-// shared memory sized by s_c and k_c (pick_dyn_bytes), so that small problems keep many blocks per SM:
-// F [s][s], r [k], y [k], x0 [s] as doubles, then the columns z [s * k + 2] (they start at z[0] or z[1]: see pick_columns).
-struct PickDyn { double* F; double* r; double* y; double* x0; uint16_t* z; };
-
-__device__ __forceinline__ PickDyn pick_dyn(const ChunkArgs& a) {
-    extern __shared__ double pick_mem[];
-    PickDyn d;
-    d.F = pick_mem; d.r = d.F + a.s * a.s; d.y = d.r + a.k; d.x0 = d.y + a.k;
-    d.z = reinterpret_cast<uint16_t*>(d.x0 + a.s);
-    return d;
+// dynamic shared memory: residual r [k], new column a [k], q [j][k]
+__device__ __forceinline__ double* pick_mem() {
+    extern __shared__ __align__(16) double pick_dyn_mem[];
+    return pick_dyn_mem;
 }
+size_t pick_dyn_bytes(int s, int k) { return (size_t)(s + 1) * k * sizeof(double); }
+int pick_threads(int k) { return k <= 32 ? 64 : (k <= 128 ? 128 : kPickMaxThreads); }
 
-size_t pick_dyn_bytes(int s, int k) {
-    return (size_t)(s * s + 2 * k + s) * sizeof(double) + ((size_t)(s * k + 2) * sizeof(uint16_t) + 7) / 8 * 8;
-}
-
-// Copies the state that pick j of a recovery reads (the j earlier columns, F, x, y and the residual) into shared memory.
-// All loads are independent of one another, so they cost one trip to global memory instead of one per phase of the update.
-// A block-wide barrier has to follow before pick_finish reads them.
-// The staged columns keep the position inside a 32-bit word that they have in global memory, so that they can be copied
-// word by word.
-__device__ __forceinline__ uint16_t* pick_columns(const PickDyn& dy, const uint16_t* zs) {
-    return dy.z + (((uintptr_t)zs >> 1) & 1u);
-}
-
+// the vectors of the earlier picks and the residual: independent loads, one trip to global memory.  A block-wide barrier has to
+// follow before pick_finish reads them.
 __device__ __forceinline__ void pick_stage(const ChunkArgs& a, const ChunkRef& ref, int m, int j) {
-    const int t = threadIdx.x, k = a.k, s = a.s;
-    const PickDyn dy = pick_dyn(a);
-    const uint16_t* zs = ref.zsel + (size_t)m * s * k;
-    {
-        uint16_t* zsh = pick_columns(dy, zs);
-        const int n = j * k, first = (int)(zsh - dy.z);               // elements before the first whole word: 0 or 1
-        if (n > 0) {
-            const int words = (n - first) / 2;
-            const uint32_t* src = reinterpret_cast<const uint32_t*>(zs + first);
-            uint32_t* dst = reinterpret_cast<uint32_t*>(zsh + first);
-            for (int w = t; w < words; w += kPickThreads) dst[w] = src[w];
-            if (t == 0 && first) zsh[0] = zs[0];
-            if (t == 1 && first + 2 * words < n) zsh[n - 1] = zs[n - 1];
-        }
-    }
-    const double* F = ref.F + (size_t)m * s * s;
-    for (int e = t; e < j * j; e += kPickThreads) {
-        const int l = e / j, i = e - l * j;
-        dy.F[l * s + i] = F[(size_t)l * s + i];
-    }
-    if (t < j) dy.x0[t] = ref.x[(size_t)m * s + t];
-    const double* r = ref.r64 + (size_t)m * k;
-    const double* y = ref.y64 + (size_t)m * k;
-    for (int row = t; row < k; row += kPickThreads) { dy.r[row] = r[row]; dy.y[row] = y[row]; }
-}
-
-// sums of two values over the block; every thread receives both
-__device__ __forceinline__ void pick_sum2(PickSmem& sh, double& a, double& b) {
-    a = warp_sum_d(a); b = warp_sum_d(b);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) { sh.red[0][threadIdx.x >> 5] = a; sh.red[1][threadIdx.x >> 5] = b; }
-    __syncthreads();
-    a = 0.0; b = 0.0;
-#pragma unroll
-    for (int w = 0; w < kPickThreads / 32; ++w) { a += sh.red[0][w]; b += sh.red[1][w]; }
+    const int k = a.k;
+    double* r = pick_mem();
+    double* q = r + 2 * k;
+    const double* src = ref.qb + (size_t)m * a.s * k;
+    for (int e = threadIdx.x; e < j * k; e += blockDim.x) q[e] = src[e];
+    const double* rg = ref.r64 + (size_t)m * k;
+    for (int row = threadIdx.x; row < k; row += blockDim.x) r[row] = rg[row];
 }
 
 // largest value over the block; every thread receives it
 __device__ __forceinline__ float pick_max(PickSmem& sh, float v) {
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    const unsigned int key = v >= 0.0f ? __float_as_uint(v) + 1u : 0u;
+    const unsigned int w = __reduce_max_sync(0xffffffffu, key);
+    const int lane = threadIdx.x & 31, warps = blockDim.x >> 5;
     __syncthreads();
-    if ((threadIdx.x & 31) == 0) sh.fred[threadIdx.x >> 5] = v;
+    if (lane == 0) sh.fred[threadIdx.x >> 5] = __uint_as_float(w);
     __syncthreads();
-    v = sh.fred[0];
-#pragma unroll
-    for (int w = 1; w < kPickThreads / 32; ++w) v = fmaxf(v, sh.fred[w]);
-    return v;
+    const unsigned int m = __reduce_max_sync(0xffffffffu, lane < warps ? __float_as_uint(sh.fred[lane]) : 0u);
+    return m ? __uint_as_float(m - 1u) : -1.0f;
 }
 
 // the decision among the nc candidates in sh.cidx and the update of the recovery `res` with the winner as pick j
-// (all kPickThreads threads of the block; nc is the same in every thread; pick_stage has run for this recovery)
+// (all threads of the block; nc is the same in every thread; pick_stage has run for this recovery)
 __device__ void pick_finish(const ChunkArgs& a, const ChunkRef& ref, PickSmem& sh, int res, int j, int nc) {
-    double* gv = sh.gv; double* cv = sh.cv; double* xs = sh.xs;
-    const uint32_t* cidx = sh.cidx;
-    const int m = res & 1, t = threadIdx.x, lane = t & 31, warp = t >> 5, k = a.k, s = a.s;
-    double* r = ref.r64 + (size_t)m * k;
-    const PickDyn dy = pick_dyn(a);
-    const double* y = dy.y;
+    const int m = res & 1, t = threadIdx.x, lane = t & 31, warp = t >> 5, warps = blockDim.x >> 5, k = a.k, s = a.s;
     if (nc == 0) {                                                   // no column left to pick (d/c = iterations made)
         if (t == 0) { ref.cnt->stopped[m] = 1; ref.cnt->done[m] = j; }
         return;
     }
-    __syncthreads();                                                 // the staged state is complete
-    // fp64 scores of the candidates
-    double best_sc = -1.0, best_dot = 0.0, best_n2 = 1.0;
-    uint32_t best_idx = kNoColumn;
-    for (int c = 0; c < nc; ++c) {
-        const uint32_t idx = cidx[c];
-        const ColKey key = column_key(a.seed_lo, a.seed_hi, idx);
+    double* r = pick_mem();
+    double* an = r + k;
+    double* qs = an + k;
+    __syncthreads();                                                 // the staged state and the candidates are complete
+    // exact scores: warp = one candidate; the first one's column is kept
+    for (int c = warp; c < nc; c += warps) {
+        const ColKey key = column_key(a.seed_lo, a.seed_hi, sh.cidx[c]);
         double dot = 0.0, n2 = 0.0;
-        for (int row = 2 * t; row < k; row += 2 * kPickThreads) {
-            const float2 zz = half2_bits_to_float2(z_pair_from_word(key.ck + (uint32_t)(row >> 1) * key.mk));
-            dot += (double)zz.x * dy.r[row];
-            n2 += (double)zz.x * (double)zz.x;
-            if (row + 1 < k) { dot += (double)zz.y * dy.r[row + 1]; n2 += (double)zz.y * (double)zz.y; }
+        for (int row = 2 * lane; row < k; row += 64) {
+            const float2 z = half2_bits_to_float2(z_pair_from_word(key.ck + (uint32_t)(row >> 1) * key.mk));
+            const double z0 = a.sigma * (double)z.x, z1 = a.sigma * (double)z.y;
+            dot = fma(z0, r[row], dot); n2 = fma(z0, z0, n2);
+            if (c == 0) an[row] = z0;
+            if (row + 1 < k) { dot = fma(z1, r[row + 1], dot); n2 = fma(z1, z1, n2); if (c == 0) an[row + 1] = z1; }
         }
-        pick_sum2(sh, dot, n2);
-        const double sc = n2 > 0.0 ? dot * dot / n2 : 0.0;
-        if (sc > best_sc || (sc == best_sc && idx < best_idx)) { best_sc = sc; best_idx = idx; best_dot = dot; best_n2 = n2; }
+        dot = warp_sum_d(dot); n2 = warp_sum_d(n2);
+        if (lane == 0) { sh.cdot[c] = dot; sh.cn2[c] = n2; }
     }
-    // the new column, binary16 bits (exact): kept in the state and beside the staged ones
-    uint16_t* zs = ref.zsel + (size_t)m * s * k;
-    uint16_t* zsh = pick_columns(dy, zs);
-    double* F = ref.F + (size_t)m * s * s;
-    double* xg = ref.x + (size_t)m * s;
+    __syncthreads();
+    int win = 0;
     {
-        const ColKey key = column_key(a.seed_lo, a.seed_hi, best_idx);
-        uint16_t* znew = zs + (size_t)j * k;
-        for (int row = 2 * t; row < k; row += 2 * kPickThreads) {
-            const uint32_t z2 = z_pair_from_word(key.ck + (uint32_t)(row >> 1) * key.mk);
-            znew[row] = (uint16_t)(z2 & 0xFFFFu);
-            zsh[j * k + row] = (uint16_t)(z2 & 0xFFFFu);
-            if (row + 1 < k) { znew[row + 1] = (uint16_t)(z2 >> 16); zsh[j * k + row + 1] = (uint16_t)(z2 >> 16); }
+        double best = -1.0;
+        for (int c = 0; c < nc; ++c) {
+            const double sc = sh.cn2[c] > 0.0 ? sh.cdot[c] * sh.cdot[c] / sh.cn2[c] : 0.0;
+            if (sc > best || (sc == best && sh.cidx[c] < sh.cidx[win])) { best = sc; win = c; }
         }
     }
-    __syncthreads();
-    const double sig2 = a.sigma * a.sigma;
-    const uint16_t* znew = zsh + j * k;
-    for (int l = warp; l < j; l += kPickThreads / 32) {              // g = A_Lambda^T a_new, one earlier column per warp
-        const uint16_t* zl = zsh + l * k;
-        double acc = 0.0;
-        for (int row = lane; row < k; row += 32) acc += (double)(half_bits_to_float(zl[row]) * half_bits_to_float(znew[row]));
-        acc = warp_sum_d(acc);
-        if (lane == 0) gv[l] = sig2 * acc;
+    const uint32_t col = sh.cidx[win];
+    const double dot = sh.cdot[win], n2 = sh.cn2[win];
+    if (win != 0) {
+        const ColKey key = column_key(a.seed_lo, a.seed_hi, col);
+        for (int row = t; row < k; row += blockDim.x) an[row] = a.sigma * (double)z_at(key, (uint32_t)row);
+        __syncthreads();
     }
-    __syncthreads();
-    if (warp == 0) {
-        double csq = 0.0;
-        if (lane < j) {                                              // c = F^T g (F upper triangular, F(l, i) at F[l*s + i])
-            double acc = 0.0;
-            for (int l = 0; l <= lane; ++l) acc += dy.F[l * s + lane] * gv[l];
-            cv[lane] = acc;
-            csq = acc * acc;
+    // c_l = <q_l, a>: warp = two vectors at a time
+    for (int l = warp; l < j; l += 2 * warps) {
+        const int l2 = l + warps < j ? l + warps : l;
+        double c0 = 0.0, c1 = 0.0;
+        for (int row = lane; row < k; row += 32) {
+            const double x = an[row];
+            c0 = fma(qs[l * k + row], x, c0); c1 = fma(qs[l2 * k + row], x, c1);
         }
-        csq = warp_sum_d(csq);
-        if (lane == 0) sh.csq = csq;
+        c0 = warp_sum_d(c0); c1 = warp_sum_d(c1);
+        if (lane == 0) { sh.cs[l] = c0; if (l2 != l) sh.cs[l2] = c1; }
     }
     __syncthreads();
-    const double gnn = sig2 * best_n2;
-    const double piv = gnn - sh.csq;
-    if (!(piv > 1e-10 * gnn)) {                                      // dependent column: this recovery ends with j picks
+    double csq = lane < j ? sh.cs[lane] * sh.cs[lane] : 0.0;         // (j < 32)
+    csq = warp_sum_d(csq);
+    const double piv = n2 - csq;
+    if (!(piv > 1e-10 * n2)) {                                       // dependent column: this recovery ends with j picks
         if (t == 0) {
             ref.cnt->stopped[m] = 1; ref.cnt->done[m] = j;
             atomicOr(&ref.cnt->status, (unsigned int)SGC_STATUS_DEPENDENT_COLUMN);
         }
         return;
     }
-    const double gamma = 1.0 / sqrt(piv);
-    const double aj = gamma * a.sigma * best_dot;
-    if (warp == 0) {
-        double fj = 0.0;                                             // this lane's entry of the new column of F
-        if (lane < j) {
-            double acc = 0.0;
-            for (int l = lane; l < j; ++l) acc += dy.F[lane * s + l] * cv[l];
-            fj = -gamma * acc;
-            F[(size_t)lane * s + j] = fj;
-        } else if (lane == j) {
-            fj = gamma;
-            F[(size_t)j * s + j] = fj;
-        }
-        if (lane <= j) {
-            const double xo = lane < j ? dy.x0[lane] : 0.0;
-            const double xn = xo + aj * fj;
-            xg[lane] = xn;
-            xs[lane] = xn;
-        }
-        if (lane == 0) { ref.acoef[(size_t)m * s + j] = aj; ref.lam[(size_t)m * s + j] = best_idx; }
-    }
-    __syncthreads();
-    double rn2 = 0.0, unused = 0.0;
-    for (int row = t; row < k; row += kPickThreads) {                // r = y - A_Lambda x
-        double acc = 0.0;
-        for (int l = 0; l <= j; ++l) acc += xs[l] * (double)half_bits_to_float(zsh[l * k + row]);
-        const double rv = y[row] - a.sigma * acc;
-        r[row] = rv;
+    const double gamma = rsqrt(piv), aj = gamma * dot;
+    double rn2 = 0.0;
+    for (int row = t; row < k; row += blockDim.x) {
+        double v0 = 0.0, v1 = 0.0;
+        int l = 0;
+#pragma unroll 4
+        for (; l + 1 < j; l += 2) { v0 = fma(sh.cs[l], qs[l * k + row], v0); v1 = fma(sh.cs[l + 1], qs[(l + 1) * k + row], v1); }
+        if (l < j) v0 = fma(sh.cs[l], qs[l * k + row], v0);
+        const double q = gamma * (an[row] - (v0 + v1));
+        ref.qb[((size_t)m * s + j) * k + row] = q;
+        const double rv = r[row] - aj * q;
+        ref.r64[(size_t)m * k + row] = rv;
         a.r32[(size_t)res * a.kp + row] = (float)rv;
-        rn2 += rv * rv;
+        rn2 = fma(rv, rv, rn2);
     }
-    pick_sum2(sh, rn2, unused);
+    if (t < j) ref.crow[((size_t)m * s + j) * s + t] = sh.cs[t];
     if (t == 0) {
-        ref.rnorm[(size_t)m * s + j] = sqrt(rn2);
+        a.lam[(size_t)res * s + j] = col;
+        ref.gam[(size_t)m * s + j] = gamma; ref.acoef[(size_t)m * s + j] = aj; ref.lam[(size_t)m * s + j] = col;
         ref.cnt->done[m] = j + 1;
+    }
+    rn2 = warp_sum_d(rn2);
+    if (lane == 0) sh.red[warp] = rn2;
+    __syncthreads();
+    if (t == 0) {
+        double v = 0.0;
+        for (int w = 0; w < warps; ++w) v += sh.red[w];
+        ref.rnorm[(size_t)m * s + j] = sqrt(v);
     }
 }
 
 // SIMT route: the candidates are the columns that phase A left within 2e-3 (relative) of the best fp32 score.
 // only != nullptr: a second chance for the recoveries that the tensor-core route marked unresolved; skipped unless *gate
 // names this iteration.
-__global__ void __launch_bounds__(kPickThreads) k_chunk_pick(ChunkArgs a, int iter, const int* gate, const unsigned char* only) {
+__global__ void __launch_bounds__(kPickMaxThreads) k_chunk_pick(ChunkArgs a, int iter, const int* gate, const unsigned char* only) {
     __shared__ PickSmem sh;
+    const int res = blockIdx.x, m = res & 1, t = threadIdx.x, j = iter;
+    const ChunkRef ref = a.table[res >> 1];
+    // what earlier picks left is complete when this grid starts (phase A, the kernel before this one, has waited for the last
+    // pick, and lets this one's blocks in only then), so it can be fetched before waiting for phase A itself
+    if (gate == nullptr) pick_stage(a, ref, m, j);
+    if (t == 0) sh.n_c = 0;
     after_previous_kernel(a.early);
     if (gate != nullptr && *gate != a.epoch0 + iter) return;
-    const int res = blockIdx.x, m = res & 1, t = threadIdx.x;
     if (only != nullptr && !only[res]) return;
-    const ChunkRef ref = a.table[res >> 1];
     if (ref.cnt->stopped[m]) return;
-    const int j = iter;
-    pick_stage(a, ref, m, j);                                    // (pick_max's barriers come before anything reads it)
+    if (gate != nullptr) pick_stage(a, ref, m, j);
     const Cand* cc = a.cand + (size_t)res * a.splits * 2;
     const int n_entries = a.splits * 2;
     float mx = -1.0f;
-    for (int e = t; e < n_entries; e += kPickThreads) if (cc[e].idx != kNoColumn) mx = fmaxf(mx, cc[e].score);
-    if (t == 0) sh.n_c = 0;
+    Cand first[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        first[u].score = -1.0f; first[u].idx = kNoColumn;
+        const int e = t + u * (int)blockDim.x;
+        if (e < n_entries) { const float2 f = __ldcg(reinterpret_cast<const float2*>(cc + e)); first[u].score = f.x; first[u].idx = __float_as_uint(f.y); }
+        if (first[u].idx != kNoColumn) mx = fmaxf(mx, first[u].score);
+    }
+    for (int e = t + 2 * (int)blockDim.x; e < n_entries; e += blockDim.x) if (cc[e].idx != kNoColumn) mx = fmaxf(mx, cc[e].score);
     mx = pick_max(sh, mx);                                          // (its barriers also publish n_c = 0)
     const float thr = mx - 2e-3f * fabsf(mx);
-    for (int e = t; e < n_entries; e += kPickThreads) {
-        const Cand c = cc[e];
+    auto offer = [&](const Cand& c) {
         if (c.idx != kNoColumn && c.score >= 0.0f && c.score >= thr) {
             const int slot = atomicAdd(&sh.n_c, 1);
             if (slot < kRescoreCap) sh.cidx[slot] = c.idx;
         }
-    }
+    };
+    offer(first[0]); offer(first[1]);
+    for (int e = t + 2 * (int)blockDim.x; e < n_entries; e += blockDim.x) offer(cc[e]);
     __syncthreads();
     int nc = sh.n_c;
     if (nc > kRescoreCap) {
@@ -587,7 +688,7 @@ __global__ void __launch_bounds__(64) k_chunk_rt(ChunkArgs a, int n_rows, int it
     }
 }
 
-__global__ void __launch_bounds__(kPickThreads) k_chunk_pick_rep(ChunkArgs a, int iter) {
+__global__ void __launch_bounds__(kPickMaxThreads) k_chunk_pick_rep(ChunkArgs a, int iter) {
     __shared__ PickSmem sh;
     const int res = blockIdx.x, m = res & 1, t = threadIdx.x, j = iter;
     const ChunkRef ref = a.table[res >> 1];
@@ -600,7 +701,7 @@ __global__ void __launch_bounds__(kPickThreads) k_chunk_pick_rep(ChunkArgs a, in
     const uint32_t* sup = ref.lam + (size_t)m * a.s;
     float smax = -1.0f;
     if (!give_up) {
-        for (unsigned int e = t; e < count; e += kPickThreads) {
+        for (unsigned int e = t; e < count; e += blockDim.x) {
             const uint2 v = rp[e];
             bool taken = false;
             for (int q = 0; q < j; ++q) taken |= (sup[q] == v.x);
@@ -619,7 +720,7 @@ __global__ void __launch_bounds__(kPickThreads) k_chunk_pick_rep(ChunkArgs a, in
     if (!give_up) {
         if (t == 0) sh.n_c = 0;
         __syncthreads();
-        for (unsigned int e = t; e < count; e += kPickThreads) {
+        for (unsigned int e = t; e < count; e += blockDim.x) {
             const uint2 v = rp[e];
             if (__uint_as_float(v.y) < lo) continue;
             bool taken = false;
@@ -641,53 +742,66 @@ __global__ void __launch_bounds__(kPickThreads) k_chunk_pick_rep(ChunkArgs a, in
     pick_finish(a, ref, sh, res, j, sh.n_c);
 }
 
-// ---- a5: Eq. (8) on the common support of the two recoveries of a chunk, one warp per chunk -------------------
-__global__ void __launch_bounds__(32) k_chunk_scatter(ChunkArgs a, float* __restrict__ weight, double alpha, double eps, double lr) {
-    __shared__ uint32_t vidx[kChunkMaxS];
-    __shared__ double vval[kChunkMaxS];
-    __shared__ int flag[kChunkMaxS];
-    const int ch = blockIdx.x, lane = threadIdx.x, s = a.s;
+// ---- a5: coefficients and Eq. (8) on the common support of the two recoveries of a chunk, one block of two warps per chunk ----
+__global__ void __launch_bounds__(64) k_chunk_scatter(ChunkArgs a, float* __restrict__ weight, double alpha, double eps, double lr) {
+    __shared__ uint32_t vidx[kChunkMaxS], lam_s[2][kChunkMaxS];
+    __shared__ double x_s[2][kChunkMaxS];
+    extern __shared__ double rows_s[];                                // [2][s][s]
+    after_previous_kernel(0);
+    const int ch = blockIdx.x, lane = threadIdx.x & 31, m = threadIdx.x >> 5, s = a.s;
     const ChunkRef ref = a.table[ch];
     float* W = weight + (size_t)ch * a.dc;
-    const int nM = ref.cnt->done[0], nV = ref.cnt->done[1];
-    uint32_t* lam = ref.lam;
-    double* x = ref.x;
-    if (lane < s) {                                                  // unpicked slots read as "none"
-        if (lane >= nM) { lam[lane] = kNoColumn; x[lane] = 0.0; }
-        if (lane >= nV) { lam[s + lane] = kNoColumn; x[s + lane] = 0.0; }
-        flag[lane] = 0;
+    const int done[2] = {ref.cnt->done[0], ref.cnt->done[1]}, n = done[m];
+    // warp = recovery, lane = pick: x_l = gamma_l (a_l - sum_{j > l} c^(j)_l x_j), last pick first
+    {
+        double* rows = rows_s + (size_t)m * s * s;
+        {
+            const double* src = ref.crow + (size_t)m * s * s;
+#pragma unroll 8
+            for (int e = lane; e < n * s; e += 32) rows[e] = src[e];
+        }
+        const uint32_t col = lane < n ? ref.lam[(size_t)m * s + lane] : kNoColumn;
+        double acc = lane < n ? ref.acoef[(size_t)m * s + lane] : 0.0, x = 0.0;
+        const double gam = lane < n ? ref.gam[(size_t)m * s + lane] : 0.0;
+        __syncwarp();
+        for (int j = n - 1; j >= 0; --j) {
+            const double xj = __shfl_sync(0xffffffffu, gam * acc, j);
+            if (lane == j) x = xj;
+            if (lane < j) acc = fma(-rows[(size_t)j * s + lane], xj, acc);
+        }
+        x_s[m][lane] = x; lam_s[m][lane] = col;
+        if (lane < s) { ref.x[(size_t)m * s + lane] = x; if (lane >= n) ref.lam[(size_t)m * s + lane] = kNoColumn; }   // unpicked slots read as "none"
     }
-    __syncwarp();
-    bool mis = false, neg = false;
-    if (lane < nM) {
-        const uint32_t li = lam[lane];
+    __syncthreads();
+    if (m != 0) return;
+    bool mis = false, neg = false, upd = false;
+    double val = 0.0;
+    const uint32_t mine = lam_s[0][lane];
+    if (lane < done[0]) {
         int hit = -1;
-        for (int b = 0; b < nV; ++b) if (lam[s + b] == li) { hit = b; break; }
+        for (int b = 0; b < done[1]; ++b) if (lam_s[1][b] == mine) { hit = b; break; }
         if (hit < 0) mis = true;
         else {
-            const double xv = x[s + hit];
+            const double xv = x_s[1][hit];
             if (!(xv > 0.0)) neg = true;
-            else {
-                const double N = alpha * x[lane] / (sqrt(xv) + eps);
-                vidx[lane] = li; vval[lane] = lr * N; flag[lane] = 1;
-            }
+            else { val = lr * (alpha * x_s[0][lane] / (sqrt(xv) + eps)); upd = true; }
         }
     }
+    vidx[lane] = upd ? mine : kNoColumn;
     __syncwarp();
     const int n_mis = __popc(__ballot_sync(0xffffffffu, mis)), n_neg = __popc(__ballot_sync(0xffffffffu, neg));
-    const bool valid = lane < nM && flag[lane];
-    const int n_valid = __popc(__ballot_sync(0xffffffffu, valid));
-    if (valid) {
+    const int n_valid = __popc(__ballot_sync(0xffffffffu, upd));
+    if (upd) {
         int rank = 0;
-        for (int b = 0; b < nM; ++b) if (flag[b] && vidx[b] < vidx[lane]) ++rank;
-        ref.upd_idx[rank] = vidx[lane];
-        ref.upd_val[rank] = vval[lane];
-        W[vidx[lane]] = (float)((double)W[vidx[lane]] - vval[lane]);
+        for (int b = 0; b < done[0]; ++b) rank += vidx[b] < mine ? 1 : 0;
+        ref.upd_idx[rank] = mine;
+        ref.upd_val[rank] = val;
+        W[mine] = (float)((double)W[mine] - val);
     }
     if (lane == 0) {
         ref.cnt->n_upd = n_valid; ref.cnt->mismatch = n_mis; ref.cnt->negv = n_neg;
         unsigned int bits = 0;
-        if (n_mis > 0 || nM != nV) bits |= (unsigned int)SGC_STATUS_SUPPORT_MISMATCH;
+        if (n_mis > 0 || done[0] != done[1]) bits |= (unsigned int)SGC_STATUS_SUPPORT_MISMATCH;
         if (n_neg > 0) bits |= (unsigned int)SGC_STATUS_NEGATIVE_V;
         if (bits) atomicOr(&ref.cnt->status, bits);
     }
@@ -712,8 +826,8 @@ unsigned long long list_key(sgc_state* const* sts, int c) {
 
 template <int KP>
 cudaError_t corr_setup(size_t* smem_out) {
-    constexpr int TC = corr_tile(KP);
-    const size_t smem = (size_t)(TC * (KP + 4 * corr_ks(KP)) + TC + kCorrBlock) * sizeof(float);
+    constexpr int TC = corr_tile(KP), KB = corr_kb(KP);
+    const size_t smem = (size_t)(TC / 16) * KB * 512 + (size_t)(TC + KB * TC) * sizeof(float);
     *smem_out = smem;
     return cudaFuncSetAttribute(k_chunk_corr<KP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
@@ -777,6 +891,7 @@ cudaError_t ensure_ws(sgc_state* const* sts, int c) {
     const size_t b_table = up((size_t)c * sizeof(ChunkRef));
     const size_t b_r32 = up((size_t)2 * c * ws->kp * sizeof(float));
     const size_t b_cand = up((size_t)2 * c * splits * 2 * sizeof(Cand));
+    const size_t b_lam = up((size_t)2 * c * st0->s * sizeof(uint32_t));
     // tensor-core route: worth it from k_c = 33 on; bounded by its report lists (n_rows * 16 KB)
     // (a pass has some 40 us of fixed cost: below ~1e9 multiply-adds per iteration the fp32 kernel is quicker)
     ws->tensor = ws->kp >= 64 && 2 * c <= 2048 && (double)st0->d * ws->kp * 2.0 * c >= 1.0e9;
@@ -793,13 +908,14 @@ cudaError_t ensure_ws(sgc_state* const* sts, int c) {
         b_un = up((size_t)2 * c);
         b_flags = 256;
     }
-    cudaError_t e = cudaMalloc(&ws->base, b_table + b_r32 + b_cand + b_rt + 3 * b_row + b_rep + b_norm + b_rn + b_un + b_flags);
+    cudaError_t e = cudaMalloc(&ws->base, b_table + b_r32 + b_cand + b_lam + b_rt + 3 * b_row + b_rep + b_norm + b_rn + b_un + b_flags);
     if (e != cudaSuccess) { delete ws; return e; }
     unsigned char* base = static_cast<unsigned char*>(ws->base);
     size_t off = 0;
     ws->table = reinterpret_cast<ChunkRef*>(base + off); off += b_table;
     ws->r32 = reinterpret_cast<float*>(base + off); off += b_r32;
     ws->cand = reinterpret_cast<Cand*>(base + off); off += b_cand;
+    ws->lam = reinterpret_cast<uint32_t*>(base + off); off += b_lam;
     if (ws->tensor) {
         ws->rt = reinterpret_cast<uint16_t*>(base + off); off += b_rt;
         ws->tau = reinterpret_cast<float*>(base + off); off += b_row;
@@ -830,7 +946,7 @@ cudaError_t ensure_ws(sgc_state* const* sts, int c) {
         ChunkRef& r = host[i];
         r.M = st->M; r.V = st->V; r.p = st->p; r.q = st->q; r.y64 = st->y64; r.r64 = st->r64;
         r.sel_idx = st->sel_idx; r.sel_val = st->sel_val;
-        r.zsel = st->zsel; r.lam = st->lam; r.F = st->F; r.acoef = st->acoef; r.x = st->x; r.rnorm = st->rnorm;
+        r.qb = st->q_basis; r.lam = st->lam; r.crow = st->F; r.gam = st->gam; r.acoef = st->acoef; r.x = st->x; r.rnorm = st->rnorm;
         r.upd_idx = st->upd_idx; r.upd_val = st->upd_val; r.cnt = st->cnt; r.ctl = st->ctl;
     }
     e = cudaMemcpy(ws->table, host.data(), (size_t)c * sizeof(ChunkRef), cudaMemcpyHostToDevice);
@@ -878,7 +994,7 @@ cudaError_t launch_chunked_batch(sgc_state* const* sts, int c, const float* grad
     a.table = ws->table; a.c = c; a.k = st0->k; a.s = st0->s; a.kp = ws->kp; a.dc = st0->d;
     a.seed_lo = (uint32_t)(st0->seed & 0xFFFFFFFFu); a.seed_hi = (uint32_t)(st0->seed >> 32);
     a.sigma = (double)(float)(1.0 / sqrt((double)st0->k));
-    a.r32 = ws->r32; a.cand = ws->cand; a.splits = ws->splits;
+    a.r32 = ws->r32; a.cand = ws->cand; a.lam = ws->lam; a.splits = ws->splits;
     {
         const int groups = (2 * c + corr_group(ws->kp) - 1) / corr_group(ws->kp);
         a.early = (ws->splits * groups <= st0->sm_count && 2 * c <= st0->sm_count) ? 1 : 0;
@@ -897,13 +1013,23 @@ cudaError_t launch_chunked_batch(sgc_state* const* sts, int c, const float* grad
     const double b1 = (double)st0->beta1, b2 = (double)st0->beta2;
     const double c1 = 1.0 - pow(b1, (double)st0->t), c2 = 1.0 - pow(b2, (double)st0->t);
     const int s = st0->s;
-    if (s <= 1) k_chunk_front<1><<<c, kFrontThreads, 0, stream>>>(a, grad, b1, b2, c1, c2);
-    else if (s <= 2) k_chunk_front<2><<<c, kFrontThreads, 0, stream>>>(a, grad, b1, b2, c1, c2);
-    else if (s <= 4) k_chunk_front<4><<<c, kFrontThreads, 0, stream>>>(a, grad, b1, b2, c1, c2);
-    else if (s <= 8) k_chunk_front<8><<<c, kFrontThreads, 0, stream>>>(a, grad, b1, b2, c1, c2);
-    else if (s <= 16) k_chunk_front<16><<<c, kFrontThreads, 0, stream>>>(a, grad, b1, b2, c1, c2);
-    else k_chunk_front<32><<<c, kFrontThreads, 0, stream>>>(a, grad, b1, b2, c1, c2);
+    {
+        // blocks per chunk: up to two blocks per SM, at least four vectors per thread
+        int split = 1;
+        while (split < kFrontMaxSplit && 2 * split * c <= 2 * st0->sm_count && st0->d >= (int64_t)2 * split * kFrontThreads * 16) split *= 2;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned int)(c * split)); cfg.blockDim = dim3(kFrontThreads); cfg.stream = stream;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)split; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr; cfg.numAttrs = 1;
+        e = cudaLaunchKernelEx(&cfg, k_chunk_front, a, grad, b1, b2, c1, c2);
+        if (e != cudaSuccess) return e;
+    }
     *launches += 1;
+    e = cudaFuncSetAttribute(k_chunk_pick, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pick_dyn_bytes(kChunkMaxS, kChunkMaxK));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_chunk_pick_rep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pick_dyn_bytes(kChunkMaxS, kChunkMaxK));
+    if (e != cudaSuccess) return e;
     size_t smem = 0;
     switch (ws->kp) {
         case 8: e = corr_setup<8>(&smem); break;
@@ -929,7 +1055,7 @@ cudaError_t launch_chunked_batch(sgc_state* const* sts, int c, const float* grad
                                 st0->sm_count, stream, nullptr, nullptr, 0, st0->wait_limit_ns);
             }
             if (e != cudaSuccess) return e;
-            k_chunk_pick_rep<<<2 * c, kPickThreads, pick_dyn_bytes(s, st0->k), stream>>>(a, iter);
+            k_chunk_pick_rep<<<2 * c, pick_threads(st0->k), pick_dyn_bytes(s, st0->k), stream>>>(a, iter);
             *launches += 2 + ws->passes;
             gate = ws->flags;
         }
@@ -942,14 +1068,18 @@ cudaError_t launch_chunked_batch(sgc_state* const* sts, int c, const float* grad
             default: e = corr_launch<256>(a, iter, smem, stream, gate); break;
         }
         {
-            ChainedLaunch l(dim3((unsigned int)(2 * c)), dim3(kPickThreads), pick_dyn_bytes(s, st0->k), stream);
+            ChainedLaunch l(dim3((unsigned int)(2 * c)), dim3(pick_threads(st0->k)), pick_dyn_bytes(s, st0->k), stream);
             const unsigned char* only = gate ? ws->unresolved : nullptr;
             if (e == cudaSuccess) e = cudaLaunchKernelEx(&l.cfg, k_chunk_pick, a, iter, gate, only);
         }
         if (e != cudaSuccess) return e;
         *launches += 2;
     }
-    k_chunk_scatter<<<c, 32, 0, stream>>>(a, weight, (double)st0->alpha, (double)st0->eps, (double)st0->lr);
+    {
+        ChainedLaunch l(dim3((unsigned int)c), dim3(64), (size_t)2 * s * s * sizeof(double), stream);
+        e = cudaLaunchKernelEx(&l.cfg, k_chunk_scatter, a, weight, (double)st0->alpha, (double)st0->eps, (double)st0->lr);
+        if (e != cudaSuccess) return e;
+    }
     *launches += 1;
     return cudaGetLastError();
 }

@@ -209,7 +209,7 @@ struct Counters {
 struct ChunkRef {
     float* M; float* V; double* p; double* q; double* y64; double* r64;
     uint32_t* sel_idx; float* sel_val;
-    uint16_t* zsel; uint32_t* lam; double* F; double* acoef; double* x; double* rnorm;
+    double* qb; uint32_t* lam; double* crow; double* gam; double* acoef; double* x; double* rnorm;
     uint32_t* upd_idx; double* upd_val; Counters* cnt; SpecCtl* ctl;
 };
 // workspace of the batched chunk path, owned by the first state of the chunk list it was built for
@@ -218,6 +218,7 @@ struct ChunkWs {
     ChunkRef* table;            // [c]
     float* r32;                 // [2c][kp] residuals of all streams (stream = 2 * chunk + moment), rows padded to kp
     Cand* cand;                 // [2c][splits][2] best two columns of every column split, per stream
+    uint32_t* lam;              // [2c][s] supports of all recoveries
     int c, kp, splits;
     unsigned long long key;     // names the chunk list (its state pointers) the table was built from
     // tensor-core route of the correlation (k_c > 32): the residuals of all recoveries go through the screening pass
@@ -274,10 +275,9 @@ struct sgc_state {
     float2* r32;                // [k] (M^ residual, V^ residual)
     unsigned long long* sel_cand; unsigned int* sel_hist;
     float4* corr_cand;          // [2][kCorrBlocks]
-    uint16_t* zsel;             // [2][s][k] selected columns of Z as binary16 bits (chunk path only)
     uint32_t* lam;              // [2][s]
     double* q_basis;            // [2][s][k] orthogonal basis of the picked columns
-    double *F, *ccol, *acoef, *gam, *x, *rnorm;   // [2][s*s] (coefficients c by pick and by row; the chunk path keeps its F there), [2][s]
+    double *F, *ccol, *acoef, *gam, *x, *rnorm;   // [2][s*s] (coefficients c by pick and by row), [2][s]
     uint32_t* upd_idx; double* upd_val;
     sgc::Counters* cnt;
     // speculative recovery
