@@ -31,11 +31,13 @@ constexpr int kChunkMaxK = 256;
 
 struct ChunkArgs {
     const ChunkRef* table;
-    int c, k, s, kp;                     // kp: k rounded up to 8, 16, 32, 64, 128 or 256 (row stride of r32)
+    int c, k, s, kp;                     // kp: k rounded up to 8, 16, 32, 64, 128 or 256
     long long dc;                        // columns per chunk
     uint32_t seed_lo, seed_hi;
     double sigma;
-    float* r32;                          // [2c][kp]
+    uint16_t* frag;                      // [2c][2][kf] residuals as two binary16 numbers each, in operand order (see frag_place)
+    float* back;                         // [2c] what undoes the power-of-two scale of a residual
+    int kf;                              // max(kp, 16)
     Cand* cand;                          // [2c][splits][2]
     uint32_t* lam;                       // [2c][s] the supports once more, side by side (a state's own copy is an allocation of its own)
     int splits, cols_per_split;
@@ -52,6 +54,24 @@ __device__ __forceinline__ double warp_sum_d(double v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
+
+// ---- residuals as operands of k_chunk_corr ----------------------------------------------------------------
+// Position of row `row` in a residual's operand: for each 16 rows, lane q of a column group holds rows 2q, 2q + 1 and 2q + 8, 2q + 9
+// as two registers of the B operand of mma.m16n8k16.
+__device__ __forceinline__ int frag_place(int row) {
+    const int r = row & 15;
+    return (row & ~15) + ((r & 7) >> 1) * 4 + (r >> 3) * 2 + (r & 1);
+}
+// one entry (scale: a power of two that brings the residual's norm into [2^10, 2^11)): the value and what it leaves
+__device__ __forceinline__ void frag_write(const ChunkArgs& a, int res, int row, double v, double scale) {
+    const float x = (float)(v * scale);
+    const __half h = __float2half_rn(x);
+    const __half l = __float2half_rn(x - __half2float(h));
+    uint16_t* f = a.frag + (size_t)res * 2 * a.kf + frag_place(row);
+    f[0] = __half_as_ushort(h);
+    f[a.kf] = __half_as_ushort(l);
+}
+__device__ __forceinline__ double frag_scale(double rn) { return 0.125 * residual_scale(rn); }      // (residual_scale: [2^12, 2^13))
 
 // ---- a1 + a2 + a3, one block or cluster of blocks per chunk -----------------------------------------------
 // Top-s of the chunk by the key (|g| bits << 32) | ~index (unique; lowest index wins equal magnitudes).  One read of the
@@ -95,6 +115,7 @@ k_chunk_front(ChunkArgs a, const float* __restrict__ grad, double b1, double b2,
     __shared__ unsigned long long sel_key[kChunkMaxS];
     __shared__ ColKey keys[kChunkMaxS];
     __shared__ float vals[kChunkMaxS];
+    __shared__ double norms[2][kFrontThreads / 32];
     __shared__ int n_list;
     cg::cluster_group cluster = cg::this_cluster();
     const int split = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();      // split: a power of two
@@ -203,7 +224,10 @@ k_chunk_front(ChunkArgs a, const float* __restrict__ grad, double b1, double b2,
     }
     __syncthreads();
     // a2 + a3: thread = row; fp64 sums in ascending column order (the arithmetic of the one-state kernel, term by term)
-    for (int row = t; row < k; row += kFrontThreads) {
+    static_assert(kChunkMaxK <= kFrontThreads, "one row per thread");
+    double mh = 0.0, vh = 0.0;
+    if (t < k) {
+        const int row = t;
         double accp = 0.0, accq = 0.0;
         for (int i = 0; i < s; ++i) {
             const double av = a.sigma * (double)z_at(keys[i], (uint32_t)row);
@@ -217,11 +241,20 @@ k_chunk_front(ChunkArgs a, const float* __restrict__ grad, double b1, double b2,
         const float v = (float)(b2 * (double)ref.V[row] + (1.0 - b2) * accq);
         ref.M[row] = m;
         ref.V[row] = v;
-        const double mh = (double)m / c1, vh = (double)v / c2;      // bias-corrected temporaries; state stays uncorrected
+        mh = (double)m / c1; vh = (double)v / c2;                    // bias-corrected temporaries; state stays uncorrected
         ref.y64[row] = mh; ref.y64[k + row] = vh;
         ref.r64[row] = mh; ref.r64[k + row] = vh;
-        a.r32[(size_t)(2 * ch) * a.kp + row] = (float)mh;
-        a.r32[(size_t)(2 * ch + 1) * a.kp + row] = (float)vh;
+    }
+    {
+        double m2 = warp_sum_d(mh * mh), v2 = warp_sum_d(vh * vh);
+        if (lane == 0) { norms[0][warp] = m2; norms[1][warp] = v2; }
+        __syncthreads();
+        m2 = v2 = 0.0;
+#pragma unroll
+        for (int w = 0; w < kFrontThreads / 32; ++w) { m2 += norms[0][w]; v2 += norms[1][w]; }
+        const double sm = frag_scale(sqrt(m2)), sv = frag_scale(sqrt(v2));
+        if (t < k) { frag_write(a, 2 * ch, t, mh, sm); frag_write(a, 2 * ch + 1, t, vh, sv); }
+        if (t == 0) { a.back[2 * ch] = (float)(1.0 / sm); a.back[2 * ch + 1] = (float)(1.0 / sv); }
     }
 }
 
@@ -230,15 +263,15 @@ k_chunk_front(ChunkArgs a, const float* __restrict__ grad, double b1, double b2,
 // register layout of mma.m16n8k16's A operand (a row pair of a column is one register) into shared memory, with 1 / ||Z_i||,
 // and every warp multiplies it with the residuals it holds as B operands: NT tiles of four recoveries, each residual as two
 // binary16 numbers (value and remainder, 22 bits, scaled by a power of two), sums in fp32.  A lane ends up with the scores of
-// one recovery for two columns of every 16; only the best two columns per recovery leave the block; columns already in the
-// support are skipped when they show up as a new best.  (The legacy matrix instruction on purpose: with 2c residuals of k_c
+// one recovery for two columns of every 16; only the best two columns per recovery leave the block.  (The legacy matrix instruction on purpose: with 2c residuals of k_c
 // rows the tensor work is small, what bounds the kernel is generating, comparing and the launch itself, and an operand in
 // registers needs no hand-off.  With one multiply-add per instruction it took 37 us at k_c = 8, 512 recoveries, 65536
 // columns, and 22 us per iteration at k_c = 217, 128 recoveries, 2048 columns.)
 __host__ __device__ constexpr int corr_kb(int kp) { return kp / 16 > 0 ? kp / 16 : 1; }              // 16-row blocks
-__host__ __device__ constexpr int corr_nt(int kp) { return kp <= 64 ? 8 : (kp <= 128 ? 4 : 2); }     // tiles of four recoveries per warp
+__host__ __device__ constexpr int corr_nt(int kp) { return kp == 64 ? 8 : (kp <= 128 ? 4 : 2); }     // tiles of four recoveries per warp
 __host__ __device__ constexpr int corr_group(int kp) { return kCorrBlock / 32 * 4 * corr_nt(kp); }   // recoveries per block
 __host__ __device__ constexpr int corr_tile(int kp) { return kp <= 64 ? 64 : 32; }                   // columns generated at a time
+constexpr int kCorrSuper = 512;                                                                      // columns that a key can tell apart
 
 // The two kernels of an iteration are launched with programmatic stream serialization: the blocks of the next kernel may
 // become resident while this one is still running, and wait here until it has completed and its writes are visible.
@@ -268,15 +301,6 @@ __device__ __forceinline__ void mma_16816(float (&c)[4], const uint4& x, uint32_
         : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(x.x), "r"(x.y), "r"(x.z), "r"(x.w), "r"(b0), "r"(b1));
 }
 
-// two binary16 numbers of a residual pair: the values (part 0) or what they leave (part 1)
-__device__ __forceinline__ uint32_t residual_part(float x, float y, int part) {
-    const __half2 h = __floats2half2_rn(x, y);
-    if (part == 0) return *reinterpret_cast<const uint32_t*>(&h);
-    const float2 f = __half22float2(h);
-    const __half2 l = __floats2half2_rn(x - f.x, y - f.y);
-    return *reinterpret_cast<const uint32_t*>(&l);
-}
-
 // the two best columns of a recovery
 struct Best2 {
     float s1, s2; uint32_t i1, i2;
@@ -289,13 +313,13 @@ struct Best2 {
 // gate != nullptr: the launch is a fallback of the tensor-core route and returns at once unless *gate names this
 // iteration (a.epoch): the word holds the epoch of the last iteration that left a recovery unresolved.
 template <int KP>
-__global__ void __launch_bounds__(kCorrBlock) k_chunk_corr(ChunkArgs a, int iter, const int* gate) {
+__global__ void __launch_bounds__(kCorrBlock, KP <= 32 ? 2 : 1) k_chunk_corr(ChunkArgs a, int iter, const int* gate) {
     constexpr int KB = corr_kb(KP), NT = corr_nt(KP), TC = corr_tile(KP), TILES = TC / 16, WARPS = kCorrBlock / 32;
     constexpr int UNITS = TILES * KB;                                 // (16 columns, 16 rows): one warp's share of the generating
     extern __shared__ uint4 smem4[];
     uint4* zt = smem4;                                                // [TILES][KB][32] A operands
-    float* inv = reinterpret_cast<float*>(zt + TILES * KB * 32);      // [TC]
-    float* n2p = inv + TC;                                            // [KB][TC] partial ||Z_i||^2
+    float2* inv = reinterpret_cast<float2*>(zt + TILES * KB * 32);    // [TC] 1 / ||Z_i||, code of the column
+    float* n2p = reinterpret_cast<float*>(inv + TC);                  // [KB][TC] partial ||Z_i||^2
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, q = lane & 3;
     const long long col0 = (long long)blockIdx.x * a.cols_per_split;
     long long col1 = col0 + a.cols_per_split;
@@ -333,123 +357,100 @@ __global__ void __launch_bounds__(kCorrBlock) k_chunk_corr(ChunkArgs a, int iter
     // residuals as B operands: n = g of a tile is value (g even) or remainder (g odd) of recovery 4 tile + g / 2.  (Recoveries
     // that have stopped are scored like the others; k_chunk_pick does not look at them.)
     const int res0 = blockIdx.y * corr_group(KP) + warp * NT * 4;
-    uint32_t bf[NT][KB][2];
-    float back[NT];                                                   // of recovery 4 tile + q, whose scores this lane gets
-    {
-        constexpr int HB = KB * NT <= 8 ? NT : (KB >= 8 ? 1 : 8 / KB);       // tiles whose loads are in flight together
-#pragma unroll
-        for (int i0 = 0; i0 < NT; i0 += HB) {
-            float2 lo[HB][KB], hi[HB][KB];
-#pragma unroll
-            for (int i = 0; i < HB; ++i) {
-                const int res = res0 + 4 * (i0 + i) + (g >> 1);
-                const float* src = a.r32 + (size_t)(res < 2 * a.c ? res : 0) * KP + 2 * q;
-#pragma unroll
-                for (int kb = 0; kb < KB; ++kb) {
-                    lo[i][kb] = *reinterpret_cast<const float2*>(src + 16 * kb);
-                    hi[i][kb] = KP >= 16 ? *reinterpret_cast<const float2*>(src + 16 * kb + 8) : make_float2(0.0f, 0.0f);
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < HB; ++i) {
-                unsigned int m = 0u;
-#pragma unroll
-                for (int kb = 0; kb < KB; ++kb) {
-                    m = max(m, max(__float_as_uint(lo[i][kb].x) & 0x7FFFFFFFu, __float_as_uint(lo[i][kb].y) & 0x7FFFFFFFu));
-                    m = max(m, max(__float_as_uint(hi[i][kb].x) & 0x7FFFFFFFu, __float_as_uint(hi[i][kb].y) & 0x7FFFFFFFu));
-                }
-                m = max(m, __shfl_xor_sync(0xffffffffu, m, 1)); m = max(m, __shfl_xor_sync(0xffffffffu, m, 2));
-                int e = (int)(m >> 23);                               // largest entry scaled into [2^10, 2^11)
-                e = e < 20 ? 20 : (e > 250 ? 250 : e);
-                const float sc = __uint_as_float((unsigned int)(264 - e) << 23);
-#pragma unroll
-                for (int kb = 0; kb < KB; ++kb) {
-                    bf[i0 + i][kb][0] = residual_part(lo[i][kb].x * sc, lo[i][kb].y * sc, g & 1);
-                    bf[i0 + i][kb][1] = residual_part(hi[i][kb].x * sc, hi[i][kb].y * sc, g & 1);
-                }
-                back[i0 + i] = __uint_as_float((unsigned int)(__shfl_sync(0xffffffffu, e, 8 * q) - 10) << 23);
-            }
-        }
-    }
-    Best2 best[NT];
-    float least[NT];                                                  // no column at or below this can be among the best two
+    uint2 bf[NT][KB];
 #pragma unroll
     for (int i = 0; i < NT; ++i) {
-        best[i].s1 = best[i].s2 = -1.0f; best[i].i1 = best[i].i2 = kNoColumn;
-        least[i] = res0 + 4 * i + q < 2 * a.c ? -1.0f : 3.0e38f;
+        const int res = res0 + 4 * i + (g >> 1);
+        const uint2* src = reinterpret_cast<const uint2*>(a.frag + ((size_t)(res < 2 * a.c ? res : 0) * 2 + (g & 1)) * (16 * KB)) + q;
+#pragma unroll
+        for (int kb = 0; kb < KB; ++kb) bf[i][kb] = src[4 * kb];
     }
-    for (long long tile0 = col0; tile0 < col1; tile0 += TC) {
-        if (tile0 != col0) { __syncthreads(); generate(tile0); }
-        __syncthreads();
-        if (threadIdx.x < TC) {
-            float n2 = 0.0f;
+    // Scores are compared as keys: the score's bits with the lowest ten replaced by a code of the column (relative error 2^-13, an
+    // eighth of the window that k_chunk_pick rescores), so that the best two follow from three integer minima and maxima, without
+    // a branch.  Columns of a recovery's support score rounding noise; should one be among the best two all the same (hardly any
+    // columns left, or a zero residual), the block goes through its columns again and leaves them out.
+    Best2 best[NT];
+    bool exclude = false;
+    for (;;) {
 #pragma unroll
-            for (int kb = 0; kb < KB; ++kb) n2 += n2p[kb * TC + threadIdx.x];
-            // (-infinity: no column of this block; its score is -infinity or not a number, and passes no comparison)
-            inv[threadIdx.x] = tile0 + threadIdx.x < col1 ? (n2 > 0.0f ? 1.0f / sqrtf(n2) : 0.0f) : __int_as_float(0xff800000);
-        }
-        __syncthreads();
-        unsigned int moved = 0u;
+        for (int i = 0; i < NT; ++i) { best[i].s1 = best[i].s2 = -1.0f; best[i].i1 = best[i].i2 = kNoColumn; }
+        for (long long super = col0; super < col1; super += kCorrSuper) {
+            unsigned int k1[NT], k2[NT];
+#pragma unroll
+            for (int i = 0; i < NT; ++i) k1[i] = k2[i] = 0u;
+            const long long super1 = super + kCorrSuper < col1 ? super + kCorrSuper : col1;
+            for (long long tile0 = super; tile0 < super1; tile0 += TC) {
+                if (tile0 != col0 || exclude) { __syncthreads(); generate(tile0); }
+                __syncthreads();
+                if (threadIdx.x < TC) {
+                    float n2 = 0.0f;
+#pragma unroll
+                    for (int kb = 0; kb < KB; ++kb) n2 += n2p[kb * TC + threadIdx.x];
+                    const bool real = tile0 + threadIdx.x < col1;     // code 0 (and score 0): no column of this block
+                    inv[threadIdx.x] = make_float2(real && n2 > 0.0f ? 1.0f / sqrtf(n2) : 0.0f,
+                                                   __uint_as_float(real ? (unsigned int)(kCorrSuper - (tile0 - super) - threadIdx.x) : 0u));
+                }
+                __syncthreads();
 #pragma unroll 1
-        for (int tl = 0; tl < TILES; ++tl) {
-            if (tile0 + tl * 16 >= col1) break;
-            float acc[NT][4];
+                for (int tl = 0; tl < TILES; ++tl) {
+                    float acc[NT][4];
 #pragma unroll
-            for (int i = 0; i < NT; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.0f;
+                    for (int i = 0; i < NT; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.0f;
 #pragma unroll
-            for (int kb = 0; kb < KB; ++kb) {
-                const uint4 x = zt[(size_t)(tl * KB + kb) * 32 + lane];
+                    for (int kb = 0; kb < KB; ++kb) {
+                        const uint4 x = zt[(size_t)(tl * KB + kb) * 32 + lane];
 #pragma unroll
-                for (int i = 0; i < NT; ++i) mma_16816(acc[i], x, bf[i][kb][0], bf[i][kb][1]);
-            }
-            const float v0 = inv[tl * 16 + g], v1 = inv[tl * 16 + g + 8];
+                        for (int i = 0; i < NT; ++i) mma_16816(acc[i], x, bf[i][kb].x, bf[i][kb].y);
+                    }
+                    const float2 v0 = inv[tl * 16 + g], v1 = inv[tl * 16 + g + 8];
 #pragma unroll
-            for (int i = 0; i < NT; ++i) {
-                const float s0 = fabsf(acc[i][0] + acc[i][1]) * v0, s1 = fabsf(acc[i][2] + acc[i][3]) * v1;
-                if (fmaxf(s0, s1) > least[i]) {
-                    const uint32_t* sup = a.lam + (size_t)(res0 + 4 * i + q) * a.s;
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const float sc = e ? s1 : s0;
-                        if (!(sc > least[i])) continue;
-                        const uint32_t col = (uint32_t)(tile0 + tl * 16 + g + 8 * e);
-                        bool taken = false;
-                        for (int l = 0; l < iter; ++l) taken |= (sup[l] == col);
-                        if (!taken) { best[i].push(sc, col); least[i] = fmaxf(least[i], best[i].s2); moved |= 1u << i; }
+                    for (int i = 0; i < NT; ++i) {
+                        unsigned int x0 = (__float_as_uint(fabsf(acc[i][0] + acc[i][1]) * v0.x) & ~1023u) | __float_as_uint(v0.y);
+                        unsigned int x1 = (__float_as_uint(fabsf(acc[i][2] + acc[i][3]) * v1.x) & ~1023u) | __float_as_uint(v1.y);
+                        if (exclude) {
+                            const int mine = res0 + 4 * i + q;
+                            const uint32_t* sup = a.lam + (size_t)(mine < 2 * a.c ? mine : 0) * a.s;
+                            const uint32_t c0 = (uint32_t)(tile0 + tl * 16 + g);
+                            for (int l = 0; l < iter; ++l) { if (sup[l] == c0) x0 = 0u; if (sup[l] == c0 + 8u) x1 = 0u; }
+                        }
+                        k2[i] = max(k2[i], min(k1[i], x0)); k1[i] = max(k1[i], x0);
+                        k2[i] = max(k2[i], min(k1[i], x1)); k1[i] = max(k1[i], x1);
                     }
                 }
             }
-        }
-        // the eight lanes of a recovery tell one another their second best (a lower bound of the block's): later columns rarely pass it
-        if (tile0 + TC < col1 && __any_sync(0xffffffffu, moved != 0u)) {
+            // the eight lanes of a recovery (same q) join their best two
 #pragma unroll
             for (int i = 0; i < NT; ++i) {
-                // second best among the lanes' best two: at least the largest s2, and at least the second largest s1
-                float hi1 = best[i].s1, hi2 = best[i].s2;
 #pragma unroll
                 for (int o = 4; o < 32; o <<= 1) {
-                    const float t1 = __shfl_xor_sync(0xffffffffu, hi1, o), t2 = __shfl_xor_sync(0xffffffffu, hi2, o);
-                    hi2 = fmaxf(fmaxf(hi2, t2), fminf(hi1, t1));
-                    hi1 = fmaxf(hi1, t1);
+                    const unsigned int t1 = __shfl_xor_sync(0xffffffffu, k1[i], o), t2 = __shfl_xor_sync(0xffffffffu, k2[i], o);
+                    k2[i] = max(max(k2[i], t2), min(k1[i], t1));
+                    k1[i] = max(k1[i], t1);
                 }
-                least[i] = fmaxf(least[i], hi2);
+                if (k1[i]) best[i].push(__uint_as_float(k1[i] & ~1023u), (uint32_t)(super + kCorrSuper - (k1[i] & 1023u)));
+                if (k2[i]) best[i].push(__uint_as_float(k2[i] & ~1023u), (uint32_t)(super + kCorrSuper - (k2[i] & 1023u)));
             }
         }
+        if (exclude || iter == 0) break;
+        // lane g = l of a recovery looks at every eighth column of its support
+        bool taken = false;
+#pragma unroll
+        for (int i = 0; i < NT; ++i) {
+            const int mine = res0 + 4 * i + q;
+            const uint32_t* sup = a.lam + (size_t)(mine < 2 * a.c ? mine : 0) * a.s;
+            for (int l = g; l < iter; l += 8) { const uint32_t v = sup[l]; taken = taken || v == best[i].i1 || v == best[i].i2; }
+        }
+        if (!__syncthreads_or(taken ? 1 : 0)) break;
+        exclude = true;
     }
-    // the eight lanes of a recovery (same q) join their best two
 #pragma unroll
     for (int i = 0; i < NT; ++i) {
-#pragma unroll
-        for (int o = 4; o < 32; o <<= 1) {
-            const float t1 = __shfl_xor_sync(0xffffffffu, best[i].s1, o), t2 = __shfl_xor_sync(0xffffffffu, best[i].s2, o);
-            const uint32_t j1 = __shfl_xor_sync(0xffffffffu, best[i].i1, o), j2 = __shfl_xor_sync(0xffffffffu, best[i].i2, o);
-            if (j1 != kNoColumn) best[i].push(t1, j1);
-            if (j2 != kNoColumn) best[i].push(t2, j2);
-        }
         const int mine = res0 + 4 * i + q;
         if (g == 0 && mine < 2 * a.c) {
+            const float back = a.back[mine];
             float4* out = reinterpret_cast<float4*>(a.cand + ((size_t)mine * a.splits + blockIdx.x) * 2);
-            *out = make_float4(best[i].s1 * back[i], __uint_as_float(best[i].i1), best[i].s2 * back[i], __uint_as_float(best[i].i2));
+            *out = make_float4(best[i].i1 != kNoColumn ? best[i].s1 * back : -1.0f, __uint_as_float(best[i].i1),
+                               best[i].i2 != kNoColumn ? best[i].s2 * back : -1.0f, __uint_as_float(best[i].i2));
         }
     }
 }
@@ -473,20 +474,20 @@ struct PickSmem {
     int n_c;
 };
 
-// dynamic shared memory: residual r [k], new column a [k], q [j][k]
+// dynamic shared memory: residual r [k], q [j][k]
 __device__ __forceinline__ double* pick_mem() {
     extern __shared__ __align__(16) double pick_dyn_mem[];
     return pick_dyn_mem;
 }
-size_t pick_dyn_bytes(int s, int k) { return (size_t)(s + 1) * k * sizeof(double); }
-int pick_threads(int k) { return k <= 32 ? 64 : (k <= 128 ? 128 : kPickMaxThreads); }
+size_t pick_dyn_bytes(int s, int k) { return (size_t)s * k * sizeof(double); }
+int pick_threads(int k) { return k <= 64 ? 64 : (k <= 128 ? 128 : kPickMaxThreads); }      // one row per thread
 
 // the vectors of the earlier picks and the residual: independent loads, one trip to global memory.  A block-wide barrier has to
 // follow before pick_finish reads them.
 __device__ __forceinline__ void pick_stage(const ChunkArgs& a, const ChunkRef& ref, int m, int j) {
     const int k = a.k;
     double* r = pick_mem();
-    double* q = r + 2 * k;
+    double* q = r + k;
     const double* src = ref.qb + (size_t)m * a.s * k;
     for (int e = threadIdx.x; e < j * k; e += blockDim.x) q[e] = src[e];
     const double* rg = ref.r64 + (size_t)m * k;
@@ -505,6 +506,47 @@ __device__ __forceinline__ float pick_max(PickSmem& sh, float v) {
     return m ? __uint_as_float(m - 1u) : -1.0f;
 }
 
+constexpr int kPickPairs = kChunkMaxK / 64;           // row pairs of a column per lane
+
+// this warp's copy of a column (scaled by sigma; rows beyond k are zero): lane holds the row pairs lane, lane + 32, ...
+__device__ __forceinline__ void pick_column(const ChunkArgs& a, uint32_t col, double (&x)[2 * kPickPairs]) {
+    const ColKey key = column_key(a.seed_lo, a.seed_hi, col);
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int u = 0; u < kPickPairs; ++u) {
+        const int p = lane + 32 * u;
+        x[2 * u] = x[2 * u + 1] = 0.0;
+        if (2 * p < a.k) {
+            const float2 z = half2_bits_to_float2(z_pair_from_word(key.ck + (uint32_t)p * key.mk));
+            x[2 * u] = a.sigma * (double)z.x;
+            if (2 * p + 1 < a.k) x[2 * u + 1] = a.sigma * (double)z.y;
+        }
+    }
+}
+// this lane's part of <v, x>
+__device__ __forceinline__ double pick_dot(const ChunkArgs& a, const double* v, const double (&x)[2 * kPickPairs]) {
+    const int lane = threadIdx.x & 31;
+    double acc = 0.0;
+#pragma unroll
+    for (int u = 0; u < kPickPairs; ++u) {
+        const int row = 2 * (lane + 32 * u);
+        if (row < a.k) acc = fma(v[row], x[2 * u], acc);
+        if (row + 1 < a.k) acc = fma(v[row + 1], x[2 * u + 1], acc);
+    }
+    return acc;
+}
+// c_l = <q_l, a> for all earlier picks: warp = two vectors at a time
+__device__ __forceinline__ void pick_products(const ChunkArgs& a, PickSmem& sh, const double* qs, int j, const double (&x)[2 * kPickPairs]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    for (int l = warp; l < j; l += 2 * warps) {
+        const int l2 = l + warps < j ? l + warps : l;
+        double c0 = pick_dot(a, qs + (size_t)l * a.k, x), c1 = pick_dot(a, qs + (size_t)l2 * a.k, x);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) { c0 += __shfl_xor_sync(0xffffffffu, c0, o); c1 += __shfl_xor_sync(0xffffffffu, c1, o); }
+        if (lane == 0) { sh.cs[l] = c0; sh.cs[l2] = l2 != l ? c1 : c0; }
+    }
+}
+
 // the decision among the nc candidates in sh.cidx and the update of the recovery `res` with the winner as pick j
 // (all threads of the block; nc is the same in every thread; pick_stage has run for this recovery)
 __device__ void pick_finish(const ChunkArgs& a, const ChunkRef& ref, PickSmem& sh, int res, int j, int nc) {
@@ -514,23 +556,20 @@ __device__ void pick_finish(const ChunkArgs& a, const ChunkRef& ref, PickSmem& s
         return;
     }
     double* r = pick_mem();
-    double* an = r + k;
-    double* qs = an + k;
+    double* qs = r + k;
     __syncthreads();                                                 // the staged state and the candidates are complete
-    // exact scores: warp = one candidate; the first one's column is kept
-    for (int c = warp; c < nc; c += warps) {
-        const ColKey key = column_key(a.seed_lo, a.seed_hi, sh.cidx[c]);
-        double dot = 0.0, n2 = 0.0;
-        for (int row = 2 * lane; row < k; row += 64) {
-            const float2 z = half2_bits_to_float2(z_pair_from_word(key.ck + (uint32_t)(row >> 1) * key.mk));
-            const double z0 = a.sigma * (double)z.x, z1 = a.sigma * (double)z.y;
-            dot = fma(z0, r[row], dot); n2 = fma(z0, z0, n2);
-            if (c == 0) an[row] = z0;
-            if (row + 1 < k) { dot = fma(z1, r[row + 1], dot); n2 = fma(z1, z1, n2); if (c == 0) an[row + 1] = z1; }
-        }
-        dot = warp_sum_d(dot); n2 = warp_sum_d(n2);
+    double x[2 * kPickPairs];
+    // exact scores (warp = one candidate, the last warp takes the first), and the products of the first candidate with the q_l
+    for (int c = (warps - 1) - warp; c < nc; c += warps) {
+        pick_column(a, sh.cidx[c], x);
+        double dot = pick_dot(a, r, x), n2 = 0.0;
+#pragma unroll
+        for (int u = 0; u < 2 * kPickPairs; ++u) n2 = fma(x[u], x[u], n2);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) { dot += __shfl_xor_sync(0xffffffffu, dot, o); n2 += __shfl_xor_sync(0xffffffffu, n2, o); }
         if (lane == 0) { sh.cdot[c] = dot; sh.cn2[c] = n2; }
     }
+    if (warp < j) { pick_column(a, sh.cidx[0], x); pick_products(a, sh, qs, j, x); }
     __syncthreads();
     int win = 0;
     {
@@ -542,23 +581,11 @@ __device__ void pick_finish(const ChunkArgs& a, const ChunkRef& ref, PickSmem& s
     }
     const uint32_t col = sh.cidx[win];
     const double dot = sh.cdot[win], n2 = sh.cn2[win];
-    if (win != 0) {
-        const ColKey key = column_key(a.seed_lo, a.seed_hi, col);
-        for (int row = t; row < k; row += blockDim.x) an[row] = a.sigma * (double)z_at(key, (uint32_t)row);
+    if (win != 0 && j > 0) {
+        __syncthreads();                                             // (a slow warp may still be reading sums of the first candidate)
+        if (warp < j) { pick_column(a, col, x); pick_products(a, sh, qs, j, x); }
         __syncthreads();
     }
-    // c_l = <q_l, a>: warp = two vectors at a time
-    for (int l = warp; l < j; l += 2 * warps) {
-        const int l2 = l + warps < j ? l + warps : l;
-        double c0 = 0.0, c1 = 0.0;
-        for (int row = lane; row < k; row += 32) {
-            const double x = an[row];
-            c0 = fma(qs[l * k + row], x, c0); c1 = fma(qs[l2 * k + row], x, c1);
-        }
-        c0 = warp_sum_d(c0); c1 = warp_sum_d(c1);
-        if (lane == 0) { sh.cs[l] = c0; if (l2 != l) sh.cs[l2] = c1; }
-    }
-    __syncthreads();
     double csq = lane < j ? sh.cs[lane] * sh.cs[lane] : 0.0;         // (j < 32)
     csq = warp_sum_d(csq);
     const double piv = n2 - csq;
@@ -570,19 +597,18 @@ __device__ void pick_finish(const ChunkArgs& a, const ChunkRef& ref, PickSmem& s
         return;
     }
     const double gamma = rsqrt(piv), aj = gamma * dot;
-    double rn2 = 0.0;
-    for (int row = t; row < k; row += blockDim.x) {
+    double rv = 0.0;                                                 // row t of the new residual (pick_threads: at least k threads)
+    if (t < k) {
+        const int row = t;
         double v0 = 0.0, v1 = 0.0;
         int l = 0;
 #pragma unroll 4
         for (; l + 1 < j; l += 2) { v0 = fma(sh.cs[l], qs[l * k + row], v0); v1 = fma(sh.cs[l + 1], qs[(l + 1) * k + row], v1); }
         if (l < j) v0 = fma(sh.cs[l], qs[l * k + row], v0);
-        const double q = gamma * (an[row] - (v0 + v1));
+        const double q = gamma * (a.sigma * (double)z_at(column_key(a.seed_lo, a.seed_hi, col), (uint32_t)row) - (v0 + v1));
         ref.qb[((size_t)m * s + j) * k + row] = q;
-        const double rv = r[row] - aj * q;
+        rv = r[row] - aj * q;
         ref.r64[(size_t)m * k + row] = rv;
-        a.r32[(size_t)res * a.kp + row] = (float)rv;
-        rn2 = fma(rv, rv, rn2);
     }
     if (t < j) ref.crow[((size_t)m * s + j) * s + t] = sh.cs[t];
     if (t == 0) {
@@ -590,14 +616,14 @@ __device__ void pick_finish(const ChunkArgs& a, const ChunkRef& ref, PickSmem& s
         ref.gam[(size_t)m * s + j] = gamma; ref.acoef[(size_t)m * s + j] = aj; ref.lam[(size_t)m * s + j] = col;
         ref.cnt->done[m] = j + 1;
     }
-    rn2 = warp_sum_d(rn2);
-    if (lane == 0) sh.red[warp] = rn2;
+    const double part = warp_sum_d(rv * rv);
+    if (lane == 0) sh.red[warp] = part;
     __syncthreads();
-    if (t == 0) {
-        double v = 0.0;
-        for (int w = 0; w < warps; ++w) v += sh.red[w];
-        ref.rnorm[(size_t)m * s + j] = sqrt(v);
-    }
+    double rn2 = 0.0;
+    for (int w = 0; w < warps; ++w) rn2 += sh.red[w];
+    const double rn = sqrt(rn2), sc = frag_scale(rn);
+    if (t < k) frag_write(a, res, t, rv, sc);
+    if (t == 0) { ref.rnorm[(size_t)m * s + j] = rn; a.back[res] = (float)(1.0 / sc); }
 }
 
 // SIMT route: the candidates are the columns that phase A left within 2e-3 (relative) of the best fp32 score.
@@ -827,7 +853,7 @@ unsigned long long list_key(sgc_state* const* sts, int c) {
 template <int KP>
 cudaError_t corr_setup(size_t* smem_out) {
     constexpr int TC = corr_tile(KP), KB = corr_kb(KP);
-    const size_t smem = (size_t)(TC / 16) * KB * 512 + (size_t)(TC + KB * TC) * sizeof(float);
+    const size_t smem = (size_t)(TC / 16) * KB * 512 + (size_t)(2 * TC + KB * TC) * sizeof(float);
     *smem_out = smem;
     return cudaFuncSetAttribute(k_chunk_corr<KP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
@@ -889,7 +915,8 @@ cudaError_t ensure_ws(sgc_state* const* sts, int c) {
     ws->splits = splits;
     auto up = [](size_t b) { return (b + 255) / 256 * 256; };
     const size_t b_table = up((size_t)c * sizeof(ChunkRef));
-    const size_t b_r32 = up((size_t)2 * c * ws->kp * sizeof(float));
+    const int kf = ws->kp < 16 ? 16 : ws->kp;
+    const size_t b_frag = up((size_t)2 * c * 2 * kf * sizeof(uint16_t)), b_back = up((size_t)2 * c * sizeof(float));
     const size_t b_cand = up((size_t)2 * c * splits * 2 * sizeof(Cand));
     const size_t b_lam = up((size_t)2 * c * st0->s * sizeof(uint32_t));
     // tensor-core route: worth it from k_c = 33 on; bounded by its report lists (n_rows * 16 KB)
@@ -908,12 +935,13 @@ cudaError_t ensure_ws(sgc_state* const* sts, int c) {
         b_un = up((size_t)2 * c);
         b_flags = 256;
     }
-    cudaError_t e = cudaMalloc(&ws->base, b_table + b_r32 + b_cand + b_lam + b_rt + 3 * b_row + b_rep + b_norm + b_rn + b_un + b_flags);
+    cudaError_t e = cudaMalloc(&ws->base, b_table + b_frag + b_back + b_cand + b_lam + b_rt + 3 * b_row + b_rep + b_norm + b_rn + b_un + b_flags);
     if (e != cudaSuccess) { delete ws; return e; }
     unsigned char* base = static_cast<unsigned char*>(ws->base);
     size_t off = 0;
     ws->table = reinterpret_cast<ChunkRef*>(base + off); off += b_table;
-    ws->r32 = reinterpret_cast<float*>(base + off); off += b_r32;
+    ws->frag = reinterpret_cast<uint16_t*>(base + off); off += b_frag;
+    ws->back = reinterpret_cast<float*>(base + off); off += b_back;
     ws->cand = reinterpret_cast<Cand*>(base + off); off += b_cand;
     ws->lam = reinterpret_cast<uint32_t*>(base + off); off += b_lam;
     if (ws->tensor) {
@@ -950,7 +978,7 @@ cudaError_t ensure_ws(sgc_state* const* sts, int c) {
         r.upd_idx = st->upd_idx; r.upd_val = st->upd_val; r.cnt = st->cnt; r.ctl = st->ctl;
     }
     e = cudaMemcpy(ws->table, host.data(), (size_t)c * sizeof(ChunkRef), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(ws->r32, 0, b_r32);         // rows k..kp of every residual stay zero
+    if (e == cudaSuccess) e = cudaMemset(ws->frag, 0, b_frag);       // rows k..kf of every residual stay zero
     if (e == cudaSuccess) e = cudaDeviceSynchronize();               // set-up done before the caller's stream runs on it
     if (e != cudaSuccess) { cudaFree(ws->base); delete ws; return e; }
     st0->chunk_ws = ws;
@@ -994,7 +1022,7 @@ cudaError_t launch_chunked_batch(sgc_state* const* sts, int c, const float* grad
     a.table = ws->table; a.c = c; a.k = st0->k; a.s = st0->s; a.kp = ws->kp; a.dc = st0->d;
     a.seed_lo = (uint32_t)(st0->seed & 0xFFFFFFFFu); a.seed_hi = (uint32_t)(st0->seed >> 32);
     a.sigma = (double)(float)(1.0 / sqrt((double)st0->k));
-    a.r32 = ws->r32; a.cand = ws->cand; a.lam = ws->lam; a.splits = ws->splits;
+    a.frag = ws->frag; a.back = ws->back; a.kf = ws->kp < 16 ? 16 : ws->kp; a.cand = ws->cand; a.lam = ws->lam; a.splits = ws->splits;
     {
         const int groups = (2 * c + corr_group(ws->kp) - 1) / corr_group(ws->kp);
         a.early = (ws->splits * groups <= st0->sm_count && 2 * c <= st0->sm_count) ? 1 : 0;

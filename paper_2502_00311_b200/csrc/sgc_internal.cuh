@@ -216,7 +216,8 @@ struct ChunkRef {
 struct ChunkWs {
     void* base;                 // one device allocation holding everything below
     ChunkRef* table;            // [c]
-    float* r32;                 // [2c][kp] residuals of all streams (stream = 2 * chunk + moment), rows padded to kp
+    uint16_t* frag;             // [2c][2][max(kp, 16)] residuals of all streams (stream = 2 * chunk + moment) as matrix operands
+    float* back;                // [2c] inverse of their scales
     Cand* cand;                 // [2c][splits][2] best two columns of every column split, per stream
     uint32_t* lam;              // [2c][s] supports of all recoveries
     int c, kp, splits;

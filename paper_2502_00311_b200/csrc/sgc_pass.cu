@@ -171,11 +171,41 @@ __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
 
+// Reports of one epilogue warp, collected in shared memory and appended to the lists many at a time: an append is two dependent
+// trips to global memory (1.4 us), which the warp would otherwise make for every report (small passes, where a few dozen
+// reports per warp meet a few microseconds of work, spent most of their time there: 215 -> 94 us at d = 129344, k = 512 when
+// fewer columns were reported).  word 0: count; then three words per entry (residual, column, score).
+struct ReportQueue {
+    uint32_t* mem; int cap;
+    __device__ __forceinline__ void init(int lane) { if (lane == 0) mem[0] = 0u; __syncwarp(); }
+};
+__device__ __forceinline__ void report_append(const PassArgs& a, uint32_t n_res, uint32_t col, float sc) {
+    const unsigned int slot = atomicAdd(&a.rep_count[n_res], 1u);
+    if (slot < (unsigned int)a.rep_cap)
+        a.rep[(size_t)n_res * a.rep_cap + slot] = make_uint2(col, __float_as_uint(a.inv_scale ? sc * a.inv_scale[n_res] : sc));
+}
+__device__ __forceinline__ void report_push(const PassArgs& a, const ReportQueue& q, uint32_t n_res, uint32_t col, float sc) {
+    const unsigned int e = atomicAdd(&q.mem[0], 1u);
+    if (e < (unsigned int)q.cap) { uint32_t* w = q.mem + 1 + 3 * e; w[0] = n_res; w[1] = col; w[2] = __float_as_uint(sc); }
+    else report_append(a, n_res, col, sc);
+}
+// the whole warp; appends what the queue holds when there is at least `least` of it
+__device__ __forceinline__ void report_flush(const PassArgs& a, const ReportQueue& q, int lane, unsigned int least) {
+    __syncwarp();
+    unsigned int n = *reinterpret_cast<volatile uint32_t*>(q.mem);
+    if (n < least) return;
+    if (n > (unsigned int)q.cap) n = (unsigned int)q.cap;
+    for (unsigned int e = lane; e < n; e += 32u) { const uint32_t* w = q.mem + 1 + 3 * e; report_append(a, w[0], w[1], __uint_as_float(w[2])); }
+    __syncwarp();
+    if (lane == 0) q.mem[0] = 0u;
+    __syncwarp();
+}
+
 // ---- the kernel -----------------------------------------------------------------------------------------
 // dynamic shared memory (after alignment to 1024 bytes):
 //   stages x { A tile 0 (16 KB) | A tile 1 (16 KB) | R^T chunk (n x 128 B) }
 //   norms  float[kNormRing][256][2]      partial ||Z_i||^2 of the two generator threads of each column
-//   tau    float[256], 1 / tau float[256], 1 / wide-list threshold float[256]
+//   tau    float[256], 1 / tau float[256], 1 / wide-list threshold float[256]; report queues u32[4][256] (without a table of norms)
 //   mbarriers: full[stages], empty[stages], acc_full[2], acc_empty[2], drain;  tensor-memory base;  abort flag
 // WIDE: the two-level screening code (wide-list harvest, list passes) is compiled in
 // SUB: 64-row chunks of A per slot of the ring, i.e. per hand-off between generators, TMA and MMA issuer (2 when the
@@ -216,7 +246,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
     float* tau_s = norms + kNormRing * kSuperCols * 2;
     float* itau_s = tau_s + 256;                                     // 1 / tau: a group of 16 residuals is skipped on one compare
     float* iwide_s = itau_s + 256;                                   // 1 / threshold of the wide lists
-    uint64_t* bars = reinterpret_cast<uint64_t*>(iwide_s + 256);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(iwide_s + 256 + 4 * kSuperCols);            // (report queues of the variant that sums its norms)
     const uint32_t bar_full = smem_u32(bars), bar_empty = bar_full + 8u * a.stages;
     const uint32_t bar_accf = bar_empty + 8u * a.stages, bar_acce = bar_accf + 16u, bar_drain = bar_acce + 16u;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * a.stages + 5);
@@ -319,6 +349,12 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
         const int quad = warp & 3;
         uint32_t sweep_i = 0;
         bool ok = true;
+        // room for the reports: what the table of norms leaves of its ring (the swapped form keeps 12 KB of it for other things)
+        ReportQueue queue_r;
+        queue_r.mem = TABLE ? reinterpret_cast<uint32_t*>(norms + (SWAP ? (size_t)(12 + quad) * kSuperCols : (size_t)quad * 4 * kSuperCols))
+                            : reinterpret_cast<uint32_t*>(norms) + kNormRing * kSuperCols * 2 + 768 + quad * kSuperCols;
+        queue_r.cap = ((TABLE && !SWAP ? 4 : 1) * kSuperCols - 1) / 3;
+        queue_r.init(lane);
         for (unsigned int sweep = blockIdx.x; ok && sweep < num_super; sweep += gridDim.x, ++sweep_i) {
             const uint32_t buf = sweep_i % a.bufs, use = sweep_i / a.bufs;
             if (!__all_sync(0xffffffffu, mbar_wait(bar_accf + 8u * buf, use & 1u, abort_flag, 512, a.wait_limit_ns))) { ok = false; break; }
@@ -393,12 +429,8 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
                         const float inv = inv_w[c0 + i];
                         const float sc = fabsf(__uint_as_float(v[i])) * inv;
                         if (sc >= tau_n && inv > 0.0f) {
-                            const unsigned int slot = atomicAdd(&a.rep_count[n_res], 1u);
-                            if (slot < (unsigned int)a.rep_cap) {
-                                const float out = a.inv_scale ? sc * a.inv_scale[n_res] : sc;
-                                const uint32_t col = listed ? col_w[c0 + i] : (uint32_t)((unsigned long long)sweep * kSuperCols + c0 + i);
-                                a.rep[(size_t)n_res * a.rep_cap + slot] = make_uint2(col, __float_as_uint(out));
-                            }
+                            const uint32_t col = listed ? col_w[c0 + i] : (uint32_t)((unsigned long long)sweep * kSuperCols + c0 + i);
+                            report_push(a, queue_r, (uint32_t)n_res, col, sc);
                         }
                     }
                 }
@@ -419,6 +451,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
                     }
                     __syncwarp();
                 }
+                report_flush(a, queue_r, lane, (unsigned int)queue_r.cap / 2);
                 continue;
             }
             const float* nr = norms + (size_t)(sweep_i % kNormRing) * kSuperCols * 2;
@@ -480,20 +513,16 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
                         const float sc = fabsf(__uint_as_float(v[i])) * inv;
-                        if (sc >= tau_s[c0 + i] && inv > 0.0f) {
-                            const unsigned int slot = atomicAdd(&a.rep_count[c0 + i], 1u);
-                            if (slot < (unsigned int)a.rep_cap) {
-                                const float out = a.inv_scale ? sc * a.inv_scale[c0 + i] : sc;
-                                a.rep[(size_t)(c0 + i) * a.rep_cap + slot] = make_uint2((uint32_t)col, __float_as_uint(out));
-                            }
-                        }
+                        if (sc >= tau_s[c0 + i] && inv > 0.0f) report_push(a, queue_r, (uint32_t)(c0 + i), (uint32_t)col, sc);
                     }
                 }
             }
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_acce + 8u * buf);
+            report_flush(a, queue_r, lane, (unsigned int)queue_r.cap / 2);
         }
+        report_flush(a, queue_r, lane, 1u);
     } else {
         // ---------------- generators: Z tiles as binary16, swizzled K-major ---------------------------------
         const int g = threadIdx.x - kFirstGenWarp * 32;
@@ -613,7 +642,7 @@ cudaError_t get_encoder(EncodeTiledFn* out) {
 }
 
 size_t pass_smem_bytes(int n, int slots, int sub) {
-    return 1024 + (size_t)slots * sub * (2 * kTileBytes + (size_t)n * 128) + sizeof(float) * (kNormRing * kSuperCols * 2 + 768) +
+    return 1024 + (size_t)slots * sub * (2 * kTileBytes + (size_t)n * 128) + sizeof(float) * (kNormRing * kSuperCols * 2 + 768 + 4 * kSuperCols) +
            8 * (2 * (size_t)slots + 5) + 16;
 }
 
