@@ -6,7 +6,8 @@
 //                     projected gradient.  64 fp64 multiply-adds per cycle and SM bound it (30 us for a 4096 x 4096 gradient at
 //                     r = 32); conversions from fp32, a quarter as fast, are kept out of the way: a thread owns four columns and
 //                     eight rows, converts each element of G once for its eight products and reads B as fp64 from a slab that
-//                     the block has converted on the way in.  (An error-free two-float form took 276 us, fp64 with both operands
+//                     the block has converted on the way in; G arrives by asynchronous copies, three slabs ahead (with one
+//                     slab ahead in registers the kernel waited for memory: 138 us).  (An error-free two-float form took 276 us, fp64 with both operands
 //                     converted per product 1.1 ms.)  The rows of G are split over the CTAs of a thread-block cluster; their
 //                     partial sums meet through distributed shared memory, added in rank order.
 //   k_cesgc_back      W += B^T U for the r x n matrix U that the SGC core left (U = -eta N has at most s non-zeros).
@@ -22,7 +23,8 @@ namespace {
 constexpr int kCesgcMaxR = 64;
 constexpr int kProjCols = 128;           // columns of G per block: 32 lanes of four
 constexpr int kProjRows = 8;             // rows of B per thread
-constexpr int kProjPer = 4;              // rows of a slab of G per thread
+constexpr int kProjPer = 8;              // rows of a slab of G per thread
+constexpr int kProjStages = 4;           // slabs of G in shared memory
 constexpr int kProjMaxSplit = 8;         // CTAs of a cluster (the portable limit), each with a range of G's rows
 constexpr int kProjResident = 148;       // one wave
 
@@ -30,9 +32,10 @@ constexpr int kProjResident = 148;       // one wave
 __host__ __device__ constexpr int proj_groups(int r) { return (r + kProjRows - 1) / kProjRows; }
 __host__ __device__ constexpr int proj_parts(int r) { return proj_groups(r) > 4 ? 2 : proj_groups(r) > 2 ? 4 : 8; }
 __host__ __device__ constexpr int proj_slab(int r) { return kProjPer * proj_parts(r); }
-// slabs of B (two, fp64) and, at the end, the partial sums of the parts
+// slabs of B (two, fp64), slabs of G; at the end the partial sums of the parts
+__host__ __device__ constexpr size_t proj_bslab(int r) { return 2 * (size_t)proj_groups(r) * kProjRows * proj_slab(r) * sizeof(double); }
 __host__ __device__ constexpr size_t proj_smem(int r) {
-    const size_t slab = 2 * (size_t)proj_groups(r) * kProjRows * proj_slab(r) * sizeof(double);
+    const size_t slab = proj_bslab(r) + (size_t)kProjStages * proj_slab(r) * kProjCols * sizeof(float);
     const size_t part = (size_t)proj_groups(r) * kProjRows * kProjCols * sizeof(double);
     return slab > part ? slab : part;
 }
@@ -50,7 +53,6 @@ k_cesgc_project(const float* __restrict__ B, const float* __restrict__ G, float*
     const int groups = proj_groups(r), rows8 = groups * kProjRows, parts = proj_parts(r), slab_rows = proj_slab(r);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ig = warp % groups, part = warp / groups;
-    const int j0 = blockIdx.x * kProjCols + 4 * lane;                 // this thread's four columns
     // this CTA's rows of G: whole slabs, the same number for every CTA of the cluster (the last ranges may be empty)
     const int slabs = (m + slab_rows - 1) / slab_rows;
     const int part_rows = (slabs + (int)gridDim.y - 1) / (int)gridDim.y * slab_rows;
@@ -61,59 +63,83 @@ k_cesgc_project(const float* __restrict__ B, const float* __restrict__ G, float*
     for (int u = 0; u < kProjRows; ++u)
 #pragma unroll
         for (int c = 0; c < 4; ++c) acc[u][c] = 0.0;
-    // slab of B as [row of G][row of B]: a thread reads its eight values of a row of G in four 16-byte broadcasts
-    auto stage = [&](double* dst, int row0) {
-        for (int e = threadIdx.x; e < rows8 * slab_rows; e += blockDim.x) {
-            const int i = e / slab_rows, q = e % slab_rows;
-            dst[q * rows8 + i] = (i < r && row0 + q < m_end) ? (double)B[(size_t)i * m + row0 + q] : 0.0;
+    // slab of B as [row of G][row of B]: a thread reads its eight values of a row of G in four 16-byte broadcasts.  Its values
+    // travel through registers, one slab ahead
+    constexpr int kBHold = kProjRows * kProjPer / 32;                  // (rows8 * slab_rows values over 32 * groups * parts threads)
+    float bh[kBHold];
+    const int b_items = rows8 * slab_rows, threads = (int)blockDim.x;
+    auto fetch_b = [&](int row0) {
+#pragma unroll
+        for (int u = 0; u < kBHold; ++u) {
+            const int e = (int)threadIdx.x + u * threads;
+            bh[u] = 0.0f;
+            if (e < b_items) { const int i = e / slab_rows, q = e % slab_rows; if (i < r && row0 + q < m_end) bh[u] = B[(size_t)i * m + row0 + q]; }
         }
     };
-    auto load = [&](int row) -> float4 {
-        float4 f = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (row < m_end) {
-            const float* src = G + (size_t)row * n + j0;
-            if (VEC) { if (j0 < n) f = __ldcs(reinterpret_cast<const float4*>(src)); }        // n is a multiple of 4
-            else {
-                if (j0 < n) f.x = src[0];
-                if (j0 + 1 < n) f.y = src[1];
-                if (j0 + 2 < n) f.z = src[2];
-                if (j0 + 3 < n) f.w = src[3];
+    auto store_b = [&](double* dst) {
+#pragma unroll
+        for (int u = 0; u < kBHold; ++u) {
+            const int e = (int)threadIdx.x + u * threads;
+            if (e < b_items) { const int i = e / slab_rows, q = e % slab_rows; dst[q * rows8 + i] = (double)bh[u]; }
+        }
+    };
+    float* gbuf = reinterpret_cast<float*>(smem + proj_bslab(r) / sizeof(double));      // [kProjStages][slab_rows][kProjCols]
+    // one slab of G; what lies outside the matrix is filled with zeros (a copy of 0 bytes)
+    auto copy_g = [&](int stage, int row0) {
+        float* dst = gbuf + (size_t)stage * slab_rows * kProjCols;
+        for (int e = threadIdx.x; e < slab_rows * (kProjCols / 4); e += threads) {
+            const int q = e / (kProjCols / 4), c = e % (kProjCols / 4) * 4, col = blockIdx.x * kProjCols + c;
+            const bool row_ok = row0 + q < m_end;
+            const uint32_t to = (uint32_t)__cvta_generic_to_shared(dst + q * kProjCols + c);
+            if (VEC) {
+                const bool ok = row_ok && col < n;                    // n is a multiple of 4
+                const float* src = ok ? G + (size_t)(row0 + q) * n + col : G;
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to), "l"(src), "r"(ok ? 16 : 0) : "memory");
+            } else {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const bool ok = row_ok && col + u < n;
+                    const float* src = ok ? G + (size_t)(row0 + q) * n + col + u : G;
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(to + 4 * u), "l"(src), "r"(ok ? 4 : 0) : "memory");
+                }
             }
         }
-        return f;
+        asm volatile("cp.async.commit_group;" ::: "memory");
     };
     double* bufs[2] = {smem, smem + (size_t)rows8 * slab_rows};
-    float4 next[kProjPer];
     if (m_begin < m_end) {
-        stage(bufs[0], m_begin);
+        fetch_b(m_begin);
+        for (int st = 0; st < kProjStages - 1; ++st) copy_g(st, m_begin + st * slab_rows);
+        store_b(bufs[0]);
+        int b = 0, stage = 0;
+        for (int row0 = m_begin; row0 < m_end; row0 += slab_rows) {
+            asm volatile("cp.async.wait_group %0;" ::"n"(kProjStages - 2) : "memory");
+            __syncthreads();                                          // slab `stage` of G and slab b of B are staged, the others used up
+            copy_g((stage + kProjStages - 1) % kProjStages, row0 + (kProjStages - 1) * slab_rows);
+            const bool more = row0 + slab_rows < m_end;
+            if (more) fetch_b(row0 + slab_rows);
+            const double* slab = bufs[b] + ig * kProjRows;
+            const float* gs = gbuf + (size_t)stage * slab_rows * kProjCols + 4 * lane;
+#pragma unroll 2
+            for (int q = 0; q < kProjPer; ++q) {
+                const int row = q * parts + part;
+                const float4 g = *reinterpret_cast<const float4*>(gs + row * kProjCols);
+                const double2* bq = reinterpret_cast<const double2*>(slab + (size_t)row * rows8);
+                const double gx = (double)g.x, gy = (double)g.y, gz = (double)g.z, gw = (double)g.w;
 #pragma unroll
-        for (int q = 0; q < kProjPer; ++q) next[q] = load(m_begin + q * parts + part);
-    }
-    int b = 0;
-    for (int row0 = m_begin; row0 < m_end; row0 += slab_rows, b ^= 1) {
-        __syncthreads();                                              // this slab is staged, the other one used up
-        float4 g[kProjPer];
-#pragma unroll
-        for (int q = 0; q < kProjPer; ++q) g[q] = next[q];
-        if (row0 + slab_rows < m_end) {
-#pragma unroll
-            for (int q = 0; q < kProjPer; ++q) next[q] = load(row0 + slab_rows + q * parts + part);
-            stage(bufs[b ^ 1], row0 + slab_rows);
-        }
-        const double* slab = bufs[b] + ig * kProjRows;
-#pragma unroll
-        for (int q = 0; q < kProjPer; ++q) {
-            const double2* bq = reinterpret_cast<const double2*>(slab + (size_t)(q * parts + part) * rows8);
-            const double gx = (double)g[q].x, gy = (double)g[q].y, gz = (double)g[q].z, gw = (double)g[q].w;
-#pragma unroll
-            for (int u = 0; u < kProjRows / 2; ++u) {
-                const double2 v = bq[u];
-                acc[2 * u][0] = fma(v.x, gx, acc[2 * u][0]); acc[2 * u][1] = fma(v.x, gy, acc[2 * u][1]);
-                acc[2 * u][2] = fma(v.x, gz, acc[2 * u][2]); acc[2 * u][3] = fma(v.x, gw, acc[2 * u][3]);
-                acc[2 * u + 1][0] = fma(v.y, gx, acc[2 * u + 1][0]); acc[2 * u + 1][1] = fma(v.y, gy, acc[2 * u + 1][1]);
-                acc[2 * u + 1][2] = fma(v.y, gz, acc[2 * u + 1][2]); acc[2 * u + 1][3] = fma(v.y, gw, acc[2 * u + 1][3]);
+                for (int u = 0; u < kProjRows / 2; ++u) {
+                    const double2 v = bq[u];
+                    acc[2 * u][0] = fma(v.x, gx, acc[2 * u][0]); acc[2 * u][1] = fma(v.x, gy, acc[2 * u][1]);
+                    acc[2 * u][2] = fma(v.x, gz, acc[2 * u][2]); acc[2 * u][3] = fma(v.x, gw, acc[2 * u][3]);
+                    acc[2 * u + 1][0] = fma(v.y, gx, acc[2 * u + 1][0]); acc[2 * u + 1][1] = fma(v.y, gy, acc[2 * u + 1][1]);
+                    acc[2 * u + 1][2] = fma(v.y, gz, acc[2 * u + 1][2]); acc[2 * u + 1][3] = fma(v.y, gw, acc[2 * u + 1][3]);
+                }
             }
+            if (more) store_b(bufs[b ^ 1]);
+            b ^= 1;
+            stage = (stage + 1) % kProjStages;
         }
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
     // the parts of this CTA, one after the other (a fixed order), into shared memory; then the CTAs of the cluster
     double* sums = smem;                                              // [rows8][kProjCols]
@@ -140,11 +166,11 @@ k_cesgc_project(const float* __restrict__ B, const float* __restrict__ G, float*
     cluster.sync();                                                   // nobody leaves while its sums may still be read
 }
 
-// Block = kBackCols columns x kBackRows rows of W: the block lists the non-zeros of its columns of U (ascending rows of B, whatever
+// Block = kBackCols columns x kBackSlabs slabs of kBackRows rows of W: the block lists the non-zeros of its columns of U (ascending rows of B, whatever
 // order they are found in), stages its rows of B^T as fp64, and its threads walk W in runs of four columns, so that reads and
 // writes are whole sectors (a block per column touched 32 bytes for every 4: 56 us at 4096 x 4096).  Runs of four without a
 // non-zero are not touched.
-constexpr int kBackCols = 64, kBackRows = 64, kBackThreads = 256;
+constexpr int kBackCols = 64, kBackRows = 64, kBackThreads = 256, kBackSlabs = 8;      // slabs of kBackRows rows per block
 
 __global__ void __launch_bounds__(kBackThreads)
 k_cesgc_back(const float* __restrict__ B, const float* __restrict__ U, float* __restrict__ W, int r, int m, int n) {
@@ -154,7 +180,7 @@ k_cesgc_back(const float* __restrict__ B, const float* __restrict__ U, float* __
     int* idx = reinterpret_cast<int*>(us + kBackCols * r);            // [kBackCols][r] rows of B
     __shared__ int count[kBackCols];
     const unsigned int col_blocks = (unsigned int)((n + kBackCols - 1) / kBackCols);
-    const int j0 = (int)(blockIdx.x % col_blocks) * kBackCols, i0 = (int)(blockIdx.x / col_blocks) * kBackRows, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int j0 = (int)(blockIdx.x % col_blocks) * kBackCols, r0 = (int)(blockIdx.x / col_blocks) * kBackRows * kBackSlabs, t = threadIdx.x, lane = t & 31, warp = t >> 5;
     // U tile, coalesced, then compacted: a warp per column and 32 rows at a time keeps the rows ascending
     for (int e = t; e < r * kBackCols; e += kBackThreads) {
         const int i = e / kBackCols, c = e % kBackCols;
@@ -184,36 +210,59 @@ k_cesgc_back(const float* __restrict__ B, const float* __restrict__ U, float* __
         any |= nz;
     }
     if (!__syncthreads_or(any)) return;
-    for (int e = t; e < r * kBackRows; e += kBackThreads) {
-        const int i = e / kBackRows, q = e % kBackRows;
-        bt[i * (kBackRows + 1) + q] = i0 + q < m ? (double)B[(size_t)i * m + i0 + q] : 0.0;
-    }
-    __syncthreads();
     const bool vec = (n & 3) == 0 && ((uintptr_t)W & 15u) == 0;
-    const int c4 = (t % (kBackCols / 4)) * 4;
+    const int c4 = (t % (kBackCols / 4)) * 4, q0 = t / (kBackCols / 4);
+    constexpr int kStep = kBackThreads / (kBackCols / 4), kRuns = kBackRows / kStep;        // this thread's runs of four in a slab
     int nz[4], most = 0;
 #pragma unroll
     for (int u = 0; u < 4; ++u) { nz[u] = count[c4 + u]; most = nz[u] > most ? nz[u] : most; }
-    if (most == 0) return;
-    for (int q = t / (kBackCols / 4); q < kBackRows && i0 + q < m; q += kBackThreads / (kBackCols / 4)) {
-        float* w = W + (size_t)(i0 + q) * n + j0 + c4;
-        float old[4];
-        if (vec) *reinterpret_cast<float4*>(old) = *reinterpret_cast<const float4*>(w);
-        else {
+    for (int i0 = r0; i0 < r0 + kBackRows * kBackSlabs && i0 < m; i0 += kBackRows) {
+        float old[kRuns][4];
+        if (most) {
 #pragma unroll
-            for (int u = 0; u < 4; ++u) old[u] = j0 + c4 + u < n ? w[u] : 0.0f;
+            for (int v = 0; v < kRuns; ++v) {
+                const int row = i0 + q0 + v * kStep;
+                if (row >= m) continue;
+                const float* w = W + (size_t)row * n + j0 + c4;
+                if (vec) *reinterpret_cast<float4*>(old[v]) = *reinterpret_cast<const float4*>(w);
+                else {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) old[v][u] = j0 + c4 + u < n ? w[u] : 0.0f;
+                }
+            }
         }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            if (nz[u] == 0) continue;
-            double acc = 0.0;
-            for (int e = 0; e < nz[u]; ++e) acc += bt[idx[(c4 + u) * r + e] * (kBackRows + 1) + q] * (double)us[(c4 + u) * r + e];
-            old[u] = (float)((double)old[u] + acc);
+        __syncthreads();                                              // the previous slab of B has been used up
+        for (int e = t; e < r * kBackRows; e += kBackThreads) {
+            const int i = e / kBackRows, q = e % kBackRows;
+            bt[i * (kBackRows + 1) + q] = i0 + q < m ? (double)B[(size_t)i * m + i0 + q] : 0.0;
         }
-        if (vec) *reinterpret_cast<float4*>(w) = *reinterpret_cast<const float4*>(old);
-        else {
+        __syncthreads();
+        if (!most) continue;
+        double acc[kRuns][4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) if (nz[u] != 0) w[u] = old[u];
+        for (int v = 0; v < kRuns; ++v)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) acc[v][u] = 0.0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            for (int e = 0; e < nz[u]; ++e) {
+                const double x = (double)us[(c4 + u) * r + e];
+                const double* bq = bt + idx[(c4 + u) * r + e] * (kBackRows + 1) + q0;
+#pragma unroll
+                for (int v = 0; v < kRuns; ++v) acc[v][u] += bq[v * kStep] * x;
+            }
+#pragma unroll
+        for (int v = 0; v < kRuns; ++v) {
+            const int row = i0 + q0 + v * kStep;
+            if (row >= m) continue;
+            float* w = W + (size_t)row * n + j0 + c4;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) if (nz[u]) old[v][u] = (float)((double)old[v][u] + acc[v][u]);
+            if (vec) *reinterpret_cast<float4*>(w) = *reinterpret_cast<const float4*>(old[v]);
+            else {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) if (nz[u]) w[u] = old[v][u];
+            }
         }
     }
 }
@@ -251,7 +300,7 @@ cudaError_t launch_cesgc_back(const float* B, const float* U, float* W, int r, i
     cudaError_t e = cudaFuncSetAttribute(k_cesgc_back, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)(kCesgcMaxR * ((kBackRows + 1) * sizeof(double) + 2 * kBackCols * sizeof(float))));
     if (e != cudaSuccess) return e;
-    const unsigned int blocks = (unsigned int)((n + kBackCols - 1) / kBackCols) * (unsigned int)((m + kBackRows - 1) / kBackRows);
+    const unsigned int blocks = (unsigned int)((n + kBackCols - 1) / kBackCols) * (unsigned int)((m + kBackRows * kBackSlabs - 1) / (kBackRows * kBackSlabs));
     k_cesgc_back<<<blocks, kBackThreads, smem, stream>>>(B, U, W, r, m, n);
     return cudaGetLastError();
 }

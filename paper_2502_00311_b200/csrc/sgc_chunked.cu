@@ -25,7 +25,6 @@ namespace sgc {
 namespace {
 
 constexpr int kFrontThreads = 512;
-constexpr int kCorrBlock = 256;          // threads per block of k_chunk_corr
 constexpr int kChunkMaxS = 32;
 constexpr int kChunkMaxK = 256;
 
@@ -62,7 +61,7 @@ __device__ __forceinline__ int frag_place(int row) {
     const int r = row & 15;
     return (row & ~15) + ((r & 7) >> 1) * 4 + (r >> 3) * 2 + (r & 1);
 }
-// one entry (scale: a power of two that brings the residual's norm into [2^10, 2^11)): the value and what it leaves
+// one entry (scale: a power of two that brings the residual's norm into [2^9, 2^10)): the value and what it leaves
 __device__ __forceinline__ void frag_write(const ChunkArgs& a, int res, int row, double v, double scale) {
     const float x = (float)(v * scale);
     const __half h = __float2half_rn(x);
@@ -267,10 +266,11 @@ k_chunk_front(ChunkArgs a, const float* __restrict__ grad, double b1, double b2,
 // rows the tensor work is small, what bounds the kernel is generating, comparing and the launch itself, and an operand in
 // registers needs no hand-off.  With one multiply-add per instruction it took 37 us at k_c = 8, 512 recoveries, 65536
 // columns, and 22 us per iteration at k_c = 217, 128 recoveries, 2048 columns.)
+__host__ __device__ constexpr int corr_threads(int kp) { return kp <= 32 ? 512 : 256; }              // (registers hold the residuals)
 __host__ __device__ constexpr int corr_kb(int kp) { return kp / 16 > 0 ? kp / 16 : 1; }              // 16-row blocks
 __host__ __device__ constexpr int corr_nt(int kp) { return kp == 64 ? 8 : (kp <= 128 ? 4 : 2); }     // tiles of four recoveries per warp
-__host__ __device__ constexpr int corr_group(int kp) { return kCorrBlock / 32 * 4 * corr_nt(kp); }   // recoveries per block
-__host__ __device__ constexpr int corr_tile(int kp) { return kp <= 64 ? 64 : 32; }                   // columns generated at a time
+__host__ __device__ constexpr int corr_group(int kp) { return corr_threads(kp) / 32 * 4 * corr_nt(kp); }   // recoveries per block
+__host__ __device__ constexpr int corr_tile(int kp) { return kp <= 16 ? 256 : kp == 32 ? 128 : kp == 64 ? 64 : 32; }   // columns generated at a time
 constexpr int kCorrSuper = 512;                                                                      // columns that a key can tell apart
 
 // The two kernels of an iteration are launched with programmatic stream serialization: the blocks of the next kernel may
@@ -310,12 +310,16 @@ struct Best2 {
     }
 };
 
+// 1 / ||Z|| of a column and the code that its keys carry
+__device__ __forceinline__ float2 corr_norm(float n2, int code, bool real) {
+    return make_float2(real && n2 > 0.0f ? 1.0f / sqrtf(n2) : 0.0f, __uint_as_float(real ? (unsigned int)code : 0u));
+}
+
 // gate != nullptr: the launch is a fallback of the tensor-core route and returns at once unless *gate names this
 // iteration (a.epoch): the word holds the epoch of the last iteration that left a recovery unresolved.
 template <int KP>
-__global__ void __launch_bounds__(kCorrBlock, KP <= 32 ? 2 : 1) k_chunk_corr(ChunkArgs a, int iter, const int* gate) {
-    constexpr int KB = corr_kb(KP), NT = corr_nt(KP), TC = corr_tile(KP), TILES = TC / 16, WARPS = kCorrBlock / 32;
-    constexpr int UNITS = TILES * KB;                                 // (16 columns, 16 rows): one warp's share of the generating
+__global__ void __launch_bounds__(corr_threads(KP)) k_chunk_corr(ChunkArgs a, int iter, const int* gate) {
+    constexpr int KB = corr_kb(KP), NT = corr_nt(KP), TC = corr_tile(KP), TILES = TC / 16, WARPS = corr_threads(KP) / 32;
     extern __shared__ uint4 smem4[];
     uint4* zt = smem4;                                                // [TILES][KB][32] A operands
     float2* inv = reinterpret_cast<float2*>(zt + TILES * KB * 32);    // [TC] 1 / ||Z_i||, code of the column
@@ -324,16 +328,22 @@ __global__ void __launch_bounds__(kCorrBlock, KP <= 32 ? 2 : 1) k_chunk_corr(Chu
     const long long col0 = (long long)blockIdx.x * a.cols_per_split;
     long long col1 = col0 + a.cols_per_split;
     if (col1 > a.dc) col1 = a.dc;
-    auto generate = [&](long long tile0) {
-        for (int u = warp; u < UNITS; u += WARPS) {
+    // code: see the keys below (columns beyond this block's range get code 0 and 1 / ||Z|| = 0)
+    // (unit of work: 16 columns, 16 rows)
+    auto generate = [&](long long tile0, int code0) {
+        const int units = (int)(col1 - tile0 < TC ? (col1 - tile0 + 15) / 16 : TILES) * KB;
+        for (int u = warp; u < units; u += WARPS) {
             const int tl = u / KB, kb = u % KB;
-            const uint32_t c0 = (uint32_t)(tile0 + tl * 16 + g), c1 = c0 + 8u;
-            const ColKey k0 = column_key(a.seed_lo, a.seed_hi, c0), k1 = column_key(a.seed_lo, a.seed_hi, c1);
-            const uint32_t h0 = k0.ck + (uint32_t)(kb * 8 + q) * k0.mk, h1 = k1.ck + (uint32_t)(kb * 8 + q) * k1.mk;
-            uint32_t z[4] = {z_pair_from_word(h0), z_pair_from_word(h1), z_pair_from_word(h0 + 4u * k0.mk), z_pair_from_word(h1 + 4u * k1.mk)};
+            // a column's key is worked out by one lane (lanes 0-15) and handed to the four that use it
+            const ColKey key = column_key(a.seed_lo, a.seed_hi, (uint32_t)(tile0 + tl * 16 + (lane & 15)));
+            const uint32_t ck0 = __shfl_sync(0xffffffffu, key.ck, g), mk0 = __shfl_sync(0xffffffffu, key.mk, g);
+            const uint32_t ck1 = __shfl_sync(0xffffffffu, key.ck, g + 8), mk1 = __shfl_sync(0xffffffffu, key.mk, g + 8);
+            const uint32_t h0 = ck0 + (uint32_t)(kb * 8 + q) * mk0, h1 = ck1 + (uint32_t)(kb * 8 + q) * mk1;
+            uint32_t z[4] = {z_pair_from_word(h0), z_pair_from_word(h1), 0u, 0u};
+            if (KP > 8) { z[2] = z_pair_from_word(h0 + 4u * mk0); z[3] = z_pair_from_word(h1 + 4u * mk1); }
             float n[2] = {0.0f, 0.0f};
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {                             // rows beyond k do not count
+            for (int e = 0; e < (KP > 8 ? 4 : 2); ++e) {              // rows beyond k do not count
                 const int row = kb * 16 + 2 * q + (e & 2 ? 8 : 0);
                 if (row >= a.k) z[e] = 0u;
                 else if (row + 1 >= a.k) z[e] &= 0xFFFFu;
@@ -344,15 +354,19 @@ __global__ void __launch_bounds__(kCorrBlock, KP <= 32 ? 2 : 1) k_chunk_corr(Chu
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
                 n[e] += __shfl_xor_sync(0xffffffffu, n[e], 1); n[e] += __shfl_xor_sync(0xffffffffu, n[e], 2);
-                if (q == 0) n2p[kb * TC + tl * 16 + g + 8 * e] = n[e];
+                const int c = tl * 16 + g + 8 * e;
+                if (q == 0) {
+                    if (KB > 1) n2p[kb * TC + c] = n[e];
+                    else inv[c] = corr_norm(n[e], code0 - c, tile0 + c < col1);
+                }
             }
         }
     };
-    if (gate == nullptr) generate(col0);                              // the first tile needs nothing of the kernels before
+    if (gate == nullptr) generate(col0, kCorrSuper);                              // the first tile needs nothing of the kernels before
     after_previous_kernel(a.early);
     if (gate != nullptr) {
         if (*gate != a.epoch0 + iter) return;
-        generate(col0);
+        generate(col0, kCorrSuper);
     }
     // residuals as B operands: n = g of a tile is value (g even) or remainder (g odd) of recovery 4 tile + g / 2.  (Recoveries
     // that have stopped are scored like the others; k_chunk_pick does not look at them.)
@@ -380,19 +394,20 @@ __global__ void __launch_bounds__(kCorrBlock, KP <= 32 ? 2 : 1) k_chunk_corr(Chu
             for (int i = 0; i < NT; ++i) k1[i] = k2[i] = 0u;
             const long long super1 = super + kCorrSuper < col1 ? super + kCorrSuper : col1;
             for (long long tile0 = super; tile0 < super1; tile0 += TC) {
-                if (tile0 != col0 || exclude) { __syncthreads(); generate(tile0); }
+                const int code0 = (int)(kCorrSuper - (tile0 - super));
+                if (tile0 != col0 || exclude) { __syncthreads(); generate(tile0, code0); }
                 __syncthreads();
-                if (threadIdx.x < TC) {
-                    float n2 = 0.0f;
+                if (KB > 1) {
+                    if (threadIdx.x < TC) {
+                        float n2 = 0.0f;
 #pragma unroll
-                    for (int kb = 0; kb < KB; ++kb) n2 += n2p[kb * TC + threadIdx.x];
-                    const bool real = tile0 + threadIdx.x < col1;     // code 0 (and score 0): no column of this block
-                    inv[threadIdx.x] = make_float2(real && n2 > 0.0f ? 1.0f / sqrtf(n2) : 0.0f,
-                                                   __uint_as_float(real ? (unsigned int)(kCorrSuper - (tile0 - super) - threadIdx.x) : 0u));
+                        for (int kb = 0; kb < KB; ++kb) n2 += n2p[kb * TC + threadIdx.x];
+                        inv[threadIdx.x] = corr_norm(n2, code0 - (int)threadIdx.x, tile0 + threadIdx.x < col1);
+                    }
+                    __syncthreads();
                 }
-                __syncthreads();
 #pragma unroll 1
-                for (int tl = 0; tl < TILES; ++tl) {
+                for (int tl = 0; tl < TILES && tile0 + tl * 16 < col1; ++tl) {
                     float acc[NT][4];
 #pragma unroll
                     for (int i = 0; i < NT; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.0f;
@@ -506,37 +521,29 @@ __device__ __forceinline__ float pick_max(PickSmem& sh, float v) {
     return m ? __uint_as_float(m - 1u) : -1.0f;
 }
 
-constexpr int kPickPairs = kChunkMaxK / 64;           // row pairs of a column per lane
+constexpr int kPickRows = kChunkMaxK / 32;            // rows of a column per lane
 
-// this warp's copy of a column (scaled by sigma; rows beyond k are zero): lane holds the row pairs lane, lane + 32, ...
-__device__ __forceinline__ void pick_column(const ChunkArgs& a, uint32_t col, double (&x)[2 * kPickPairs]) {
+// this warp's copy of a column (scaled by sigma; rows beyond k are zero): lane holds the rows lane, lane + 32, ... (a generated word
+// serves two rows, so it is worked out twice; in exchange the reads of the q_l are consecutive)
+__device__ __forceinline__ void pick_column(const ChunkArgs& a, uint32_t col, double (&x)[kPickRows]) {
     const ColKey key = column_key(a.seed_lo, a.seed_hi, col);
     const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int u = 0; u < kPickPairs; ++u) {
-        const int p = lane + 32 * u;
-        x[2 * u] = x[2 * u + 1] = 0.0;
-        if (2 * p < a.k) {
-            const float2 z = half2_bits_to_float2(z_pair_from_word(key.ck + (uint32_t)p * key.mk));
-            x[2 * u] = a.sigma * (double)z.x;
-            if (2 * p + 1 < a.k) x[2 * u + 1] = a.sigma * (double)z.y;
-        }
+    for (int u = 0; u < kPickRows; ++u) {
+        const int row = lane + 32 * u;
+        x[u] = row < a.k ? a.sigma * (double)z_at(key, (uint32_t)row) : 0.0;
     }
 }
 // this lane's part of <v, x>
-__device__ __forceinline__ double pick_dot(const ChunkArgs& a, const double* v, const double (&x)[2 * kPickPairs]) {
+__device__ __forceinline__ double pick_dot(const ChunkArgs& a, const double* v, const double (&x)[kPickRows]) {
     const int lane = threadIdx.x & 31;
     double acc = 0.0;
 #pragma unroll
-    for (int u = 0; u < kPickPairs; ++u) {
-        const int row = 2 * (lane + 32 * u);
-        if (row < a.k) acc = fma(v[row], x[2 * u], acc);
-        if (row + 1 < a.k) acc = fma(v[row + 1], x[2 * u + 1], acc);
-    }
+    for (int u = 0; u < kPickRows; ++u) if (lane + 32 * u < a.k) acc = fma(v[lane + 32 * u], x[u], acc);
     return acc;
 }
 // c_l = <q_l, a> for all earlier picks: warp = two vectors at a time
-__device__ __forceinline__ void pick_products(const ChunkArgs& a, PickSmem& sh, const double* qs, int j, const double (&x)[2 * kPickPairs]) {
+__device__ __forceinline__ void pick_products(const ChunkArgs& a, PickSmem& sh, const double* qs, int j, const double (&x)[kPickRows]) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     for (int l = warp; l < j; l += 2 * warps) {
         const int l2 = l + warps < j ? l + warps : l;
@@ -558,13 +565,13 @@ __device__ void pick_finish(const ChunkArgs& a, const ChunkRef& ref, PickSmem& s
     double* r = pick_mem();
     double* qs = r + k;
     __syncthreads();                                                 // the staged state and the candidates are complete
-    double x[2 * kPickPairs];
+    double x[kPickRows];
     // exact scores (warp = one candidate, the last warp takes the first), and the products of the first candidate with the q_l
     for (int c = (warps - 1) - warp; c < nc; c += warps) {
         pick_column(a, sh.cidx[c], x);
         double dot = pick_dot(a, r, x), n2 = 0.0;
 #pragma unroll
-        for (int u = 0; u < 2 * kPickPairs; ++u) n2 = fma(x[u], x[u], n2);
+        for (int u = 0; u < kPickRows; ++u) n2 = fma(x[u], x[u], n2);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) { dot += __shfl_xor_sync(0xffffffffu, dot, o); n2 += __shfl_xor_sync(0xffffffffu, n2, o); }
         if (lane == 0) { sh.cdot[c] = dot; sh.cn2[c] = n2; }
@@ -864,7 +871,7 @@ int corr_resident() {
     size_t smem = 0;
     int blocks = 0;
     if (corr_setup<KP>(&smem) != cudaSuccess) return 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_chunk_corr<KP>, kCorrBlock, smem) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_chunk_corr<KP>, corr_threads(KP), smem) != cudaSuccess) return 0;
     return blocks;
 }
 
@@ -882,7 +889,7 @@ int corr_resident(int kp) {
 template <int KP>
 cudaError_t corr_launch(const ChunkArgs& a, int iter, size_t smem, cudaStream_t stream, const int* gate) {
     dim3 grid((unsigned int)a.splits, (unsigned int)((2 * a.c + corr_group(KP) - 1) / corr_group(KP)));
-    ChainedLaunch l(grid, dim3(kCorrBlock), smem, stream);
+    ChainedLaunch l(grid, dim3((unsigned int)corr_threads(KP)), smem, stream);
     return cudaLaunchKernelEx(&l.cfg, k_chunk_corr<KP>, a, iter, gate);
 }
 
@@ -902,9 +909,11 @@ cudaError_t ensure_ws(sgc_state* const* sts, int c) {
     ws->c = c; ws->key = key; ws->kp = padded_k(st0->k);
     // column splits: as many blocks as the SMs hold at a time (one wave), at least one tile per split
     const int groups = (2 * c + corr_group(ws->kp) - 1) / corr_group(ws->kp);
-    const int tile = corr_tile(ws->kp);
+    constexpr int tile = 16;                                         // columns that an operand of the correlation holds
     int resident = corr_resident(ws->kp);
     if (resident < 1) { delete ws; return cudaErrorLaunchOutOfResources; }
+    // with few columns per SM one block each will do: the kernel that follows then finds room beside it (see `early`)
+    if ((double)st0->d * groups <= 256.0 * st0->sm_count) resident = 1;
     int splits = resident * st0->sm_count / groups;
     const long long max_splits = (st0->d + tile - 1) / tile;
     if (splits > max_splits) splits = (int)max_splits;
@@ -1028,8 +1037,7 @@ cudaError_t launch_chunked_batch(sgc_state* const* sts, int c, const float* grad
         a.early = (ws->splits * groups <= st0->sm_count && 2 * c <= st0->sm_count) ? 1 : 0;
     }
     a.cols_per_split = (int)((st0->d + ws->splits - 1) / ws->splits);
-    const int tile = corr_tile(ws->kp);
-    a.cols_per_split = (a.cols_per_split + tile - 1) / tile * tile;
+    a.cols_per_split = (a.cols_per_split + 15) / 16 * 16;
     a.kp64 = ws->kp64; a.rt = ws->rt; a.tau = ws->tau; a.inv_scale = ws->inv_scale; a.rep_count = ws->rep_count; a.rep = ws->rep;
     a.rnv = ws->rnv; a.unresolved = ws->unresolved; a.flags = ws->flags; a.z_rep = ws->z_rep;
     // names the iterations of this step in the gate word: 1 + (step count mod 2^20) * 64 + iteration, never 0
@@ -1042,7 +1050,7 @@ cudaError_t launch_chunked_batch(sgc_state* const* sts, int c, const float* grad
     const double c1 = 1.0 - pow(b1, (double)st0->t), c2 = 1.0 - pow(b2, (double)st0->t);
     const int s = st0->s;
     {
-        // blocks per chunk: up to two blocks per SM, at least four vectors per thread
+        // blocks per chunk: up to two blocks per SM, at least four vectors per thread (256 chunks of 65536 in 512 blocks: 22 -> 35 us)
         int split = 1;
         while (split < kFrontMaxSplit && 2 * split * c <= 2 * st0->sm_count && st0->d >= (int64_t)2 * split * kFrontThreads * 16) split *= 2;
         cudaLaunchConfig_t cfg = {};

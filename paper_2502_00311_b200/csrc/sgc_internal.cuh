@@ -147,10 +147,9 @@ __device__ __forceinline__ double screen_margin(double rn, double ps, int k) {
 // power-of-two scale that brings a residual of norm rn into [2^12, 2^13): no binary16 overflow, and entries
 // down to 2^-26 of the norm stay normal numbers
 __device__ __forceinline__ double residual_scale(double rn) {
-    if (!(rn > 0.0) || !isfinite(rn)) return 1.0;
-    int e;
-    frexp(rn, &e);
-    return ldexp(1.0, 13 - e);
+    const int e = (int)((unsigned long long)__double_as_longlong(rn) >> 52);        // 2^(e - 1023) <= rn < 2^(e - 1022); a norm is not negative
+    if (e < 32 || e >= 2047) return 1.0;
+    return __longlong_as_double((long long)(2058 - e) << 52);
 }
 
 constexpr uint32_t kNoColumn = 0xFFFFFFFFu;

@@ -65,7 +65,7 @@ __device__ __forceinline__ bool in_list(const uint32_t* lam, int n, uint32_t col
 
 // shared memory of k_omp that has a fixed size
 struct OmpSmem {
-    unsigned int wkey[kWarps], wkey2[kWarps];
+    unsigned int wkey[kWarps], wkey2[kWarps], floor_key[2];
     float npart[64][16];
     double wsum[kWarps];
     Top wtop[2][kWarps];
@@ -127,9 +127,15 @@ __device__ __forceinline__ bool in_support4(const uint32_t* sup, int n, uint32_t
     return hit;
 }
 
-// (a column of the support scores rounding noise: the look-up is needed only for what would enter the best two)
-__device__ __forceinline__ void offer(const OmpSmem& sh, Top& best, const int* picks, int m, float score, uint32_t col) {
-    if (score > best.s2 && !in_support4(sh.sup[m], picks[m], col)) best.push(score, col);
+// The threads of the block tell one another the second best score that each has seen: a column at or below any of these can be
+// neither the block's best nor its second best, so that after the first few columns hardly any gets further than one compare.
+// (A column of the support scores rounding noise: the look-up is needed only for what passes.)
+__device__ __forceinline__ void offer(OmpSmem& sh, Top& best, const int* picks, int m, float score, uint32_t col) {
+    if (!(score > best.s2) || score_key(score) <= *reinterpret_cast<volatile unsigned int*>(&sh.floor_key[m])) return;
+    if (in_support4(sh.sup[m], picks[m], col)) return;
+    const float before = best.s2;
+    best.push(score, col);
+    if (best.s2 > before && best.s2 >= 0.0f) atomicMax(&sh.floor_key[m], score_key(best.s2));
 }
 
 __device__ __forceinline__ void mma_16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
@@ -176,6 +182,7 @@ __device__ void stage_residuals(const OmpArgs& a, OmpSmem& sh, uint2* frag, floa
     }
     m0 = __reduce_max_sync(0xffffffffu, m0); m1 = __reduce_max_sync(0xffffffffu, m1);
     if (lane == 0) { sh.wkey[warp] = m0; sh.wkey2[warp] = m1; }
+    if (t < 2) sh.floor_key[t] = 0u;
     __syncthreads();
     m0 = __reduce_max_sync(0xffffffffu, lane < kWarps ? sh.wkey[lane] : 0u);
     m1 = __reduce_max_sync(0xffffffffu, lane < kWarps ? sh.wkey2[lane] : 0u);
@@ -213,18 +220,22 @@ __device__ void correlate(const OmpArgs& a, OmpSmem& sh, const CorrPlan& c, cons
     const bool have = filled && c.norms, read = filled && c.cached;
     Top best;                                                         // of residual q & 1
     best.init();
-    const int units = c.tiles * c.ks, kper = (c.kblocks + c.ks - 1) / c.ks;
+    const int ks_log = 31 - __clz(c.ks), units = c.tiles * c.ks, kper = (c.kblocks + c.ks - 1) / c.ks;
     for (int u = warp; u < units; u += kWarps) {
-        const int tile = u / c.ks, part_k = u % c.ks;
+        const int tile = u >> ks_log, part_k = u & (c.ks - 1);
         const int kb0 = part_k * kper, kb1 = kb0 + kper < c.kblocks ? kb0 + kper : c.kblocks;
         const int i0 = tile * 16 + g, i1 = i0 + 8;
         const bool ok0 = i0 < c.cnt, ok1 = i1 < c.cnt;
         float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
         float n0 = 0.0f, n1 = 0.0f;
-        uint32_t col0 = kNoColumn, col1 = kNoColumn;
-        if (ok0) col0 = col_list ? (have ? col_s[i0] : col_list[c.e0 + i0]) : (uint32_t)(c.e0 + i0);
-        if (ok1) col1 = col_list ? (have ? col_s[i1] : col_list[c.e0 + i1]) : (uint32_t)(c.e0 + i1);
-        if (c.norms && !have && part_k == 0 && q == 0) { col_s[i0] = col0; col_s[i1] = col1; }
+        // lane l < 16 looks up column l of the tile (and works out its key); the others get theirs from it
+        uint32_t col_l = kNoColumn;
+        {
+            const int il = tile * 16 + (lane & 15);
+            if (il < c.cnt) col_l = col_list ? (have ? col_s[il] : col_list[c.e0 + il]) : (uint32_t)(c.e0 + il);
+            if (c.norms && !have && part_k == 0 && lane < 16) col_s[il] = col_l;
+        }
+        const uint32_t col0 = __shfl_sync(0xffffffffu, col_l, g), col1 = __shfl_sync(0xffffffffu, col_l, g + 8);
         const uint2* fb = frag + lane;
         uint4* zt = zc + (size_t)tile * c.kblocks * 32 + lane;
         if (read) {
@@ -235,7 +246,10 @@ __device__ void correlate(const OmpArgs& a, OmpSmem& sh, const CorrPlan& c, cons
                 mma_16816(acc, z.x, z.y, z.z, z.w, b.x, b.y);
             }
         } else {
-            const ColKey k0 = column_key(a.seed_lo, a.seed_hi, col0), k1 = column_key(a.seed_lo, a.seed_hi, col1);
+            const ColKey key = column_key(a.seed_lo, a.seed_hi, col_l);
+            ColKey k0, k1;
+            k0.ck = __shfl_sync(0xffffffffu, key.ck, g); k0.mk = __shfl_sync(0xffffffffu, key.mk, g);
+            k1.ck = __shfl_sync(0xffffffffu, key.ck, g + 8); k1.mk = __shfl_sync(0xffffffffu, key.mk, g + 8);
             uint32_t h00 = k0.ck + (uint32_t)(kb0 * 8 + q) * k0.mk, h01 = h00 + 4u * k0.mk;
             uint32_t h10 = k1.ck + (uint32_t)(kb0 * 8 + q) * k1.mk, h11 = h10 + 4u * k1.mk;
             const uint32_t st0 = 8u * k0.mk, st1 = 8u * k1.mk;

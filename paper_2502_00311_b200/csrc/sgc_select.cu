@@ -1,15 +1,15 @@
 // a1: G~ = Sparsify_s(G)  (Section 3.2: keep the s entries of largest magnitude, zero the rest).
 //
 // The answer is the set of the s largest keys  key(i) = (|g_i| bit pattern) << 32 | ~i  (unique; the
-// ~i part sends ties to the lower index).  HBM traffic is one read of the gradient:
-//   1. k_sample   reads <= 2^18..2^24 strided elements, builds a 12-bit magnitude histogram and derives a
-//                 threshold tau under which roughly max(2048, 8s) elements of the whole vector lie above;
-//   2. k_filter   streams the gradient once with 128-bit loads and appends every key >= tau to a
-//                 candidate list (a few thousand entries);
-//   3. k_pick     one block: exact radix select of the s largest candidate keys, sort by index.
-// If the candidate list ends up with fewer than s or more than its capacity (degenerate value
-// distributions, e.g. all magnitudes equal), k_pick instead runs the same exact radix select over the
-// whole gradient (slow, still correct) and reports SGC_STATUS_SELECT_FALLBACK.
+// ~i part sends ties to the lower index).  Three ways, by what is known beforehand and by size:
+//   k_select_fast    a state's second and later steps: one launch with the threshold that the previous step left behind;
+//   k_unit_max,      no threshold known (a state's first step, sgc_sparsify_static): one read of the gradient gives the
+//   k_unit_pick      largest magnitude of each of up to 4096 units (interleaved shares); the s-th largest of those maxima is a
+//                    bound that at least s elements reach, so only the units whose maximum reaches it are read again, and the
+//                    last block to finish makes the exact pick from the elements found;
+//   k_select_small   vectors of at most kSelCap elements: the same idea inside one block.
+// If too many elements reach the bound (degenerate value distributions, e.g. all magnitudes equal), the exact radix
+// selection runs over the whole gradient instead (slow, still correct) and reports SGC_STATUS_SELECT_FALLBACK.
 #include <mutex>
 
 #include "sgc_internal.cuh"
@@ -17,60 +17,7 @@
 namespace sgc {
 namespace {
 
-constexpr int kSampleThreads = 256;
-constexpr int kSampleChunk = 256;
-
 __device__ __forceinline__ uint32_t mag_bits(float g) { return __float_as_uint(g) & 0x7FFFFFFFu; }
-
-__global__ void __launch_bounds__(kSampleThreads)
-k_sample(const float* __restrict__ grad, unsigned long long d, unsigned int n_chunks, unsigned int target,
-         unsigned int* __restrict__ hist, Counters* __restrict__ cnt, int direct) {
-    if (direct) {   // the whole vector fits in the candidate list: no threshold needed
-        if (blockIdx.x == 0 && threadIdx.x == 0) { cnt->sel_tau = 0u; cnt->sel_count = 0u; }
-        return;
-    }
-    __shared__ unsigned int sh[kSelBins];
-    __shared__ unsigned int part[kSampleThreads];
-    __shared__ bool last;
-    for (int b = threadIdx.x; b < kSelBins; b += kSampleThreads) sh[b] = 0u;
-    __syncthreads();
-    for (unsigned int c = blockIdx.x; c < n_chunks; c += gridDim.x) {
-        const unsigned long long start = (((unsigned long long)c * d) / n_chunks) & ~3ull;
-        const unsigned long long next = (c + 1 == n_chunks) ? d : ((((unsigned long long)(c + 1) * d) / n_chunks) & ~3ull);
-        const unsigned long long i = start + threadIdx.x;
-        if (i < next && i < start + kSampleChunk) atomicAdd(&sh[mag_bits(__ldg(grad + i)) >> 19], 1u);
-    }
-    __syncthreads();
-    for (int b = threadIdx.x; b < kSelBins; b += kSampleThreads)
-        if (sh[b]) atomicAdd(&hist[b], sh[b]);
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) last = (atomicAdd(&cnt->sel_ticket, 1u) == gridDim.x - 1);
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    // last block: largest bin b such that (number of sampled keys in bins >= b) >= target
-    constexpr int per = kSelBins / kSampleThreads;      // 16 bins per thread
-    unsigned int mine = 0;
-    for (int u = 0; u < per; ++u) mine += __ldcg(&hist[threadIdx.x * per + u]);
-    part[threadIdx.x] = mine;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned int acc = 0, tau = 0;
-        int t = kSampleThreads - 1;
-        for (; t >= 0; --t) { if (acc + part[t] >= target) break; acc += part[t]; }
-        if (t >= 0) {
-            int b = t * per + per - 1;
-            for (; b >= t * per; --b) { acc += __ldcg(&hist[b]); if (acc >= target) break; }
-            tau = (unsigned int)b << 19;
-        }
-        cnt->sel_tau = tau;
-        cnt->sel_count = 0u;
-        cnt->sel_ticket = 0u;
-    }
-    __syncthreads();
-    for (int b = threadIdx.x; b < kSelBins; b += kSampleThreads) hist[b] = 0u;    // ready for the next step
-}
 
 __device__ __forceinline__ void consider(float g, unsigned long long i, unsigned int tau, unsigned long long* cand,
                                          Counters* cnt) {
@@ -82,42 +29,7 @@ __device__ __forceinline__ void consider(float g, unsigned long long i, unsigned
     }
 }
 
-__global__ void __launch_bounds__(512)
-k_filter(const float* __restrict__ grad, unsigned long long d, unsigned long long* __restrict__ cand,
-         Counters* __restrict__ cnt) {
-    const unsigned int tau = cnt->sel_tau;
-    const unsigned long long n4 = d >> 2;
-    const float4* g4 = reinterpret_cast<const float4*>(grad);
-    const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
-    unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
-    for (; i + 3 * stride < n4; i += 4 * stride) {            // four independent 128-bit loads in flight
-        const float4 a = __ldcs(g4 + i), b = __ldcs(g4 + i + stride), c = __ldcs(g4 + i + 2 * stride),
-                     e = __ldcs(g4 + i + 3 * stride);
-        // largest sign-cleared bit pattern of the 16 values (orders magnitudes; NaN and infinity sort on top)
-        const uint32_t m0 = max(max(mag_bits(a.x), mag_bits(a.y)), max(mag_bits(a.z), mag_bits(a.w)));
-        const uint32_t m1 = max(max(mag_bits(b.x), mag_bits(b.y)), max(mag_bits(b.z), mag_bits(b.w)));
-        const uint32_t m2 = max(max(mag_bits(c.x), mag_bits(c.y)), max(mag_bits(c.z), mag_bits(c.w)));
-        const uint32_t m3 = max(max(mag_bits(e.x), mag_bits(e.y)), max(mag_bits(e.z), mag_bits(e.w)));
-        const bool hit = max(max(m0, m1), max(m2, m3)) >= tau;
-        if (hit) {
-            const float v[16] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w, e.x, e.y, e.z, e.w};
-#pragma unroll
-            for (int u = 0; u < 16; ++u) consider(v[u], (i + (u >> 2) * stride) * 4 + (u & 3), tau, cand, cnt);
-        }
-    }
-    for (; i < n4; i += stride) {
-        const float4 a = __ldcs(g4 + i);
-        consider(a.x, i * 4 + 0, tau, cand, cnt); consider(a.y, i * 4 + 1, tau, cand, cnt);
-        consider(a.z, i * 4 + 2, tau, cand, cnt); consider(a.w, i * 4 + 3, tau, cand, cnt);
-    }
-    if (blockIdx.x == 0 && threadIdx.x < (d & 3ull)) {       // ragged tail
-        const unsigned long long t = (n4 << 2) + threadIdx.x;
-        consider(grad[t], t, tau, cand, cnt);
-    }
-}
-
 // ---- exact selection of the s largest 64-bit keys by one block ---------------------------------------
-constexpr int kPickThreads = 1024;
 constexpr int kDigitBits = 11;
 constexpr int kDigits = 1 << kDigitBits;
 
@@ -241,16 +153,213 @@ __device__ void pick_block(PickSmem& sm, const float* __restrict__ grad, unsigne
     }
 }
 
-// carry_out: the sampled threshold is left for the next call's one-kernel selection, which appends to an empty list
-__global__ void __launch_bounds__(kPickThreads)
-k_pick(const float* __restrict__ grad, unsigned long long d, unsigned int s, const unsigned long long* __restrict__ cand,
-       Counters* __restrict__ cnt, uint32_t* __restrict__ sel_idx, float* __restrict__ sel_val, int carry_out) {
-    __shared__ PickSmem sm;
-    pick_block<kPickThreads>(sm, grad, d, s, cand, cnt->sel_count, cnt, sel_idx, sel_val);
-    if (carry_out && threadIdx.x == 0) {
-        cnt->sel_tau_next = cnt->sel_tau;
-        cnt->sel_count = 0u;
+// next threshold of a state from a result: a quarter octave below the smallest kept magnitude
+__device__ __forceinline__ unsigned int tau_below(const float* sel_val, unsigned int s) {
+    uint32_t lo = 0xFFFFFFFFu;
+    for (unsigned int e = 0; e < s; ++e) lo = min(lo, mag_bits(sel_val[e]));
+    return ((lo >> 19) > 4u ? (lo >> 19) - 4u : 1u) << 19;
+}
+
+// ---- selection without a threshold ---------------------------------------------------------------------------
+// unit = `lanes` neighbouring threads of the grid (8 or 32) and what they read in a grid-stride walk over 16-byte vectors: the
+// elements of unit u are the vectors i with (i % T) / lanes == u, T the number of threads.  Units without a vector report 0.
+// bound: HBM, 4 d bytes; eight vectors per thread in flight (180 MB: 31 us, then 12 us for k_unit_pick; the sampled threshold
+// that this replaces took 23 us to find before a 31 us filter).
+constexpr int kUnitLoads = 8;
+constexpr int kUnitPickThreads = 512;
+constexpr int kHotUnits = 512;                       // units that one block can list for reading again
+
+__global__ void __launch_bounds__(512)
+k_unit_max(const float* __restrict__ grad, unsigned long long d, int lanes, unsigned int* __restrict__ unit_max, Counters* __restrict__ cnt,
+           int clear_status) {
+    const unsigned long long n4 = d >> 2, T = (unsigned long long)gridDim.x * blockDim.x;
+    const float4* g4 = reinterpret_cast<const float4*>(grad);
+    const unsigned long long t = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t == 0) { cnt->sel_count = 0u; cnt->sel_ticket = 0u; if (clear_status) cnt->status = 0u; }
+    uint32_t m = 0u;
+    unsigned long long i = t;
+    for (; i + (kUnitLoads - 1) * T < n4; i += kUnitLoads * T) {
+        float4 v[kUnitLoads];
+#pragma unroll
+        for (int u = 0; u < kUnitLoads; ++u) v[u] = g4[i + u * T];
+#pragma unroll
+        for (int u = 0; u < kUnitLoads; ++u)
+            m = max(m, max(max(mag_bits(v[u].x), mag_bits(v[u].y)), max(mag_bits(v[u].z), mag_bits(v[u].w))));
     }
+    for (; i < n4; i += T) {
+        const float4 v = g4[i];
+        m = max(m, max(max(mag_bits(v.x), mag_bits(v.y)), max(mag_bits(v.z), mag_bits(v.w))));
+    }
+    if (t < (d & 3ull)) m = max(m, mag_bits(grad[(n4 << 2) + t]));       // ragged tail: threads 0..2, that is unit 0
+    if (lanes == 32) m = __reduce_max_sync(0xffffffffu, m);
+    else for (int o = 4; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & (lanes - 1)) == 0) unit_max[t / lanes] = m;
+}
+
+// same grid and block as k_unit_max (T and the units must agree); n_units <= kSelBins.  out_status may be null.
+__global__ void __launch_bounds__(kUnitPickThreads)
+k_unit_pick(const float* __restrict__ grad, unsigned long long d, unsigned int s, int lanes, unsigned long long T, unsigned int n_units,
+            unsigned int* __restrict__ unit_max, unsigned long long* __restrict__ cand, Counters* __restrict__ cnt,
+            uint32_t* __restrict__ sel_idx, float* __restrict__ sel_val, int carry_out, uint32_t* __restrict__ out_status) {
+    __shared__ __align__(16) unsigned int hist[kSelBins];
+    __shared__ PickSmem sm;
+    __shared__ unsigned int part[32];
+    __shared__ unsigned int hot[kHotUnits];
+    __shared__ unsigned int tau_bin, n_hot;
+    __shared__ bool last;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    for (int b = t; b < kSelBins; b += kUnitPickThreads) hist[b] = 0u;
+    if (t == 0) { tau_bin = 0u; n_hot = 0u; }
+    __syncthreads();
+    // the bin of the s-th largest maximum (1/16 octave wide); its lower edge is the bound
+    constexpr int kPer = kSelBins / kUnitPickThreads;
+    unsigned int mine[kPer];
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) { const unsigned int e = t + u * kUnitPickThreads; mine[u] = e < n_units ? __ldcg(unit_max + e) : 0u; }
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) if (t + u * kUnitPickThreads < (int)n_units) atomicAdd(&hist[mine[u] >> 19], 1u);
+    __syncthreads();
+    {
+        unsigned int own = 0u;
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) own += hist[t * kPer + u];
+        unsigned int incl = own;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const unsigned int v = __shfl_down_sync(0xffffffffu, incl, o); if (lane + o < 32) incl += v; }
+        if (lane == 0) part[warp] = incl;
+        __syncthreads();
+        for (int w = warp + 1; w < kUnitPickThreads / 32; ++w) incl += part[w];
+        unsigned int above = incl - own;
+        if (above < s && s <= incl)
+            for (int u = kPer - 1; u >= 0; --u) { above += hist[t * kPer + u]; if (above >= s) { tau_bin = t * kPer + u; break; } }
+    }
+    __syncthreads();
+    const unsigned int tau = tau_bin << 19;                              // (fewer than s units: 0, everything qualifies)
+    // this block's units whose maximum reaches the bound, read again by the whole block, one after the other
+    const unsigned long long n4 = d >> 2;
+    const float4* g4 = reinterpret_cast<const float4*>(grad);
+    const unsigned int per_block = (n_units + gridDim.x - 1) / gridDim.x, u0 = blockIdx.x * per_block;
+    for (unsigned int u = u0 + t; u < u0 + per_block && u < n_units; u += kUnitPickThreads)
+        if (__ldcg(unit_max + u) >= tau) { const unsigned int q = atomicAdd(&n_hot, 1u); if (q < (unsigned int)kHotUnits) hot[q] = u; }
+    __syncthreads();
+    const unsigned int nh = min(n_hot, (unsigned int)kHotUnits);
+    const int groups = kUnitPickThreads / lanes, grp = t / lanes, in = t % lanes;
+    for (unsigned int q = 0; q < nh; ++q) {
+        const unsigned long long first = (unsigned long long)hot[q] * lanes + in;
+#pragma unroll 4
+        for (unsigned long long i = first + (unsigned long long)grp * T; i < n4; i += (unsigned long long)groups * T) {
+            const float4 v = g4[i];
+            const float e[4] = {v.x, v.y, v.z, v.w};
+            if (max(max(mag_bits(v.x), mag_bits(v.y)), max(mag_bits(v.z), mag_bits(v.w))) >= tau) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) consider(e[c], i * 4 + c, tau, cand, cnt);
+            }
+        }
+        if (hot[q] == 0u && (unsigned long long)t < (d & 3ull)) consider(grad[(n4 << 2) + t], (n4 << 2) + t, tau, cand, cnt);
+    }
+    if (n_hot > (unsigned int)kHotUnits && t == 0) atomicAdd(&cnt->sel_count, (unsigned int)kSelCap + 1u);   // more than can be listed: the exact path serves
+    __threadfence();
+    __syncthreads();
+    if (t == 0) last = (atomicAdd(&cnt->sel_ticket, 1u) == gridDim.x - 1);
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const unsigned int count = __ldcg(&cnt->sel_count);
+    const unsigned long long* src = cand;
+    if (count >= s && count <= (unsigned int)(kSelBins / 2)) {
+        unsigned long long* staged = reinterpret_cast<unsigned long long*>(hist);
+        __syncthreads();
+        for (unsigned int e = t; e < count; e += kUnitPickThreads) staged[e] = __ldcg(cand + e);
+        __syncthreads();
+        src = staged;
+    }
+    pick_block<kUnitPickThreads>(sm, grad, d, s, src, count, cnt, sel_idx, sel_val);
+    for (unsigned int e = t; e < n_units; e += kUnitPickThreads) unit_max[e] = 0u;        // the histogram of k_select_fast lives here
+    __syncthreads();
+    if (t == 0) {
+        if (carry_out) cnt->sel_tau_next = tau_below(sel_val, s);
+        cnt->sel_count = 0u; cnt->sel_ticket = 0u;
+        if (out_status) *out_status = cnt->status;
+    }
+}
+
+// A vector of at most kSelCap elements, one block: thread maxima, the smallest over the warps of a warp's e-th largest one as the
+// bound (e = ceil(s / warps): at least s elements reach it), and the exact pick among what reaches it.  Replaces three launches.
+constexpr int kSmallThreads = 1024;
+
+__global__ void __launch_bounds__(kSmallThreads)
+k_select_small(const float* __restrict__ grad, unsigned int d, unsigned int s, unsigned long long* __restrict__ cand, Counters* __restrict__ cnt,
+               uint32_t* __restrict__ sel_idx, float* __restrict__ sel_val, int clear_status, uint32_t* __restrict__ out_status) {
+    __shared__ PickSmem sm;
+    __shared__ unsigned long long list[2048];
+    __shared__ unsigned int wtau[kSmallThreads / 32];
+    __shared__ unsigned int n_list;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    if (t == 0) { n_list = 0u; cnt->sel_count = 0u; if (clear_status) cnt->status = 0u; }
+    const unsigned int n4 = d >> 2;
+    const float4* g4 = reinterpret_cast<const float4*>(grad);
+    constexpr int kHold = kSelCap / 4 / kSmallThreads;                   // 8 vectors per thread at most
+    float4 v[kHold];
+    float tail = 0.0f;
+    const bool has_tail = (unsigned int)t < (d & 3u);
+#pragma unroll
+    for (int u = 0; u < kHold; ++u) { const unsigned int i = t + u * kSmallThreads; v[u] = i < n4 ? g4[i] : make_float4(0.0f, 0.0f, 0.0f, 0.0f); }
+    if (has_tail) tail = grad[(n4 << 2) + t];
+    uint32_t top = mag_bits(tail);
+#pragma unroll
+    for (int u = 0; u < kHold; ++u) top = max(top, max(max(mag_bits(v[u].x), mag_bits(v[u].y)), max(mag_bits(v[u].z), mag_bits(v[u].w))));
+    if (__syncthreads_or(top >= 0x7F800000u) && t == 0) atomicOr(&cnt->status, (unsigned int)SGC_STATUS_NONFINITE_INPUT);
+    {
+        const int e = (int)((s + kSmallThreads / 32 - 1) / (kSmallThreads / 32));
+        unsigned int m = 0u;
+        bool out = false;
+        for (int q = 0; q < e; ++q) {
+            m = __reduce_max_sync(0xffffffffu, out ? 0u : top);
+            const unsigned int who = __ballot_sync(0xffffffffu, !out && top == m);
+            if (who != 0u && lane == __ffs(who) - 1) out = true;
+        }
+        if (lane == 0) wtau[warp] = m;
+    }
+    __syncthreads();
+    const unsigned int tau = __reduce_min_sync(0xffffffffu, wtau[lane]);
+    auto offer = [&](float g, unsigned int i) {
+        if (i < d && mag_bits(g) >= tau) {
+            const unsigned int q = atomicAdd(&n_list, 1u);
+            const unsigned long long key = ((unsigned long long)mag_bits(g) << 32) | (uint32_t)(~i);
+            if (q < 2048u) list[q] = key;
+            cand[q] = key;                                               // (at most d <= kSelCap of them)
+        }
+    };
+#pragma unroll
+    for (int u = 0; u < kHold; ++u) {
+        const unsigned int i = 4u * (t + u * kSmallThreads);
+        if (i >= (n4 << 2)) continue;
+        offer(v[u].x, i); offer(v[u].y, i + 1u); offer(v[u].z, i + 2u); offer(v[u].w, i + 3u);
+    }
+    if (has_tail) offer(tail, (n4 << 2) + t);
+    __syncthreads();
+    const unsigned int n = n_list;
+    if (n <= kSmallThreads) {
+        // rank of each among all: the s largest, then their order by index
+        const unsigned long long mine = t < (int)n ? list[t] : 0ull;
+        unsigned int r = 0;
+        for (unsigned int q = 0; q < n; ++q) r += list[q] > mine ? 1u : 0u;
+        const bool keep = t < (int)n && r < s;
+        if (keep) sm.picked[r] = ~(uint32_t)mine;
+        __syncthreads();
+        if (t < (int)s) {
+            const uint32_t idx = sm.picked[t];
+            unsigned int rank = 0;
+            for (unsigned int q = 0; q < s; ++q) rank += sm.picked[q] < idx ? 1u : 0u;
+            sel_idx[rank] = idx; sel_val[rank] = grad[idx];
+        }
+    } else {
+        __threadfence();
+        __syncthreads();
+        pick_block<kSmallThreads>(sm, grad, d, s, n <= 2048u ? list : cand, n, cnt, sel_idx, sel_val);
+    }
+    if (out_status && t == 0) *out_status = cnt->status;
 }
 
 // ---- the one-kernel selection of a warm state ---------------------------------------------------------------
@@ -261,7 +370,7 @@ k_pick(const float* __restrict__ grad, unsigned long long d, unsigned int s, con
 // histogram and makes the exact pick.  A miss (fewer than s survivors, or more than the list holds: the law moved by
 // a factor of several from one step to the next) is served by the same block with the exact selection over the whole
 // gradient -- milliseconds instead of microseconds, flagged SGC_STATUS_SELECT_FALLBACK -- which also yields the next tau.
-// The first step of a state has no tau and takes the sampled path (k_sample, k_filter, k_pick) instead.
+// The first step of a state has no tau and takes the path without a threshold instead.
 constexpr int kFastLoads = 4;                       // 128-bit loads in flight per thread
 constexpr int kFastThreads = 512;                   // three blocks per SM, four loads each: 96 KB in flight per SM
 constexpr int kTailBins = 8;                        // histogram bins kept below tau
@@ -386,9 +495,7 @@ k_select_fast(const float* __restrict__ grad, unsigned long long d, unsigned int
         unsigned int nb = next_bin;
         if (!hit) {
             // next threshold from the result itself: a quarter octave below the smallest kept magnitude
-            uint32_t lo = 0xFFFFFFFFu;
-            for (unsigned int e = 0; e < s; ++e) lo = min(lo, mag_bits(sel_val[e]));
-            nb = (lo >> 19) > 4u ? (lo >> 19) - 4u : 1u;
+            nb = tau_below(sel_val, s) >> 19;
         }
         if (nb < 1u) nb = 1u;
         cnt->sel_tau_next = nb << 19;
@@ -397,78 +504,56 @@ k_select_fast(const float* __restrict__ grad, unsigned long long d, unsigned int
     }
 }
 
-// Launch geometry of the selection for a vector of length d with s kept entries: one definition for every caller.
-struct SelectPlan {
-    int direct;                 // the whole vector fits in the candidate list: no threshold needed
-    unsigned int n_chunks;      // sample: 256-element chunks, between 2^10 and 2^16 of them
-    unsigned int target;        // rank in the sample that corresponds to max(2048, 8 s) survivors in the vector
-    int sample_grid;
-    unsigned int filter_blocks;
-    unsigned int want;          // survivors aimed at: max(2048, 8 s)
-};
-
-SelectPlan plan_select(unsigned long long d, int s, int sm_count) {
-    SelectPlan p;
-    p.direct = d <= (unsigned long long)kSelCap;
-    unsigned long long n_chunks = d / 16384ull;
-    if (n_chunks < 1024ull) n_chunks = 1024ull;
-    if (n_chunks > 65536ull) n_chunks = 65536ull;
-    unsigned long long n_sample = n_chunks * kSampleChunk;
-    if (n_sample > d) n_sample = d;
-    unsigned long long want = 8ull * (unsigned long long)s;
-    if (want < 2048ull) want = 2048ull;
-    unsigned long long target = (want * n_sample + d - 1) / d;       // rank in the sample
-    if (target < 32ull) target = 32ull;
-    p.want = (unsigned int)want;
-    p.n_chunks = (unsigned int)n_chunks;
-    p.target = (unsigned int)target;
-    p.sample_grid = (int)(n_chunks < 4096ull ? n_chunks / 8 : 512);
-    if (p.sample_grid < 1) p.sample_grid = 1;
-    const unsigned long long n4 = d >> 2;
-    unsigned long long blocks = (n4 + 512ull * 4ull - 1) / (512ull * 4ull);
-    const unsigned long long max_blocks = (unsigned long long)sm_count * 4ull;
-    if (blocks > max_blocks) blocks = max_blocks;
-    if (blocks < 1) blocks = 1;
-    p.filter_blocks = (unsigned int)blocks;
-    return p;
-}
-
-// The launches of the selection on `stream`; hist and the counters must be zero on entry (the kernels leave them so for
-// the next call).  warm: a threshold carried from the previous call exists, and the one-kernel selection runs; otherwise
-// the sampled path (sample, filter, pick), which leaves its threshold behind when carry_out is set.  `timed` (may be null)
-// receives the per-kernel timing when profiling is on.
+// The launches of the selection on `stream`; hist must be zero on entry (the kernels leave it so for the next call).
+// warm: a threshold carried from the previous call exists, and the one-kernel selection runs; otherwise a threshold is left
+// behind when carry_out is set.  `timed` (may be null) receives the per-kernel timing when profiling is on.  own_status: the
+// counters belong to this call alone (their status word is cleared, and copied to out_status at the end).
 cudaError_t enqueue_select(const float* grad, unsigned long long d, int s, int sm_count, unsigned int* hist,
                            unsigned long long* cand, Counters* cnt, uint32_t* out_idx, float* out_val, cudaStream_t stream,
-                           sgc_state* timed, bool warm, bool carry_out, int* launches) {
-    const SelectPlan p = plan_select(d, s, sm_count);
-    if (warm && !p.direct) {
-        PhaseTimer timer(timed, stream, kPhaseFilter, 1);
-        k_select_fast<<<3 * sm_count, kFastThreads, 0, stream>>>(grad, d, (unsigned int)s, p.want, cand, hist, cnt, out_idx, out_val);
+                           sgc_state* timed, bool warm, bool carry_out, bool own_status, uint32_t* out_status, int* launches) {
+    if (d <= (unsigned long long)kSelCap) {
+        PhaseTimer timer(timed, stream, kPhasePick, 1);
+        k_select_small<<<1, kSmallThreads, 0, stream>>>(grad, (unsigned int)d, (unsigned int)s, cand, cnt, out_idx, out_val, own_status ? 1 : 0, out_status);
         *launches += 1;
         return cudaGetLastError();
     }
-    {
-        PhaseTimer timer(timed, stream, kPhaseSample, 1);
-        k_sample<<<p.direct ? 1 : p.sample_grid, kSampleThreads, 0, stream>>>(grad, d, p.n_chunks, p.target, hist, cnt, p.direct);
+    if (warm) {
+        unsigned long long want = 8ull * (unsigned long long)s;          // survivors aimed at
+        if (want < 2048ull) want = 2048ull;
+        PhaseTimer timer(timed, stream, kPhaseFilter, 1);
+        k_select_fast<<<3 * sm_count, kFastThreads, 0, stream>>>(grad, d, (unsigned int)s, (unsigned int)want, cand, hist, cnt, out_idx, out_val);
+        *launches += 1;
+        return cudaGetLastError();
     }
+    // units: 32 threads each for long vectors (two blocks of at most 512 threads per SM, as many as give 4096 units); 8 threads
+    // each for short ones, so that there are at least as many units with an element as entries to keep (s <= 1024, d > 32768)
+    const int lanes = d >= (1ull << 22) ? 32 : 8;
+    int blocks, threads;
+    if (lanes == 32) { blocks = 2 * sm_count; threads = kSelBins / blocks * 32; if (threads > 512) threads = 512; if (threads < 32) { threads = 32; blocks = kSelBins; } }
+    else { blocks = 128; threads = 256; }
+    const unsigned int n_units = (unsigned int)(blocks * (threads / lanes));
     {
         PhaseTimer timer(timed, stream, kPhaseFilter, 1);
-        k_filter<<<p.filter_blocks, 512, 0, stream>>>(grad, d, cand, cnt);
+        k_unit_max<<<blocks, threads, 0, stream>>>(grad, d, lanes, hist, cnt, own_status ? 1 : 0);
     }
-    {
-        PhaseTimer timer(timed, stream, kPhasePick, 1);
-        k_pick<<<1, kPickThreads, 0, stream>>>(grad, d, (unsigned int)s, cand, cnt, out_idx, out_val, carry_out && !p.direct ? 1 : 0);
-    }
-    *launches += 3;
-    return cudaGetLastError();
+    PhaseTimer timer(timed, stream, kPhasePick, 1);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(n_units < (unsigned)sm_count ? n_units : (unsigned)sm_count)); cfg.blockDim = dim3(kUnitPickThreads); cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    *launches += 2;
+    return cudaLaunchKernelEx(&cfg, k_unit_pick, grad, d, (unsigned int)s, lanes, (unsigned long long)blocks * threads, n_units, hist, cand, cnt,
+                              out_idx, out_val, carry_out ? 1 : 0, out_status);
 }
 
 }  // namespace
 
 cudaError_t launch_select(sgc_state* st, const float* grad, cudaStream_t stream, int* launches) {
-    // the first selection of a state samples its threshold; every later one carries it
+    // the first selection of a state finds its threshold; every later one carries it
     const cudaError_t e = enqueue_select(grad, (unsigned long long)st->d, st->s, st->sm_count, st->sel_hist, st->sel_cand,
-                                         st->cnt, st->sel_idx, st->sel_val, stream, st, st->sel_warm, true, launches);
+                                         st->cnt, st->sel_idx, st->sel_val, stream, st, st->sel_warm, true, false, nullptr, launches);
     if (e == cudaSuccess) st->sel_warm = true;
     return e;
 }
@@ -509,8 +594,6 @@ struct StaticSetup { bool ready; unsigned char* ptr; int sm_count; };
 StaticSetup g_static_setup[kMaxDevices];            // zero-initialised; written once per device
 std::mutex g_static_mutex;
 
-__global__ void k_copy_status(const Counters* __restrict__ cnt, uint32_t* __restrict__ out) { *out = cnt->status; }
-
 }  // namespace
 }  // namespace sgc
 
@@ -544,13 +627,9 @@ extern "C" SGC_API int sgc_sparsify_static(const float* grad, int64_t d, int32_t
     Counters* cnt = reinterpret_cast<Counters*>(setup.ptr + kStaticCntOff);
     unsigned int* hist = reinterpret_cast<unsigned int*>(setup.ptr + kStaticHistOff);
     unsigned long long* cand = reinterpret_cast<unsigned long long*>(setup.ptr + kStaticCandOff);
-    // counters and histogram must start at zero; the candidate list is overwritten before it is read
-    e = cudaMemsetAsync(setup.ptr, 0, kStaticCandOff, cs);
-    if (e != cudaSuccess) return (int)e;
     int launches = 0;
-    e = enqueue_select(grad, (unsigned long long)d, s, setup.sm_count, hist, cand, cnt, out_idx, out_val, cs, nullptr, false, false,
-                       &launches);
+    e = enqueue_select(grad, (unsigned long long)d, s, setup.sm_count, hist, cand, cnt, out_idx, out_val, cs, nullptr, false, false, true,
+                       out_status, &launches);
     if (e != cudaSuccess) return (int)e;
-    if (out_status) k_copy_status<<<1, 1, 0, cs>>>(cnt, out_status);
     return (int)cudaGetLastError();
 }
