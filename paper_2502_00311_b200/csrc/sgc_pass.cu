@@ -16,7 +16,7 @@
 // speculated pick, and it harvests new candidates.
 //
 // One persistent CTA per SM; warp roles: 0 = TMA producer, 1 = MMA issuer (owns the tensor-memory
-// allocation), 2-5 = epilogue (one per 32-lane quadrant of tensor memory), 6-21 = generators.
+// allocation), 2-9 = epilogue (two per 32-lane quadrant of tensor memory), 10-25 = generators.
 // Every wait on an mbarrier is bounded (two seconds unless the caller sets another limit); on expiry the CTA records an
 // error, leaves all loops, waits for the matrix operations and copies it still has in flight, frees its tensor memory and
 // returns.
@@ -30,8 +30,9 @@ namespace sgc {
 namespace {
 
 constexpr int kGenWarps = 16;                                // 512 generator threads: two per column of a sweep
-constexpr int kFirstGenWarp = 6;                             // warps 2..5 are the epilogue
-constexpr int kPassThreads = 32 * (kFirstGenWarp + kGenWarps);   // 704
+constexpr int kEpiWarps = 8;                                 // warps 2..9: two per tensor-memory quadrant, half of the columns each
+constexpr int kFirstGenWarp = 2 + kEpiWarps;
+constexpr int kPassThreads = 32 * (kFirstGenWarp + kGenWarps);   // 832
 constexpr int kTileCols = 128;                               // UMMA M: columns of A per accumulator tile
 constexpr int kSuperCols = 2 * kTileCols;                    // columns of A per sweep over k
 constexpr int kChunkRows = 64;                               // rows of A per pipeline stage (128 B of binary16)
@@ -262,7 +263,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(bar_accf + 8u * b, 1);
-            mbar_init(bar_acce + 8u * b, 4);
+            mbar_init(bar_acce + 8u * b, kEpiWarps);
         }
         mbar_init(bar_drain, 1);
         *abort_flag = 0;
@@ -346,30 +347,31 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
         }
     } else if (warp < kFirstGenWarp) {
         // ---------------- epilogue: scores against thresholds ----------------------------------------------
-        const int quad = warp & 3;
+        const int quad = warp & 3, side = (warp - 2) >> 2, ew = side * 4 + quad;      // this warp's quadrant and half of the columns
+        constexpr int kHalf = kSuperCols / 2;
         uint32_t sweep_i = 0;
         bool ok = true;
         // room for the reports: what the table of norms leaves of its ring (the swapped form keeps 12 KB of it for other things)
         ReportQueue queue_r;
-        queue_r.mem = TABLE ? reinterpret_cast<uint32_t*>(norms + (SWAP ? (size_t)(12 + quad) * kSuperCols : (size_t)quad * 4 * kSuperCols))
-                            : reinterpret_cast<uint32_t*>(norms) + kNormRing * kSuperCols * 2 + 768 + quad * kSuperCols;
-        queue_r.cap = ((TABLE && !SWAP ? 4 : 1) * kSuperCols - 1) / 3;
+        queue_r.mem = TABLE ? reinterpret_cast<uint32_t*>(norms + (SWAP ? 12 * (size_t)kSuperCols + ew * kHalf : (size_t)ew * 2 * kSuperCols))
+                            : reinterpret_cast<uint32_t*>(norms) + kNormRing * kSuperCols * 2 + 768 + ew * kHalf;
+        queue_r.cap = ((TABLE && !SWAP ? 4 : 1) * kHalf - 1) / 3;
         queue_r.init(lane);
         for (unsigned int sweep = blockIdx.x; ok && sweep < num_super; sweep += gridDim.x, ++sweep_i) {
             const uint32_t buf = sweep_i % a.bufs, use = sweep_i / a.bufs;
-            if (!__all_sync(0xffffffffu, mbar_wait(bar_accf + 8u * buf, use & 1u, abort_flag, 512, a.wait_limit_ns))) { ok = false; break; }
-            tc_fence_after();
+            // (what the sweep's scores are divided by is fetched before its accumulators are waited for)
             if (SWAP) {
                 // this thread owns residual n_res; the 256 columns of the sweep run along the tensor-memory columns.  Each
                 // epilogue warp keeps its own copy of the sweep's 1 / ||Z_i|| as floats (no barrier between the warps)
                 const int n_res = quad * 32 + lane;
                 const float tau_n = tau_s[n_res];
-                float* inv_w = norms + (size_t)quad * kSuperCols;
-                uint32_t* col_w = reinterpret_cast<uint32_t*>(norms + (size_t)(4 + quad) * kSuperCols);   // list pass: the columns
+                float* inv_w = norms + (size_t)ew * kHalf;
+                uint32_t* col_w = reinterpret_cast<uint32_t*>(norms + 4 * (size_t)kSuperCols + ew * kHalf);      // list pass: the columns
+                const unsigned long long col_first = (unsigned long long)sweep * kSuperCols + side * kHalf;
                 __syncwarp();
 #pragma unroll
-                for (int q = 0; q < kSuperCols / 32; ++q) {
-                    unsigned long long col = (unsigned long long)sweep * kSuperCols + q * 32 + lane;
+                for (int q = 0; q < kHalf / 32; ++q) {
+                    unsigned long long col = col_first + q * 32 + lane;
                     if (listed) {
                         const unsigned int idx = (unsigned int)col;
                         col = idx < list_n0 ? a.big_list[idx] : (idx < list_n ? a.big_list[(size_t)a.big_cap + idx - list_n0] : a.d);
@@ -378,20 +380,22 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
                     inv_w[q * 32 + lane] = col < a.d ? half_bits_to_float(a.inv_norm[col]) : 0.0f;
                 }
                 __syncwarp();
+                if (!__all_sync(0xffffffffu, mbar_wait(bar_accf + 8u * buf, use & 1u, abort_flag, 512, a.wait_limit_ns))) { ok = false; break; }
+                tc_fence_after();
                 // some residuals feed the wide list of their stream (full passes of the two-level screening)
                 const float wide_tau_n = WIDE && a.big_tau != nullptr && !listed ? a.big_tau[n_res] : __int_as_float(0x7f800000);
                 const bool feeds = WIDE && wide_tau_n < __int_as_float(0x7f800000);
                 // wide-list hits of this warp are queued in shared memory and appended after the sweep, all at once: the two
                 // dependent global atomics of an append then cost the warp two round trips per sweep instead of two per hit
                 // (the warp's 32 residuals belong to one stream whenever the streams' blocks are multiples of 32 rows)
-                uint32_t* queue = reinterpret_cast<uint32_t*>(norms + (size_t)(8 + quad) * kSuperCols);
+                uint32_t* queue = reinterpret_cast<uint32_t*>(norms + 8 * (size_t)kSuperCols + ew * kHalf);
                 const bool queued = WIDE && (a.big_half & 31) == 0;
                 if (WIDE && lane == 0) queue[0] = 0u;
                 if (WIDE) __syncwarp();
 #pragma unroll 1
-                for (int c0 = 0; c0 < kSuperCols; c0 += 16) {
+                for (int c0 = 0; c0 < kHalf; c0 += 16) {
                     uint32_t v[16];
-                    tmem_ld16(tmem_base + ((uint32_t)(quad * 32) << 16) + buf * acc_cols + c0, v);
+                    tmem_ld16(tmem_base + ((uint32_t)(quad * 32) << 16) + buf * acc_cols + side * kHalf + c0, v);
                     float peak = 0.0f;
                     const float4* in4 = reinterpret_cast<const float4*>(inv_w + c0);
 #pragma unroll
@@ -411,10 +415,10 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
                         while (hits) {
                             const int i = __ffs(hits) - 1;
                             hits &= hits - 1u;
-                            const unsigned long long col = (unsigned long long)sweep * kSuperCols + c0 + i;
+                            const unsigned long long col = col_first + c0 + i;
                             if (queued) {
                                 const unsigned int qs = atomicAdd(&queue[0], 1u) + 1u;
-                                if (qs < (unsigned int)kSuperCols) { queue[qs] = (uint32_t)col; continue; }
+                                if (qs < (unsigned int)kHalf) { queue[qs] = (uint32_t)col; continue; }
                             }
                             const unsigned int bit = 1u << ((unsigned int)col & 31u);
                             if (!(atomicOr(&a.big_bits[(size_t)m * ((a.d + 31) >> 5) + (col >> 5)], bit) & bit)) {
@@ -429,7 +433,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
                         const float inv = inv_w[c0 + i];
                         const float sc = fabsf(__uint_as_float(v[i])) * inv;
                         if (sc >= tau_n && inv > 0.0f) {
-                            const uint32_t col = listed ? col_w[c0 + i] : (uint32_t)((unsigned long long)sweep * kSuperCols + c0 + i);
+                            const uint32_t col = listed ? col_w[c0 + i] : (uint32_t)(col_first + c0 + i);
                             report_push(a, queue_r, (uint32_t)n_res, col, sc);
                         }
                     }
@@ -439,7 +443,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
                 if (lane == 0) mbar_arrive(bar_acce + 8u * buf);     // the accumulator is free; the queued appends follow
                 if (WIDE && queued) {
                     unsigned int qn = queue[0];
-                    if (qn > (unsigned int)kSuperCols - 1u) qn = (unsigned int)kSuperCols - 1u;
+                    if (qn > (unsigned int)kHalf - 1u) qn = (unsigned int)kHalf - 1u;
                     const int m = quad * 32 >= a.big_half ? 1 : 0;
                     for (unsigned int e = 1u + lane; e <= qn; e += 32u) {
                         const unsigned long long col = queue[e];
@@ -455,23 +459,30 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
                 continue;
             }
             const float* nr = norms + (size_t)(sweep_i % kNormRing) * kSuperCols * 2;
+            unsigned long long cols[2];
+            float invs[2] = {0.0f, 0.0f};
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                cols[t] = (unsigned long long)sweep * kSuperCols + t * kTileCols + quad * 32 + lane;
+                if (listed) {
+                    const unsigned int idx = (unsigned int)cols[t];
+                    cols[t] = idx < list_n0 ? a.big_list[idx] : (idx < list_n ? a.big_list[(size_t)a.big_cap + idx - list_n0] : a.d);
+                }
+                if (TABLE && cols[t] < a.d) invs[t] = half_bits_to_float(a.inv_norm[cols[t]]);
+            }
+            if (!__all_sync(0xffffffffu, mbar_wait(bar_accf + 8u * buf, use & 1u, abort_flag, 512, a.wait_limit_ns))) { ok = false; break; }
+            tc_fence_after();
 #pragma unroll 1
             for (int t = 0; t < 2; ++t) {
-                const int col_local = t * kTileCols + quad * 32 + lane;
-                unsigned long long col = (unsigned long long)sweep * kSuperCols + col_local;
-                if (listed) {
-                    const unsigned int idx = (unsigned int)col;
-                    col = idx < list_n0 ? a.big_list[idx] : (idx < list_n ? a.big_list[(size_t)a.big_cap + idx - list_n0] : a.d);
-                }
-                float inv = 0.0f;
-                if (TABLE) {
-                    if (col < a.d) inv = half_bits_to_float(a.inv_norm[col]);
-                } else {
+                const unsigned long long col = t ? cols[1] : cols[0];
+                float inv = t ? invs[1] : invs[0];
+                if (!TABLE) {
+                    const int col_local = t * kTileCols + quad * 32 + lane;
                     const float n2 = nr[col_local * 2] + nr[col_local * 2 + 1];
                     if (col < a.d && n2 > 0.0f) inv = 1.0f / sqrtf(n2);
                 }
 #pragma unroll 1
-                for (int c0 = 0; c0 < a.n; c0 += 16) {
+                for (int c0 = side * (a.n / 2); c0 < (side + 1) * (a.n / 2); c0 += 16) {
                     uint32_t v[16];
                     tmem_ld16(tmem_base + ((uint32_t)(quad * 32) << 16) + buf * acc_cols + t * a.n + c0, v);
                     if (WIDE && a.big_tau != nullptr && !listed && inv > 0.0f) {
