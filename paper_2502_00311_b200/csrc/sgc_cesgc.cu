@@ -5,11 +5,11 @@
 //   k_cesgc_project   P = B G in fp64, rounded to fp32 once, so that the top-s selection that follows decides on the exactly
 //                     projected gradient.  64 fp64 multiply-adds per cycle and SM bound it (30 us for a 4096 x 4096 gradient at
 //                     r = 32); conversions from fp32, a quarter as fast, are kept out of the way: a thread owns four columns and
-//                     eight rows, converts each element of G once for its eight products and reads B as fp64 from a slab that
-//                     the block has converted on the way in; G arrives by asynchronous copies, three slabs ahead (with one
-//                     slab ahead in registers the kernel waited for memory: 138 us).  (An error-free two-float form took 276 us, fp64 with both operands
-//                     converted per product 1.1 ms.)  The rows of G are split over the CTAs of a thread-block cluster; their
-//                     partial sums meet through distributed shared memory, added in rank order.
+//                     eight rows and reads both operands as fp64 from slabs that the block has converted, each element once.  G
+//                     arrives by asynchronous copies, three slabs ahead (with one slab ahead in registers the kernel waited for
+//                     memory: 138 us; an error-free two-float form took 276 us, fp64 with both operands converted per product
+//                     1.1 ms).  The rows of G are split over the CTAs of a thread-block cluster; their partial sums meet through
+//                     distributed shared memory, added in rank order.
 //   k_cesgc_back      W += B^T U for the r x n matrix U that the SGC core left (U = -eta N has at most s non-zeros).
 #include "sgc_internal.cuh"
 
@@ -30,12 +30,13 @@ constexpr int kProjResident = 148;       // one wave
 
 // groups of 8 rows of B (warps of a part), parts (each with every parts-th row of G) that make up 16 warps at most, rows of G per slab
 __host__ __device__ constexpr int proj_groups(int r) { return (r + kProjRows - 1) / kProjRows; }
-__host__ __device__ constexpr int proj_parts(int r) { return proj_groups(r) > 4 ? 2 : proj_groups(r) > 2 ? 4 : 8; }
+__host__ __device__ constexpr int proj_parts(int r) { return proj_groups(r) > 4 ? 2 : 4; }
 __host__ __device__ constexpr int proj_slab(int r) { return kProjPer * proj_parts(r); }
 // slabs of B (two, fp64), slabs of G; at the end the partial sums of the parts
-__host__ __device__ constexpr size_t proj_bslab(int r) { return 2 * (size_t)proj_groups(r) * kProjRows * proj_slab(r) * sizeof(double); }
+// (rows of a staged slab of B are two doubles longer than there are values: the stores that transpose it then spread over the banks)
+__host__ __device__ constexpr size_t proj_bslab(int r) { return 2 * (size_t)(proj_groups(r) * kProjRows + 2) * proj_slab(r) * sizeof(double); }
 __host__ __device__ constexpr size_t proj_smem(int r) {
-    const size_t slab = proj_bslab(r) + (size_t)kProjStages * proj_slab(r) * kProjCols * sizeof(float);
+    const size_t slab = proj_bslab(r) + (size_t)proj_slab(r) * kProjCols * (kProjStages * sizeof(float) + 2 * sizeof(double));
     const size_t part = (size_t)proj_groups(r) * kProjRows * kProjCols * sizeof(double);
     return slab > part ? slab : part;
 }
@@ -50,7 +51,7 @@ __global__ void __launch_bounds__(512, 1)
 k_cesgc_project(const float* __restrict__ B, const float* __restrict__ G, float* __restrict__ P, int r, int m, int n) {
     extern __shared__ double smem[];
     cg::cluster_group cluster = cg::this_cluster();
-    const int groups = proj_groups(r), rows8 = groups * kProjRows, parts = proj_parts(r), slab_rows = proj_slab(r);
+    const int groups = proj_groups(r), rows8 = groups * kProjRows, bstride = rows8 + 2, parts = proj_parts(r), slab_rows = proj_slab(r);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ig = warp % groups, part = warp / groups;
     // this CTA's rows of G: whole slabs, the same number for every CTA of the cluster (the last ranges may be empty)
@@ -80,7 +81,7 @@ k_cesgc_project(const float* __restrict__ B, const float* __restrict__ G, float*
 #pragma unroll
         for (int u = 0; u < kBHold; ++u) {
             const int e = (int)threadIdx.x + u * threads;
-            if (e < b_items) { const int i = e / slab_rows, q = e % slab_rows; dst[q * rows8 + i] = (double)bh[u]; }
+            if (e < b_items) { const int i = e / slab_rows, q = e % slab_rows; dst[q * bstride + i] = (double)bh[u]; }
         }
     };
     float* gbuf = reinterpret_cast<float*>(smem + proj_bslab(r) / sizeof(double));      // [kProjStages][slab_rows][kProjCols]
@@ -106,33 +107,50 @@ k_cesgc_project(const float* __restrict__ B, const float* __restrict__ G, float*
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    double* bufs[2] = {smem, smem + (size_t)rows8 * slab_rows};
+    double* bufs[2] = {smem, smem + (size_t)bstride * slab_rows};
+    double* gd[2];                                                    // [slab_rows][kProjCols] a slab of G as fp64: converted once, used by every group of rows
+    gd[0] = reinterpret_cast<double*>(gbuf + (size_t)kProjStages * slab_rows * kProjCols);
+    gd[1] = gd[0] + (size_t)slab_rows * kProjCols;
+    // columns 4 c .. 4 c + 3 go to places 2 c, 2 c + 1 and 64 + 2 c, 64 + 2 c + 1: two consecutive 16-byte reads per lane
+    auto convert_g = [&](int stage, double* dst) {
+        const float* src = gbuf + (size_t)stage * slab_rows * kProjCols;
+        for (int e = threadIdx.x; e < slab_rows * (kProjCols / 4); e += threads) {
+            const int q = e / (kProjCols / 4), c = e % (kProjCols / 4);
+            const float4 f = *reinterpret_cast<const float4*>(src + q * kProjCols + 4 * c);
+            double2* d = reinterpret_cast<double2*>(dst + q * kProjCols);
+            d[c] = make_double2((double)f.x, (double)f.y);
+            d[kProjCols / 4 + c] = make_double2((double)f.z, (double)f.w);
+        }
+    };
     if (m_begin < m_end) {
         fetch_b(m_begin);
         for (int st = 0; st < kProjStages - 1; ++st) copy_g(st, m_begin + st * slab_rows);
         store_b(bufs[0]);
+        asm volatile("cp.async.wait_group %0;" ::"n"(kProjStages - 2) : "memory");
+        __syncthreads();
+        convert_g(0, gd[0]);
         int b = 0, stage = 0;
         for (int row0 = m_begin; row0 < m_end; row0 += slab_rows) {
-            asm volatile("cp.async.wait_group %0;" ::"n"(kProjStages - 2) : "memory");
-            __syncthreads();                                          // slab `stage` of G and slab b of B are staged, the others used up
+            // slab `stage` + 1 of G has arrived; slab b of B and of the converted G are complete, the others used up
+            asm volatile("cp.async.wait_group %0;" ::"n"(kProjStages - 3) : "memory");
+            __syncthreads();
             copy_g((stage + kProjStages - 1) % kProjStages, row0 + (kProjStages - 1) * slab_rows);
             const bool more = row0 + slab_rows < m_end;
-            if (more) fetch_b(row0 + slab_rows);
+            if (more) { fetch_b(row0 + slab_rows); convert_g((stage + 1) % kProjStages, gd[b ^ 1]); }
             const double* slab = bufs[b] + ig * kProjRows;
-            const float* gs = gbuf + (size_t)stage * slab_rows * kProjCols + 4 * lane;
+            const double2* gs = reinterpret_cast<const double2*>(gd[b]) + lane;
 #pragma unroll 2
             for (int q = 0; q < kProjPer; ++q) {
                 const int row = q * parts + part;
-                const float4 g = *reinterpret_cast<const float4*>(gs + row * kProjCols);
-                const double2* bq = reinterpret_cast<const double2*>(slab + (size_t)row * rows8);
-                const double gx = (double)g.x, gy = (double)g.y, gz = (double)g.z, gw = (double)g.w;
+                const double2 g0 = gs[row * (kProjCols / 2)], g1 = gs[row * (kProjCols / 2) + kProjCols / 4];
+                const double2* bq = reinterpret_cast<const double2*>(slab + (size_t)row * bstride);
 #pragma unroll
                 for (int u = 0; u < kProjRows / 2; ++u) {
                     const double2 v = bq[u];
-                    acc[2 * u][0] = fma(v.x, gx, acc[2 * u][0]); acc[2 * u][1] = fma(v.x, gy, acc[2 * u][1]);
-                    acc[2 * u][2] = fma(v.x, gz, acc[2 * u][2]); acc[2 * u][3] = fma(v.x, gw, acc[2 * u][3]);
-                    acc[2 * u + 1][0] = fma(v.y, gx, acc[2 * u + 1][0]); acc[2 * u + 1][1] = fma(v.y, gy, acc[2 * u + 1][1]);
-                    acc[2 * u + 1][2] = fma(v.y, gz, acc[2 * u + 1][2]); acc[2 * u + 1][3] = fma(v.y, gw, acc[2 * u + 1][3]);
+                    acc[2 * u][0] = fma(v.x, g0.x, acc[2 * u][0]); acc[2 * u][1] = fma(v.x, g0.y, acc[2 * u][1]);
+                    acc[2 * u][2] = fma(v.x, g1.x, acc[2 * u][2]); acc[2 * u][3] = fma(v.x, g1.y, acc[2 * u][3]);
+                    acc[2 * u + 1][0] = fma(v.y, g0.x, acc[2 * u + 1][0]); acc[2 * u + 1][1] = fma(v.y, g0.y, acc[2 * u + 1][1]);
+                    acc[2 * u + 1][2] = fma(v.y, g1.x, acc[2 * u + 1][2]); acc[2 * u + 1][3] = fma(v.y, g1.y, acc[2 * u + 1][3]);
                 }
             }
             if (more) store_b(bufs[b ^ 1]);

@@ -379,6 +379,18 @@ __global__ void __launch_bounds__(corr_threads(KP)) k_chunk_corr(ChunkArgs a, in
 #pragma unroll
         for (int kb = 0; kb < KB; ++kb) bf[i][kb] = src[4 * kb];
     }
+    // lane g of a recovery's eight holds every eighth column of its support, for the check at the end
+    constexpr int kHeld = kChunkMaxS / 8;
+    uint32_t held[NT][kHeld];
+    if (NT <= 4) {
+#pragma unroll
+        for (int i = 0; i < NT; ++i) {
+            const int mine = res0 + 4 * i + q;
+            const uint32_t* sup = a.lam + (size_t)(mine < 2 * a.c ? mine : 0) * a.s;
+#pragma unroll
+            for (int h = 0; h < kHeld; ++h) held[i][h] = g + 8 * h < iter ? sup[g + 8 * h] : kNoColumn;
+        }
+    }
     // Scores are compared as keys: the score's bits with the lowest ten replaced by a code of the column (relative error 2^-13, an
     // eighth of the window that k_chunk_pick rescores), so that the best two follow from three integer minima and maxima, without
     // a branch.  Columns of a recovery's support score rounding noise; should one be among the best two all the same (hardly any
@@ -447,13 +459,18 @@ __global__ void __launch_bounds__(corr_threads(KP)) k_chunk_corr(ChunkArgs a, in
             }
         }
         if (exclude || iter == 0) break;
-        // lane g = l of a recovery looks at every eighth column of its support
         bool taken = false;
 #pragma unroll
         for (int i = 0; i < NT; ++i) {
-            const int mine = res0 + 4 * i + q;
-            const uint32_t* sup = a.lam + (size_t)(mine < 2 * a.c ? mine : 0) * a.s;
-            for (int l = g; l < iter; l += 8) { const uint32_t v = sup[l]; taken = taken || v == best[i].i1 || v == best[i].i2; }
+            if (NT <= 4) {
+#pragma unroll
+                for (int h = 0; h < kHeld; ++h)
+                    taken = taken || (held[i][h] != kNoColumn && (held[i][h] == best[i].i1 || held[i][h] == best[i].i2));
+            } else {
+                const int mine = res0 + 4 * i + q;
+                const uint32_t* sup = a.lam + (size_t)(mine < 2 * a.c ? mine : 0) * a.s;
+                for (int l = g; l < iter; l += 8) { const uint32_t v = sup[l]; taken = taken || v == best[i].i1 || v == best[i].i2; }
+            }
         }
         if (!__syncthreads_or(taken ? 1 : 0)) break;
         exclude = true;

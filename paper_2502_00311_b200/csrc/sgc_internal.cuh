@@ -117,7 +117,11 @@ constexpr int kWideCap = 2097152;       // columns per wide list (two-level scre
 constexpr int kResolveBlocks = 16;        // blocks of the resolve kernel: all sweep the report lists, the last to finish walks the picks
 constexpr int kPassFastRows = 128;      // a pass over up to this many residual rows costs half of a wider one (A is generated once either way)
 constexpr int kMiniRounds = 8;          // list passes between two full passes, at most
-constexpr int kMiniDepth = 32;          // picks speculated ahead of one list pass
+// Picks speculated ahead of one list pass; half as many with few rows of A, where a pick changes the residual more and a list pass
+// costs less beside the picks that a refuted one throws away (ms per step at depth 32 / 16: d = 3 M, k = 700, s = 100: 19.7 / 17.2;
+// four states of 1.7 M, k = 448: 37.7 / 31.5; 16.8 M, k = 1024: 86.7 / 85.5; three of 1.5 M, k = 1216: 54.4 / 59.8; 45 M, k = 2048: 118 / 122).
+constexpr int kMiniDepth = 32;
+constexpr int kMiniShallowK = 1024;
 constexpr int kGramList = 256;          // lists up to this length run OMP on their Gram matrix (Algorithm 3 as printed)
 constexpr int kRepCap = 8192;           // report slots per residual of one screening pass
 constexpr int kPassMaxN = 256;          // residuals per screening pass (UMMA N)

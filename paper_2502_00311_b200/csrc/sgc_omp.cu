@@ -409,21 +409,22 @@ __device__ __forceinline__ void warp_sums(double (&v)[N]) {
 constexpr int kLanePairs = 4;                              // row pairs of a column that a lane generates at a time (256 rows per warp)
 
 // Partial products of column `col` over this slice with q_0 .. q_(j-1) and the residual, and (full) its squared norm and the
-// residual's, sent to slot g of the exchange buffer of every block of the group.  Warp = four vectors at a time; every warp
-// generates the slice of the column for itself (a few words per lane), which saves a barrier.
-template <int GS>
-__device__ void send_products(cg::cluster_group& cluster, const OmpArgs& a, const BookMem& b, int m, int j, uint32_t col, bool full,
-                              double* xbuf, int rank0, int g) {
+// residual's, sent to slot g of the exchange buffer of every block of the group.  Warp = V vectors at a time (as many as it takes
+// to keep all warps busy: the sums of a vector over the lanes are most of the work); every warp generates the slice of the column
+// for itself (a few words per lane), which saves a barrier.
+template <int GS, int V>
+__device__ __forceinline__ void send_vectors(cg::cluster_group& cluster, const OmpArgs& a, const BookMem& b, int m, int j, const ColKey& key,
+                                             double* xbuf, int rank0, int g) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, pairs = b.R / 2, xstride = exchange_stride(a.s);
-    const ColKey key = column_key(a.seed_lo, a.seed_hi, col);
     const bool vec = (a.k & 1) == 0 || j <= a.q_cols;
-    for (int l0 = warp; l0 <= j; l0 += 4 * kWarps) {
-        double acc[4] = {0.0, 0.0, 0.0, 0.0};
-        const double* v[4];
-        bool live[4];
+    for (int l0 = warp; l0 <= j; l0 += V * kWarps) {
+        double acc[V];
+        const double* v[V];
+        bool live[V];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < V; ++u) {
             const int l = l0 + u * kWarps;
+            acc[u] = 0.0;
             live[u] = l <= j;
             v[u] = l < j ? q_slice(a, b, m, l) : b.rr;
         }
@@ -432,7 +433,7 @@ __device__ void send_products(cg::cluster_group& cluster, const OmpArgs& a, cons
 #pragma unroll
             for (int i = 0; i < kLanePairs; ++i) x[i] = p0 + 32 * i < pairs ? column_rows(a, b, key, p0 + 32 * i) : make_double2(0.0, 0.0);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
+            for (int u = 0; u < V; ++u) {
                 if (!live[u]) continue;
 #pragma unroll
                 for (int i = 0; i < kLanePairs; ++i) {
@@ -452,9 +453,15 @@ __device__ void send_products(cg::cluster_group& cluster, const OmpArgs& a, cons
         if (lane < GS) {
             double* dst = cluster.map_shared_rank(xbuf, rank0 + lane) + (size_t)g * xstride;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) if (live[u]) dst[l0 + u * kWarps] = acc[u];
+            for (int u = 0; u < V; ++u) if (live[u]) dst[l0 + u * kWarps] = acc[u];
         }
     }
+}
+template <int GS>
+__device__ void send_products(cg::cluster_group& cluster, const OmpArgs& a, const BookMem& b, int m, int j, uint32_t col, bool full,
+                              double* xbuf, int rank0, int g) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, pairs = b.R / 2, xstride = exchange_stride(a.s);
+    const ColKey key = column_key(a.seed_lo, a.seed_hi, col);
     if (full && warp == kWarps - 1) {
         double acc[2] = {0.0, 0.0};
         for (int p = lane; p < pairs; p += 32) {
@@ -468,6 +475,9 @@ __device__ void send_products(cg::cluster_group& cluster, const OmpArgs& a, cons
             dst[a.s] = acc[0]; dst[a.s + 1] = acc[1];
         }
     }
+    if (j < kWarps) send_vectors<GS, 1>(cluster, a, b, m, j, key, xbuf, rank0, g);
+    else if (j < 2 * kWarps) send_vectors<GS, 2>(cluster, a, b, m, j, key, xbuf, rank0, g);
+    else send_vectors<GS, 4>(cluster, a, b, m, j, key, xbuf, rank0, g);
 }
 
 // a further candidate: its product with the residual and its squared norm (warp = one candidate)
@@ -1226,10 +1236,10 @@ __global__ void __launch_bounds__(kT, 1) k_omp(OmpArgs a, int mode) {
                 if (!(piv > kPivot * n2)) rc = 2;
                 else {
                     const double gamma = rsqrt(piv), aj = gamma * dot;
-                    const int R = bk.R, P = bk.P;
+                    const int R = bk.R, P = bk.P < (j + 3) / 4 ? bk.P : (j + 3) / 4 > 0 ? (j + 3) / 4 : 1;      // at least four vectors per part
                     const int r0 = P == 1 ? t : t % R, h = P == 1 ? 0 : t / R;
                     if (h < P)
-                        for (int r = r0; r < bk.rows; r += P == 1 ? kT : R) {
+                        for (int r = r0; r < bk.rows; r += P == 1 ? kT : R) {                       // (P > 1: one row per thread)
                             double va = 0.0, vb = 0.0;
                             int l = h;
 #pragma unroll 4

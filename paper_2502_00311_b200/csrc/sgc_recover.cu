@@ -838,7 +838,7 @@ static cudaError_t recover_batches(sgc_state* const* sts, float* const* weights,
                 {
                     PhaseTimer timer(st, stream, kPhaseCorr, 1);
                     OmpArgs am = args[0];
-                    am.mini = 1; am.depth = kMiniDepth;
+                    am.mini = 1; am.depth = st->k < kMiniShallowK ? kMiniDepth / 2 : kMiniDepth;
                     e = launch_omp(st, am, 0, stream);
                     *launches += 1;
                 }
