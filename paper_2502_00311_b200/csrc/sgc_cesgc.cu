@@ -4,12 +4,12 @@
 // are the kernels of this file.
 //   k_cesgc_project   P = B G in fp64, rounded to fp32 once, so that the top-s selection that follows decides on the exactly
 //                     projected gradient.  64 fp64 multiply-adds per cycle and SM bound it (30 us for a 4096 x 4096 gradient at
-//                     r = 32); conversions from fp32, a quarter as fast, are kept out of the way: a thread owns four columns and
-//                     eight rows and reads both operands as fp64 from slabs that the block has converted, each element once.  G
-//                     arrives by asynchronous copies, three slabs ahead (with one slab ahead in registers the kernel waited for
-//                     memory: 138 us; an error-free two-float form took 276 us, fp64 with both operands converted per product
-//                     1.1 ms).  The rows of G are split over the CTAs of a thread-block cluster; their partial sums meet through
-//                     distributed shared memory, added in rank order.
+//                     r = 32), and shared memory comes next: a thread owns four columns and eight rows, converts each element of G
+//                     once for its eight products, and reads B, which the block converts slab by slab, as eight 8-byte broadcasts
+//                     (a 16-byte broadcast costs four of them).  Both matrices arrive by asynchronous copies, three slabs ahead
+//                     (with one slab ahead in registers the kernel waited for memory: 138 us; an error-free two-float form took
+//                     276 us, fp64 with both operands converted per product 1.1 ms).  The rows of G are split over the CTAs of a
+//                     thread-block cluster; their partial sums meet through distributed shared memory, added in rank order.
 //   k_cesgc_back      W += B^T U for the r x n matrix U that the SGC core left (U = -eta N has at most s non-zeros).
 #include "sgc_internal.cuh"
 
@@ -32,11 +32,11 @@ constexpr int kProjResident = 148;       // one wave
 __host__ __device__ constexpr int proj_groups(int r) { return (r + kProjRows - 1) / kProjRows; }
 __host__ __device__ constexpr int proj_parts(int r) { return proj_groups(r) > 4 ? 2 : 4; }
 __host__ __device__ constexpr int proj_slab(int r) { return kProjPer * proj_parts(r); }
-// slabs of B (two, fp64), slabs of G; at the end the partial sums of the parts
-// (rows of a staged slab of B are two doubles longer than there are values: the stores that transpose it then spread over the banks)
-__host__ __device__ constexpr size_t proj_bslab(int r) { return 2 * (size_t)(proj_groups(r) * kProjRows + 2) * proj_slab(r) * sizeof(double); }
+// two slabs of B as fp64 (rows two doubles longer than there are values: the stores that transpose it then spread over the banks),
+// the rings of slabs of B and of G as they arrive; at the end the partial sums of the parts
+__host__ __device__ constexpr size_t proj_bslab(int r) { return (size_t)(proj_groups(r) * kProjRows + 2) * proj_slab(r) * sizeof(double); }
 __host__ __device__ constexpr size_t proj_smem(int r) {
-    const size_t slab = proj_bslab(r) + (size_t)proj_slab(r) * kProjCols * (kProjStages * sizeof(float) + 2 * sizeof(double));
+    const size_t slab = 2 * proj_bslab(r) + (size_t)kProjStages * proj_slab(r) * (kProjCols + proj_groups(r) * kProjRows) * sizeof(float);
     const size_t part = (size_t)proj_groups(r) * kProjRows * kProjCols * sizeof(double);
     return slab > part ? slab : part;
 }
@@ -64,29 +64,24 @@ k_cesgc_project(const float* __restrict__ B, const float* __restrict__ G, float*
     for (int u = 0; u < kProjRows; ++u)
 #pragma unroll
         for (int c = 0; c < 4; ++c) acc[u][c] = 0.0;
-    // slab of B as [row of G][row of B]: a thread reads its eight values of a row of G in four 16-byte broadcasts.  Its values
-    // travel through registers, one slab ahead
-    constexpr int kBHold = kProjRows * kProjPer / 32;                  // (rows8 * slab_rows values over 32 * groups * parts threads)
-    float bh[kBHold];
-    const int b_items = rows8 * slab_rows, threads = (int)blockDim.x;
-    auto fetch_b = [&](int row0) {
-#pragma unroll
-        for (int u = 0; u < kBHold; ++u) {
-            const int e = (int)threadIdx.x + u * threads;
-            bh[u] = 0.0f;
-            if (e < b_items) { const int i = e / slab_rows, q = e % slab_rows; if (i < r && row0 + q < m_end) bh[u] = B[(size_t)i * m + row0 + q]; }
-        }
+    const int threads = (int)blockDim.x;
+    double* bufs[2] = {smem, smem + proj_bslab(r) / sizeof(double)};      // [slab_rows][bstride]: row of G, row of B
+    float* gbuf = reinterpret_cast<float*>(smem + 2 * proj_bslab(r) / sizeof(double));      // [kProjStages][slab_rows][kProjCols]
+    float* bbuf = gbuf + (size_t)kProjStages * slab_rows * kProjCols;      // [kProjStages][rows8][slab_rows]
+    // the slab of B that arrived in `stage`, transposed and as fp64
+    auto convert_b = [&](int stage, double* dst) {
+        const float* src = bbuf + (size_t)stage * rows8 * slab_rows;
+        for (int e = threadIdx.x; e < rows8 * slab_rows; e += threads) dst[e % slab_rows * bstride + e / slab_rows] = (double)src[e];
     };
-    auto store_b = [&](double* dst) {
-#pragma unroll
-        for (int u = 0; u < kBHold; ++u) {
-            const int e = (int)threadIdx.x + u * threads;
-            if (e < b_items) { const int i = e / slab_rows, q = e % slab_rows; dst[q * bstride + i] = (double)bh[u]; }
+    // one slab of G and of B; what lies outside the matrices is filled with zeros (a copy of 0 bytes)
+    auto copy_slabs = [&](int stage, int row0) {
+        float* bd = bbuf + (size_t)stage * rows8 * slab_rows;
+        for (int e = threadIdx.x; e < rows8 * slab_rows; e += threads) {
+            const int i = e / slab_rows, q = e % slab_rows;
+            const bool ok = i < r && row0 + q < m_end;
+            const float* src = ok ? B + (size_t)i * m + row0 + q : B;
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(bd + e)), "l"(src), "r"(ok ? 4 : 0) : "memory");
         }
-    };
-    float* gbuf = reinterpret_cast<float*>(smem + proj_bslab(r) / sizeof(double));      // [kProjStages][slab_rows][kProjCols]
-    // one slab of G; what lies outside the matrix is filled with zeros (a copy of 0 bytes)
-    auto copy_g = [&](int stage, int row0) {
         float* dst = gbuf + (size_t)stage * slab_rows * kProjCols;
         for (int e = threadIdx.x; e < slab_rows * (kProjCols / 4); e += threads) {
             const int q = e / (kProjCols / 4), c = e % (kProjCols / 4) * 4, col = blockIdx.x * kProjCols + c;
@@ -107,53 +102,34 @@ k_cesgc_project(const float* __restrict__ B, const float* __restrict__ G, float*
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    double* bufs[2] = {smem, smem + (size_t)bstride * slab_rows};
-    double* gd[2];                                                    // [slab_rows][kProjCols] a slab of G as fp64: converted once, used by every group of rows
-    gd[0] = reinterpret_cast<double*>(gbuf + (size_t)kProjStages * slab_rows * kProjCols);
-    gd[1] = gd[0] + (size_t)slab_rows * kProjCols;
-    // columns 4 c .. 4 c + 3 go to places 2 c, 2 c + 1 and 64 + 2 c, 64 + 2 c + 1: two consecutive 16-byte reads per lane
-    auto convert_g = [&](int stage, double* dst) {
-        const float* src = gbuf + (size_t)stage * slab_rows * kProjCols;
-        for (int e = threadIdx.x; e < slab_rows * (kProjCols / 4); e += threads) {
-            const int q = e / (kProjCols / 4), c = e % (kProjCols / 4);
-            const float4 f = *reinterpret_cast<const float4*>(src + q * kProjCols + 4 * c);
-            double2* d = reinterpret_cast<double2*>(dst + q * kProjCols);
-            d[c] = make_double2((double)f.x, (double)f.y);
-            d[kProjCols / 4 + c] = make_double2((double)f.z, (double)f.w);
-        }
-    };
     if (m_begin < m_end) {
-        fetch_b(m_begin);
-        for (int st = 0; st < kProjStages - 1; ++st) copy_g(st, m_begin + st * slab_rows);
-        store_b(bufs[0]);
+        for (int st = 0; st < kProjStages - 1; ++st) copy_slabs(st, m_begin + st * slab_rows);
         asm volatile("cp.async.wait_group %0;" ::"n"(kProjStages - 2) : "memory");
         __syncthreads();
-        convert_g(0, gd[0]);
+        convert_b(0, bufs[0]);
         int b = 0, stage = 0;
         for (int row0 = m_begin; row0 < m_end; row0 += slab_rows) {
-            // slab `stage` + 1 of G has arrived; slab b of B and of the converted G are complete, the others used up
+            // the slabs after this one have arrived; this one's B is converted, the buffers of the previous one are used up
             asm volatile("cp.async.wait_group %0;" ::"n"(kProjStages - 3) : "memory");
             __syncthreads();
-            copy_g((stage + kProjStages - 1) % kProjStages, row0 + (kProjStages - 1) * slab_rows);
-            const bool more = row0 + slab_rows < m_end;
-            if (more) { fetch_b(row0 + slab_rows); convert_g((stage + 1) % kProjStages, gd[b ^ 1]); }
-            const double* slab = bufs[b] + ig * kProjRows;
-            const double2* gs = reinterpret_cast<const double2*>(gd[b]) + lane;
+            copy_slabs((stage + kProjStages - 1) % kProjStages, row0 + (kProjStages - 1) * slab_rows);
+            if (row0 + slab_rows < m_end) convert_b((stage + 1) % kProjStages, bufs[b ^ 1]);
+            const uint32_t slab = (uint32_t)__cvta_generic_to_shared(bufs[b] + ig * kProjRows);
+            const float* gs = gbuf + (size_t)stage * slab_rows * kProjCols + 4 * lane;
 #pragma unroll 2
             for (int q = 0; q < kProjPer; ++q) {
                 const int row = q * parts + part;
-                const double2 g0 = gs[row * (kProjCols / 2)], g1 = gs[row * (kProjCols / 2) + kProjCols / 4];
-                const double2* bq = reinterpret_cast<const double2*>(slab + (size_t)row * bstride);
+                const float4 g = *reinterpret_cast<const float4*>(gs + row * kProjCols);
+                const uint32_t bq = slab + (uint32_t)(row * bstride) * 8u;
+                const double gx = (double)g.x, gy = (double)g.y, gz = (double)g.z, gw = (double)g.w;
 #pragma unroll
-                for (int u = 0; u < kProjRows / 2; ++u) {
-                    const double2 v = bq[u];
-                    acc[2 * u][0] = fma(v.x, g0.x, acc[2 * u][0]); acc[2 * u][1] = fma(v.x, g0.y, acc[2 * u][1]);
-                    acc[2 * u][2] = fma(v.x, g1.x, acc[2 * u][2]); acc[2 * u][3] = fma(v.x, g1.y, acc[2 * u][3]);
-                    acc[2 * u + 1][0] = fma(v.y, g0.x, acc[2 * u + 1][0]); acc[2 * u + 1][1] = fma(v.y, g0.y, acc[2 * u + 1][1]);
-                    acc[2 * u + 1][2] = fma(v.y, g1.x, acc[2 * u + 1][2]); acc[2 * u + 1][3] = fma(v.y, g1.y, acc[2 * u + 1][3]);
+                for (int u = 0; u < kProjRows; ++u) {
+                    double v;
+                    asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(bq + 8u * u) : "memory");
+                    acc[u][0] = fma(v, gx, acc[u][0]); acc[u][1] = fma(v, gy, acc[u][1]);
+                    acc[u][2] = fma(v, gz, acc[u][2]); acc[u][3] = fma(v, gw, acc[u][3]);
                 }
             }
-            if (more) store_b(bufs[b ^ 1]);
             b ^= 1;
             stage = (stage + 1) % kProjStages;
         }
@@ -188,7 +164,7 @@ k_cesgc_project(const float* __restrict__ B, const float* __restrict__ G, float*
 // order they are found in), stages its rows of B^T as fp64, and its threads walk W in runs of four columns, so that reads and
 // writes are whole sectors (a block per column touched 32 bytes for every 4: 56 us at 4096 x 4096).  Runs of four without a
 // non-zero are not touched.
-constexpr int kBackCols = 64, kBackRows = 64, kBackThreads = 256, kBackSlabs = 8;      // slabs of kBackRows rows per block
+constexpr int kBackCols = 64, kBackRows = 64, kBackThreads = 256, kBackSlabs = 4;      // slabs of kBackRows rows per block
 
 __global__ void __launch_bounds__(kBackThreads)
 k_cesgc_back(const float* __restrict__ B, const float* __restrict__ U, float* __restrict__ W, int r, int m, int n) {
