@@ -16,7 +16,7 @@
 // speculated pick, and it harvests new candidates.
 //
 // One persistent CTA per SM; warp roles: 0 = TMA producer, 1 = MMA issuer (owns the tensor-memory
-// allocation), 2-9 = epilogue (two per 32-lane quadrant of tensor memory), 10-25 = generators.
+// allocation), 2-9 = epilogue (two per 32-lane quadrant of tensor memory; one in long sweeps), the next 16 = generators.
 // Every wait on an mbarrier is bounded (two seconds unless the caller sets another limit); on expiry the CTA records an
 // error, leaves all loops, waits for the matrix operations and copies it still has in flight, frees its tensor memory and
 // returns.
@@ -30,9 +30,7 @@ namespace sgc {
 namespace {
 
 constexpr int kGenWarps = 16;                                // 512 generator threads: two per column of a sweep
-constexpr int kEpiWarps = 8;                                 // warps 2..9: two per tensor-memory quadrant, half of the columns each
-constexpr int kFirstGenWarp = 2 + kEpiWarps;
-constexpr int kPassThreads = 32 * (kFirstGenWarp + kGenWarps);   // 832
+constexpr int pass_threads(int epi_warps) { return 32 * (2 + epi_warps + kGenWarps); }      // 832 or 704
 constexpr int kTileCols = 128;                               // UMMA M: columns of A per accumulator tile
 constexpr int kSuperCols = 2 * kTileCols;                    // columns of A per sweep over k
 constexpr int kChunkRows = 64;                               // rows of A per pipeline stage (128 B of binary16)
@@ -42,6 +40,10 @@ constexpr int kNormRing = 8;
 #define SGC_PASS_SWAP 1
 #endif
 constexpr bool kPassSwap = SGC_PASS_SWAP != 0;
+// Rows of A from which the 128-row form has four epilogue warps that append their reports directly instead of eight with queues:
+// generating a sweep then takes longer than any epilogue, and the eight warps' issue slots are what the generators lack
+// (steps of 2^24 x 2048, s = 64: 11.48 -> 11.40 ms;  3e6, 4096: 4.26 -> 4.24;  2^24, 1024: equal;  8e6, 512: 16.6 -> 21.2)
+constexpr int kLongSweep = 1024;
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // default bound of every mbarrier wait
 
 struct PassArgs {
@@ -214,8 +216,12 @@ __device__ __forceinline__ void report_flush(const PassArgs& a, const ReportQueu
 // SWAP (128 residual rows, table of norms, no wide lists): the residual chunk is the M operand and all 256 generated columns
 // the N operand of one MMA per 16 rows (instead of two MMAs of N = 128 that both read the residual chunk); the accumulator then
 // holds residuals along the lanes and columns of A along the tensor-memory columns
-template <bool TABLE, bool WIDE, int SUB, bool SWAP>
-__global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant__ CUtensorMap tmap, PassArgs a) {
+// EPI: epilogue warps.  8: two per tensor-memory quadrant, half of the columns each, reports queued in shared memory.  4 (swapped
+// form alone): one per quadrant, reports appended directly (see kLongSweep)
+template <bool TABLE, bool WIDE, int SUB, bool SWAP, int EPI>
+__global__ void __launch_bounds__(pass_threads(EPI), 1) k_pass(const __grid_constant__ CUtensorMap tmap, PassArgs a) {
+    static_assert(EPI == 8 || (EPI == 4 && SWAP), "four epilogue warps serve the swapped form alone");
+    constexpr int kFirstGenWarp = 2 + EPI;
     if (a.gate[0] != nullptr) {
         bool any = false;
 #pragma unroll
@@ -263,14 +269,14 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(bar_accf + 8u * b, 1);
-            mbar_init(bar_acce + 8u * b, kEpiWarps);
+            mbar_init(bar_acce + 8u * b, EPI);
         }
         mbar_init(bar_drain, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_async_smem();
     }
-    for (int i = threadIdx.x; i < 256; i += kPassThreads) {
+    for (int i = threadIdx.x; i < 256; i += 32 * (kFirstGenWarp + kGenWarps)) {
         const float tv = i < a.n ? a.tau[i] : __int_as_float(0x7f800000);
         tau_s[i] = tv;
         itau_s[i] = tv > 0.0f ? 1.0f / tv : 3.0e38f;                 // tau = +inf (unused residual) -> 0
@@ -347,8 +353,9 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
         }
     } else if (warp < kFirstGenWarp) {
         // ---------------- epilogue: scores against thresholds ----------------------------------------------
-        const int quad = warp & 3, side = (warp - 2) >> 2, ew = side * 4 + quad;      // this warp's quadrant and half of the columns
-        constexpr int kHalf = kSuperCols / 2;
+        const int quad = warp & 3, side = (warp - 2) >> 2, ew = side * 4 + quad;      // this warp's quadrant and share of the columns
+        constexpr int kHalf = kSuperCols * 4 / EPI;
+        constexpr bool kQueue = EPI == 8;
         uint32_t sweep_i = 0;
         bool ok = true;
         // room for the reports: what the table of norms leaves of its ring (the swapped form keeps 12 KB of it for other things)
@@ -356,7 +363,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
         queue_r.mem = TABLE ? reinterpret_cast<uint32_t*>(norms + (SWAP ? 12 * (size_t)kSuperCols + ew * kHalf : (size_t)ew * 2 * kSuperCols))
                             : reinterpret_cast<uint32_t*>(norms) + kNormRing * kSuperCols * 2 + 768 + ew * kHalf;
         queue_r.cap = ((TABLE && !SWAP ? 4 : 1) * kHalf - 1) / 3;
-        queue_r.init(lane);
+        if (kQueue) queue_r.init(lane);
         for (unsigned int sweep = blockIdx.x; ok && sweep < num_super; sweep += gridDim.x, ++sweep_i) {
             const uint32_t buf = sweep_i % a.bufs, use = sweep_i / a.bufs;
             // (what the sweep's scores are divided by is fetched before its accumulators are waited for)
@@ -434,7 +441,8 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
                         const float sc = fabsf(__uint_as_float(v[i])) * inv;
                         if (sc >= tau_n && inv > 0.0f) {
                             const uint32_t col = listed ? col_w[c0 + i] : (uint32_t)(col_first + c0 + i);
-                            report_push(a, queue_r, (uint32_t)n_res, col, sc);
+                            if (kQueue) report_push(a, queue_r, (uint32_t)n_res, col, sc);
+                            else report_append(a, (uint32_t)n_res, col, sc);
                         }
                     }
                 }
@@ -455,7 +463,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
                     }
                     __syncwarp();
                 }
-                report_flush(a, queue_r, lane, (unsigned int)queue_r.cap / 2);
+                if (kQueue) report_flush(a, queue_r, lane, (unsigned int)queue_r.cap / 2);
                 continue;
             }
             const float* nr = norms + (size_t)(sweep_i % kNormRing) * kSuperCols * 2;
@@ -533,7 +541,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
             if (lane == 0) mbar_arrive(bar_acce + 8u * buf);
             report_flush(a, queue_r, lane, (unsigned int)queue_r.cap / 2);
         }
-        report_flush(a, queue_r, lane, 1u);
+        if (kQueue) report_flush(a, queue_r, lane, 1u);
     } else {
         // ---------------- generators: Z tiles as binary16, swizzled K-major ---------------------------------
         const int g = threadIdx.x - kFirstGenWarp * 32;
@@ -677,9 +685,9 @@ cudaError_t pass_encode_map(void* tmap_out, const void* rt, int n, int k) {
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-template <bool TABLE, bool WIDE, int SUB, bool SWAP = false>
+template <bool TABLE, bool WIDE, int SUB, bool SWAP = false, int EPI = 8>
 cudaError_t pass_opt_in(int need) {
-    return cudaFuncSetAttribute(k_pass<TABLE, WIDE, SUB, SWAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, need);
+    return cudaFuncSetAttribute(k_pass<TABLE, WIDE, SUB, SWAP, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, need);
 }
 
 cudaError_t pass_configure(int) {
@@ -698,6 +706,8 @@ cudaError_t pass_configure(int) {
     if (e == cudaSuccess) e = pass_opt_in<true, false, 2>((int)need);
     if (e == cudaSuccess) e = pass_opt_in<true, false, 2, true>((int)need);
     if (e == cudaSuccess) e = pass_opt_in<true, true, 2, true>((int)need);
+    if (e == cudaSuccess) e = pass_opt_in<true, false, 2, true, 4>((int)need);
+    if (e == cudaSuccess) e = pass_opt_in<true, true, 2, true, 4>((int)need);
     return e;
 }
 
@@ -732,16 +742,21 @@ cudaError_t launch_pass(const void* tmap, uint64_t seed, uint64_t d, int k, int 
     CUtensorMap map;
     memcpy(&map, tmap, sizeof(map));
     const size_t smem = pass_smem_bytes(n, a.stages, sub);
-    if (sub == 2) {
-        if (inv_norm && wide && n == kTileCols && kPassSwap) k_pass<true, true, 2, true><<<grid, kPassThreads, smem, stream>>>(map, a);
-        else if (inv_norm && wide) k_pass<true, true, 2, false><<<grid, kPassThreads, smem, stream>>>(map, a);
-        else if (inv_norm && n == kTileCols && kPassSwap) k_pass<true, false, 2, true><<<grid, kPassThreads, smem, stream>>>(map, a);
-        else if (inv_norm) k_pass<true, false, 2, false><<<grid, kPassThreads, smem, stream>>>(map, a);
-        else k_pass<false, false, 2, false><<<grid, kPassThreads, smem, stream>>>(map, a);
+    const dim3 block8(pass_threads(8)), block4(pass_threads(4));
+    if (sub == 2 && inv_norm && n == kTileCols && kPassSwap) {
+        const bool lng = k >= kLongSweep;
+        if (wide && lng) k_pass<true, true, 2, true, 4><<<grid, block4, smem, stream>>>(map, a);
+        else if (wide) k_pass<true, true, 2, true, 8><<<grid, block8, smem, stream>>>(map, a);
+        else if (lng) k_pass<true, false, 2, true, 4><<<grid, block4, smem, stream>>>(map, a);
+        else k_pass<true, false, 2, true, 8><<<grid, block8, smem, stream>>>(map, a);
+    } else if (sub == 2) {
+        if (inv_norm && wide) k_pass<true, true, 2, false, 8><<<grid, block8, smem, stream>>>(map, a);
+        else if (inv_norm) k_pass<true, false, 2, false, 8><<<grid, block8, smem, stream>>>(map, a);
+        else k_pass<false, false, 2, false, 8><<<grid, block8, smem, stream>>>(map, a);
     } else {
-        if (inv_norm && wide) k_pass<true, true, 1, false><<<grid, kPassThreads, smem, stream>>>(map, a);
-        else if (inv_norm) k_pass<true, false, 1, false><<<grid, kPassThreads, smem, stream>>>(map, a);
-        else k_pass<false, false, 1, false><<<grid, kPassThreads, smem, stream>>>(map, a);
+        if (inv_norm && wide) k_pass<true, true, 1, false, 8><<<grid, block8, smem, stream>>>(map, a);
+        else if (inv_norm) k_pass<true, false, 1, false, 8><<<grid, block8, smem, stream>>>(map, a);
+        else k_pass<false, false, 1, false, 8><<<grid, block8, smem, stream>>>(map, a);
     }
     return cudaGetLastError();
 }

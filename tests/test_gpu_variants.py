@@ -1,0 +1,85 @@
+"""The variants the dispatch rules choose between, at the sizes where they change over or leave remainders.
+
+Same bar as test_gpu_parity (index sets bit-exact, state 1e-5, update 1e-4): the comparisons are its own.
+"""
+import numpy as np
+import pytest
+
+import oracle
+import test_gpu_parity as parity
+from paper_2502_00311_b200 import inputs
+from test_gpu_parity import cuda, run_both, sgc  # noqa: F401  (sgc is the module's fixture)
+
+pytestmark = pytest.mark.gpu
+
+
+# one block holds the whole gradient up to 32768 entries; above, maxima of units of vectors; remainders of four and of a unit
+@pytest.mark.parametrize("d,s", [(3, 2), (1024, 1024), (4097, 1), (32767, 1024), (32768, 31), (32770, 1024), (65_537, 3),
+                                 ((1 << 22) - 1, 200), ((1 << 22) + 5, 1024)])
+def test_selection_without_a_threshold(sgc, d, s):  # noqa: F811
+    import torch
+    rng = np.random.default_rng(d + s)
+    idx, val = torch.empty(s, dtype=torch.int32, device="cuda"), torch.empty(s, device="cuda")
+    cases = [(rng.standard_t(3.0, size=d) * 1e-3).astype(np.float32), np.round(rng.standard_normal(d) * 2).astype(np.float32) / 2]
+    cluster = cases[0].copy()
+    cluster[max(0, d - 3 * s):] += 4.0                                    # all kept entries in the last units
+    for g in cases + [cluster, np.full(d, -0.75, dtype=np.float32)]:
+        sgc.sparsify_static(cuda(g), s, idx, val)
+        widx, wval = oracle.sparsify(g, s)
+        assert np.array_equal(idx.cpu().numpy().view(np.uint32), widx) and np.array_equal(val.cpu().numpy(), wval)
+
+
+def test_selection_after_the_scale_of_the_gradient_jumps(sgc):  # noqa: F811
+    # the threshold of the last step is far too high, far too low, then right again
+    d, s = 300_001, 40
+    st = sgc.Sgc(d, 64, s, 3, 1e-3, 0.9, 0.999, 1e-8)
+    w = cuda(np.zeros(d, dtype=np.float32))
+    for step, scale in enumerate([1.0, 1.0, 1e-4, 1e4, 1.0, 1.0]):
+        g = (np.random.default_rng(step).standard_t(3.0, size=d) * scale).astype(np.float32)
+        st.step(cuda(g), w)
+        widx, wval = oracle.sparsify(g, s)
+        assert np.array_equal(st.get("sel_idx"), widx) and np.array_equal(st.get("sel_val"), wval), step
+    st.close()
+
+
+# lock-step: one cluster up to k d = 1.2e6, groups of eight blocks, pairs from 2e8 on; fewer columns than blocks, odd k, many rows
+@pytest.mark.parametrize("d,k,s", [(37, 5, 1), (4800, 250, 9), (4801, 250, 9), (700, 257, 130), (1001, 1199, 3), (66_000, 3100, 4),
+                                   (1_000_003, 201, 6), (30_000, 7001, 3)])
+def test_lockstep_cluster_shapes(sgc, d, k, s):  # noqa: F811
+    run_both(sgc, d, k, s, 6, "student", 2, cfg_id=2, mode=1)
+
+
+# the screening pass: rows of A in one or two chunks per slot, the long and the short sweep of the 128-row form, wide lists
+@pytest.mark.parametrize("d,k,s,redraw", [(30_001, 64, 2, False), (40_000, 960, 64, False), (40_003, 1024, 64, False),
+                                          (200_000, 1024, 60, True), (20_000, 1088, 120, False)])
+def test_screening_pass_forms(sgc, d, k, s, redraw):  # noqa: F811
+    run_both(sgc, d, k, s, 7, "student", 3, cfg_id=2, mode=2, redraw_support=redraw)
+
+
+def test_a_state_chooses_between_speculation_and_lockstep(sgc):  # noqa: F811
+    # k no multiple of 64 speculates on its own accord when k > 1.2 s ln d; below that size and below d = 65536 it does not
+    for d, k, s, speculates in [(70_000, 333, 10, True), (65_535, 333, 10, False), (70_000, 70, 10, False)]:
+        stats = []
+        run_both(sgc, d, k, s, 5, "student", 2, cfg_id=2, stats=stats)
+        assert all((rounds >= 1) == speculates for rounds, _, _ in stats), (d, k, s, stats)
+
+
+# chunks: several blocks per chunk in the first kernel, one, equal magnitudes across the blocks of a chunk, as many picks as a
+# chunk has rows but one
+@pytest.mark.parametrize("c,dc,k,sc", [(2, 200_000, 217, 31), (3, 65_540, 7, 1), (12, 3000, 8, 7), (150, 4100, 16, 2)])
+def test_chunk_variants(sgc, c, dc, k, sc):  # noqa: F811
+    parity.test_mesgc_small_chunks_batched_path_matches_independent_oracles(sgc, c, dc, k, sc, "student")
+    m = sgc.Mesgc(c * dc, c, k, sc, 8, *(inputs.ADAM[n] for n in ("lr", "beta1", "beta2", "eps")))
+    g = np.full(c * dc, 0.25, dtype=np.float32)
+    g[1::2] *= -1
+    m.step(cuda(g), cuda(np.zeros(c * dc, dtype=np.float32)))
+    for st in m.chunks:
+        assert np.array_equal(st.get("sel_idx"), np.arange(sc, dtype=np.uint32))
+    m.close()
+
+
+# projection: columns that are no multiple of four (no 16-byte copies) or of a block's columns, r at its ends, ragged rows
+@pytest.mark.parametrize("m,n,r,c,k,sc", [(333, 97, 8, 2, 28, 4), (70, 33, 12, 1, 40, 5), (130, 68, 64, 4, 56, 7),
+                                          (257, 260, 1, 1, 40, 5), (4099, 130, 34, 5, 60, 6)])
+def test_cesgc_remainders(sgc, m, n, r, c, k, sc):  # noqa: F811
+    parity.test_cesgc_step_matches_its_oracle(sgc, m, n, r, c, k, sc)
