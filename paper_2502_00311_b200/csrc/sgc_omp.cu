@@ -18,6 +18,8 @@
 // Lists of up to kGramList columns (the steady state of a run with a stable support) need no iteration of that kind: with
 // the Gram matrix G of the list at hand, block m runs all picks of recovery m on it alone (gram_picks), and the whole grid
 // then forms the residuals of all picks at once (gram_rows, gram_emit).
+#include <mutex>
+
 #include <cooperative_groups.h>
 
 #include "sgc_omp.cuh"
@@ -32,7 +34,7 @@ constexpr int kWarps = kT / 32;
 constexpr size_t kOmpDynBytes = 196 * 1024;           // dynamic shared memory of every launch (one block per SM)
 constexpr int kRescanCap = 64;
 constexpr double kOmpOneWork = 1.2e6;                  // k * d up to which one cluster of 16 serves the lock-step recovery
-constexpr double kOmpPairWork = 2.0e8;                 // k * d from which pairs do
+constexpr double kOmpPairCols = 1000.0;                // columns per pick from which pairs do
 constexpr double kPivot = 1e-10;                      // a new column whose orthogonal part is below this share is dependent
 
 // the best column seen (lowest index on ties), and the largest score among all others (what is dropped: the caller can tell
@@ -207,6 +209,106 @@ __device__ void stage_residuals(const OmpArgs& a, OmpSmem& sh, uint2* frag, floa
     for (int it = t + kHold * kT; it < items; it += kT) put(it, fetch(it));
 }
 
+// Tiles of a block from which they are streamed: four per warp, two rounds of two (rows are split over warps up to here).  From 64
+// instead of 128 tiles, steps: d = 200000, k = 210, s = 30: 1001 -> 919 us;  250000, 64, 9: 258 -> 236 us.
+constexpr int kStreamTiles = 64;
+
+// The columns of a block in lock-step when they are too many to keep: a warp takes 32 columns a round.  Each lane works out the
+// key of one of them, and the two tiles' eight generated words overlap one another.  The norms (HAVE: those kept from the first
+// iteration, inv_s) are the diagonals of two more products with the tile itself as B operand (lane (g, t) holds the very words
+// that B wants of columns g and g + 8), which saves the conversions and multiply-adds; their accumulators are emptied into a sum
+// every kNormBlocks blocks of rows, so that a norm is as exact as one summed entry by entry.  A column that cannot pass the
+// block's second best score so far costs one compare and no division.  Issue slots bound it: 16 rows of 2e6 columns take 10 us
+// (3.2e12 entries/s; the generator alone allows 5.1e12), and what a column costs whatever k is another 16 us.  Per pick, d = 2e6,
+// k = 42: 96 -> 55 us;  1.2e6, 224: 110 -> 88;  5e5, 700: 140 -> 105.
+constexpr int kNormBlocks = 16;
+template <bool HAVE>
+__device__ __forceinline__ void correlate_stream(const OmpArgs& a, OmpSmem& sh, const CorrPlan& c, const uint2* frag, float* inv_s,
+                                                 const float (&back)[2], const int* picks, Top& best) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, q = lane & 3;
+    const int diag = g * 4 + (g >> 1);                                // lane of column g's own norm, element g & 1 of its pair
+    const bool odd = g & 1;
+    const float bq = q == 0 ? back[0] : back[1];
+    for (int base = warp * 32; base < c.cnt; base += 32 * kWarps) {
+        const ColKey key = column_key(a.seed_lo, a.seed_hi, (uint32_t)(c.e0 + base + lane));
+        uint32_t h[4], st[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const uint32_t mk = __shfl_sync(0xffffffffu, key.mk, g + 8 * u);
+            h[u] = __shfl_sync(0xffffffffu, key.ck, g + 8 * u) + (uint32_t)q * mk;
+            st[u] = 4u * mk;
+        }
+        float acc0[4] = {0.0f, 0.0f, 0.0f, 0.0f}, acc1[4] = {0.0f, 0.0f, 0.0f, 0.0f}, n[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        // rows 2q, 2q + 1 (lo) and 2q + 8, 2q + 9 (hi) of columns g + 8 u
+        auto words = [&](uint32_t (&lo)[4], uint32_t (&hi)[4]) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                lo[u] = z_pair_from_word(h[u]); h[u] += st[u];
+                hi[u] = z_pair_from_word(h[u]); h[u] += st[u];
+            }
+        };
+        if (HAVE) {
+            // (rows beyond k meet zeros of the residuals)
+#pragma unroll 2
+            for (int kb = 0; kb < c.kblocks; ++kb) {
+                const uint2 b = lane < 16 ? frag[(size_t)kb * 16 + lane] : make_uint2(0u, 0u);
+                uint32_t lo[4], hi[4];
+                words(lo, hi);
+                mma_16816(acc0, lo[0], lo[1], hi[0], hi[1], b.x, b.y);
+                mma_16816(acc1, lo[2], lo[3], hi[2], hi[3], b.x, b.y);
+            }
+        } else {
+            for (int kg = 0; kg < c.kblocks; kg += kNormBlocks) {
+                const int kend = kg + kNormBlocks < c.kblocks ? kg + kNormBlocks : c.kblocks;
+                float na[4] = {0.0f, 0.0f, 0.0f, 0.0f}, nb[4] = {0.0f, 0.0f, 0.0f, 0.0f}, nc[4] = {0.0f, 0.0f, 0.0f, 0.0f}, nd[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 1
+                for (int kb = kg; kb < kend; ++kb) {
+                    const uint2 b = lane < 16 ? frag[(size_t)kb * 16 + lane] : make_uint2(0u, 0u);
+                    uint32_t lo[4], hi[4];
+                    words(lo, hi);
+                    if (kb == c.kblocks - 1) {                        // rows beyond k do not count
+                        const int r0 = kb * 16 + 2 * q, r1 = r0 + 8;
+                        const uint32_t m0 = r0 >= a.k ? 0u : r0 + 1 >= a.k ? 0xFFFFu : 0xFFFFFFFFu;
+                        const uint32_t m1 = r1 >= a.k ? 0u : r1 + 1 >= a.k ? 0xFFFFu : 0xFFFFFFFFu;
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) { lo[u] &= m0; hi[u] &= m1; }
+                    }
+                    mma_16816(acc0, lo[0], lo[1], hi[0], hi[1], b.x, b.y);
+                    mma_16816(acc1, lo[2], lo[3], hi[2], hi[3], b.x, b.y);
+                    mma_16816(na, lo[0], lo[1], hi[0], hi[1], lo[0], hi[0]);
+                    mma_16816(nb, lo[0], lo[1], hi[0], hi[1], lo[1], hi[1]);
+                    mma_16816(nc, lo[2], lo[3], hi[2], hi[3], lo[2], hi[2]);
+                    mma_16816(nd, lo[2], lo[3], hi[2], hi[3], lo[3], hi[3]);
+                }
+                n[0] += odd ? na[1] : na[0]; n[1] += odd ? nb[3] : nb[2];
+                n[2] += odd ? nc[1] : nc[0]; n[3] += odd ? nd[3] : nd[2];
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) n[u] = __shfl_sync(0xffffffffu, n[u], diag);
+            if (c.norms) {                                            // (room for whole tiles; an odd one may end the block's columns)
+                const float nq = q == 0 ? n[0] : q == 1 ? n[1] : q == 2 ? n[2] : n[3];
+                if (base + 8 * q < c.tiles * 16) inv_s[base + g + 8 * q] = nq > 0.0f ? 1.0f / nq : 0.0f;
+            }
+        }
+        if (q < 2) {
+            // lane (g, 0): M^ products (value part and remainder part); lane (g, 1): V^'s
+            const float e[4] = {(acc0[0] + acc0[1]) * bq, (acc0[2] + acc0[3]) * bq, (acc1[0] + acc1[1]) * bq, (acc1[2] + acc1[3]) * bq};
+            // (a hair below the bound: offer() decides exactly)
+            const float bound = fmaxf(best.s2, key_score(*reinterpret_cast<volatile unsigned int*>(&sh.floor_key[q]))) * 0.999999f;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int i = base + g + 8 * u;
+                if (HAVE) {
+                    const float score = i < c.cnt ? e[u] * e[u] * inv_s[i] : -1.0f;
+                    if (score >= bound && i < c.cnt) offer(sh, best, picks, q, score, (uint32_t)(c.e0 + i));
+                } else if (e[u] * e[u] >= bound * n[u] && i < c.cnt)
+                    offer(sh, best, picks, q, e[u] * e[u] * (n[u] > 0.0f ? 1.0f / n[u] : 0.0f), (uint32_t)(c.e0 + i));
+            }
+        }
+        __syncwarp();
+    }
+}
+
 __device__ void correlate(const OmpArgs& a, OmpSmem& sh, const CorrPlan& c, const uint32_t* col_list, uint2* frag, float* mem,
                           bool filled, const int* picks, int blk, int nblk) {
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5, g = lane >> 2, q = lane & 3;
@@ -220,7 +322,10 @@ __device__ void correlate(const OmpArgs& a, OmpSmem& sh, const CorrPlan& c, cons
     const bool have = filled && c.norms, read = filled && c.cached;
     Top best;                                                         // of residual q & 1
     best.init();
-    const int ks_log = 31 - __clz(c.ks), units = c.tiles * c.ks, kper = (c.kblocks + c.ks - 1) / c.ks;
+    const bool stream = col_list == nullptr && !c.cached && c.tiles > kStreamTiles;
+    if (stream && have) correlate_stream<true>(a, sh, c, frag, inv_s, back, picks, best);
+    else if (stream) correlate_stream<false>(a, sh, c, frag, inv_s, back, picks, best);
+    const int ks_log = 31 - __clz(c.ks), units = stream ? 0 : c.tiles * c.ks, kper = (c.kblocks + c.ks - 1) / c.ks;
     for (int u = warp; u < units; u += kWarps) {
         const int tile = u >> ks_log, part_k = u & (c.ks - 1);
         const int kb0 = part_k * kper, kb1 = kb0 + kper < c.kblocks ? kb0 + kper : c.kblocks;
@@ -1392,14 +1497,30 @@ cudaError_t omp_launch(OmpArgs a, int mode, int grid, cudaStream_t stream) {
 }  // namespace
 
 cudaError_t omp_configure(sgc_state* st) {
+    // How many clusters a device holds is a property of the device: asked once for each (the three questions would otherwise be
+    // most of what the creation of a small state takes, and chunked optimizers create hundreds)
+    struct Resident { int n2, n8, n16; bool known; };
+    constexpr int kDevices = 64;
+    static std::mutex lock;
+    static Resident table[kDevices];
     cudaError_t e = omp_opt_in<2>();
     if (e == cudaSuccess) e = omp_opt_in<8>();
     if (e != cudaSuccess) return e;
-    int n2 = 0, n8 = 0, n16 = 0;
-    e = resident_clusters<2>(&n2);
-    if (e == cudaSuccess) e = resident_clusters<8>(&n8);
-    if (e != cudaSuccess) return e;
-    if (omp_opt_in<16>() != cudaSuccess || resident_clusters<16>(&n16) != cudaSuccess) { n16 = 0; cudaGetLastError(); }
+    const bool clusters16 = omp_opt_in<16>() == cudaSuccess;
+    if (!clusters16) cudaGetLastError();
+    Resident r = {};
+    const bool listed = st->device >= 0 && st->device < kDevices;
+    if (listed) { std::lock_guard<std::mutex> hold(lock); r = table[st->device]; }
+    if (!r.known) {
+        e = resident_clusters<2>(&r.n2);
+        if (e == cudaSuccess) e = resident_clusters<8>(&r.n8);
+        if (e != cudaSuccess) return e;
+        if (!clusters16 || resident_clusters<16>(&r.n16) != cudaSuccess) { r.n16 = 0; cudaGetLastError(); }
+        r.known = true;
+        if (listed) { std::lock_guard<std::mutex> hold(lock); table[st->device] = r; }
+    }
+    int n2 = r.n2, n8 = r.n8;
+    const int n16 = r.n16;
     if (2 * n2 > kCorrBlocks) n2 = kCorrBlocks / 2;
     if (8 * n8 > kCorrBlocks) n8 = kCorrBlocks / 8;
     st->omp_grid2 = 2 * n2; st->omp_grid8 = 8 * n8; st->omp_one = n16 >= 1 ? 1 : 0;
@@ -1408,14 +1529,15 @@ cudaError_t omp_configure(sgc_state* st) {
 }
 
 // Which cluster shape: the one-cluster form while a pick's correlation takes 16 SMs no longer than the grid barriers cost
-// the others; pairs (all 148 SMs correlate, two blocks keep the books) once the correlation of a pick dwarfs its
-// bookkeeping; groups of 8 (120 SMs, the most that clusters of 8 can occupy) in between and for lists.
+// the others; pairs (all 148 SMs correlate, two blocks keep each recovery's books) when the correlation of a pick (k d) dwarfs
+// its bookkeeping (k s), whatever k is; groups of 8 (120 SMs, the most that clusters of 8 can occupy) otherwise and for lists.
+// Step in groups of 8 / in pairs, us: d = 500000, k = 210, s = 30: 2187 / 1832; 65000, 350, 50: 1312 / 1126; 10000, 200, 8:
+// 143 / 136;  60000, 512, 64 (940 columns per pick): 1692 / 1694;  60000, 1024, 64: 2359 / 2521;  25000, 1400, 200: 7708 / 13020.
 cudaError_t launch_omp(sgc_state* st, const OmpArgs& a, int mode, cudaStream_t stream) {
-    const double work = (double)a.k * (double)a.d;
     if (mode == 1) {
         const bool pairs_fit = book_doubles(a.k, a.s, 2, false) * sizeof(double) + frag_bytes(a.k) + 40 * 1024 <= kOmpDynBytes;
-        if (st->omp_one && work <= kOmpOneWork) return omp_launch<16>(a, mode, 16, stream);
-        if (pairs_fit && work >= kOmpPairWork) return omp_launch<2>(a, mode, st->omp_grid2, stream);
+        if (st->omp_one && (double)a.k * (double)a.d <= kOmpOneWork) return omp_launch<16>(a, mode, 16, stream);
+        if (pairs_fit && (double)a.d >= kOmpPairCols * a.s) return omp_launch<2>(a, mode, st->omp_grid2, stream);
     }
     return omp_launch<8>(a, mode, st->omp_grid8, stream);
 }

@@ -701,11 +701,11 @@ cudaError_t configure_recover(sgc_state* st) {
     // k = 256, s = 16: 16.2 (2.80) / 14.7 (2.45) / 14.1 ms (2.25); k = 2048, s = 128: 125 (3.50) / 117 (3.19) / 119 ms (3.19);
     // k = 4096, s = 256: 247 (2.55) / 259 (2.60) / 263 ms (2.60): denser feeding makes the lists longer.
     st->wide_every = st->k < 512 ? 2 : st->k <= 2048 ? 4 : 8;
-    return pass_configure(kPassMaxN);
+    return cudaSuccess;
 }
 
 cudaError_t finish_recover_setup(sgc_state* st) {
-    cudaError_t e = cudaSuccess;
+    cudaError_t e = pass_configure(kPassMaxN);
     for (int g = 1; g <= kPassMaxN / st->pass_n && e == cudaSuccess; ++g)      // one map per number of states in a batch
         e = pass_encode_map(st->tmap[g - 1], st->rt, g * st->pass_n, st->kp);
     if (e != cudaSuccess) return e;
@@ -722,18 +722,19 @@ cudaError_t finish_recover_setup(sgc_state* st) {
 // correlations, list passes and resolving.  Which of the two a state meets is known once it has speculated for two steps; before,
 // the sizes tell: steps of d = 129344, k = 512, s = 33 (k = 1.32 s ln d) are confirmed by one pass, those of 1721085, 384, 26
 // (1.03) and 2^24, 1024, 64 (0.96) are not.
-//   lock-step, us per pick:  d = 50304, k = 128: 15.9;  31820, 1024: 28;  200000, 512: 60      (11 + k d / 2.0e6)
+//   lock-step, us per pick:  d = 65000, k = 350: 22;  200000, 210: 30;  270000, 300: 41;  1200000, 224: 88;  500000, 700: 105
+//                                                                                             (11 + k d / 2.8e6)
 //   refuted speculation:     d = 151700, k = 320, s = 37: 100;  117656, 832, 102: 81;  1876582, 960, 123: 168;  3001000, 700, 100: 270
 //                                                                                             (100 + k d / 2.0e7)
 //   confirmed speculation, us per step: d = 143488, k = 1600, s = 25: 370 (with the launches; 140 + 1.2 s + k d / 3.3e6)
 // A state that has come to prefer lock-step tries a speculating step now and then: its gradients may have changed.
 constexpr int kRetrySteps = 32;
-constexpr double kFewRoundsWork = 3.0e8;              // k * d up to which a pick in lock-step costs at most 160 us
+constexpr double kFewRoundsWork = 3.0e8;              // k * d up to which a pick in lock-step costs at most 120 us
 constexpr double kTwoLevelWork = 1.0e8;               // k * d from which list passes can be cheaper than full ones
 
 static bool prefers_speculation(const sgc_state* st) {
     const double kd = (double)st->k * (double)st->d, s = (double)st->s;
-    const double lock = s * (11.0 + kd / 2.0e6);
+    const double lock = s * (11.0 + kd / 2.8e6);
     const int seen = *reinterpret_cast<volatile int*>(st->h_rounds);
     const bool refuted = (seen & 255) != 0 ? ((seen >> 10) & 3) >= 2 : (double)st->k < 1.2 * s * log((double)st->d);
     const double spec = refuted ? s * (100.0 + kd / 2.0e7) : 140.0 + 1.2 * s + kd / 3.3e6;
