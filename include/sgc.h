@@ -68,7 +68,7 @@ enum {
                                                 score of one pick (a block that keeps such a column beyond the two it
                                                 forwards has its range screened again, so up to 16 always reach the fp64
                                                 decision): the pick may then differ from the exact argmax by a near-tie */
-    SGC_STATUS_SELECT_FALLBACK = 1u << 5,  /* the sampled top-s threshold missed; exact fallback ran */
+    SGC_STATUS_SELECT_FALLBACK = 1u << 5,  /* the bound on the kept magnitudes missed; exact fallback ran */
     SGC_STATUS_TIMEOUT = 1u << 6           /* a bounded wait inside a tensor-core screening pass ran out; the pass's
                                               reports were discarded and the step finished on its slower exact path */
 };

@@ -13,7 +13,7 @@
 // (0.28 us each) instead of the chain of a dozen block barriers and L2 round trips that one block needs for it.  All other
 // blocks (in lock-step: all blocks) correlate the columns with the current residuals.  An iteration is
 //     correlate | grid barrier | decide in fp64, update q, r | grid barrier
-// Measured at k = 2048 with a list of 8 to 21 thousand columns: see the table at k_omp.
+// What an iteration takes: see the table at k_omp.
 //
 // Lists of up to kGramList columns (the steady state of a run with a stable support) need no iteration of that kind: with
 // the Gram matrix G of the list at hand, block m runs all picks of recovery m on it alone (gram_picks), and the whole grid
@@ -84,9 +84,8 @@ struct OmpSmem {
 // Warp = 16 columns at a time, mma.m16n8k16: a generated row pair of a column is exactly one register of the A operand, and
 // the B operand holds both residuals, each as two binary16 numbers (value and remainder, 22 bits), so that the products
 // are summed in fp32 by the tensor cores and a row pair costs its 13 generator instructions and little else (26 with the
-// conversions and multiply-adds done one by one: 36 -> see k_omp for what an iteration takes).  This is the legacy matrix
-// instruction on purpose: N is 4, so a tcgen05 tile would be idle but for one in sixty columns, and the generator bounds it
-// anyway.  A tile's rows are split over several warps when the block has fewer tiles than warps.  When the generated entries
+// conversions and multiply-adds done one by one).  This is the legacy matrix instruction on purpose: N is 4, so a tcgen05 tile
+// would be idle but for one in sixty columns, and the generator bounds it anyway.  A tile's rows are split over several warps when the block has fewer tiles than warps.  When the generated entries
 // of the block's columns fit its shared memory they are kept from the first iteration on, as operand registers: an iteration
 // then reads 16 bytes per lane and 16 rows instead of regenerating them.  The norms are summed in the first iteration.
 struct CorrPlan { int e0, cnt, tiles, ks, kblocks; bool cached, norms; size_t part_off, inv_off, col_off, z_off; };
@@ -800,7 +799,7 @@ __device__ void gram_matrix(const OmpArgs& a, int n) {
 // not fit).  A pick reads c_l = sigma w_l(pick) and updates
 //     w_j(i) = gamma (sigma G(pick, i) - sum_l c_l w_l(i)),    p_i -= a_j w_j(i):
 // one block barrier per pick and j fp64 multiply-adds per member.  64 picks on 64 columns: 270 us with the k-free form of
-// the printed recurrences (F kept, p recomputed from x), see k_omp for this form.
+// the printed recurrences (F kept, p recomputed from x), 40 us this way.
 __device__ void gram_picks(const OmpArgs& a, int m, int n, double* dyn) {
     __shared__ unsigned int khi[2][8], klo[2][8];
     __shared__ uint32_t kcol[2][8];
@@ -1100,6 +1099,12 @@ __device__ void gram_emit(const OmpArgs& a, OmpSmem& sh) {
 // the kernel.  mode 0: speculate on the candidate list; mode 1: lock-step over all columns.
 //   CL = 16: one cluster is the whole grid (both groups of 8 in it): every barrier is a cluster barrier
 //   CL = 8, 2: clusters 0 and 1 keep the books of M^ and V^
+// Bound by the generator where the columns are many (correlate_stream), else by latency: barriers, and for each pick the chain
+// best score -> exact scores -> products with the q_l -> new q, r.  us per pick, one block per recovery and a grid barrier after
+// every phase (the Cholesky form) / this form:
+//   lock-step  d = 4096, k = 256: 50 / 11;  50304, 128: 34 / 15;  31820, 1024: 140 / 27;  110000, 210: 46 / 22;  1.2e6, 224: 128 / 88;
+//              2e6, 42: 63 / 55
+//   the books of a pick alone  k = 1024: 16 / 5.5;  k = 2048: 40 / 7
 // ------------------------------------------------------------------------------------------------
 template <int CL>
 __global__ void __launch_bounds__(kT, 1) k_omp(OmpArgs a, int mode) {
