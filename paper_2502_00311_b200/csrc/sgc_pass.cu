@@ -204,6 +204,36 @@ __device__ __forceinline__ void report_flush(const PassArgs& a, const ReportQueu
     __syncwarp();
 }
 
+// largest |v_i| w_i of 16 accumulators, in four chains (one chain of 16 dependent maxima took as long as the load)
+__device__ __forceinline__ float peak16(const uint32_t (&v)[16], const float* w) {
+    float p[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    const float4* w4 = reinterpret_cast<const float4*>(w);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float4 x = w4[i];
+        p[0] = fmaxf(p[0], fabsf(__uint_as_float(v[4 * i])) * x.x);
+        p[1] = fmaxf(p[1], fabsf(__uint_as_float(v[4 * i + 1])) * x.y);
+        p[2] = fmaxf(p[2], fabsf(__uint_as_float(v[4 * i + 2])) * x.z);
+        p[3] = fmaxf(p[3], fabsf(__uint_as_float(v[4 * i + 3])) * x.w);
+    }
+    return fmaxf(fmaxf(p[0], p[1]), fmaxf(p[2], p[3]));
+}
+// which of 16 accumulators reach their thresholds: all compared before the first report is written, because the compiler cannot
+// fetch a threshold ahead of a store to shared memory
+__device__ __forceinline__ unsigned int hits16(const uint32_t (&v)[16], const float* tau, float inv) {
+    unsigned int h = 0u;
+    const float4* t4 = reinterpret_cast<const float4*>(tau);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float4 x = t4[i];
+        h |= fabsf(__uint_as_float(v[4 * i])) * inv >= x.x ? 1u << (4 * i) : 0u;
+        h |= fabsf(__uint_as_float(v[4 * i + 1])) * inv >= x.y ? 2u << (4 * i) : 0u;
+        h |= fabsf(__uint_as_float(v[4 * i + 2])) * inv >= x.z ? 4u << (4 * i) : 0u;
+        h |= fabsf(__uint_as_float(v[4 * i + 3])) * inv >= x.w ? 8u << (4 * i) : 0u;
+    }
+    return h;
+}
+
 // ---- the kernel -----------------------------------------------------------------------------------------
 // dynamic shared memory (after alignment to 1024 bytes):
 //   stages x { A tile 0 (16 KB) | A tile 1 (16 KB) | R^T chunk (n x 128 B) }
@@ -403,16 +433,7 @@ __global__ void __launch_bounds__(pass_threads(EPI), 1) k_pass(const __grid_cons
                 for (int c0 = 0; c0 < kHalf; c0 += 16) {
                     uint32_t v[16];
                     tmem_ld16(tmem_base + ((uint32_t)(quad * 32) << 16) + buf * acc_cols + side * kHalf + c0, v);
-                    float peak = 0.0f;
-                    const float4* in4 = reinterpret_cast<const float4*>(inv_w + c0);
-#pragma unroll
-                    for (int i4 = 0; i4 < 4; ++i4) {
-                        const float4 w = in4[i4];
-                        peak = fmaxf(peak, fabsf(__uint_as_float(v[4 * i4])) * w.x);
-                        peak = fmaxf(peak, fabsf(__uint_as_float(v[4 * i4 + 1])) * w.y);
-                        peak = fmaxf(peak, fabsf(__uint_as_float(v[4 * i4 + 2])) * w.z);
-                        peak = fmaxf(peak, fabsf(__uint_as_float(v[4 * i4 + 3])) * w.w);
-                    }
+                    const float peak = peak16(v, inv_w + c0);
                     if (feeds && peak >= wide_tau_n) {
                         const int m = n_res >= a.big_half ? 1 : 0;
                         unsigned int hits = 0u;
@@ -516,24 +537,12 @@ __global__ void __launch_bounds__(pass_threads(EPI), 1) k_pass(const __grid_cons
                     }
                     // one compare settles the usual case that none of the 16 residuals reaches its threshold
                     // (|v| inv >= tau  <=>  |v| / tau >= 1 / inv, with a little slack for the rounding of 1 / tau)
-                    float peak = 0.0f;
-                    {
-                        const float4* it4 = reinterpret_cast<const float4*>(itau_s + c0);
-#pragma unroll
-                        for (int i4 = 0; i4 < 4; ++i4) {
-                            const float4 w = it4[i4];
-                            peak = fmaxf(peak, fabsf(__uint_as_float(v[4 * i4])) * w.x);
-                            peak = fmaxf(peak, fabsf(__uint_as_float(v[4 * i4 + 1])) * w.y);
-                            peak = fmaxf(peak, fabsf(__uint_as_float(v[4 * i4 + 2])) * w.z);
-                            peak = fmaxf(peak, fabsf(__uint_as_float(v[4 * i4 + 3])) * w.w);
-                        }
-                    }
+                    const float peak = peak16(v, itau_s + c0);
                     if (!(peak * inv >= 0.999f)) continue;
+                    const unsigned int hits = inv > 0.0f ? hits16(v, tau_s + c0, inv) : 0u;
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        const float sc = fabsf(__uint_as_float(v[i])) * inv;
-                        if (sc >= tau_s[c0 + i] && inv > 0.0f) report_push(a, queue_r, (uint32_t)(c0 + i), (uint32_t)col, sc);
-                    }
+                    for (int i = 0; i < 16; ++i)
+                        if (hits >> i & 1u) report_push(a, queue_r, (uint32_t)(c0 + i), (uint32_t)col, fabsf(__uint_as_float(v[i])) * inv);
                 }
             }
             tc_fence_before();
