@@ -170,6 +170,13 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
         : "memory");
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
+// one accumulator column once more: a loop over the few that hold a report, instead of sixteen copies of the report code
+__device__ __forceinline__ float tmem_ld1(uint32_t taddr) {
+    uint32_t v;
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(v) : "r"(taddr) : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    return __uint_as_float(v);
+}
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
@@ -455,12 +462,17 @@ __global__ void __launch_bounds__(pass_threads(EPI), 1) k_pass(const __grid_cons
                             }
                         }
                     }
-                    if (!(peak >= tau_n)) continue;
+                    if (!__any_sync(0xffffffffu, peak >= tau_n)) continue;
+                    unsigned int hits = 0u;
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
                         const float inv = inv_w[c0 + i];
-                        const float sc = fabsf(__uint_as_float(v[i])) * inv;
-                        if (sc >= tau_n && inv > 0.0f) {
+                        hits |= fabsf(__uint_as_float(v[i])) * inv >= tau_n && inv > 0.0f ? 1u << i : 0u;
+                    }
+                    for (unsigned int any = __reduce_or_sync(0xffffffffu, hits); any; any &= any - 1u) {
+                        const int i = __ffs(any) - 1;
+                        const float sc = fabsf(tmem_ld1(tmem_base + ((uint32_t)(quad * 32) << 16) + buf * acc_cols + side * kHalf + c0 + i)) * inv_w[c0 + i];
+                        if (hits >> i & 1u) {
                             const uint32_t col = listed ? col_w[c0 + i] : (uint32_t)(col_first + c0 + i);
                             if (kQueue) report_push(a, queue_r, (uint32_t)n_res, col, sc);
                             else report_append(a, (uint32_t)n_res, col, sc);
@@ -537,12 +549,13 @@ __global__ void __launch_bounds__(pass_threads(EPI), 1) k_pass(const __grid_cons
                     }
                     // one compare settles the usual case that none of the 16 residuals reaches its threshold
                     // (|v| inv >= tau  <=>  |v| / tau >= 1 / inv, with a little slack for the rounding of 1 / tau)
-                    const float peak = peak16(v, itau_s + c0);
-                    if (!(peak * inv >= 0.999f)) continue;
+                    if (!__any_sync(0xffffffffu, peak16(v, itau_s + c0) * inv >= 0.999f)) continue;
                     const unsigned int hits = inv > 0.0f ? hits16(v, tau_s + c0, inv) : 0u;
-#pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        if (hits >> i & 1u) report_push(a, queue_r, (uint32_t)(c0 + i), (uint32_t)col, fabsf(__uint_as_float(v[i])) * inv);
+                    for (unsigned int any = __reduce_or_sync(0xffffffffu, hits); any; any &= any - 1u) {
+                        const int i = __ffs(any) - 1;
+                        const float sc = fabsf(tmem_ld1(tmem_base + ((uint32_t)(quad * 32) << 16) + buf * acc_cols + t * a.n + c0 + i)) * inv;
+                        if (hits >> i & 1u) report_push(a, queue_r, (uint32_t)(c0 + i), (uint32_t)col, sc);
+                    }
                 }
             }
             tc_fence_before();
