@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "sgc.h"
+#include "sgc_omp_plan.h"
 
 namespace sgc {
 
@@ -105,7 +106,6 @@ constexpr int kMaxS = 1024;
 constexpr int kSelCap = 32768;          // candidate slots of the top-s filter
 constexpr int kSelBins = 4096;          // 12-bit magnitude histogram of the sample
 constexpr int kCorrBlocks = 160;        // blocks that correlate, at most (a multiple of 32)
-constexpr int kRescoreCap = 16;         // candidates rescored in fp64 per iteration and residual
 constexpr int kOmpThreads = 1024;       // threads per block of the resolve and finish kernels
 constexpr int kCandCap = 32768;         // candidate columns kept for the restricted (speculative) OMP
 constexpr int kCandKeep = 24576;        // the list is rebuilt from the supports once it grows beyond this

@@ -29,12 +29,9 @@ namespace cg = cooperative_groups;
 namespace sgc {
 namespace {
 
-constexpr int kT = 512;                               // threads per block of k_omp
+constexpr int kT = kOmpBlock;
 constexpr int kWarps = kT / 32;
-constexpr size_t kOmpDynBytes = 196 * 1024;           // dynamic shared memory of every launch (one block per SM)
 constexpr int kRescanCap = 64;
-constexpr double kOmpOneWork = 1.2e6;                  // k * d up to which one cluster of 16 serves the lock-step recovery
-constexpr double kOmpPairCols = 1000.0;                // columns per pick from which pairs do
 constexpr double kPivot = 1e-10;                      // a new column whose orthogonal part is below this share is dependent
 
 // the best column seen (lowest index on ties), and the largest score among all others (what is dropped: the caller can tell
@@ -89,8 +86,6 @@ struct OmpSmem {
 // of the block's columns fit its shared memory they are kept from the first iteration on, as operand registers: an iteration
 // then reads 16 bytes per lane and 16 rows instead of regenerating them.  The norms are summed in the first iteration.
 struct CorrPlan { int e0, cnt, tiles, ks, kblocks; bool cached, norms; size_t part_off, inv_off, col_off, z_off; };
-
-__host__ __device__ inline size_t frag_bytes(int k) { return (size_t)((k + 15) / 16) * 128; }
 
 __device__ CorrPlan corr_plan(const OmpArgs& a, unsigned int n, int blk, int nblk) {
     CorrPlan c;
@@ -456,24 +451,13 @@ __device__ void correlate(const OmpArgs& a, OmpSmem& sh, const CorrPlan& c, cons
 // ------------------------------------------------------------------------------------------------
 // bookkeeping: one group of GS blocks per recovery, block g owns rows [row0, row0 + R) of A
 // ------------------------------------------------------------------------------------------------
-template <int CL> struct Group { static constexpr int GS = CL == 16 ? 8 : CL; };
-
-// row slices: an even number of rows per block (a generated word holds two rows)
-__host__ __device__ inline int slice_rows(int k, int gs) { return 2 * ((k + 2 * gs - 1) / (2 * gs)); }
+template <int CL> struct Group { static constexpr int GS = group_blocks(CL); };
 
 // dynamic shared memory of a bookkeeping block, in doubles: residual slice | partial sums | exchanged sums | exchange slots | q
 struct BookMem {
     double *rr, *part, *cs, *x0, *x1, *xrn, *qs;
     int R, P, row0, rows;                                  // slice length, parts per row in the update, first row, rows owned
 };
-__host__ __device__ inline int even(int n) { return (n + 1) & ~1; }
-// a slot of the exchange: products with q_l and the residual (by l), then ||a||^2, ||r||^2, and two values per further candidate
-__host__ __device__ inline int exchange_stride(int s) { return even(s + 2 + 2 * kRescoreCap); }
-__host__ __device__ inline size_t book_doubles(int k, int s, int gs, bool two) {
-    const int R = slice_rows(k, gs);
-    return (size_t)R + (R > kT ? R : kT) + even(s + 4) + (size_t)(two ? 2 : 1) * gs * exchange_stride(s) + 2 * gs;
-}
-
 __device__ BookMem book_mem(const OmpArgs& a, double* base, int gs, int g, bool two) {
     BookMem b;
     b.R = slice_rows(a.k, gs);
@@ -1473,28 +1457,11 @@ cudaError_t resident_clusters(int* out) {
     return cudaOccupancyMaxActiveClusters(out, k_omp<CL>, &l.cfg);
 }
 
-// columns of q and generated entries that fit beside the fixed buffers
-template <int CL>
-void omp_budget(OmpArgs& a, int mode) {
-    constexpr int GS = Group<CL>::GS;
-    const size_t total = kOmpDynBytes, pb = frag_bytes(a.k), bb = book_doubles(a.k, a.s, GS, CL == 16) * sizeof(double);
-    const size_t col = (size_t)slice_rows(a.k, GS) * sizeof(double);
-    // bookkeeping blocks correlate as well in lock-step, as far as both fit
-    const size_t least = 40 * 1024;                                   // partial sums and norms of the correlation
-    a.book_correlates = (CL == 16 || (mode == 1 && bb + pb + least <= total)) ? 1 : 0;
-    size_t room = total > bb ? total - bb : 0;
-    if (a.book_correlates) room -= pb;
-    size_t q = a.book_correlates ? (room - least) / 2 : room;
-    if (q > col * a.s) q = col * a.s;
-    a.q_cols = (int)(q / col);
-    if (a.book_correlates) room -= (size_t)a.q_cols * col;
-    else room = total - pb;
-    a.z_words = (int)(room / 4) - 8;
-}
-
 template <int CL>
 cudaError_t omp_launch(OmpArgs a, int mode, int grid, cudaStream_t stream) {
-    omp_budget<CL>(a, mode);
+    const OmpBudget b = omp_budget(CL, a.k, a.s, mode);
+    if (!b.fits) return cudaErrorInvalidConfiguration;
+    a.q_cols = b.q_cols; a.book_correlates = b.book_correlates; a.z_words = b.z_words;
     OmpLaunch l(CL, grid, stream);
     return cudaLaunchKernelEx(&l.cfg, k_omp<CL>, a, mode);
 }
@@ -1533,18 +1500,12 @@ cudaError_t omp_configure(sgc_state* st) {
     return cudaSuccess;
 }
 
-// Which cluster shape: the one-cluster form while a pick's correlation takes 16 SMs no longer than the grid barriers cost
-// the others; pairs (all 148 SMs correlate, two blocks keep each recovery's books) when the correlation of a pick (k d) dwarfs
-// its bookkeeping (k s), whatever k is; groups of 8 (120 SMs, the most that clusters of 8 can occupy) otherwise and for lists.
-// Step in groups of 8 / in pairs, us: d = 500000, k = 210, s = 30: 2187 / 1832; 65000, 350, 50: 1312 / 1126; 10000, 200, 8:
-// 143 / 136;  60000, 512, 64 (940 columns per pick): 1692 / 1694;  60000, 1024, 64: 2359 / 2521;  25000, 1400, 200: 7708 / 13020.
 cudaError_t launch_omp(sgc_state* st, const OmpArgs& a, int mode, cudaStream_t stream) {
-    if (mode == 1) {
-        const bool pairs_fit = book_doubles(a.k, a.s, 2, false) * sizeof(double) + frag_bytes(a.k) + 40 * 1024 <= kOmpDynBytes;
-        if (st->omp_one && (double)a.k * (double)a.d <= kOmpOneWork) return omp_launch<16>(a, mode, 16, stream);
-        if (pairs_fit && (double)a.d >= kOmpPairCols * a.s) return omp_launch<2>(a, mode, st->omp_grid2, stream);
+    switch (omp_shape(st->d, a.k, a.s, mode, st->omp_one != 0)) {
+        case 16: return omp_launch<16>(a, mode, 16, stream);
+        case 2: return omp_launch<2>(a, mode, st->omp_grid2, stream);
+        default: return omp_launch<8>(a, mode, st->omp_grid8, stream);
     }
-    return omp_launch<8>(a, mode, st->omp_grid8, stream);
 }
 
 }  // namespace sgc

@@ -83,3 +83,9 @@ def test_chunk_variants(sgc, c, dc, k, sc):  # noqa: F811
                                           (257, 260, 1, 1, 40, 5), (4099, 130, 34, 5, 60, 6)])
 def test_cesgc_remainders(sgc, m, n, r, c, k, sc):  # noqa: F811
     parity.test_cesgc_step_matches_its_oracle(sgc, m, n, r, c, k, sc)
+
+
+# many rows and a handful of columns: the one-cluster form has no room for its books there, groups of eight serve
+@pytest.mark.parametrize("d,k,s", [(73, 16384, 4), (83, 14369, 83), (40, 16384, 33), (80, 13999, 16)])
+def test_lockstep_with_far_more_rows_than_columns(sgc, d, k, s):  # noqa: F811
+    run_both(sgc, d, k, s, 6, "student", 2, cfg_id=2, mode=1)
