@@ -784,21 +784,24 @@ __device__ void gram_matrix(const OmpArgs& a, int n) {
 //     w_j(i) = gamma (sigma G(pick, i) - sum_l c_l w_l(i)),    p_i -= a_j w_j(i):
 // one block barrier per pick and j fp64 multiply-adds per member.  64 picks on 64 columns: 270 us with the k-free form of
 // the printed recurrences (F kept, p recomputed from x), 40 us this way.
-__device__ void gram_picks(const OmpArgs& a, int m, int n, double* dyn) {
+//
+// fin, vc, fc: what the control block said of both recoveries before this phase, read by the whole grid ahead of a grid barrier.
+// Both blocks look both recoveries up in the list and have to come to the same answer, while each moves its own recovery's words on
+// as it goes: neither may read the other's here.
+__device__ void gram_picks(const OmpArgs& a, int m, int n, double* dyn, const int (&fin)[2], const int (&vc)[2], const uint32_t (&fc)[2]) {
     __shared__ unsigned int khi[2][8], klo[2][8];
     __shared__ uint32_t kcol[2][8];
     __shared__ int kidx[2][8];
     __shared__ double ps[2][kGramList], gd[kGramList];
     __shared__ int li[kGramList + 1];
     __shared__ int found;
-    volatile SpecCtl* ctl = a.ctl;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5, s = a.s;
     for (int c = t; c < a.half_n; c += kT) {
         a.rep_count[m * a.half_n + c] = 0u;
         a.tau[m * a.half_n + c] = __int_as_float(0x7f800000);
     }
-    const int v0 = ctl->v[m];
-    const uint32_t forced0 = ctl->forced[m];
+    const int v0 = m ? vc[1] : vc[0];
+    const uint32_t forced0 = m ? fc[1] : fc[0];
     const int base = v0 + (forced0 != kNoColumn ? 1 : 0);
     int end = base + a.half_n < s ? base + a.half_n : s;
     if (end > n + 1) end = n + 1;
@@ -824,10 +827,11 @@ __device__ void gram_picks(const OmpArgs& a, int m, int n, double* dyn) {
     __syncthreads();
     double my_g = 1.0;
     int want = 0;
-    for (int u = 0; u < 2; ++u) {                                     // both blocks look both recoveries up: they decide alike
-        if (ctl->finished[u]) continue;
-        const int vu = ctl->v[u];
-        const uint32_t fu = ctl->forced[u];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        if (fin[u]) continue;
+        const int vu = vc[u];
+        const uint32_t fu = fc[u];
         want += vu + (fu != kNoColumn ? 1 : 0);
         if (!member) continue;
         for (int l = 0; l < vu; ++l) if (a.lam[(size_t)u * s + l] == my_col) { if (u == m) li[l] = t; atomicAdd(&found, 1); }
@@ -843,7 +847,7 @@ __device__ void gram_picks(const OmpArgs& a, int m, int n, double* dyn) {
         if (t == 0) a.ctl->gram_ok = 0;
         return;
     }
-    if (ctl->finished[m]) return;
+    if (m ? fin[1] : fin[0]) return;
     const double inv_g = my_g > 0.0 ? 1.0 / my_g : 0.0;
     int hi = base, extra = 0, dep = 0;
     const int nw = (n + 31) >> 5;                                     // the warps that hold members go on by themselves
@@ -1104,6 +1108,9 @@ __global__ void __launch_bounds__(kT, 1) k_omp(OmpArgs a, int mode) {
     const int k = a.k, s = a.s;
     auto barrier = [&]() { if (kOneCluster) cluster.sync(); else grid.sync(); };
     // ---- gate: identical in every block, because nothing below changes the control block before the first barrier
+    const int fin[2] = {ctl->finished[0], ctl->finished[1]};
+    const int vc[2] = {ctl->v[0], ctl->v[1]};                            // confirmed picks
+    const uint32_t fc[2] = {ctl->forced[0], ctl->forced[1]};             // confirmed winner for pick vc, if any
     if (mode == 0) {
         if (!ctl->round_active || ctl->fallback) return;
         if (a.mini && (ctl->mini_done || ctl->n_cand <= kGramList || (a.wide_count[0] == 0u && a.wide_count[1] == 0u))) return;
@@ -1117,7 +1124,7 @@ __global__ void __launch_bounds__(kT, 1) k_omp(OmpArgs a, int mode) {
                 if (blockIdx.x == 0 && t == 0) a.ctl->gram_version = ctl->list_version;
                 barrier();
             }
-            if (blockIdx.x < 2) gram_picks(a, (int)blockIdx.x, n, dyn);
+            if (blockIdx.x < 2) gram_picks(a, (int)blockIdx.x, n, dyn, fin, vc, fc);
             barrier();
             if (ctl->gram_ok) {
                 gram_rows(a, dyn);
@@ -1127,10 +1134,7 @@ __global__ void __launch_bounds__(kT, 1) k_omp(OmpArgs a, int mode) {
             }
         }
     }
-    const int fin[2] = {ctl->finished[0], ctl->finished[1]};
     if (mode == 1 && fin[0] && fin[1]) return;
-    const int vc[2] = {ctl->v[0], ctl->v[1]};                            // confirmed picks
-    const uint32_t fc[2] = {ctl->forced[0], ctl->forced[1]};             // confirmed winner for pick vc, if any
     const int n_cand = ctl->n_cand;
     const int base[2] = {vc[0] + (fc[0] != kNoColumn ? 1 : 0), vc[1] + (fc[1] != kNoColumn ? 1 : 0)};
     // where this kernel starts: the speculation resumes after the tentative picks (those confirmed against the wide

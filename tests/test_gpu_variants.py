@@ -89,3 +89,12 @@ def test_cesgc_remainders(sgc, m, n, r, c, k, sc):  # noqa: F811
 @pytest.mark.parametrize("d,k,s", [(73, 16384, 4), (83, 14369, 83), (40, 16384, 33), (80, 13999, 16)])
 def test_lockstep_with_far_more_rows_than_columns(sgc, d, k, s):  # noqa: F811
     run_both(sgc, d, k, s, 6, "student", 2, cfg_id=2, mode=1)
+
+
+# picks refuted while the list stays short: a round on the Gram matrix starts from a prescribed pick, of one recovery or of both
+@pytest.mark.parametrize("d,k,s", [(200, 64, 10), (256, 128, 40), (250, 64, 3)])
+def test_prescribed_picks_on_a_short_list(sgc, d, k, s):  # noqa: F811
+    stats = []
+    run_both(sgc, d, k, s, 7, "student", 12, cfg_id=2, mode=2, redraw_support=True, n_planted=2 * s, stats=stats)
+    assert any(rounds > 1 and not fallback for rounds, fallback, _ in stats), stats
+    assert all(n_cand <= 256 for _, _, n_cand in stats)
