@@ -13,6 +13,7 @@
 // Every record lands in the chunk's own state, so sgc_get works per chunk exactly as after sgc_step.
 #include <algorithm>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include <cooperative_groups.h>
@@ -118,6 +119,9 @@ k_chunk_front(ChunkArgs a, const float* __restrict__ grad, double b1, double b2,
     __shared__ int n_list;
     cg::cluster_group cluster = cg::this_cluster();
     const int split = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();      // split: a power of two
+    // every block of the cluster has to run before another writes to its shared memory: announced here, waited for after the read
+    cg::cluster_group::arrival_token started;
+    if (split > 1) started = cluster.barrier_arrive();
     const int ch = blockIdx.x / split, s = a.s, k = a.k, t = threadIdx.x;
     const ChunkRef ref = a.table[ch];
     const float* g = grad + (size_t)ch * a.dc;
@@ -149,6 +153,7 @@ k_chunk_front(ChunkArgs a, const float* __restrict__ grad, double b1, double b2,
             const unsigned int who = __ballot_sync(0xffffffffu, !out && top == m);
             if (who != 0u && lane == __ffs(who) - 1) out = true;
         }
+        if (split > 1) cluster.barrier_wait(std::move(started));
         if (lane < split) *cluster.map_shared_rank(&wtau[rank * (kFrontThreads / 32) + warp], lane) = m;
     }
     if (split > 1) cluster.sync(); else __syncthreads();

@@ -98,3 +98,17 @@ def test_prescribed_picks_on_a_short_list(sgc, d, k, s):  # noqa: F811
     run_both(sgc, d, k, s, 7, "student", 12, cfg_id=2, mode=2, redraw_support=True, n_planted=2 * s, stats=stats)
     assert any(rounds > 1 and not fallback for rounds, fallback, _ in stats), stats
     assert all(n_cand <= 256 for _, _, n_cand in stats)
+
+
+# several blocks per chunk with short shares: each writes its bound into the others' shared memory
+@pytest.mark.parametrize("c,dc,sc", [(1, 16_384, 31), (20, 65_536, 5), (70, 16_388, 1), (9, 32_772, 17)])
+def test_chunk_selection_over_a_cluster(sgc, c, dc, sc):  # noqa: F811
+    m = sgc.Mesgc(c * dc, c, 8 * sc, sc, 8, *(inputs.ADAM[n] for n in ("lr", "beta1", "beta2", "eps")))
+    w = cuda(np.zeros(c * dc, dtype=np.float32))
+    for step in range(20):
+        g = np.random.default_rng(100 * c + step).standard_t(3.0, size=c * dc).astype(np.float32)
+        m.step(cuda(g), w)
+        for i, st in enumerate(m.chunks):
+            idx, val = oracle.sparsify(g[i * dc:(i + 1) * dc], sc)
+            assert np.array_equal(st.get("sel_idx"), idx) and np.array_equal(st.get("sel_val"), val), (step, i)
+    m.close()
