@@ -85,34 +85,6 @@ struct OmpSmem {
 // would be idle but for one in sixty columns, and the generator bounds it anyway.  A tile's rows are split over several warps when the block has fewer tiles than warps.  When the generated entries
 // of the block's columns fit its shared memory they are kept from the first iteration on, as operand registers: an iteration
 // then reads 16 bytes per lane and 16 rows instead of regenerating them.  The norms are summed in the first iteration.
-struct CorrPlan { int e0, cnt, tiles, ks, kblocks; bool cached, norms; size_t part_off, inv_off, col_off, z_off; };
-
-__device__ CorrPlan corr_plan(const OmpArgs& a, unsigned int n, int blk, int nblk) {
-    CorrPlan c;
-    const unsigned int per = (n + nblk - 1) / nblk;
-    const unsigned long long e0 = (unsigned long long)per * blk;
-    c.e0 = e0 < n ? (int)e0 : (int)n;
-    c.cnt = e0 >= n ? 0 : (int)((n - e0) < per ? (n - e0) : per);
-    const int tiles = (int)((per + 15) / 16);                         // the same plan in every block
-    c.kblocks = (a.k + 15) / 16;
-    int best = 1; float cost = 3e38f;
-    for (int ks = 1; ks <= 16 && ks <= c.kblocks && tiles * ks <= 64; ks <<= 1) {
-        const float rounds = (float)((tiles * ks + kWarps - 1) / kWarps);
-        const float t = rounds * ((float)((c.kblocks + ks - 1) / ks) + 3.0f);
-        if (t < cost * 0.99f) { cost = t; best = ks; }
-    }
-    c.ks = best;
-    c.tiles = tiles;
-    // word offsets in the correlation's part of shared memory: partial sums of split tiles, norms, generated entries
-    c.part_off = 0;
-    c.inv_off = best > 1 ? (size_t)tiles * best * 32 : 0;
-    c.norms = c.inv_off + (size_t)tiles * 32 <= (size_t)a.z_words;      // norms, and the columns themselves (lists)
-    c.col_off = c.inv_off + (size_t)tiles * 16;
-    c.z_off = (c.inv_off + (c.norms ? (size_t)tiles * 32 : 0) + 3) & ~(size_t)3;
-    c.cached = c.norms && c.z_off + (size_t)tiles * c.kblocks * 128 <= (size_t)a.z_words;
-    return c;
-}
-
 // membership in a support staged in shared memory (padded with kNoColumn to a multiple of 4)
 __device__ __forceinline__ bool in_support4(const uint32_t* sup, int n, uint32_t col) {
     bool hit = false;
@@ -610,7 +582,7 @@ __device__ void emit_row(const OmpArgs& a, const BookMem& b, size_t n, double rn
 // rescoring window as well.  Its columns are screened again here and every free one inside the window (with a little slack:
 // the sums run in another order) that was not forwarded is noted, so that all of them reach the fp64 decision.
 __device__ void rescan_block(const OmpArgs& a, OmpSmem& sh, int m, int j, int blk, int nblk, float thr, uint32_t forwarded) {
-    const CorrPlan c = corr_plan(a, (unsigned int)a.d, blk, nblk);
+    const CorrPlan c = corr_plan((unsigned int)a.d, a.k, a.z_words, blk, nblk);
     const float2* r = reinterpret_cast<const float2*>(a.r32);
     for (int idx = threadIdx.x; idx < c.cnt; idx += kT) {
         const uint32_t col = (uint32_t)(c.e0 + idx);
@@ -1225,7 +1197,7 @@ __global__ void __launch_bounds__(kT, 1) k_omp(OmpArgs a, int mode) {
             }
         }
     }
-    CorrPlan plan = corr_plan(a, n_cols, corr ? cblk : 0, nblk);
+    CorrPlan plan = corr_plan(n_cols, k, a.z_words, corr ? cblk : 0, nblk);
     bool filled = false;
     barrier();
     for (int i = 0;; ++i) {

@@ -64,6 +64,35 @@ inline OmpBudget omp_budget(int cl, int k, int s, int mode) {
     return b;
 }
 
+// The share of block blk of nblk in the correlation of n columns, and where its sums, norms and generated entries lie (word offsets
+// in the z_words of shared memory that it has).
+struct CorrPlan { uint32_t e0; int cnt, tiles, ks, kblocks; bool cached, norms; size_t part_off, inv_off, col_off, z_off; };
+
+SGC_HD inline CorrPlan corr_plan(uint32_t n, int k, int z_words, int blk, int nblk) {
+    CorrPlan c;
+    const uint64_t per = ((uint64_t)n + nblk - 1) / nblk, e0 = per * blk;      // (up to 2^32 - 1 columns)
+    c.e0 = e0 < n ? (uint32_t)e0 : n;
+    c.cnt = (int)(n - c.e0 < per ? n - c.e0 : per);
+    const int tiles = (int)((per + 15) / 16);                         // the same plan in every block
+    c.kblocks = (k + 15) / 16;
+    int best = 1; float cost = 3e38f;
+    for (int ks = 1; ks <= 16 && ks <= c.kblocks && tiles * ks <= 64; ks <<= 1) {
+        const float rounds = (float)((tiles * ks + kOmpBlock / 32 - 1) / (kOmpBlock / 32));
+        const float t = rounds * ((float)((c.kblocks + ks - 1) / ks) + 3.0f);
+        if (t < cost * 0.99f) { cost = t; best = ks; }
+    }
+    c.ks = best;
+    c.tiles = tiles;
+    // partial sums of split tiles, norms, generated entries
+    c.part_off = 0;
+    c.inv_off = best > 1 ? (size_t)tiles * best * 32 : 0;
+    c.norms = c.inv_off + (size_t)tiles * 32 <= (size_t)z_words;      // norms, and the columns themselves (lists)
+    c.col_off = c.inv_off + (size_t)tiles * 16;
+    c.z_off = (c.inv_off + (c.norms ? (size_t)tiles * 32 : 0) + 3) & ~(size_t)3;
+    c.cached = c.norms && c.z_off + (size_t)tiles * c.kblocks * 128 <= (size_t)z_words;
+    return c;
+}
+
 // Which cluster shape (16, 2 or 8; one: a cluster of 16 can be resident): the one-cluster form while a pick's correlation takes
 // 16 SMs no longer than the grid barriers cost the others; pairs (all 148 SMs correlate, two blocks keep each recovery's books)
 // when the correlation of a pick (k d) dwarfs its bookkeeping (k s), whatever k is; groups of 8 (120 SMs, the most that

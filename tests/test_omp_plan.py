@@ -47,6 +47,18 @@ extern "C" int sweep_budget(int k0, int k1, long long* out) {
         }
     return 0;
 }
+// are the blocks' shares of n columns whole, one after the other and inside their memory?
+extern "C" int shares(unsigned n, int k, int nblk) {
+    unsigned long long at = 0;
+    for (int b = 0; b < nblk; ++b) {
+        const CorrPlan c = corr_plan(n, k, 20000, b, nblk);
+        if (c.cnt < 0 || (unsigned long long)c.tiles * 16 < (unsigned long long)c.cnt || (c.cnt > 0 && c.e0 != at)) return 0;
+        at += (unsigned long long)c.cnt;
+        if (c.norms && c.inv_off + (size_t)c.tiles * 32 > 20000) return 0;
+        if (c.cached && c.z_off + (size_t)c.tiles * c.kblocks * 128 > 20000) return 0;
+    }
+    return at == n;
+}
 extern "C" int shape(long long d, int k, int s, int mode, int one) { return omp_shape(d, k, s, mode, one != 0); }
 """
 
@@ -71,3 +83,11 @@ def test_many_rows_and_few_columns_leave_the_one_cluster_form(plan):
     # books and operands of the one cluster do not fit one block there
     assert [plan.shape(C.c_longlong(d), k, s, 1, 1) for d, k, s in [(73, 16384, 4), (83, 14369, 83), (64, 16384, 64)]] == [8, 8, 8]
     assert [plan.shape(C.c_longlong(d), k, s, 1, 1) for d, k, s in [(4096, 256, 16), (80, 14000, 16), (1171, 1024, 1024)]] == [16, 16, 16]
+
+
+@pytest.mark.parametrize("nblk", [8, 16, 104, 120, 148, 160])
+def test_shares_of_the_correlation_are_whole(plan, nblk):
+    for n in [1, 7, nblk - 1, nblk, nblk + 1, 16 * nblk + 1, 24_576, 45_088_768, 2**31 - 1, 2**31, 2**31 + 12_345, 3 * 2**30 + 5,
+              2**32 - nblk, 2**32 - nblk + 1, 2**32 - 2, 2**32 - 1]:
+        for k in (1, 64, 300, 16384):
+            assert plan.shares(C.c_uint(n), k, nblk), (n, k)
