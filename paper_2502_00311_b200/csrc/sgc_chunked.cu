@@ -306,14 +306,22 @@ __device__ __forceinline__ void mma_16816(float (&c)[4], const uint4& x, uint32_
         : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(x.x), "r"(x.y), "r"(x.z), "r"(x.w), "r"(b0), "r"(b1));
 }
 
-// the two best columns of a recovery
+// the two best columns of a recovery, and a bound on the score of all others
 struct Best2 {
-    float s1, s2; uint32_t i1, i2;
+    float s1, s2, s3; uint32_t i1, i2;
     __device__ __forceinline__ void push(float s, uint32_t i) {      // i != i1, i2; lower index first on ties
-        if (s > s1 || (s == s1 && i < i1)) { s2 = s1; i2 = i1; s1 = s; i1 = i; }
-        else if (s > s2 || (s == s2 && i < i2)) { s2 = s; i2 = i; }
+        if (s > s1 || (s == s1 && i < i1)) { s3 = fmaxf(s3, s2); s2 = s1; i2 = i1; s1 = s; i1 = i; }
+        else if (s > s2 || (s == s2 && i < i2)) { s3 = fmaxf(s3, s2); s2 = s; i2 = i; }
+        else s3 = fmaxf(s3, s);
     }
 };
+
+// Keys (see k_chunk_corr) order columns to 2^-13 of their score, so that one which is left out may yet be the best when three agree
+// that closely.  A block that may have left a key within kKeyWindow of its first out marks its first candidate's index, and k_chunk_pick
+// goes through that block's columns again if they can hold the best one (as long as three columns have to agree the keys themselves
+// cost nothing more; kept per column, a third key cost 8 % of a step).  The window: one step of the keys, and 4e-5 for the fp32 sums.
+constexpr float kKeyWindow = 3e-4f;
+constexpr uint32_t kThirdMark = 0x80000000u;                          // (a chunk has fewer than 2^31 columns)
 
 // 1 / ||Z|| of a column and the code that its keys carry
 __device__ __forceinline__ float2 corr_norm(float n2, int code, bool real) {
@@ -404,7 +412,7 @@ __global__ void __launch_bounds__(corr_threads(KP)) k_chunk_corr(ChunkArgs a, in
     bool exclude = false;
     for (;;) {
 #pragma unroll
-        for (int i = 0; i < NT; ++i) { best[i].s1 = best[i].s2 = -1.0f; best[i].i1 = best[i].i2 = kNoColumn; }
+        for (int i = 0; i < NT; ++i) { best[i].s1 = best[i].s2 = best[i].s3 = -1.0f; best[i].i1 = best[i].i2 = kNoColumn; }
         for (long long super = col0; super < col1; super += kCorrSuper) {
             unsigned int k1[NT], k2[NT];
 #pragma unroll
@@ -450,17 +458,22 @@ __global__ void __launch_bounds__(corr_threads(KP)) k_chunk_corr(ChunkArgs a, in
                     }
                 }
             }
-            // the eight lanes of a recovery (same q) join their best two
+            // the eight lanes of a recovery (same q) join their best two; k3: the largest key that may be left out (a lane has not kept
+            // its third, which its second bounds)
 #pragma unroll
             for (int i = 0; i < NT; ++i) {
+                unsigned int k3 = k2[i];
 #pragma unroll
                 for (int o = 4; o < 32; o <<= 1) {
                     const unsigned int t1 = __shfl_xor_sync(0xffffffffu, k1[i], o), t2 = __shfl_xor_sync(0xffffffffu, k2[i], o);
+                    const unsigned int t3 = __shfl_xor_sync(0xffffffffu, k3, o);
+                    k3 = max(max(k3, t3), max(min(k2[i], t1), min(k1[i], t2)));
                     k2[i] = max(max(k2[i], t2), min(k1[i], t1));
                     k1[i] = max(k1[i], t1);
                 }
                 if (k1[i]) best[i].push(__uint_as_float(k1[i] & ~1023u), (uint32_t)(super + kCorrSuper - (k1[i] & 1023u)));
                 if (k2[i]) best[i].push(__uint_as_float(k2[i] & ~1023u), (uint32_t)(super + kCorrSuper - (k2[i] & 1023u)));
+                best[i].s3 = fmaxf(best[i].s3, __uint_as_float(k3 & ~1023u));
             }
         }
         if (exclude || iter == 0) break;
@@ -486,7 +499,8 @@ __global__ void __launch_bounds__(corr_threads(KP)) k_chunk_corr(ChunkArgs a, in
         if (g == 0 && mine < 2 * a.c) {
             const float back = a.back[mine];
             float4* out = reinterpret_cast<float4*>(a.cand + ((size_t)mine * a.splits + blockIdx.x) * 2);
-            *out = make_float4(best[i].i1 != kNoColumn ? best[i].s1 * back : -1.0f, __uint_as_float(best[i].i1),
+            const bool third = best[i].s3 > 0.0f && best[i].s3 >= best[i].s1 * (1.0f - kKeyWindow);
+            *out = make_float4(best[i].i1 != kNoColumn ? best[i].s1 * back : -1.0f, __uint_as_float(third ? best[i].i1 | kThirdMark : best[i].i1),
                                best[i].i2 != kNoColumn ? best[i].s2 * back : -1.0f, __uint_as_float(best[i].i2));
         }
     }
@@ -508,7 +522,8 @@ struct PickSmem {
     double red[kPickMaxThreads / 32];
     float fred[kPickMaxThreads / 32];
     uint32_t cidx[kRescoreCap];
-    int n_c;
+    int redo[8];
+    int n_c, n_redo;
 };
 
 // dynamic shared memory: residual r [k], q [j][k]
@@ -655,6 +670,29 @@ __device__ void pick_finish(const ChunkArgs& a, const ChunkRef& ref, PickSmem& s
     if (t == 0) { ref.rnorm[(size_t)m * s + j] = rn; a.back[res] = (float)(1.0 / sc); }
 }
 
+// The columns col0 .. col1 of a split once more, whose third key came too close: every free column with score >= thr that the split
+// did not forward (f0, f1) joins the candidates (fp64, thread = column; once in some 10^5 picks of a noisy recovery).
+__device__ __noinline__ void pick_redo_split(PickSmem* sh, uint32_t seed_lo, uint32_t seed_hi, int k, const uint32_t* sup, int j,
+                                             uint32_t col0, uint32_t col1, uint32_t f0, uint32_t f1, double thr) {
+    const double* r = pick_mem();
+    for (uint32_t col = col0 + threadIdx.x; col < col1; col += blockDim.x) {
+        const ColKey key = column_key(seed_lo, seed_hi, col);
+        double dot = 0.0, n2 = 0.0;
+        for (int row = 0; row < k; row += 2) {
+            const float2 z = half2_bits_to_float2(z_pair_from_word(key.ck + (uint32_t)(row >> 1) * key.mk));
+            dot = fma((double)z.x, r[row], dot); n2 = fma((double)z.x, (double)z.x, n2);
+            if (row + 1 < k) { dot = fma((double)z.y, r[row + 1], dot); n2 = fma((double)z.y, (double)z.y, n2); }
+        }
+        if (!(n2 > 0.0) || fabs(dot) < thr * sqrt(n2) || col == f0 || col == f1) continue;
+        bool taken = false;
+        for (int l = 0; l < j; ++l) taken = taken || sup[l] == col;
+        if (taken) continue;
+        const int slot = atomicAdd(&sh->n_c, 1);
+        if (slot < kRescoreCap) sh->cidx[slot] = col;
+    }
+    __syncthreads();
+}
+
 // SIMT route: the candidates are the columns that phase A left within 2e-3 (relative) of the best fp32 score.
 // only != nullptr: a second chance for the recoveries that the tensor-core route marked unresolved; skipped unless *gate
 // names this iteration.
@@ -665,7 +703,7 @@ __global__ void __launch_bounds__(kPickMaxThreads) k_chunk_pick(ChunkArgs a, int
     // what earlier picks left is complete when this grid starts (phase A, the kernel before this one, has waited for the last
     // pick, and lets this one's blocks in only then), so it can be fetched before waiting for phase A itself
     if (gate == nullptr) pick_stage(a, ref, m, j);
-    if (t == 0) sh.n_c = 0;
+    if (t == 0) sh.n_c = sh.n_redo = 0;
     after_previous_kernel(a.early);
     if (gate != nullptr && *gate != a.epoch0 + iter) return;
     if (only != nullptr && !only[res]) return;
@@ -685,15 +723,29 @@ __global__ void __launch_bounds__(kPickMaxThreads) k_chunk_pick(ChunkArgs a, int
     for (int e = t + 2 * (int)blockDim.x; e < n_entries; e += blockDim.x) if (cc[e].idx != kNoColumn) mx = fmaxf(mx, cc[e].score);
     mx = pick_max(sh, mx);                                          // (its barriers also publish n_c = 0)
     const float thr = mx - 2e-3f * fabsf(mx);
-    auto offer = [&](const Cand& c) {
+    auto offer = [&](const Cand& c, int e) {
         if (c.idx != kNoColumn && c.score >= 0.0f && c.score >= thr) {
             const int slot = atomicAdd(&sh.n_c, 1);
-            if (slot < kRescoreCap) sh.cidx[slot] = c.idx;
+            if (slot < kRescoreCap) sh.cidx[slot] = c.idx & ~kThirdMark;
+            if ((c.idx & kThirdMark) && c.score >= mx * (1.0f - kKeyWindow) && mx > 0.0f) {
+                const int q = atomicAdd(&sh.n_redo, 1);
+                if (q < 8) sh.redo[q] = e >> 1;
+            }
         }
     };
-    offer(first[0]); offer(first[1]);
-    for (int e = t + 2 * (int)blockDim.x; e < n_entries; e += blockDim.x) offer(cc[e]);
+    offer(first[0], t); offer(first[1], t + (int)blockDim.x);
+    for (int e = t + 2 * (int)blockDim.x; e < n_entries; e += blockDim.x) offer(cc[e], e);
     __syncthreads();
+    if (sh.n_redo > 0) {
+        // (more than eight such splits hold more than kRescoreCap candidates by themselves)
+        const int n_redo = sh.n_redo < 8 ? sh.n_redo : 8;
+        for (int q = 0; q < n_redo; ++q) {
+            const Cand* fwd = cc + 2 * sh.redo[q];
+            const long long col0 = (long long)sh.redo[q] * a.cols_per_split, col1 = col0 + a.cols_per_split;
+            pick_redo_split(&sh, a.seed_lo, a.seed_hi, a.k, a.lam + (size_t)res * a.s, j, (uint32_t)col0, (uint32_t)(col1 < a.dc ? col1 : a.dc),
+                            fwd[0].idx & ~kThirdMark, fwd[1].idx, (double)thr);
+        }
+    }
     int nc = sh.n_c;
     if (nc > kRescoreCap) {
         if (t == 0) atomicOr(&ref.cnt->status, (unsigned int)SGC_STATUS_CANDIDATE_OVERFLOW);

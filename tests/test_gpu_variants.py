@@ -112,3 +112,28 @@ def test_chunk_selection_over_a_cluster(sgc, c, dc, sc):  # noqa: F811
             idx, val = oracle.sparsify(g[i * dc:(i + 1) * dc], sc)
             assert np.array_equal(st.get("sel_idx"), idx) and np.array_equal(st.get("sel_val"), val), (step, i)
     m.close()
+
+
+# Columns of 16 neighbours, all in the share of one block of the chunk correlation, whose scores agree to 1e-5: closer than the keys
+# resolve that pick what the block forwards (2^-13), far above the fp64 scores that decide.  More of them than it forwards.
+@pytest.mark.parametrize("dc,k,c,tied", [(2048, 64, 1, 3), (2048, 24, 1, 3), (4096, 200, 2, 3), (512, 8, 3, 3), (2048, 100, 1, 5),
+                                         (4096, 16, 40, 4)])
+def test_chunk_picks_among_near_tied_columns(sgc, dc, k, c, tied):  # noqa: F811
+    hp = [inputs.ADAM[n] for n in ("lr", "beta1", "beta2", "eps")]
+    for trial in range(12):
+        rng, seed = np.random.default_rng(trial), 100 + trial
+        cols = 16 * int(rng.integers(0, dc // 16)) + np.sort(rng.choice(16, tied, replace=False))
+        A = float(oracle.sigma(k)) * np.concatenate([oracle.z_block(seed, 0, k, int(q), 1) for q in cols], axis=1).astype(np.float64)
+        G = (A.T @ A) / np.sqrt((A * A).sum(axis=0))[:, None]
+        x = np.linalg.solve(G, 1.0 + 1e-5 * np.arange(tied))              # the last of the columns wins by 1e-5
+        g = np.zeros(dc, dtype=np.float32)
+        g[cols] = x.astype(np.float32)
+        m = sgc.Mesgc(c * dc, c, k, tied, seed, *hp)
+        ref = oracle.Oracle(dc, k, tied, seed, *hp)
+        m.step(cuda(np.tile(g, c)), cuda(np.zeros(c * dc, dtype=np.float32)))
+        ref.step(g, np.zeros(dc, dtype=np.float32))
+        for st in (m.chunks[0], m.chunks[-1]):
+            assert np.array_equal(st.get("lamM"), ref.get("lamM")), (trial, st.get("lamM"), ref.get("lamM"))
+            assert np.array_equal(st.get("lamV"), ref.get("lamV")), trial
+        m.close()
+        ref.close()
