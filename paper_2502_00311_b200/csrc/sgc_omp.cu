@@ -578,14 +578,41 @@ __device__ void emit_row(const OmpArgs& a, const BookMem& b, size_t n, double rn
     if (g == 0 && threadIdx.x == 0) a.inv_scale[n] = (float)(1.0 / sc);
 }
 
-// Lock-step only.  Block `blk` of the screen forwarded its best column for residual m, but another scored inside the
-// rescoring window as well.  Its columns are screened again here and every free one inside the window (with a little slack:
-// the sums run in another order) that was not forwarded is noted, so that all of them reach the fp64 decision.
-__device__ void rescan_block(const OmpArgs& a, OmpSmem& sh, int m, int j, int blk, int nblk, float thr, uint32_t forwarded) {
-    const CorrPlan c = corr_plan((unsigned int)a.d, a.k, a.z_words, blk, nblk);
+// Block `blk` of the screen forwarded its best column for residual m, but another scored inside the rescoring window as well.
+// Its columns are screened again here and every free one inside the window (with a little slack: the sums run in another order)
+// that was not forwarded is noted, so that all of them reach the fp64 decision.  Lock-step (col_list == nullptr): thread = column;
+// a block's share of a list is a few columns of as many rows: warp = column.
+__device__ void rescan_block(const OmpArgs& a, OmpSmem& sh, const uint32_t* col_list, unsigned int n_cols, int m, int j, int blk, int nblk,
+                             float thr, uint32_t forwarded) {
+    const CorrPlan c = corr_plan(n_cols, a.k, a.z_words, blk, nblk);
     const float2* r = reinterpret_cast<const float2*>(a.r32);
+    auto note = [&](uint32_t col, float acc, float n2) {
+        const float sc = n2 > 0.0f ? acc * acc / n2 : 0.0f;
+        if (sc >= thr * 0.9999f && col != forwarded && !in_list(a.lam + (size_t)m * a.s, j, col)) {
+            const int slot = atomicAdd(&sh.rbuf_n, 1);
+            if (slot < kRescanCap) sh.rbuf[slot] = col;
+        }
+    };
+    if (col_list != nullptr) {
+        const int lane = threadIdx.x & 31;
+        for (int idx = threadIdx.x >> 5; idx < c.cnt; idx += kWarps) {
+            const uint32_t col = col_list[c.e0 + idx];
+            const ColKey key = column_key(a.seed_lo, a.seed_hi, col);
+            float acc = 0.0f, n2 = 0.0f;
+            for (int p = lane; 2 * p < a.k; p += 32) {
+                const float4 rr = __ldcg(reinterpret_cast<const float4*>(r) + p);        // (padded by two rows)
+                const float2 z = half2_bits_to_float2(z_pair_from_word(key.ck + (uint32_t)p * key.mk));
+                acc = __fmaf_rn(z.x, m ? rr.y : rr.x, acc); n2 = __fmaf_rn(z.x, z.x, n2);
+                if (2 * p + 1 < a.k) { acc = __fmaf_rn(z.y, m ? rr.w : rr.z, acc); n2 = __fmaf_rn(z.y, z.y, n2); }
+            }
+            for (int o = 16; o > 0; o >>= 1) { acc += __shfl_xor_sync(0xffffffffu, acc, o); n2 += __shfl_xor_sync(0xffffffffu, n2, o); }
+            if (lane == 0) note(col, acc, n2);
+        }
+        __syncthreads();
+        return;
+    }
     for (int idx = threadIdx.x; idx < c.cnt; idx += kT) {
-        const uint32_t col = (uint32_t)(c.e0 + idx);
+        const uint32_t col = c.e0 + (uint32_t)idx;
         const ColKey key = column_key(a.seed_lo, a.seed_hi, col);
         uint32_t h = key.ck;
         float acc = 0.0f, n2 = 0.0f;
@@ -596,20 +623,18 @@ __device__ void rescan_block(const OmpArgs& a, OmpSmem& sh, int m, int j, int bl
             acc = __fmaf_rn(z.x, m ? r0.y : r0.x, acc); n2 = __fmaf_rn(z.x, z.x, n2);
             if (row + 1 < a.k) { acc = __fmaf_rn(z.y, m ? r1.y : r1.x, acc); n2 = __fmaf_rn(z.y, z.y, n2); }
         }
-        const float sc = n2 > 0.0f ? acc * acc / n2 : 0.0f;
-        if (sc >= thr * 0.9999f && col != forwarded && !in_list(a.lam + (size_t)m * a.s, j, col)) {
-            const int slot = atomicAdd(&sh.rbuf_n, 1);
-            if (slot < kRescanCap) sh.rbuf[slot] = col;
-        }
+        note(col, acc, n2);
     }
     __syncthreads();
 }
 
 // The screened candidates of pick j: everything within 2e-3 (relative, squared scores) of the best fp32 score, the best one
 // first; every block of a group finds the same list.  Returns their number; *first: the best one (a list of more than one is in
-// sh.cidx); *inexact: a column inside the window was not forwarded (list mode only: the screening pass judges it).  Every warp
-// reads all blocks' entries: the usual case of one candidate needs no barrier.
-__device__ int gather_candidates(const OmpArgs& a, OmpSmem& sh, int m, int j, int nblk, bool lock, uint32_t* first, bool* inexact) {
+// sh.cidx); *inexact: not every column inside the window is in it (list mode: the screening pass then judges the list's members as
+// it does all others).  col_list, n_cols: the columns that the blocks share, all of them (nullptr) or a list's.  Every warp reads all
+// blocks' entries: the usual case of one candidate needs no barrier.
+__device__ int gather_candidates(const OmpArgs& a, OmpSmem& sh, int m, int j, int nblk, const uint32_t* col_list, unsigned int n_cols,
+                                 uint32_t* first, bool* inexact) {
     constexpr int kPer = kCorrBlocks / 32;
     const int t = threadIdx.x, lane = t & 31;
     const float4* cc = a.corr_cand + (size_t)m * nblk;
@@ -639,9 +664,8 @@ __device__ int gather_candidates(const OmpArgs& a, OmpSmem& sh, int m, int j, in
     best = __reduce_min_sync(0xffffffffu, best);
     kept = __any_sync(0xffffffffu, kept);
     *first = best;
-    if (kept && !lock) *inexact = true;
-    if (total == 1 && !(kept && lock)) return 1;
-    // several candidates, or columns that a block of the lock-step screen kept to itself
+    if (total == 1 && !kept) return 1;
+    // several candidates, or columns that a block kept to itself
     __syncthreads();
     if (t == 0) { sh.nc = 0; sh.rescan_n = 0; sh.rbuf_n = 0; }
     __syncthreads();
@@ -664,13 +688,14 @@ __device__ int gather_candidates(const OmpArgs& a, OmpSmem& sh, int m, int j, in
         if (lane == 0) sh.cidx[0] = best;
     }
     __syncthreads();
-    if (kept && lock) {
+    if (kept) {
         const int n_blk = sh.rescan_n < 8 ? sh.rescan_n : 8;
-        for (int q = 0; q < n_blk; ++q) rescan_block(a, sh, m, j, sh.rescan_blk[q], nblk, thr, sh.rescan_col[q]);
+        for (int q = 0; q < n_blk; ++q) rescan_block(a, sh, col_list, n_cols, m, j, sh.rescan_blk[q], nblk, thr, sh.rescan_col[q]);
         const bool over = sh.rescan_n > 8 || sh.rbuf_n > kRescanCap || total + sh.rbuf_n > kRescoreCap;
+        if (over) *inexact = true;
         if (t == 0) {
-            if (over) atomicOr(&a.cnt->status, (unsigned int)SGC_STATUS_CANDIDATE_OVERFLOW);
-            else
+            if (over && col_list == nullptr) atomicOr(&a.cnt->status, (unsigned int)SGC_STATUS_CANDIDATE_OVERFLOW);
+            if (!over)
                 // ascending order, so that every block of the group has the same list whatever order the atomics gave
                 for (int e = 0; e < sh.rbuf_n; ++e) {
                     int lo = e;
@@ -1226,7 +1251,7 @@ __global__ void __launch_bounds__(kT, 1) k_omp(OmpArgs a, int mode) {
         // ---- 1. candidates, their exact scores, the products of the best one with the q_l, ||r||
         if (active) {
             if (i == 0 && first_col[mb] != kNoColumn) { col = first_col[mb]; nc = 1; }
-            else nc = gather_candidates(a, sh, m, j, nblk, mode == 1, &col, &inexact);
+            else nc = gather_candidates(a, sh, m, j, nblk, mode == 0 ? a.cand_list : nullptr, n_cols, &col, &inexact);
             if (nc > 0) {
                 send_products<GS>(cluster, a, bk, m, j, col, true, bk.x0, rank0, g);
                 for (int e = 1 + (t >> 5); e < nc; e += kWarps) send_candidate<GS>(cluster, a, bk, sh.cidx[e], e, bk.x0, rank0, g);

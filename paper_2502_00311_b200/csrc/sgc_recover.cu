@@ -41,12 +41,17 @@ __device__ double block_sum(double v, double* red) {
     return t;
 }
 
+// Challengers of one pick that the walk rescores (3 us each at k = 16384) before it gives the step up to lock-step, where a pick
+// costs a generation of all columns.  The margin grows with k: with 16384 rows and kept entries of nearly equal size more than the 16
+// that the other kernels have room for come within it (d = 65600, s = 250: half of the steps were given up, 41 -> 110 to 170 ms).
+constexpr int kResolveCap = 256;
+
 // shared memory of the resolve kernel's walk
 struct BookSmem {
     double red[32];
     double best_dot, best_n2, best_score;
     uint32_t best_idx;
-    uint32_t cand_idx[kRescoreCap];
+    uint32_t cand_idx[kResolveCap];
     int n_cand;
     unsigned int smax_bits;
 };
@@ -124,12 +129,12 @@ __device__ int collect_challengers(BookSmem& sh, const uint2* rep, unsigned int 
         const float sc = __uint_as_float(rp.y);
         if (sc >= floor_sc && sc >= lo && rp.x != skip && !in_support(lam, n_sup, rp.x)) {
             const int slot = atomicAdd(&sh.n_cand, 1);
-            if (slot < kRescoreCap) sh.cand_idx[slot] = rp.x;
+            if (slot < kResolveCap) sh.cand_idx[slot] = rp.x;
         }
     }
     __syncthreads();
     const int n = sh.n_cand;
-    return n > kRescoreCap ? -1 : n;
+    return n > kResolveCap ? -1 : n;
 }
 
 // appends the columns `cols` that the list does not hold yet; n_s is the running length (shared memory)

@@ -137,3 +137,30 @@ def test_chunk_picks_among_near_tied_columns(sgc, dc, k, c, tied):  # noqa: F811
             assert np.array_equal(st.get("lamV"), ref.get("lamV")), trial
         m.close()
         ref.close()
+
+
+# lists a little longer than the Gram path takes, many rows of A and kept entries of nearly equal size: two columns of one block's
+# share come within the rescoring window, and more columns than 16 within the screening margin of a pick
+@pytest.mark.parametrize("drift", [3, 30])
+def test_near_equal_entries_on_a_list_of_some_hundred_columns(sgc, drift):  # noqa: F811
+    d, k, s = 65_600, 16_384, 250
+    hp = [inputs.ADAM[n] for n in ("lr", "beta1", "beta2", "eps")]
+    supp, sign = inputs.planted_support(d, s, 30 + drift)
+    supp, rng = supp.astype(np.int64), np.random.default_rng(drift)
+    st, twin = sgc.Sgc(d, k, s, 5, *hp), sgc.Sgc(d, k, s, 5, *hp)
+    twin.set_mode(sgc.MODE_LOCKSTEP)
+    w, wt = cuda(np.zeros(d, dtype=np.float32)), cuda(np.zeros(d, dtype=np.float32))
+    for step in range(10):
+        if 0 < step <= 4:
+            supp[rng.choice(s, drift, replace=False)] = np.setdiff1d(rng.integers(0, d, size=200), supp)[:drift]
+        g = (rng.standard_t(3.0, size=d) * 1e-3).astype(np.float32)
+        g[supp] = sign * (1.0 + 0.02 * rng.random(s)).astype(np.float32)
+        st.step(cuda(g), w)
+        twin.step(cuda(g), wt)
+        assert int(st.get("fallback")) == 0 and int(st.get("rounds")) >= 2, step
+        for name in ("lamM", "lamV"):
+            assert np.array_equal(st.get(name), twin.get(name)), (step, name)
+        assert np.array_equal(w.cpu().numpy(), wt.cpu().numpy())
+    assert 256 < int(st.get("n_cand")) < 768
+    st.close()
+    twin.close()
