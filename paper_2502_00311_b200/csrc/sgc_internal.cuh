@@ -192,7 +192,7 @@ struct SpecCtl {
     int hist_count, hist_next;  // ring of the kept index sets of the last steps: valid slots, slot of the next step
     int trace[kMaxRounds][3];   // per round: confirmed picks of both streams and the list length after it
     double ynorm[2];        // ||y|| per residual
-    int inexact_streak;     // speculating steps in a row that needed more than one confirming pass
+    int inexact_streak;     // speculating steps in a row that were refuted (more passes than s picks fill, or a refuted pick)
 };
 
 // device-resident counters of one state

@@ -610,10 +610,13 @@ __global__ void __launch_bounds__(kOmpThreads, 1) k_finish(FinishArgs f) {
     SpecCtl* ctl = a.ctl;
     // how many rounds this step took (the enqueued rounds if even they were not enough): sizes the next step's launches
     // bit 8: a list pass refuted a pick (the wide lists earned their keep); bit 9: a full pass refuted a pick; bits 10, 11: how
-    // many speculating steps in a row needed more than one confirming pass (at most 3)
+    // many speculating steps in a row were refuted, that is, needed more passes than the residuals of s picks fill (at most 3)
     if (t == 0 && f.speculate) {
-        const bool one = !ctl->fallback && ctl->rounds <= 1 && ctl->list_rounds == 0;
-        const int streak = one ? 0 : (ctl->inexact_streak < 3 ? ctl->inexact_streak + 1 : 3);
+        // (list passes that refute nothing count against a state of one pass alone: the next step then does without them)
+        const int fewest = (s + a.half_n - 1) / a.half_n;
+        const bool confirmed = !ctl->fallback && ctl->refuted == 0 && ctl->rounds <= fewest && ctl->list_refuted == 0 &&
+                               (fewest > 1 || ctl->list_rounds == 0);
+        const int streak = confirmed ? 0 : (ctl->inexact_streak < 3 ? ctl->inexact_streak + 1 : 3);
         ctl->inexact_streak = streak;
         *f.rounds_out = (ctl->fallback ? kMaxRounds : ctl->rounds) | (ctl->list_refuted > 0 ? 256 : 0) | (ctl->refuted > 0 ? 512 : 0) |
                         (streak << 10);
@@ -731,18 +734,22 @@ cudaError_t finish_recover_setup(sgc_state* st) {
 //                                                                                             (11 + k d / 2.8e6)
 //   refuted speculation:     d = 151700, k = 320, s = 37: 100;  117656, 832, 102: 81;  1876582, 960, 123: 168;  3001000, 700, 100: 270
 //                                                                                             (100 + k d / 2.0e7)
-//   confirmed speculation, us per step: d = 143488, k = 1600, s = 25: 370 (with the launches; 140 + 1.2 s + k d / 3.3e6)
+//   confirmed speculation, us per step: d = 143488, k = 1600, s = 25: 370 (with the launches; 140 + k d / 3.3e6 per pass, + 1.2 s)
 // A state that has come to prefer lock-step tries a speculating step now and then: its gradients may have changed.
 constexpr int kRetrySteps = 32;
 constexpr double kFewRoundsWork = 3.0e8;              // k * d up to which a pick in lock-step costs at most 120 us
 constexpr double kTwoLevelWork = 1.0e8;               // k * d from which list passes can be cheaper than full ones
+
+// passes over all columns that a step takes when nothing is refuted: a pass has room for pass_n / 2 residuals per recovery
+static int fewest_passes(const sgc_state* st) { return (st->s + st->pass_n / 2 - 1) / (st->pass_n / 2); }
 
 static bool prefers_speculation(const sgc_state* st) {
     const double kd = (double)st->k * (double)st->d, s = (double)st->s;
     const double lock = s * (11.0 + kd / 2.8e6);
     const int seen = *reinterpret_cast<volatile int*>(st->h_rounds);
     const bool refuted = (seen & 255) != 0 ? ((seen >> 10) & 3) >= 2 : (double)st->k < 1.2 * s * log((double)st->d);
-    const double spec = refuted ? s * (100.0 + kd / 2.0e7) : 140.0 + 1.2 * s + kd / 3.3e6;
+    const double passes = (double)fewest_passes(st);
+    const double spec = refuted ? s * (100.0 + kd / 2.0e7) : passes * (140.0 + kd / 3.3e6) + 1.2 * s;
     return spec < lock;
 }
 
@@ -811,8 +818,10 @@ static cudaError_t recover_batches(sgc_state* const* sts, float* const* weights,
         if (st->max_rounds > 0 && want > st->max_rounds) want = st->max_rounds;
         if (want > n_rounds) n_rounds = want;
         // two-level screening pays where steps need several full passes (recovery picks columns outside the kept sets);
-        // it is dropped again when a step needed one pass and its list passes refuted nothing
-        if (last >= 3 && (double)st->k * (double)st->d >= kTwoLevelWork) st->two_level = true;
+        // it is dropped again when a step needed one pass and its list passes refuted nothing.  Several passes that refute nothing
+        // because s picks do not fit one are no reason for it
+        const bool contested = (hint >> 10) != 0;
+        if (last >= 3 && contested && (double)st->k * (double)st->d >= kTwoLevelWork) st->two_level = true;
         else if (last == 1 && !(hint & 256)) st->two_level = false;
     }
     if (n_rounds > kMaxRounds) n_rounds = kMaxRounds;

@@ -164,3 +164,23 @@ def test_near_equal_entries_on_a_list_of_some_hundred_columns(sgc, drift):  # no
     assert 256 < int(st.get("n_cand")) < 768
     st.close()
     twin.close()
+
+
+# more picks than one pass has room for: two or three passes without a refuted pick are a confirmed step, and the state goes on
+# speculating
+@pytest.mark.parametrize("d,k,s,passes", [(131_072, 2048, 130, 2), (70_001, 4096, 260, 3)])
+def test_a_state_confirmed_in_several_passes_keeps_speculating(sgc, d, k, s, passes):  # noqa: F811
+    hp = [inputs.ADAM[n] for n in ("lr", "beta1", "beta2", "eps")]
+    supp, sign = inputs.planted_support(d, s, 3)
+    st, twin = sgc.Sgc(d, k, s, 5, *hp), sgc.Sgc(d, k, s, 5, *hp)
+    twin.set_mode(sgc.MODE_LOCKSTEP)
+    w, wt = cuda(np.zeros(d, dtype=np.float32)), cuda(np.zeros(d, dtype=np.float32))
+    for step in range(6):
+        g = cuda(inputs.gradient(d, "student", supp, sign, 100 + step))
+        st.step(g, w)
+        twin.step(g, wt)
+        assert (int(st.get("rounds")), int(st.get("fallback"))) == (passes, 0), step
+        assert np.array_equal(st.get("lamM"), twin.get("lamM")) and np.array_equal(st.get("lamV"), twin.get("lamV"))
+    assert np.array_equal(w.cpu().numpy(), wt.cpu().numpy())
+    st.close()
+    twin.close()
