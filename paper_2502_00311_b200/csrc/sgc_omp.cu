@@ -95,11 +95,12 @@ __device__ __forceinline__ bool in_support4(const uint32_t* sup, int n, uint32_t
     return hit;
 }
 
-// The threads of the block tell one another the second best score that each has seen: a column at or below any of these can be
-// neither the block's best nor its second best, so that after the first few columns hardly any gets further than one compare.
+// The threads of the block tell one another the second best score that each has seen: a column below any of these can be
+// neither the block's best nor its second best, so that after the first few columns hardly any gets further than one compare.  (One at
+// the bound goes on: of equal scores, those of a zero residual, the lowest column has to win.)
 // (A column of the support scores rounding noise: the look-up is needed only for what passes.)
 __device__ __forceinline__ void offer(OmpSmem& sh, Top& best, const int* picks, int m, float score, uint32_t col) {
-    if (!(score > best.s2) || score_key(score) <= *reinterpret_cast<volatile unsigned int*>(&sh.floor_key[m])) return;
+    if (!(score > best.s2) || score_key(score) < *reinterpret_cast<volatile unsigned int*>(&sh.floor_key[m])) return;
     if (in_support4(sh.sup[m], picks[m], col)) return;
     const float before = best.s2;
     best.push(score, col);

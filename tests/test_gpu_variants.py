@@ -184,3 +184,17 @@ def test_a_state_confirmed_in_several_passes_keeps_speculating(sgc, d, k, s, pas
     assert np.array_equal(w.cpu().numpy(), wt.cpu().numpy())
     st.close()
     twin.close()
+
+
+# a zero gradient leaves zero residuals: all scores are equal and the lowest free column is picked every time
+@pytest.mark.parametrize("d,k,s", [(4096, 256, 16), (16_384, 64, 16), (50_000, 16, 5), (300_000, 40, 6), (30_000, 128, 8)])
+def test_lockstep_on_a_zero_gradient(sgc, d, k, s):  # noqa: F811
+    st = sgc.Sgc(d, k, s, 5, *(inputs.ADAM[n] for n in ("lr", "beta1", "beta2", "eps")))
+    st.set_mode(sgc.MODE_LOCKSTEP)
+    g, w = cuda(np.zeros(d, dtype=np.float32)), cuda(np.ones(d, dtype=np.float32))
+    for _ in range(40):
+        st.step(g, w)
+        assert np.array_equal(st.get("lamM"), np.arange(s)) and np.array_equal(st.get("lamV"), np.arange(s))
+        assert int(st.get("doneM")) == s and int(st.get("n_upd")) == 0
+    assert bool((w == 1).all())
+    st.close()
