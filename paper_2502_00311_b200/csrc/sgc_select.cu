@@ -166,7 +166,7 @@ __device__ __forceinline__ unsigned int tau_below(const float* sel_val, unsigned
 // bound: HBM, 4 d bytes; eight vectors per thread in flight (180 MB: 31 us, then 12 us for k_unit_pick; the sampled threshold
 // that this replaces took 23 us to find before a 31 us filter).
 constexpr int kUnitLoads = 8;
-constexpr int kUnitPickThreads = 512;
+constexpr int kUnitPickThreads = 1024;
 constexpr int kHotUnits = 512;                       // units that one block can list for reading again
 
 __global__ void __launch_bounds__(512)
@@ -197,7 +197,7 @@ k_unit_max(const float* __restrict__ grad, unsigned long long d, int lanes, unsi
 }
 
 // same grid and block as k_unit_max (T and the units must agree); n_units <= kSelBins.  out_status may be null.
-__global__ void __launch_bounds__(kUnitPickThreads)
+__global__ void __launch_bounds__(kUnitPickThreads, 1)
 k_unit_pick(const float* __restrict__ grad, unsigned long long d, unsigned int s, int lanes, unsigned long long T, unsigned int n_units,
             unsigned int* __restrict__ unit_max, unsigned long long* __restrict__ cand, Counters* __restrict__ cnt,
             uint32_t* __restrict__ sel_idx, float* __restrict__ sel_val, int carry_out, uint32_t* __restrict__ out_status) {
@@ -235,7 +235,7 @@ k_unit_pick(const float* __restrict__ grad, unsigned long long d, unsigned int s
             for (int u = kPer - 1; u >= 0; --u) { above += hist[t * kPer + u]; if (above >= s) { tau_bin = t * kPer + u; break; } }
     }
     __syncthreads();
-    const unsigned int tau = tau_bin << 19;                              // (fewer than s units: 0, everything qualifies)
+    const unsigned int tau = tau_bin << 19;                              // (0: fewer than s units hold anything but zeros, the exact path serves)
     // this block's units whose maximum reaches the bound, read again by the whole block, one after the other
     const unsigned long long n4 = d >> 2;
     const float4* g4 = reinterpret_cast<const float4*>(grad);
@@ -245,7 +245,7 @@ k_unit_pick(const float* __restrict__ grad, unsigned long long d, unsigned int s
     __syncthreads();
     const unsigned int nh = min(n_hot, (unsigned int)kHotUnits);
     const int groups = kUnitPickThreads / lanes, grp = t / lanes, in = t % lanes;
-    for (unsigned int q = 0; q < nh; ++q) {
+    for (unsigned int q = 0; q < nh && tau != 0u; ++q) {
         const unsigned long long first = (unsigned long long)hot[q] * lanes + in;
 #pragma unroll 4
         for (unsigned long long i = first + (unsigned long long)grp * T; i < n4; i += (unsigned long long)groups * T) {
@@ -258,7 +258,7 @@ k_unit_pick(const float* __restrict__ grad, unsigned long long d, unsigned int s
         }
         if (hot[q] == 0u && (unsigned long long)t < (d & 3ull)) consider(grad[(n4 << 2) + t], (n4 << 2) + t, tau, cand, cnt);
     }
-    if (n_hot > (unsigned int)kHotUnits && t == 0) atomicAdd(&cnt->sel_count, (unsigned int)kSelCap + 1u);   // more than can be listed: the exact path serves
+    if ((n_hot > (unsigned int)kHotUnits || tau == 0u) && t == 0) atomicAdd(&cnt->sel_count, (unsigned int)kSelCap + 1u);   // more than can be listed: the exact path serves
     __threadfence();
     __syncthreads();
     if (t == 0) last = (atomicAdd(&cnt->sel_ticket, 1u) == gridDim.x - 1);
