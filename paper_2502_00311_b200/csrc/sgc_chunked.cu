@@ -162,6 +162,7 @@ k_chunk_front(ChunkArgs a, const float* __restrict__ grad, double b1, double b2,
     tau = __reduce_min_sync(0xffffffffu, tau);
     int* count = cluster.map_shared_rank(&n_list, 0);
     unsigned long long* dst = cluster.map_shared_rank(list, 0);
+    if (tau == 0u) tau = 1u;                                          // (fewer than s shares with a non-zero: zeros are added below)
     unsigned int redo = __ballot_sync(0xffffffffu, top >= tau);
     while (redo) {
         const int owner = __ffs(redo) - 1;
@@ -182,7 +183,14 @@ k_chunk_front(ChunkArgs a, const float* __restrict__ grad, double b1, double b2,
     }
     if (split > 1) { cluster.sync(); if (rank != 0) return; }          // (nobody reads this block's memory after this)
     __syncthreads();
-    const int n = n_list;
+    int n = n_list;
+    if (n < s) {
+        // fewer than s non-zeros: the first zeros of the chunk are kept as well, and those that are missing lie among its first
+        // s + n entries (a bound of zero let everything through: 1024 x 1024 zeros cost 160 us)
+        if (t < s + n && t < a.dc && (__float_as_uint(g[t]) & 0x7FFFFFFFu) == 0u) list[atomicAdd(&n_list, 1)] = front_key(0.0f, (uint32_t)t);
+        __syncthreads();
+        n = n_list;
+    }
     if (n <= kFrontRank) {
         // rank of every survivor among the others: the s largest
         if (t < n) {
@@ -407,7 +415,8 @@ __global__ void __launch_bounds__(corr_threads(KP)) k_chunk_corr(ChunkArgs a, in
     // Scores are compared as keys: the score's bits with the lowest ten replaced by a code of the column (relative error 2^-13, an
     // eighth of the window that k_chunk_pick rescores), so that the best two follow from three integer minima and maxima, without
     // a branch.  Columns of a recovery's support score rounding noise; should one be among the best two all the same (hardly any
-    // columns left, or a zero residual), the block goes through its columns again and leaves them out.
+    // columns left), the block goes through its columns again and leaves them out.  A zero residual scores zero everywhere: what it
+    // is handed does not matter.
     Best2 best[NT];
     bool exclude = false;
     for (;;) {
@@ -480,6 +489,7 @@ __global__ void __launch_bounds__(corr_threads(KP)) k_chunk_corr(ChunkArgs a, in
         bool taken = false;
 #pragma unroll
         for (int i = 0; i < NT; ++i) {
+            if (best[i].s1 == 0.0f) continue;                         // a zero residual: k_chunk_pick knows what to do
             if (NT <= 4) {
 #pragma unroll
                 for (int h = 0; h < kHeld; ++h)
@@ -670,25 +680,38 @@ __device__ void pick_finish(const ChunkArgs& a, const ChunkRef& ref, PickSmem& s
     if (t == 0) { ref.rnorm[(size_t)m * s + j] = rn; a.back[res] = (float)(1.0 / sc); }
 }
 
-// The columns col0 .. col1 of a split once more, whose third key came too close: every free column with score >= thr that the split
-// did not forward (f0, f1) joins the candidates (fp64, thread = column; once in some 10^5 picks of a noisy recovery).
-__device__ __noinline__ void pick_redo_split(PickSmem* sh, uint32_t seed_lo, uint32_t seed_hi, int k, const uint32_t* sup, int j,
-                                             uint32_t col0, uint32_t col1, uint32_t f0, uint32_t f1, double thr) {
-    const double* r = pick_mem();
-    for (uint32_t col = col0 + threadIdx.x; col < col1; col += blockDim.x) {
-        const ColKey key = column_key(seed_lo, seed_hi, col);
-        double dot = 0.0, n2 = 0.0;
-        for (int row = 0; row < k; row += 2) {
-            const float2 z = half2_bits_to_float2(z_pair_from_word(key.ck + (uint32_t)(row >> 1) * key.mk));
-            dot = fma((double)z.x, r[row], dot); n2 = fma((double)z.x, (double)z.x, n2);
-            if (row + 1 < k) { dot = fma((double)z.y, r[row + 1], dot); n2 = fma((double)z.y, (double)z.y, n2); }
+// What hardly any pick needs, out of the way of the others.  thr = 0: a zero residual; all scores are equal, and the lowest free
+// column it is (one of the first j + 1).  Otherwise: the columns of the splits in sh->redo once more, whose third key came too close;
+// every free column with score >= thr that its split did not forward joins the candidates (fp64, thread = column; once in some 10^5
+// picks of a noisy recovery).
+__device__ __noinline__ void pick_rare(PickSmem* sh, const Cand* fwd, uint32_t seed_lo, uint32_t seed_hi, int k, uint32_t dc,
+                                       uint32_t cols_per_split, const uint32_t* sup, int j, double thr) {
+    auto taken = [&](uint32_t col) { bool v = false; for (int l = 0; l < j; ++l) v = v || sup[l] == col; return v; };
+    if (thr == 0.0) {
+        if (threadIdx.x < 32) {
+            const unsigned int who = __ballot_sync(0xffffffffu, (int)threadIdx.x <= j && threadIdx.x < dc && !taken(threadIdx.x));
+            if (threadIdx.x == 0 && who != 0u) { sh->cidx[0] = (uint32_t)(__ffs(who) - 1); sh->n_c = 1; }
         }
-        if (!(n2 > 0.0) || fabs(dot) < thr * sqrt(n2) || col == f0 || col == f1) continue;
-        bool taken = false;
-        for (int l = 0; l < j; ++l) taken = taken || sup[l] == col;
-        if (taken) continue;
-        const int slot = atomicAdd(&sh->n_c, 1);
-        if (slot < kRescoreCap) sh->cidx[slot] = col;
+        __syncthreads();
+        return;
+    }
+    const double* r = pick_mem();
+    const int n_redo = sh->n_redo < 8 ? sh->n_redo : 8;              // (more than eight such splits hold more than kRescoreCap candidates by themselves)
+    for (int q = 0; q < n_redo; ++q) {
+        const uint32_t split = (uint32_t)sh->redo[q], f0 = fwd[2 * split].idx & ~kThirdMark, f1 = fwd[2 * split + 1].idx;
+        const uint32_t col0 = split * cols_per_split, col1 = dc - col0 < cols_per_split ? dc : col0 + cols_per_split;
+        for (uint32_t col = col0 + threadIdx.x; col < col1; col += blockDim.x) {
+            const ColKey key = column_key(seed_lo, seed_hi, col);
+            double dot = 0.0, n2 = 0.0;
+            for (int row = 0; row < k; row += 2) {
+                const float2 z = half2_bits_to_float2(z_pair_from_word(key.ck + (uint32_t)(row >> 1) * key.mk));
+                dot = fma((double)z.x, r[row], dot); n2 = fma((double)z.x, (double)z.x, n2);
+                if (row + 1 < k) { dot = fma((double)z.y, r[row + 1], dot); n2 = fma((double)z.y, (double)z.y, n2); }
+            }
+            if (!(n2 > 0.0) || fabs(dot) < thr * sqrt(n2) || col == f0 || col == f1 || taken(col)) continue;
+            const int slot = atomicAdd(&sh->n_c, 1);
+            if (slot < kRescoreCap) sh->cidx[slot] = col;
+        }
     }
     __syncthreads();
 }
@@ -696,7 +719,7 @@ __device__ __noinline__ void pick_redo_split(PickSmem* sh, uint32_t seed_lo, uin
 // SIMT route: the candidates are the columns that phase A left within 2e-3 (relative) of the best fp32 score.
 // only != nullptr: a second chance for the recoveries that the tensor-core route marked unresolved; skipped unless *gate
 // names this iteration.
-__global__ void __launch_bounds__(kPickMaxThreads) k_chunk_pick(ChunkArgs a, int iter, const int* gate, const unsigned char* only) {
+__global__ void __launch_bounds__(kPickMaxThreads, 4) k_chunk_pick(ChunkArgs a, int iter, const int* gate, const unsigned char* only) {
     __shared__ PickSmem sh;
     const int res = blockIdx.x, m = res & 1, t = threadIdx.x, j = iter;
     const ChunkRef ref = a.table[res >> 1];
@@ -724,10 +747,10 @@ __global__ void __launch_bounds__(kPickMaxThreads) k_chunk_pick(ChunkArgs a, int
     mx = pick_max(sh, mx);                                          // (its barriers also publish n_c = 0)
     const float thr = mx - 2e-3f * fabsf(mx);
     auto offer = [&](const Cand& c, int e) {
-        if (c.idx != kNoColumn && c.score >= 0.0f && c.score >= thr) {
+        if (c.idx != kNoColumn && c.score >= thr && c.score > 0.0f) {
             const int slot = atomicAdd(&sh.n_c, 1);
             if (slot < kRescoreCap) sh.cidx[slot] = c.idx & ~kThirdMark;
-            if ((c.idx & kThirdMark) && c.score >= mx * (1.0f - kKeyWindow) && mx > 0.0f) {
+            if ((c.idx & kThirdMark) && c.score >= mx * (1.0f - kKeyWindow)) {
                 const int q = atomicAdd(&sh.n_redo, 1);
                 if (q < 8) sh.redo[q] = e >> 1;
             }
@@ -736,16 +759,8 @@ __global__ void __launch_bounds__(kPickMaxThreads) k_chunk_pick(ChunkArgs a, int
     offer(first[0], t); offer(first[1], t + (int)blockDim.x);
     for (int e = t + 2 * (int)blockDim.x; e < n_entries; e += blockDim.x) offer(cc[e], e);
     __syncthreads();
-    if (sh.n_redo > 0) {
-        // (more than eight such splits hold more than kRescoreCap candidates by themselves)
-        const int n_redo = sh.n_redo < 8 ? sh.n_redo : 8;
-        for (int q = 0; q < n_redo; ++q) {
-            const Cand* fwd = cc + 2 * sh.redo[q];
-            const long long col0 = (long long)sh.redo[q] * a.cols_per_split, col1 = col0 + a.cols_per_split;
-            pick_redo_split(&sh, a.seed_lo, a.seed_hi, a.k, a.lam + (size_t)res * a.s, j, (uint32_t)col0, (uint32_t)(col1 < a.dc ? col1 : a.dc),
-                            fwd[0].idx & ~kThirdMark, fwd[1].idx, (double)thr);
-        }
-    }
+    if (sh.n_redo > 0 || mx == 0.0f)
+        pick_rare(&sh, cc, a.seed_lo, a.seed_hi, a.k, (uint32_t)a.dc, (uint32_t)a.cols_per_split, a.lam + (size_t)res * a.s, j, (double)thr);
     int nc = sh.n_c;
     if (nc > kRescoreCap) {
         if (t == 0) atomicOr(&ref.cnt->status, (unsigned int)SGC_STATUS_CANDIDATE_OVERFLOW);

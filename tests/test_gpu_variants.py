@@ -198,3 +198,33 @@ def test_lockstep_on_a_zero_gradient(sgc, d, k, s):  # noqa: F811
         assert int(st.get("doneM")) == s and int(st.get("n_upd")) == 0
     assert bool((w == 1).all())
     st.close()
+
+
+# chunks without a gradient beside ordinary ones, and chunks with fewer non-zeros than are kept: the first zeros fill up, and a zero
+# residual takes the lowest free columns
+@pytest.mark.parametrize("c,dc,k,s", [(5, 4096, 16, 2), (3, 40_000, 112, 16), (40, 2048, 217, 31), (2, 1 << 17, 8, 1), (6, 32, 40, 31)])
+def test_chunks_of_zeros(sgc, c, dc, k, s):  # noqa: F811
+    hp = [inputs.ADAM[n] for n in ("lr", "beta1", "beta2", "eps")]
+    m = sgc.Mesgc(c * dc, c, k, s, 8, *hp)
+    refs = [oracle.Oracle(dc, k, s, 8, *hp) for _ in range(c)]
+    w, wr = cuda(np.zeros(c * dc, dtype=np.float32)), np.zeros((c, dc), dtype=np.float32)
+    rng = np.random.default_rng(c)
+    for step in range(2):
+        g = rng.standard_t(3.0, size=(c, dc)).astype(np.float32)
+        g[0] = 0.0
+        g[1] = 0.0
+        g[1, rng.choice(dc, s // 2, replace=False)] = 1.0 + rng.random(s // 2).astype(np.float32)
+        m.step(cuda(g.reshape(-1)), w)
+        for i, (st, ref) in enumerate(zip(m.chunks, refs)):
+            idx, val = oracle.sparsify(g[i], s)
+            assert np.array_equal(st.get("sel_idx"), idx) and np.array_equal(st.get("sel_val"), val), (step, i)
+            if i > 3:
+                continue
+            ref.step(g[i], wr[i])
+            if i != 1:                                                    # (past the non-zeros its residual is rounding noise)
+                for name in ("lamM", "lamV", "doneM", "doneV"):
+                    assert np.array_equal(st.get(name), ref.get(name)), (step, i, name)
+            assert not int(st.get("status")) & sgc.STATUS_CANDIDATE_OVERFLOW or i == 1
+        got = w.cpu().numpy().reshape(c, dc)
+        assert not got[0].any() and parity.rel(got[:min(c, 4)], wr[:min(c, 4)]) < 1e-4
+    m.close()
