@@ -189,7 +189,8 @@ SGC_API int sgc_reproject(sgc_state* st, uint64_t new_seed, void* stream);
  * SGC_ERR_DIM when SGC_MODE_SPECULATIVE is requested and k is not a multiple of 64.  States with d < 65536 never
  * speculate on their own accord and are created without the buffers of that strategy (some 50 MB plus 6.5 bytes per
  * column), and so are those whose k is no multiple of 64: with d >= 65536 these allocate them at their first sgc_step or
- * sgc_step_group that is not being captured (lock-step when the allocation fails); asking for SGC_MODE_SPECULATIVE allocates them here (one cudaMalloc, synchronises; a CUDA error code if it fails). */
+ * sgc_step_group that would speculate and is not being captured, from the device's memory pool in the order of the step's
+ * stream, without synchronising (lock-step when the allocation fails); asking for SGC_MODE_SPECULATIVE allocates them here (one cudaMalloc, synchronises; a CUDA error code if it fails). */
 SGC_API int sgc_set_mode(sgc_state* st, int32_t mode);
 
 /* Opt-in variant of the recovery, built on the remark after Eq. (8) that OMP_A(M_t) and OMP_A(V_t) have their

@@ -92,18 +92,32 @@ size_t layout_spec(sgc_state* st, unsigned char* base) {
 
 bool finite_f(float v) { return isfinite(v); }
 
-cudaError_t ensure_spec(sgc_state* st) {
+// gives the buffers of the speculative recovery back to where they came from (pooled ones once `stream` has come this far)
+void free_spec(sgc_state* st, cudaStream_t stream) {
+    if (!st->spec_base) return;
+    if (st->spec_pooled) { cudaFreeAsync(st->spec_base, stream); cudaStreamSynchronize(stream); }
+    else cudaFree(st->spec_base);
+    st->spec_base = nullptr;
+}
+
+// The buffers of the speculative recovery.  At creation and at sgc_set_mode (stream == nullptr): cudaMalloc, done when the call
+// returns.  Inside a step: everything in the order of the caller's stream, from the device's memory pool, so that the step neither
+// synchronises nor disturbs a capture on another stream (a cudaMalloc would end that).
+cudaError_t ensure_spec(sgc_state* st, const cudaStream_t* stream) {
     if (st->spec_ready) return cudaSuccess;
     {
         sgc_state probe = *st;                                       // measuring must not leave pointers behind
         st->spec_bytes = layout_spec(&probe, nullptr);
     }
-    cudaError_t e = cudaMalloc(&st->spec_base, st->spec_bytes);
+    const cudaStream_t cs = stream ? *stream : 0;
+    cudaError_t e = stream ? cudaMallocAsync(&st->spec_base, st->spec_bytes, cs) : cudaMalloc(&st->spec_base, st->spec_bytes);
     if (e != cudaSuccess) { st->spec_base = nullptr; return e; }
+    st->spec_pooled = stream != nullptr;
     layout_spec(st, static_cast<unsigned char*>(st->spec_base));
-    e = cudaMemset(st->spec_base, 0, st->spec_bytes);             // empty candidate list, bitmaps, wide lists
-    if (e == cudaSuccess) e = sgc::finish_recover_setup(st);      // tensor maps of R^T, column norms (synchronises)
-    if (e != cudaSuccess) { cudaFree(st->spec_base); st->spec_base = nullptr; return e; }
+    e = cudaMemsetAsync(st->spec_base, 0, st->spec_bytes, cs);    // empty candidate list, bitmaps, wide lists
+    if (e == cudaSuccess) e = sgc::finish_recover_setup(st, cs);  // tensor maps of R^T, column norms
+    if (e == cudaSuccess && !stream) e = cudaDeviceSynchronize();
+    if (e != cudaSuccess) { free_spec(st, cs); return e; }
     st->spec_ready = true;
     return cudaSuccess;
 }
@@ -115,7 +129,12 @@ void prepare_spec(sgc_state* st, cudaStream_t stream) {
     if (st->spec_ready || st->spec_refused || !sgc::will_speculate(st)) return;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) { cudaGetLastError(); return; }
-    if (ensure_spec(st) != cudaSuccess) { st->spec_refused = true; cudaGetLastError(); }
+    // an allocation counts as unsafe while any stream is captured in the global mode, in whichever order it is made; this one touches
+    // nothing that a capture could record
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) { cudaGetLastError(); return; }
+    if (ensure_spec(st, &stream) != cudaSuccess) { st->spec_refused = true; cudaGetLastError(); }
+    cudaThreadExchangeStreamCaptureMode(&mode);
 }
 
 }  // namespace
@@ -153,7 +172,7 @@ SGC_API int sgc_create(sgc_state** out, int64_t d, int32_t k, int32_t s, uint64_
     }
     // SGC_MODE_AUTO speculates from d = 65536 on.  States whose k is no multiple of 64 are mostly chunks of MESGC, which do not
     // need these buffers: they get them at their first sgc_step instead.
-    if (e == cudaSuccess && st->d >= sgc::kSpecMinD && st->k % 64 == 0) e = ensure_spec(st);
+    if (e == cudaSuccess && st->d >= sgc::kSpecMinD && st->k % 64 == 0) e = ensure_spec(st, nullptr);
     if (e == cudaSuccess) {
         e = cudaHostAlloc(reinterpret_cast<void**>(&st->h_rounds), sizeof(int), cudaHostAllocMapped);
         if (e == cudaSuccess) { st->h_rounds[0] = 0; e = cudaHostGetDevicePointer(reinterpret_cast<void**>(&st->d_rounds), st->h_rounds, 0); }
@@ -284,7 +303,7 @@ SGC_API int sgc_destroy(sgc_state* st) {
     cudaError_t e = cudaSuccess;
     if (st->has_stream) e = cudaStreamSynchronize(st->last_stream);
     sgc::free_chunk_ws(st);
-    if (st->spec_base) cudaFree(st->spec_base);
+    free_spec(st, st->has_stream ? st->last_stream : 0);
     cudaError_t e2 = cudaFree(st->base);
     if (st->h_rounds) cudaFreeHost(st->h_rounds);
     for (cudaEvent_t ev : *st->ev_pool) cudaEventDestroy(ev);
@@ -316,7 +335,7 @@ SGC_API int sgc_set_mode(sgc_state* st, int32_t mode) {
     if (mode < SGC_MODE_AUTO || mode > SGC_MODE_SPECULATIVE) return SGC_ERR_WHAT;
     if (mode == SGC_MODE_SPECULATIVE && st->k % 64 != 0) return SGC_ERR_DIM;
     if (mode == SGC_MODE_SPECULATIVE) {
-        const cudaError_t e = ensure_spec(st);                       // small states get their speculative buffers here
+        const cudaError_t e = ensure_spec(st, nullptr);              // small states get their speculative buffers here
         if (e != cudaSuccess) return (int)e;
     }
     st->mode = mode;

@@ -256,6 +256,7 @@ struct sgc_state {
     int mode;                   // 0 auto, 1 lock-step only, 2 speculative whenever k allows it
     int shared_support;         // 1: OMP(M^) alone selects, V^ is fitted on its support (sgc_set_recovery)
     double residual_tol;        // > 0: recoveries are cut at the first pick that leaves ||r|| <= residual_tol ||y||
+    bool spec_pooled;           // they came from the device's memory pool (allocated in the order of a stream)
     bool spec_refused;          // its buffers could not be allocated at a step
     bool spec_ready;            // its buffers exist (second allocation: at creation for d >= 65536, else at sgc_set_mode)
     void* spec_base; size_t spec_bytes;
@@ -363,7 +364,7 @@ cudaError_t launch_cesgc_project(const float* B, const float* G, float* P, int r
 cudaError_t launch_cesgc_back(const float* B, const float* U, float* W, int r, int m, int n, cudaStream_t stream);
 double normal_tail_threshold(double d, double target);   // z with d * P(|N(0,1)| > z) = target
 cudaError_t configure_recover(sgc_state* st);   // occupancy / shared-memory set-up at create time
-cudaError_t finish_recover_setup(sgc_state* st); // after the workspace exists: tensor map of R^T
+cudaError_t finish_recover_setup(sgc_state* st, cudaStream_t stream); // after the workspace exists: tensor map of R^T, column norms
 
 // wide lists of the two-level screening (sgc_pass.cu): a full pass fills them, a list pass screens only their columns
 struct PassWide {

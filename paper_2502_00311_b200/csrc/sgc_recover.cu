@@ -712,16 +712,14 @@ cudaError_t configure_recover(sgc_state* st) {
     return cudaSuccess;
 }
 
-cudaError_t finish_recover_setup(sgc_state* st) {
+cudaError_t finish_recover_setup(sgc_state* st, cudaStream_t stream) {
     cudaError_t e = pass_configure(kPassMaxN);
     for (int g = 1; g <= kPassMaxN / st->pass_n && e == cudaSuccess; ++g)      // one map per number of states in a batch
         e = pass_encode_map(st->tmap[g - 1], st->rt, g * st->pass_n, st->kp);
     if (e != cudaSuccess) return e;
     e = pass_encode_map(st->tmap_half, st->rt, st->pass_n_half, st->kp);
     if (e != cudaSuccess) return e;
-    e = launch_inv_norms(st->seed, (uint64_t)st->d, st->k, st->inv_norm, 0);     // column norms: a property of (seed, k)
-    if (e != cudaSuccess) return e;
-    return cudaDeviceSynchronize();
+    return launch_inv_norms(st->seed, (uint64_t)st->d, st->k, st->inv_norm, stream);     // column norms: a property of (seed, k)
 }
 
 // Whether the next step of a state speculates.  Requested modes are obeyed.  SGC_MODE_AUTO compares estimates (us, from the

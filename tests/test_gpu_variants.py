@@ -228,3 +228,29 @@ def test_chunks_of_zeros(sgc, c, dc, k, s):  # noqa: F811
         got = w.cpu().numpy().reshape(c, dc)
         assert not got[0].any() and parity.rel(got[:min(c, 4)], wr[:min(c, 4)]) < 1e-4
     m.close()
+
+
+def test_the_first_speculating_step_leaves_another_streams_capture_alone(sgc):  # noqa: F811
+    # k no multiple of 64: the buffers of the speculation are allocated inside that step
+    import torch
+    d, k, s = 70_000, 333, 10
+    hp = [inputs.ADAM[n] for n in ("lr", "beta1", "beta2", "eps")]
+    supp, sign = inputs.planted_support(d, s, 3)
+    g, w = cuda(inputs.gradient(d, "student", supp, sign, 1)), cuda(np.zeros(d, dtype=np.float32))
+    warm = sgc.Sgc(d, k, s, 5, *hp)                                       # (a kernel's first launch loads it, which no capture survives)
+    warm.step(g, w.clone())
+    warm.close()
+    st, x, side, graph = sgc.Sgc(d, k, s, 5, *hp), cuda(np.ones(4, dtype=np.float32)), torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, capture_error_mode="global"):
+        x.mul_(2.0)
+        st.step(g, w, stream=side)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert x.tolist() == [2.0] * 4
+    assert int(st.get("rounds")) >= 1 and int(st.get("fallback")) == 0
+    ref = oracle.Oracle(d, k, s, 5, *hp)
+    ref.step(inputs.gradient(d, "student", supp, sign, 1), np.zeros(d, dtype=np.float32))
+    assert np.array_equal(st.get("lamM"), ref.get("lamM")) and np.array_equal(st.get("lamV"), ref.get("lamV"))
+    graph.reset()
+    st.close()
