@@ -250,7 +250,7 @@ struct sgc_state {
     cudaStream_t last_stream; bool has_stream;
     int32_t last_launches; bool stepped;
     bool sel_warm;              // a top-s threshold from the previous step is on the device (one-kernel selection)
-    int omp_grid2, omp_grid8;   // blocks of the recovery kernel in clusters of 2 and of 8
+    int omp_grid2, omp_grid8;   // blocks of the recovery kernel in clusters of 2 and of 8 (0: the device holds fewer than three)
     int omp_one;                // 1: a cluster of 16 can be resident
     int kp;                     // k rounded up to a multiple of 64: row stride of rt and zlist
     int mode;                   // 0 auto, 1 lock-step only, 2 speculative whenever k allows it

@@ -1497,13 +1497,12 @@ cudaError_t omp_configure(sgc_state* st) {
     const int n16 = r.n16;
     if (2 * n2 > kCorrBlocks) n2 = kCorrBlocks / 2;
     if (8 * n8 > kCorrBlocks) n8 = kCorrBlocks / 8;
-    st->omp_grid2 = 2 * n2; st->omp_grid8 = 8 * n8; st->omp_one = n16 >= 1 ? 1 : 0;
-    if (n8 < 3 || n2 < 2) return cudaErrorInvalidConfiguration;
-    return cudaSuccess;
+    st->omp_grid2 = 2 * n2; st->omp_grid8 = n8 >= 3 ? 8 * n8 : 0; st->omp_one = n16 >= 1 ? 1 : 0;
+    return n2 >= 3 ? cudaSuccess : cudaErrorInvalidConfiguration;
 }
 
 cudaError_t launch_omp(sgc_state* st, const OmpArgs& a, int mode, cudaStream_t stream) {
-    switch (omp_shape(st->d, a.k, a.s, mode, st->omp_one != 0)) {
+    switch (omp_shape(st->d, a.k, a.s, mode, st->omp_one != 0, st->omp_grid8 != 0)) {
         case 16: return omp_launch<16>(a, mode, 16, stream);
         case 2: return omp_launch<2>(a, mode, st->omp_grid2, stream);
         default: return omp_launch<8>(a, mode, st->omp_grid8, stream);

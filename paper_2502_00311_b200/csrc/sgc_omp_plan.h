@@ -93,20 +93,21 @@ SGC_HD inline CorrPlan corr_plan(uint32_t n, int k, int z_words, int blk, int nb
     return c;
 }
 
-// Which cluster shape (16, 2 or 8; one: a cluster of 16 can be resident): the one-cluster form while a pick's correlation takes
+// Which cluster shape (16, 2 or 8; one: a cluster of 16 can be resident; groups: the device holds three clusters of 8 at a time, two
+// for the books and one that correlates; a small partition of a GPU does not, and pairs serve everything there): the one-cluster form while a pick's correlation takes
 // 16 SMs no longer than the grid barriers cost the others; pairs (all 148 SMs correlate, two blocks keep each recovery's books)
 // when the correlation of a pick (k d) dwarfs its bookkeeping (k s), whatever k is; groups of 8 (120 SMs, the most that
 // clusters of 8 can occupy) otherwise and for lists.  The first two only where their buffers fit: with k in the ten thousands and a
 // handful of columns the one cluster has no room for the books beside the operands, with many rows and picks the pairs have none.
 // Step in groups of 8 / in pairs, us: d = 500000, k = 210, s = 30: 2187 / 1832; 65000, 350, 50: 1312 / 1126; 10000, 200, 8:
 // 143 / 136;  60000, 512, 64 (940 columns per pick): 1692 / 1694;  60000, 1024, 64: 2359 / 2521;  25000, 1400, 200: 7708 / 13020.
-inline int omp_shape(long long d, int k, int s, int mode, bool one) {
+inline int omp_shape(long long d, int k, int s, int mode, bool one, bool groups) {
     if (mode == 1) {
         if (one && (double)k * (double)d <= kOmpOneWork && omp_budget(16, k, s, mode).fits) return 16;
         const OmpBudget pair = omp_budget(2, k, s, mode);
         if (pair.fits && pair.book_correlates && (double)d >= kOmpPairCols * s) return 2;
     }
-    return 8;
+    return groups ? 8 : 2;
 }
 
 }  // namespace sgc

@@ -36,10 +36,10 @@ extern "C" int sweep_budget(int k0, int k1, long long* out) {
             for (long long d : ds) {
                 if (d < s || d < 1) continue;
                 for (int mode = 0; mode < 2; ++mode)
-                    for (int one = 0; one < 2; ++one) {
-                        const int cl = omp_shape(d, k, s, mode, one != 0);
+                    for (int device = 0; device < 3; ++device) {      // a whole GPU, one without clusters of 16, one with few of 8
+                        const int cl = omp_shape(d, k, s, mode, device == 0, device < 2);
                         const OmpBudget b = omp_budget(cl, k, s, mode);
-                        if (b.fits && inside(cl, k, s, b)) continue;
+                        if (b.fits && inside(cl, k, s, b) && (device < 2 || cl == 2)) continue;
                         out[0] = k; out[1] = s; out[2] = d;
                         return 1;
                     }
@@ -59,7 +59,7 @@ extern "C" int shares(unsigned n, int k, int nblk) {
     }
     return at == n;
 }
-extern "C" int shape(long long d, int k, int s, int mode, int one) { return omp_shape(d, k, s, mode, one != 0); }
+extern "C" int shape(long long d, int k, int s, int mode, int one) { return omp_shape(d, k, s, mode, one != 0, true); }
 """
 
 
