@@ -65,7 +65,7 @@ enum {
     SGC_STATUS_CANDIDATE_OVERFLOW = 1u << 4, /* a bounded candidate buffer overflowed.  In the speculative recovery the
                                                 step then fell back to its slower exact path (result unaffected).  In the
                                                 lock-step recovery more than 16 columns came within 2e-3 of the best fp32
-                                                score of one pick (a block that keeps such a column beyond the two it
+                                                score of one pick (a block that keeps such a column beyond the one it
                                                 forwards has its range screened again, so up to 16 always reach the fp64
                                                 decision): the pick may then differ from the exact argmax by a near-tie */
     SGC_STATUS_SELECT_FALLBACK = 1u << 5,  /* the bound on the kept magnitudes missed; exact fallback ran */
@@ -108,7 +108,8 @@ enum {
 
 /* How the recovery (a4) finds the picks of Algorithm 3; the picks themselves do not depend on it. */
 enum {
-    SGC_MODE_AUTO = 0,        /* speculative when d >= 65536, lock-step otherwise                           */
+    SGC_MODE_AUTO = 0,        /* from d = 65536 on whichever is estimated to be quicker, by d, k, s and what the
+                                 last steps needed; lock-step below                                          */
     SGC_MODE_LOCKSTEP = 1,    /* one pass over all d columns per OMP iteration                             */
     SGC_MODE_SPECULATIVE = 2  /* OMP on a candidate list, confirmed by batched tensor-core screening passes */
 };
@@ -263,7 +264,7 @@ SGC_API int sgc_sparsify_static(const float* grad, int64_t d, int32_t s, uint32_
 /* Per-kernel timing of the steps that follow (no counterpart in the paper: measurement support).
  * While enabled, sgc_step brackets every kernel launch with CUDA events on the caller's stream;
  * sgc_get_profile synchronises and returns the totals accumulated since sgc_set_profile(st, 1):
- *   ms[0] top-s sample    ms[1] top-s filter (the pass over the gradient)   ms[2] top-s pick
+ *   ms[0] unused          ms[1] top-s, the pass over the gradient           ms[2] top-s pick
  *   ms[3] projection+Adam ms[4] OMP kernels (candidate-list and lock-step)   ms[5] resolve + bookkeeping
  *   ms[6] combine+scatter ms[7] tensor-core screening passes
  *   launches[i] = number of kernel launches behind ms[i].   Both are host arrays of 8 entries. */

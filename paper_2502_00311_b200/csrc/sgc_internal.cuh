@@ -100,7 +100,7 @@ __device__ __forceinline__ float z_at(const ColKey& key, uint32_t row) { return 
 // ------------------------------------------------------------------------------------------------
 // limits
 // ------------------------------------------------------------------------------------------------
-constexpr int kMaxK = 16384;           // rows of A of a state: the lock-step kernel keeps both residuals (8 bytes per row) in shared memory
+constexpr int kMaxK = 16384;           // rows of A of a state: the recovery kernel keeps both residuals (8 bytes per row) in shared memory
 constexpr int kPassMaxK = 65536;       // rows of A of the stand-alone screening pass (sgc_screen)
 constexpr int kMaxS = 1024;
 constexpr int kSelCap = 32768;          // candidate slots of the top-s filter
@@ -115,14 +115,14 @@ constexpr int kLookAhead = 12;          // after a refuted pick, every kLookAhea
 constexpr double kLookAheadShare = 0.78; // ... as far as its columns reach this share of the residual's pick score
 constexpr int kWideCap = 2097152;       // columns per wide list (two-level screening)
 constexpr int kResolveBlocks = 16;        // blocks of the resolve kernel: all sweep the report lists, the last to finish walks the picks
-constexpr int kPassFastRows = 128;      // a pass over up to this many residual rows costs half of a wider one (A is generated once either way)
+constexpr int kPassFastRows = 128;      // a pass over up to this many residual rows costs 10.2 ms at d = 2^24, k = 2048, one over 256 rows 14.1 (A is generated once either way)
 constexpr int kMiniRounds = 8;          // list passes between two full passes, at most
 // Picks speculated ahead of one list pass; half as many with few rows of A, where a pick changes the residual more and a list pass
 // costs less beside the picks that a refuted one throws away (ms per step at depth 32 / 16: d = 3 M, k = 700, s = 100: 19.7 / 17.2;
 // four states of 1.7 M, k = 448: 37.7 / 31.5; 16.8 M, k = 1024: 86.7 / 85.5; three of 1.5 M, k = 1216: 54.4 / 59.8; 45 M, k = 2048: 118 / 122).
 constexpr int kMiniDepth = 32;
 constexpr int kMiniShallowK = 1024;
-constexpr int kGramList = 256;          // lists up to this length run OMP on their Gram matrix (Algorithm 3 as printed)
+constexpr int kGramList = 256;          // lists up to this length run OMP on their Gram matrix
 constexpr int kRepCap = 8192;           // report slots per residual of one screening pass
 constexpr int kPassMaxN = 256;          // residuals per screening pass (UMMA N)
 constexpr int kPassMaxBatch = 8;        // states whose residuals one screening pass can serve (kPassMaxN / 32)

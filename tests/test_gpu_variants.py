@@ -42,7 +42,7 @@ def test_selection_after_the_scale_of_the_gradient_jumps(sgc):  # noqa: F811
     st.close()
 
 
-# lock-step: one cluster up to k d = 1.2e6, groups of eight blocks, pairs from 2e8 on; fewer columns than blocks, odd k, many rows
+# lock-step: one cluster up to k d = 1.2e6, groups of eight blocks, pairs from d = 1000 s on; fewer columns than blocks, odd k, many rows
 @pytest.mark.parametrize("d,k,s", [(37, 5, 1), (4800, 250, 9), (4801, 250, 9), (700, 257, 130), (1001, 1199, 3), (66_000, 3100, 4),
                                    (1_000_003, 201, 6), (30_000, 7001, 3)])
 def test_lockstep_cluster_shapes(sgc, d, k, s):  # noqa: F811
