@@ -375,6 +375,9 @@ __global__ void __launch_bounds__(kCT, 1) k_chunk_cluster(const __grid_constant_
         const int n_own = rank < n_rec ? ((n_rec - 1 - rank) >> p.cl_log) + 1 : 0;
         const uint32_t res_bytes = (uint32_t)(n_rec * p.kb * 64), cand_bytes = (uint32_t)(n_own * p.cl * 16);
         if (t == 0) mbar_arrive_expect_tx(bar_res, res_bytes);
+        // (the last pick of a batch sends nothing that anybody waits for: a team's last warp may still be writing its records, for which it
+        // reads the books that are set up anew here, and a recovery that has just ended may still have to say so)
+        if (c0 > first) __syncthreads();
         for (int own = tm.id; own < n_own; own += teams) {
             const int rec = own * p.cl + rank, m = rec & 1;
             const ChunkRef& ref = chunk_ref(a, c0 + (rec >> 1));

@@ -161,11 +161,16 @@ inline GridPlan grid_plan(int c, long long dc, int k, int sms) {
 // the pass over 256 residuals takes most): us per step.
 inline bool chunk_on_tensor_cores(int c, long long dc, int kp) { return kp >= 64 && 2 * c <= 2048 && (double)dc * kp * 2.0 * c >= 1.0e9; }
 inline int chunk_passes(int c) { return ((2 * c + 31) / 32 * 32 + 255) / 256; }
-inline double chunk_general_us(int c, long long dc, int k, int kp, int s, int sms) {
+inline int chunk_padded_k(int k) { return k <= 8 ? 8 : k <= 16 ? 16 : k <= 32 ? 32 : k <= 64 ? 64 : k <= 128 ? 128 : 256; }
+inline double chunk_general_us(int c, long long dc, int k, int s, int sms) {
+    const int kp = chunk_padded_k(k);
     if (chunk_on_tensor_cores(c, dc, kp)) return s * (22.0 + 16.0 * chunk_passes(c));
     const double units = (double)((dc + 15) / 16) * ((2 * c + 3) / 4) / sms;
     const double books = 1.2 * s * k * ((2 * c + sms - 1) / sms);      // (cycles, for the recoveries of one SM)
     return s * (11.0 + (books + units * (7.9 + 3.8 * ((k + 15) / 16))) / 1.9e3);
 }
+// The cluster form is taken where its estimate beats that one by a tenth.  (The general form of a single vector is the lock-step recovery of
+// a whole matrix: it is taken for one wherever it fits.)
+inline bool cluster_form_taken(const ChunkPlan& p, int c, double general_us) { return p.cl > 0 && (c == 1 || 1.1 * p.us < general_us); }
 
 }  // namespace sgc

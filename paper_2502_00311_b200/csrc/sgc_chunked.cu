@@ -895,8 +895,6 @@ __global__ void __launch_bounds__(64) k_chunk_scatter(ChunkArgs a, float* __rest
 // ---- host side ----------------------------------------------------------------------------------------------
 namespace {
 
-int padded_k(int k) { return k <= 8 ? 8 : k <= 16 ? 16 : k <= 32 ? 32 : k <= 64 ? 64 : k <= 128 ? 128 : 256; }
-
 unsigned long long list_key(sgc_state* const* sts, int c) {
     unsigned long long h = 1469598103934665603ull;                   // FNV-1a
     for (int i = 0; i < c; ++i) {                                     // host object and its device allocation
@@ -958,8 +956,8 @@ ChunkRef ref_of(const sgc_state* st) {
 // 16 of 40520, 28, 4: 85 / 58;  300 of 2068, 200, 25: 783 / 550;  100 of 24712, 14, 2: 47 / 54;  300 of 3276, 21, 3: 53 / 56;
 // 256 of 65536, 8, 1: 52 / 83;  one of 4096, 256, 16: 212 / 111 (the general form of a single vector is the lock-step recovery).
 ChunkPlan plan_for(const sgc_state* st0, int c) {
-    const double general = chunk_general_us(c, st0->d, st0->k, padded_k(st0->k), st0->s, st0->sm_count);
-    auto better = [&](const ChunkPlan& p) { return p.cl > 0 && (c == 1 || 1.1 * p.us < general); };
+    const double general = chunk_general_us(c, st0->d, st0->k, st0->s, st0->sm_count);
+    auto better = [&](const ChunkPlan& p) { return cluster_form_taken(p, c, general); };
     // what a device of this size holds as a rule; it is asked (some ms, once per process) only where that form would be taken
     const int rule[kChunkShapes] = {st0->sm_count, st0->sm_count / 2, st0->sm_count * 2 / 9, st0->sm_count / 9, st0->sm_count / 18};
     if (!better(chunk_plan(c, st0->d, st0->k, st0->s, rule))) return ChunkPlan{};
@@ -992,7 +990,7 @@ cudaError_t ensure_ws(sgc_state* const* sts, int c) {
     free_chunk_ws(st0);
     ChunkWs* ws = new (std::nothrow) ChunkWs();
     if (!ws) return cudaErrorMemoryAllocation;
-    ws->c = c; ws->key = key; ws->kp = padded_k(st0->k);
+    ws->c = c; ws->key = key; ws->kp = chunk_padded_k(st0->k);
     ws->plan = plan_for(st0, c);
     if (ws->plan.cl == 0) ws->grid = grid_plan_for(st0, c);
     auto up = [](size_t b) { return (b + 255) / 256 * 256; };
@@ -1138,7 +1136,7 @@ bool chunked_batch_eligible(sgc_state* const* sts, int c) {
 static ChunkArgs common_args(const sgc_state* st0, int c) {
     ChunkArgs a;
     memset(&a, 0, sizeof(a));
-    a.c = c; a.k = st0->k; a.s = st0->s; a.kp = padded_k(st0->k); a.dc = st0->d;
+    a.c = c; a.k = st0->k; a.s = st0->s; a.kp = chunk_padded_k(st0->k); a.dc = st0->d;
     a.seed_lo = (uint32_t)(st0->seed & 0xFFFFFFFFu); a.seed_hi = (uint32_t)(st0->seed >> 32);
     a.sigma = (double)(float)(1.0 / sqrt((double)st0->k));
     a.wait_ns = st0->wait_limit_ns;

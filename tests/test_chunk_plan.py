@@ -11,6 +11,10 @@ import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
+# lists (chunks, columns of a chunk, rows of A, picks) whose chunks come in batches: more of them than the clusters have room for at a time.
+# One pick, where a batch ends as soon as it has begun, and several; 4, 8 and 16 warps on a recovery
+BATCHED = [(256, 8064, 164, 1), (400, 1684, 248, 8), (800, 856, 200, 8), (80, 6448, 212, 12)]
+
 SHIM = r"""
 #include "sgc_chunk_plan.h"
 using namespace sgc;
@@ -67,6 +71,14 @@ extern "C" int sweep(int k, long long* out, long long* taken) {
             }
     return 0;
 }
+// the cluster form of that list as the dispatch decides it on 148 SMs that hold `eight` / `sixteen` clusters of those widths: batches, warps per
+// recovery, whether the q_l are in shared memory; all zero where the list takes another form
+extern "C" void cluster_form(int c, long long dc, int k, int s, int eight, int sixteen, int* out) {
+    const int resident[kChunkShapes] = {148, 74, 2 * eight, eight, sixteen};
+    const ChunkPlan p = chunk_plan(c, dc, k, s, resident);
+    const bool taken = cluster_form_taken(p, c, chunk_general_us(c, dc, k, s, 148));
+    out[0] = taken ? p.batches : 0; out[1] = taken ? p.gw : 0; out[2] = taken ? p.q_shared : 0;
+}
 extern "C" double tail(double d, int k, double target) { return sphere_tail_threshold(d, k, target); }
 """
 
@@ -79,6 +91,7 @@ def plan(tmp_path_factory):
     subprocess.check_call(["g++", "-O2", "-std=c++17", "-Wall", "-Werror", "-shared", "-fPIC", "-I", os.path.join(ROOT, "paper_2502_00311_b200", "csrc"),
                            str(d / "shim.cpp"), "-o", lib])
     L = C.CDLL(lib)
+    L.cluster_form.argtypes = [C.c_int, C.c_longlong, C.c_int, C.c_int, C.c_int, C.c_int, C.POINTER(C.c_int)]
     L.tail.restype, L.tail.argtypes = C.c_double, [C.c_double, C.c_int, C.c_double]
     return L
 
@@ -89,6 +102,15 @@ def test_every_plan_holds_what_its_blocks_address(plan):
         out = (C.c_longlong * 5)()
         assert plan.sweep(k, out, taken) == 0, list(out)
     assert taken[0] > 10_000 and taken[1] > 1_000                         # both forms are taken
+
+
+@pytest.mark.parametrize("eight,sixteen", [(15, 7), (16, 8), (16, 7)])
+@pytest.mark.parametrize("c,dc,k,s", BATCHED)
+def test_lists_that_come_in_batches(plan, c, dc, k, s, eight, sixteen):
+    # what test_gpu_variants runs as lists whose clusters take several batches, with several warps on a recovery
+    out = (C.c_int * 3)()
+    plan.cluster_form(c, dc, k, s, eight, sixteen, out)
+    assert out[0] > 1 and out[1] > 1, list(out)
 
 
 @pytest.mark.parametrize("d,k", [(65_536, 112), (20_000, 40), (30_000, 256)])

@@ -8,6 +8,7 @@ import pytest
 import oracle
 import test_gpu_parity as parity
 from paper_2502_00311_b200 import inputs
+from test_chunk_plan import BATCHED
 from test_gpu_parity import cuda, run_both, sgc  # noqa: F401  (sgc is the module's fixture)
 
 pytestmark = pytest.mark.gpu
@@ -261,6 +262,12 @@ def test_the_first_speculating_step_leaves_another_streams_capture_alone(sgc):  
 @pytest.mark.parametrize("c,dc,k,sc", [(3, 12, 9, 3), (1, 2052, 255, 32), (7, 1300, 256, 32), (40, 508, 3, 1), (200, 640, 33, 2), (700, 260, 17, 2),
                                        (1000, 52, 250, 2), (33, 2064, 241, 12), (2, 60_000, 15, 4), (260, 20_000, 7, 1)])
 def test_chunk_recoveries_in_clusters(sgc, c, dc, k, sc):  # noqa: F811
+    parity.test_mesgc_small_chunks_batched_path_matches_independent_oracles(sgc, c, dc, k, sc, "student")
+
+
+# the same with more chunks than the clusters have room for: a batch begins while the records of the one before are still being written
+@pytest.mark.parametrize("c,dc,k,sc", BATCHED)
+def test_chunk_recoveries_in_batches(sgc, c, dc, k, sc):  # noqa: F811
     parity.test_mesgc_small_chunks_batched_path_matches_independent_oracles(sgc, c, dc, k, sc, "student")
 
 
