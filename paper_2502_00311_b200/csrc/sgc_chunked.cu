@@ -1002,6 +1002,7 @@ cudaError_t ensure_ws(sgc_state* const* sts, int c) {
         if (e != cudaSuccess) { delete ws; return e; }
         ws->table = static_cast<ChunkRef*>(ws->base);
         e = cudaMemcpy(ws->table, host.data(), (size_t)c * sizeof(ChunkRef), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaDeviceSynchronize();           // (a copy from pageable memory returns before it has arrived)
         if (e != cudaSuccess) { cudaFree(ws->base); delete ws; return e; }
         st0->chunk_ws = ws;
         return cudaSuccess;

@@ -271,6 +271,26 @@ def test_chunk_recoveries_in_batches(sgc, c, dc, k, sc):  # noqa: F811
     parity.test_mesgc_small_chunks_batched_path_matches_independent_oracles(sgc, c, dc, k, sc, "student")
 
 
+# the first step of a list builds its table; a stream that does not wait for the default one finds it complete, whichever form the list takes
+# (cluster, whole GPU, general)
+@pytest.mark.parametrize("c,dc,k,sc", [(600, 64, 20, 4), (3, 40_004, 130, 3), (1000, 512, 8, 1)])
+def test_first_chunked_step_on_a_side_stream(sgc, c, dc, k, sc):  # noqa: F811
+    import torch
+    hp = [inputs.ADAM[q] for q in ("lr", "beta1", "beta2", "eps")]
+    g = cuda(np.random.default_rng(c).standard_t(3.0, size=c * dc).astype(np.float32))
+    side, want = torch.cuda.Stream(), None
+    torch.cuda.synchronize()
+    for turn in range(4):
+        me, w = sgc.Mesgc(c * dc, c, k, sc, 3, *hp), torch.zeros(c * dc, device="cuda")
+        torch.cuda.synchronize()
+        me.step(g, w, stream=side if turn else None)
+        side.synchronize()
+        got = w.cpu().numpy()
+        want = got if want is None else want
+        assert np.array_equal(got, want) and (got != 0).any()
+        me.close()
+
+
 # chunk recoveries on the whole GPU (too many columns for a cluster): 64 to 256 rows of A, a ragged last block, tiles of residual rows
 # that are full, nearly empty, and brought in one after the other where there is room for one only
 @pytest.mark.parametrize("c,dc,k,sc", [(65, 60_000, 40, 2), (3, 40_004, 130, 3), (130, 22_004, 250, 1), (70, 30_000, 97, 2), (1, 70_016, 64, 5)])
