@@ -69,8 +69,9 @@ enum {
                                                 forwards has its range screened again, so up to 16 always reach the fp64
                                                 decision): the pick may then differ from the exact argmax by a near-tie */
     SGC_STATUS_SELECT_FALLBACK = 1u << 5,  /* the bound on the kept magnitudes missed; exact fallback ran */
-    SGC_STATUS_TIMEOUT = 1u << 6           /* a bounded wait inside a tensor-core screening pass ran out; the pass's
-                                              reports were discarded and the step finished on its slower exact path */
+    SGC_STATUS_TIMEOUT = 1u << 6           /* a bounded wait ran out, inside a tensor-core screening pass (its reports were
+                                              discarded) or in one of the kernels that make all picks of small problems; the
+                                              step finished on its slower exact path */
 };
 
 /* selectors for sgc_get: records of the LAST step, copied to a host buffer */
@@ -224,9 +225,8 @@ SGC_API int sgc_status(sgc_state* st, uint32_t* out);
  * that make all picks of small problems in one launch (these are the only kernels of this library whose warps wait for one another
  * through memory).  When a wait runs out, the pass records the fact,
  * lets the copies and matrix operations in flight finish, releases its tensor memory and returns; the step then
- * discards the pass's reports, finishes on the exact lock-step path and sets SGC_STATUS_TIMEOUT.  The
- * kernel that runs on the whole GPU goes through all columns instead, sets SGC_STATUS_TIMEOUT and makes the same picks; the one that
- * runs in clusters lets what it has sent arrive, sets SGC_STATUS_TIMEOUT and returns: the picks made so far stand, the others are missing.  The paper has no
+ * discards the pass's reports, finishes on the exact lock-step path and sets SGC_STATUS_TIMEOUT.  The two kernels of small
+ * problems let what they have sent arrive, set SGC_STATUS_TIMEOUT and make the same picks by going through all columns.  The paper has no
  * counterpart: this is failure handling, and the setter exists so that the path can be exercised (a bound of a few
  * nanoseconds makes ordinary waits run out without anything being broken).
  *   st   the state whose passes are meant; NULL sets the bound used by sgc_screen (process-wide)

@@ -12,8 +12,8 @@
 // block waits for what it needs and for nothing else (a cluster-wide barrier of 16 blocks takes 0.6 us, and an iteration needs two).
 // Latency bounds it: 5.6 us per pick for one vector of 4096 (k = 256; three cluster barriers and L2 trips of the lock-step kernel: 11), 9.2 us for 20 recoveries per
 // cluster over 2048 columns (k = 217; two launches: 17), of which scoring takes a quarter, bound by shared-memory reads of the operands.
-// Every wait is bounded; on expiry the block marks its chunks, leaves the loops, gives what is still on its way time to land and
-// meets the others at the end.
+// Every wait is bounded; on expiry the block marks its chunks, leaves the loops, gives what is still on its way time to land, meets the
+// others, and makes the picks that its recoveries lack by itself, going through all columns in fp64.
 #include <mutex>
 
 #include <cooperative_groups.h>
@@ -343,6 +343,52 @@ __device__ __forceinline__ void make_pick(const ChunkArgs& a, const ChunkPlan& p
     }
 }
 
+// books of a recovery as its chunk's first kernel left it; returns the squared norm of its residual, to all of the team
+__device__ __forceinline__ double open_books(const ChunkArgs& a, ChunkBook& bk, const ChunkRef& ref, double* r, int m, const Team& tm) {
+    double part = 0.0;
+    for (int i = tm.t; i < a.k; i += 32 * tm.warps) {
+        const double v = ref.r64[(size_t)m * a.k + i];
+        r[i] = v;
+        part = fma(v, v, part);
+    }
+    if (tm.t == 0) { bk.stopped = 0; bk.ref = ref; }
+    return team_sum(bk, part, tm, a.k);
+}
+
+// A wait has expired at pick j0 of the batch that starts with chunk c0: this block goes on without the others.  Its recoveries go through all
+// columns in fp64, which decides as the kernel does (of equal scores the lowest column), from pick j0 on, and those of the batches behind it
+// from their first.
+template <bool SHARED>
+__device__ __noinline__ void finish_alone(const ChunkArgs& a, const ChunkPlan& p, unsigned char* sm, int rank, int c0, int last, int j0, const Team& tm) {
+    const int teams = kClusterWarps / p.gw;
+    double* xs = reinterpret_cast<double*>(sm + p.off_x) + (size_t)tm.id * p.kq;
+    for (bool open = true; c0 < last; c0 += p.batch, j0 = 0, open = false) {
+        const int n_rec = 2 * (last - c0 < p.batch ? last - c0 : p.batch);
+        for (int own = tm.id; own * p.cl + rank < n_rec; own += teams) {
+            const int rec = own * p.cl + rank, m = rec & 1;
+            ChunkBook& bk = *reinterpret_cast<ChunkBook*>(sm + p.off_book + (size_t)own * kClusterBook);
+            double* r = reinterpret_cast<double*>(sm + p.off_r) + (size_t)own * p.kq;
+            if (!open) open_books(a, bk, chunk_ref(a, c0 + (rec >> 1)), r, m, tm);
+            const ChunkRef& ref = bk.ref;
+            double* qs = SHARED ? reinterpret_cast<double*>(sm + p.off_q) + (size_t)own * a.s * p.kq : ref.qb + (size_t)m * a.s * a.k;
+            for (int j = j0; j < a.s && !bk.stopped; ++j) {
+                BestColumn b;
+                scan_columns(a, bk, r, tm, j, 0, a.dc, b);
+                uint32_t col = join_columns(bk, tm, b);
+                double gamma = 0.0, aj = 0.0, rn2 = 0.0;
+                if (col == kNoColumn) { if (tm.t == 0) { ref.cnt->stopped[m] = 1; ref.cnt->done[m] = j; } }
+                else if (!extend_basis<SHARED>(a, bk, ref, r, qs, SHARED ? p.kq : a.k, xs, m, j, col, tm, &gamma, &aj, &rn2)) col = kNoColumn;
+                tm.meet();
+                if (tm.warp == tm.warps - 1) {
+                    if (col == kNoColumn) { if (tm.lane == 0) bk.stopped = 1; }
+                    else record_pick(a, bk, ref, m, j, col, gamma, aj, rn2, tm.lane);
+                }
+                tm.meet();
+            }
+        }
+    }
+}
+
 // ---- the kernel --------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(kCT, 1) k_chunk_cluster(const __grid_constant__ ChunkArgs a, const __grid_constant__ ChunkPlan p) {
     extern __shared__ __align__(16) unsigned char sm[];
@@ -369,6 +415,7 @@ __global__ void __launch_bounds__(kCT, 1) k_chunk_cluster(const __grid_constant_
     const unsigned long long limit_ns = a.wait_ns ? a.wait_ns : kClusterWaitNs;
     uint32_t ph_cand = 0, ph_res = 0;
     bool ok = true;
+    int c_left = first, j_left = 0;                                   // where a wait expired: first chunk of the batch, picks made
     for (int c0 = first; ok && c0 < last; c0 += p.batch) {
         // recovery rec of the batch: chunk c0 + rec / 2, moment rec & 1; kept by block rec % cl as its rec / cl-th
         const int n_rec = 2 * (last - c0 < p.batch ? last - c0 : p.batch);
@@ -383,18 +430,11 @@ __global__ void __launch_bounds__(kCT, 1) k_chunk_cluster(const __grid_constant_
             const ChunkRef& ref = chunk_ref(a, c0 + (rec >> 1));
             ChunkBook& bk = *reinterpret_cast<ChunkBook*>(sm + p.off_book + (size_t)own * kClusterBook);
             double* r = reinterpret_cast<double*>(sm + p.off_r) + (size_t)own * p.kq;
-            double part = 0.0;
-            for (int i = tm.t; i < a.k; i += 32 * tm.warps) {
-                const double v = ref.r64[(size_t)m * a.k + i];
-                r[i] = v;
-                part = fma(v, v, part);
-            }
-            if (tm.t == 0) { bk.stopped = 0; bk.ref = ref; }
-            const double rn2 = team_sum(bk, part, tm, a.k);
-            send_residual(p, sm, rec, r, rn2, tm);
+            send_residual(p, sm, rec, r, open_books(a, bk, ref, r, m, tm), tm);
         }
         for (int j = 0; j < a.s; ++j) {
             if (t == 0 && n_own > 0) mbar_arrive_expect_tx(bar_cand, cand_bytes);
+            c_left = c0; j_left = j;
             if (!(ok = block_wait(bar_res, ph_res & 1u, &head->abort_flag, limit_ns))) break;
             ++ph_res;
             if (t == 0 && j + 1 < a.s) mbar_arrive_expect_tx(bar_res, res_bytes);
@@ -408,15 +448,18 @@ __global__ void __launch_bounds__(kCT, 1) k_chunk_cluster(const __grid_constant_
                 else make_pick<false>(a, p, sm, rec, rec & 1, own, j, tm);
             }
         }
-        if (!ok)                                                      // the picks made so far stand
+        if (!ok)
             for (int ch = c0 + t; ch < last; ch += kCT) atomicOr(&chunk_ref(a, ch).cnt->status, (unsigned int)SGC_STATUS_TIMEOUT);
     }
-    if (!ok) {
-        // what was sent may still be on its way: it lands in microseconds
-        const unsigned long long t0 = global_ns();
-        while (global_ns() - t0 < 200000ull) __nanosleep(1000);
-    }
+    // after an expired wait: what was sent, by this block and to it, may still be on its way; it lands in microseconds
+    auto settle = [] { const unsigned long long t0 = global_ns(); while (global_ns() - t0 < 200000ull) __nanosleep(1000); };
+    if (!ok) settle();
     cluster.sync();
+    if (!ok) {
+        settle();
+        if (p.q_shared) finish_alone<true>(a, p, sm, rank, c_left, last, j_left, tm);
+        else finish_alone<false>(a, p, sm, rank, c_left, last, j_left, tm);
+    }
 }
 
 struct ClusterLaunch {

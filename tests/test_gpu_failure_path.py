@@ -122,10 +122,12 @@ def test_chunked_tensor_route_survives_an_expired_wait(sgc):
         ref.close()
 
 
-def test_cluster_recoveries_return_when_a_wait_expires(sgc):
+# one batch of chunks per cluster; several batches, with the orthogonal vectors in shared memory and in global memory
+@pytest.mark.parametrize("c,dc,k,sc", [(5, 4096, 100, 8), (256, 8064, 164, 2), (400, 1684, 248, 8)])
+def test_cluster_recoveries_go_on_when_a_wait_expires(sgc, c, dc, k, sc):
     # the picks of small problems are made inside clusters whose blocks wait for one another's data; an expired wait (step 1) is
-    # reported, the kernel returns, and the next step is an ordinary one
-    c, dc, k, sc, seed = 5, 4096, 100, 8, 9
+    # reported, every block makes the picks of its recoveries by itself, and the next step is an ordinary one
+    seed = 9
     hp = inputs.ADAM
     me = sgc.Mesgc(c * dc, c, k, sc, seed, hp["lr"], hp["beta1"], hp["beta2"], hp["eps"])
     refs = [oracle.Oracle(dc, k, sc, seed, hp["lr"], hp["beta1"], hp["beta2"], hp["eps"]) for _ in range(c)]
@@ -137,15 +139,31 @@ def test_cluster_recoveries_return_when_a_wait_expires(sgc):
         me.step(cuda(g), w_gpu)
         for i, ref in enumerate(refs):
             ref.step(g[i * dc:(i + 1) * dc], w_ref[i * dc:(i + 1) * dc])
-            done = int(me.chunks[i].get("doneM"))
-            assert np.array_equal(me.chunks[i].get("lamM")[:done], ref.get("lamM")[:done]), (step, i)
-            assert done == sc or step == 1
+            for name in ("doneM", "doneV", "lamM", "lamV", "upd_idx"):
+                assert np.array_equal(me.chunks[i].get(name), ref.get(name)), (step, i, name)
         assert any(ch.status() & sgc.STATUS_TIMEOUT for ch in me.chunks) == (step == 1)
         for ch in me.chunks:
             ch.clear_status()
+        np.testing.assert_allclose(w_gpu.cpu().numpy(), w_ref, rtol=0, atol=1e-6)
     me.close()
     for ref in refs:
         ref.close()
+
+
+def test_small_state_goes_on_when_a_wait_expires(sgc):
+    d, k, s, seed = 4096, 256, 16, 4
+    hp = inputs.ADAM
+    st = sgc.Sgc(d, k, s, seed, hp["lr"], hp["beta1"], hp["beta2"], hp["eps"])
+    ref = oracle.Oracle(d, k, s, seed, hp["lr"], hp["beta1"], hp["beta2"], hp["eps"])
+    supp, sign = inputs.planted_support(d, s, 31)
+    w_gpu, w_ref = cuda(inputs.weights(d, 3)), inputs.weights(d, 3)
+    for step in range(3):
+        st.set_wait_limit(1 if step == 1 else 0)
+        compare_step(st, ref, inputs.gradient(d, "student", supp, sign, 900 + step), w_gpu, w_ref)
+        assert bool(st.status() & sgc.STATUS_TIMEOUT) == (step == 1)
+        st.clear_status()
+    st.close()
+    ref.close()
 
 
 def test_states_of_very_different_k_live_side_by_side(sgc):
