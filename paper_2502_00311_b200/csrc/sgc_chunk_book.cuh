@@ -25,7 +25,11 @@ struct ChunkBook {
 };
 static_assert(sizeof(ChunkBook) <= kClusterBook, "a recovery's records");
 
-// The whole block waits for a barrier and agrees on whether the wait expired.  Where the caller wants waits to expire (a limit under a
+// The whole block waits for a barrier and agrees on whether the wait expired.  The waits acquire at the scope of the block, as those on TMA
+// loads do, also where another block of the cluster has sent what is waited for: it lies in this block's own shared memory, of which there is
+// one copy, the barrier counts bytes that have been written there, and blocks exchange nothing through global memory while the kernel runs,
+// which is all that the cluster's scope would add (it empties the SM's L1: with one acquire of that scope behind every wait 111 instead of 109 us at
+// 64 x 64, k = 256, and 457 instead of 442 for the projected 4096 x 4096; polled with it 105 instead of 94 us).  Where the caller wants waits to expire (a limit under a
 // millisecond) the barrier is polled without the hardware's own pause.
 static __device__ __noinline__ bool block_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_flag, unsigned long long limit_ns) {
     const bool brief = limit_ns < 1000000ull;
