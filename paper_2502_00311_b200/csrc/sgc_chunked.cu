@@ -1209,7 +1209,8 @@ cudaError_t launch_chunked_batch(sgc_state* const* sts, int c, const float* grad
     const int phases = 2 + st0->s * (chunk_on_tensor_cores(c, st0->d, ws->kp) ? 4 + chunk_passes(c) : 2);
     if (ws->plan.cl > 0) {
         e = launch_front(st0, a, true, grad, stream, launches);
-        if (e == cudaSuccess) e = launch_chunk_cluster(a, ws->plan, true, stream);
+        if (e != cudaSuccess) return e;                              // (nothing is counted: the caller takes the step count back)
+        e = launch_chunk_cluster(a, ws->plan, true, stream);
         if (e == cudaSuccess) e = launch_scatter(st0, a, weight, stream, launches);
         *launches += phases - 2;
         return e;
@@ -1217,7 +1218,8 @@ cudaError_t launch_chunked_batch(sgc_state* const* sts, int c, const float* grad
     if (ws->grid.blocks > 0) {
         a.kp64 = ws->kp64; a.rt = ws->rt; a.tau = ws->tau; a.rep_count = ws->rep_count; a.rep = ws->rep; a.flags = ws->flags; a.z_rep = ws->z_rep;
         e = launch_front(st0, a, false, grad, stream, launches);
-        if (e == cudaSuccess) e = launch_chunk_grid(a, ws->grid, stream);
+        if (e != cudaSuccess) return e;
+        e = launch_chunk_grid(a, ws->grid, stream);
         if (e == cudaSuccess) e = launch_scatter(st0, a, weight, stream, launches);
         *launches += phases - 2;
         return e;

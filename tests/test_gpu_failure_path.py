@@ -166,6 +166,43 @@ def test_small_state_goes_on_when_a_wait_expires(sgc):
     ref.close()
 
 
+# a list in clusters, on the whole GPU and in the general form; a single small state and one that is not small
+@pytest.mark.parametrize("c,dc,k,s", [(6, 512, 100, 8), (3, 40_004, 130, 3), (1000, 512, 8, 1), (0, 4096, 256, 16), (0, 40_000, 300, 4)])
+def test_a_step_whose_first_launch_fails_does_not_count(sgc, c, dc, k, s):
+    # launches into a stream whose capture has become invalid are refused by the runtime: M, V and t stay what they were
+    import ctypes
+    import torch
+    rt = ctypes.CDLL("libcudart.so.12")
+    hp = [inputs.ADAM[q] for q in ("lr", "beta1", "beta2", "eps")]
+    grads = [cuda(np.random.default_rng(i).standard_t(3.0, size=max(c, 1) * dc).astype(np.float32)) for i in range(2)]
+    side, outs = torch.cuda.Stream(), []
+    torch.cuda.synchronize()
+    for refused in (False, True):
+        opt = sgc.Mesgc(c * dc, c, k, s, 3, *hp) if c else sgc.Sgc(dc, k, s, 3, *hp)
+        st, w = opt.chunks[-1] if c else opt, torch.zeros(max(c, 1) * dc, device="cuda")
+        torch.cuda.synchronize()
+        opt.step(grads[0], w, stream=side)
+        if refused:
+            before = st.get("M"), st.get("V"), w.cpu().numpy()
+            cs = ctypes.c_void_p(side.cuda_stream)
+            assert rt.cudaStreamBeginCapture(cs, 2) == 0
+            assert rt.cudaStreamSynchronize(cs) != 0                       # not allowed while capturing, which ends the capture's validity
+            with pytest.raises(sgc.SgcError):
+                opt.step(grads[1], w, stream=side)
+            graph = ctypes.c_void_p()
+            assert rt.cudaStreamEndCapture(cs, ctypes.byref(graph)) != 0 and not graph.value
+            rt.cudaGetLastError()
+            assert int(st.get("t")) == 1
+            for a, b in zip(before, (st.get("M"), st.get("V"), w.cpu().numpy())):
+                assert np.array_equal(a, b)
+        opt.step(grads[1], w, stream=side)
+        side.synchronize()
+        assert int(st.get("t")) == 2
+        outs.append((st.get("M"), w.cpu().numpy()))
+        opt.close()
+    assert np.array_equal(outs[0][0], outs[1][0]) and np.array_equal(outs[0][1], outs[1][1])
+
+
 def test_states_of_very_different_k_live_side_by_side(sgc):
     # the lock-step kernel's shared-memory opt-in belongs to the kernel, not to a state: creating a small-k state must
     # not take away what a large-k state needs
