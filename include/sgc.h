@@ -103,6 +103,11 @@ enum {
     SGC_GET_LIST_ROUNDS = 25, /* int32     list passes (screening passes over the wide lists only) that the last step resolved */
     SGC_GET_PASS_ROWS = 26, /* int32       residual rows screened by the passes over all d columns of the last step, summed over
                                those passes (a state stepped alone; 2 k d flops of contraction per row)       */
+    SGC_GET_CHUNK_FORM = 27, /* int32[4]   which kernels made the picks of the last step (known to the host, nothing is waited for): [0] 0: those of
+                               a whole matrix; 1: for all chunks a correlation and a decision per pick; 2: the same with the correlations on
+                               the tensor cores; 3: one launch, inside thread-block clusters; 4: one launch, on the whole GPU;
+                               [1] batches in which a cluster takes its chunks (3); [2] warps that work on one recovery (3, 4);
+                               [3] 1: the orthogonal vectors are in shared memory (3)                       */
     SGC_GET_ROUND_TRACE = 24 /* int32[24][3] per screening pass of the last step: picks of M^ confirmed so far, picks of V^ confirmed so
                                 far, length of the candidate list after it (rows past SGC_GET_ROUNDS are zero)               */
 };
@@ -240,9 +245,8 @@ SGC_API int sgc_set_wait_limit(sgc_state* st, uint64_t ns);
  *            plus three, at most 24); negative: SGC_ERR_DIM.  In a group (sgc_step_group) the largest bound of a batch holds. */
 SGC_API int sgc_set_max_rounds(sgc_state* st, int32_t rounds);
 
-/* Number of kernel launches the last sgc_step / sgc_step_group enqueued for this state.  After sgc_step_chunked and sgc_cesgc_step:
- * the number of the step's phases (selection, a correlation and a decision per pick, update; with the correlations on the tensor
- * cores their launches), which is the number of its launches unless one kernel carries all the picks' phases. */
+/* Number of kernel launches the last sgc_step / sgc_step_group enqueued for this state.  Those that serve all states of a group or
+ * of a chunk list are booked on the first; sgc_cesgc_step adds its two projections, which are not counted. */
 SGC_API int sgc_last_launches(sgc_state* st, int32_t* out);
 
 /* Top-s selection (step a1 alone) for callers that cannot allocate device memory.  The paper has no

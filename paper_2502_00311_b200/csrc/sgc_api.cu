@@ -207,6 +207,7 @@ SGC_API int sgc_step(sgc_state* st, const float* grad, float* weight, void* stre
         if (e == cudaSuccess) e = sgc::launch_project_adam(st, cs, &launches);
         if (e != cudaSuccess) { st->t -= 1; return (int)e; }
         e = sgc::launch_recover(st, weight, cs, &launches);
+        memset(st->form, 0, sizeof(st->form));
     }
     st->last_stream = cs; st->has_stream = true; st->stepped = true; st->last_launches = launches;
     return (int)e;
@@ -239,6 +240,7 @@ static int step_group(sgc_state* const* states, const float* const* grads, float
             continue;
         }
         rest.push_back(st); rest_w.push_back(weights[i]);
+        memset(st->form, 0, sizeof(st->form));
         e = sgc::launch_select(st, grads[i], cs, &launches[i]);
         if (e == cudaSuccess) e = sgc::launch_project_adam(st, cs, &launches[i]);
         if (e != cudaSuccess) st->t -= 1;                           // this state's moments were not touched
@@ -374,6 +376,12 @@ SGC_API int sgc_get(sgc_state* st, int32_t what, void* dst, size_t bytes) {
         case SGC_GET_T: {
             if (bytes < 8) return SGC_ERR_SIZE;
             memcpy(dst, &st->t, 8);
+            return SGC_OK;
+        }
+        case SGC_GET_CHUNK_FORM: {
+            if (!st->stepped) return SGC_ERR_NOSTEP;
+            if (bytes < sizeof(st->form)) return SGC_ERR_SIZE;
+            memcpy(dst, st->form, sizeof(st->form));
             return SGC_OK;
         }
         case SGC_GET_M: src = st->M; n = 4 * k; needs_step = false; break;

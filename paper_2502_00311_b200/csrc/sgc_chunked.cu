@@ -1173,6 +1173,10 @@ static cudaError_t launch_scatter(const sgc_state* st0, const ChunkArgs& a, floa
     return cudaGetLastError();
 }
 
+static void set_form(sgc_state* st, int form, int batches, int warps, int q_shared) {
+    st->form[0] = form; st->form[1] = batches; st->form[2] = warps; st->form[3] = q_shared;
+}
+
 // A single small state as a list of one chunk: selection, projection and moments in one launch, the recovery in one cluster.  It is what a
 // state that recovers in lock-step does, faster (see k_chunk_cluster): a state that speculates, or has, keeps lists that this form does
 // not know.
@@ -1184,7 +1188,7 @@ static bool small_step_plan(const sgc_state* st, ChunkPlan* plan) {
     return plan->cl > 0;
 }
 bool takes_small_step(const sgc_state* st) { ChunkPlan p; return small_step_plan(st, &p); }
-cudaError_t launch_small_step(const sgc_state* st, const float* grad, float* weight, cudaStream_t stream, int* launches) {
+cudaError_t launch_small_step(sgc_state* st, const float* grad, float* weight, cudaStream_t stream, int* launches) {
     ChunkPlan plan;
     if (!small_step_plan(st, &plan)) return cudaErrorInvalidConfiguration;
     ChunkArgs a = common_args(st, 1);
@@ -1193,6 +1197,7 @@ cudaError_t launch_small_step(const sgc_state* st, const float* grad, float* wei
     if (e == cudaSuccess) e = launch_chunk_cluster(a, plan, true, stream);
     if (e != cudaSuccess) return e;
     *launches += 1;
+    set_form(st, 3, plan.batches, plan.gw, plan.q_shared);
     return launch_scatter(st, a, weight, stream, launches);
 }
 
@@ -1205,24 +1210,26 @@ cudaError_t launch_chunked_batch(sgc_state* const* sts, int c, const float* grad
     const ChunkWs* ws = st0->chunk_ws;
     ChunkArgs a = common_args(st0, c);
     a.table = ws->table;
-    // what sgc_last_launches reports of a chunked step: its phases, whichever kernels carry them
-    const int phases = 2 + st0->s * (chunk_on_tensor_cores(c, st0->d, ws->kp) ? 4 + chunk_passes(c) : 2);
+    for (int i = 0; i < c; ++i)
+        if (ws->plan.cl > 0) set_form(sts[i], 3, ws->plan.batches, ws->plan.gw, ws->plan.q_shared);
+        else if (ws->grid.blocks > 0) set_form(sts[i], 4, 0, ws->grid.gw, 0);
+        else set_form(sts[i], ws->tensor ? 2 : 1, 0, 0, 0);
     if (ws->plan.cl > 0) {
         e = launch_front(st0, a, true, grad, stream, launches);
         if (e != cudaSuccess) return e;                              // (nothing is counted: the caller takes the step count back)
         e = launch_chunk_cluster(a, ws->plan, true, stream);
-        if (e == cudaSuccess) e = launch_scatter(st0, a, weight, stream, launches);
-        *launches += phases - 2;
-        return e;
+        if (e != cudaSuccess) return e;
+        *launches += 1;
+        return launch_scatter(st0, a, weight, stream, launches);
     }
     if (ws->grid.blocks > 0) {
         a.kp64 = ws->kp64; a.rt = ws->rt; a.tau = ws->tau; a.rep_count = ws->rep_count; a.rep = ws->rep; a.flags = ws->flags; a.z_rep = ws->z_rep;
         e = launch_front(st0, a, false, grad, stream, launches);
         if (e != cudaSuccess) return e;
         e = launch_chunk_grid(a, ws->grid, stream);
-        if (e == cudaSuccess) e = launch_scatter(st0, a, weight, stream, launches);
-        *launches += phases - 2;
-        return e;
+        if (e != cudaSuccess) return e;
+        *launches += 1;
+        return launch_scatter(st0, a, weight, stream, launches);
     }
     a.frag = ws->frag; a.back = ws->back; a.kf = ws->kp < 16 ? 16 : ws->kp; a.cand = ws->cand; a.lam = ws->lam; a.splits = ws->splits;
     {

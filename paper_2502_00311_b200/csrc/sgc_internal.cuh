@@ -252,6 +252,7 @@ struct sgc_state {
     int device; int sm_count;
     cudaStream_t last_stream; bool has_stream;
     int32_t last_launches; bool stepped;
+    int32_t form[4];            // which kernels made the last step's picks (SGC_GET_CHUNK_FORM)
     bool sel_warm;              // a top-s threshold from the previous step is on the device (one-kernel selection)
     int omp_grid2, omp_grid8;   // blocks of the recovery kernel in clusters of 2 and of 8 (0: the device holds fewer than three)
     int omp_one;                // 1: a cluster of 16 can be resident
@@ -362,7 +363,7 @@ cudaError_t launch_chunked_batch(sgc_state* const* sts, int c, const float* grad
                                  int* launches);
 void free_chunk_ws(sgc_state* st);
 bool takes_small_step(const sgc_state* st);     // the next step of this state is small enough for one cluster, and recovers in lock-step
-cudaError_t launch_small_step(const sgc_state* st, const float* grad, float* weight, cudaStream_t stream, int* launches);
+cudaError_t launch_small_step(sgc_state* st, const float* grad, float* weight, cudaStream_t stream, int* launches);
 // CESGC projections (sgc_cesgc.cu): P = B G and W += B^T U
 bool cesgc_shape_ok(int r, int m, int n);
 cudaError_t launch_cesgc_project(const float* B, const float* G, float* P, float* U, int r, int m, int n, cudaStream_t stream);     // and U = 0
