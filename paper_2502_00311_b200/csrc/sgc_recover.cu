@@ -102,10 +102,8 @@ struct ResolveArgs {
     const unsigned int* wide_count;
 };
 
-// Whether a challenger's exact score reaches that of the pick, as one warp sees it: sums in another order than the walk's, so that what comes
-// within 1e-9 of the pick (ties among it) is left to the walk.
-constexpr int kSweepCap = 8;                           // challengers per pick that the sweep rescores
-__device__ __forceinline__ bool may_win(const OmpArgs& a, uint32_t col, const double* r, double ps) {
+// <z, r> and ||z||^2 of a column, as one warp sums them
+__device__ __forceinline__ void warp_products(const OmpArgs& a, uint32_t col, const double* r, double* dot_out, double* n2_out) {
     const int lane = threadIdx.x & 31;
     const ColKey key = column_key(a.seed_lo, a.seed_hi, col);
     double dot = 0.0, n2 = 0.0;
@@ -117,9 +115,9 @@ __device__ __forceinline__ bool may_win(const OmpArgs& a, uint32_t col, const do
         dot = fma((double)z.x, r0, dot); dot = fma(z1, r1, dot);
         n2 = fma((double)z.x, (double)z.x, n2); n2 = fma(z1, z1, n2);
     }
-    dot = warp_sum(dot); n2 = warp_sum(n2);
-    return dot * dot >= ps * ps * n2 * (1.0 - 1e-9);
+    *dot_out = warp_sum(dot); *n2_out = warp_sum(n2);
 }
+constexpr int kSweepCap = 8;                           // challengers per pick that the sweep rescores
 
 __device__ __forceinline__ bool in_support(const uint32_t* lam, int n, uint32_t col) {
     for (int q = 0; q < n; ++q) if (lam[q] == col) return true;
@@ -268,6 +266,11 @@ __global__ void __launch_bounds__(kOmpThreads, 1) k_resolve(ResolveArgs ra) {
                     const bool skip_members = ctl->list_exact[m] != 0;
                     const uint2* list = ra.rep + (size_t)n * ra.rep_cap;
                     const int lane = threadIdx.x & 31;
+                    // Whether a challenger reaches the pick is asked of this residual for both, as the walk does, in another order of the sums:
+                    // what comes within 1e-9 of the pick (ties among it) is left to the walk.  (pick_score would not do: on the Gram
+                    // path it comes from a recursion whose error is relative to ||y||, some 1e-8 of the score once ||r|| is at 1e-7 of ||y||.)
+                    const double* res = a.rhist + (size_t)n * a.k;
+                    double pd = 0.0, pn2 = 0.0;                          // the pick's products, from the first challenger on
                     int met = 0;                                         // challengers so far, the same in every lane
                     for (unsigned int e0 = 0; e0 < count && !hit; e0 += 8 * 32) {
                         uint2 rp8[8];                                    // eight reports in flight per lane
@@ -285,7 +288,11 @@ __global__ void __launch_bounds__(kOmpThreads, 1) k_resolve(ResolveArgs ra) {
                             if (in && in_support(a.lam + (size_t)m * s, j, rp.x)) in = false;
                             for (unsigned int who = __ballot_sync(0xffffffffu, in); who && !hit; who &= who - 1u) {
                                 const uint32_t col = __shfl_sync(0xffffffffu, rp.x, __ffs(who) - 1);
-                                hit = ++met > kSweepCap || may_win(a, col, a.rhist + (size_t)n * a.k, ps);
+                                double dot, n2;
+                                if (++met > kSweepCap) { hit = true; break; }
+                                if (met == 1) warp_products(a, pick, res, &pd, &pn2);
+                                warp_products(a, col, res, &dot, &n2);
+                                hit = dot * dot * pn2 >= pd * pd * n2 * (1.0 - 1e-9);
                             }
                         }
                     }

@@ -321,3 +321,64 @@ def test_small_states_recover_in_one_cluster(sgc, d, k, s, n):  # noqa: F811
         assert parity.rel(w.cpu().numpy(), r) < 1e-5
     for st in sts + refs:
         st.close()
+
+
+def _near_tie(k, seed, supp, p, c, gap, rng):
+    """A float32 vector of the columns `supp`, some 2e-7 of it left over once they are projected out, and column c ahead of column p there by `gap` of a
+    score.  The lead is linear in the vector, so that units in the last place of its entries set it, to some 1e-10."""
+    ext = np.longdouble                                                    # (a mantissa of 64 bits)
+    z = np.stack([oracle.z_block(seed, 0, k, int(i), 1).reshape(-1) for i in [*supp, p, c]], 1).astype(ext)
+    z /= np.sqrt((z * z).sum(0))
+    q = np.zeros((k, len(supp)), ext)
+
+    def rest(v, n=len(supp)):
+        for _ in range(2):
+            v = v - q[:, :n] @ (q[:, :n].T @ v)
+        return v
+    for j in range(len(supp)):
+        v = rest(z[:, j], j)
+        q[:, j] = v / np.sqrt(v @ v)
+    hp, hc = rest(z[:, -2]), rest(z[:, -1])
+    y = (z[:, :-2] @ (np.linspace(1.0, 0.6, len(supp)) * rng.choice([-1, 1], len(supp))).astype(ext) + ext(2e-7) * (z[:, -2] + z[:, -1])).astype(np.float32)
+    unit = np.spacing(np.abs(y)).astype(ext)
+    step, left, n = (hc - hp) * unit, ext(gap) * (hc @ y.astype(ext)) - (hc - hp) @ y.astype(ext), np.zeros(k, int)
+    coarse = np.argsort(-np.abs(step))[::8]
+    for i in coarse:
+        n[i] = int(np.clip(np.rint(float(left / step[i])), -4, 4))
+        left -= n[i] * step[i]
+    fine = np.setdiff1d(np.arange(k), coarse)                              # one unit up here, one down there, and one more of a third entry
+    a, b, sign = fine[:300], np.tile(fine[300:], 2), np.repeat([1, -1], fine.size - 300)
+    pair = (step[a][:, None] - step[a][None, :]).astype(float).ravel()
+    order, want = np.argsort(pair), (left - sign * step[b]).astype(float)
+    at = np.clip(np.searchsorted(pair[order], want), 0, pair.size - 1)
+    i = int(np.argmin(np.abs(pair[order][at] - want)))
+    u, v = divmod(int(order[at[i]]), 300)
+    n[b[i]] += sign[i]; n[a[u]] += 1; n[a[v]] -= 1
+    y = (y.astype(ext) + n * unit).astype(np.float32)
+    lead = float((hc - hp) @ y.astype(ext) / (hc @ y.astype(ext)))
+    assert abs(lead - gap) < 0.25 * abs(gap)
+    return y
+
+
+# a pick of the candidate list against a column that only the screening pass has seen, 2e-9 of a score apart (some 2e-10 is what double precision
+# leaves open at a residual of 1e-7): the confirmed order is that of the scores
+@pytest.mark.parametrize("gap", [2e-9, -2e-9])
+def test_a_pick_and_its_challenger_a_hair_apart(sgc, gap):  # noqa: F811
+    import torch
+    d, k, s, seed = 1 << 18, 1024, 18, 5
+    rng = np.random.default_rng(3)
+    for _ in range(4):
+        cols = rng.choice(d, s + 1, replace=False)
+        supp, p, c = cols[:16], cols[16], cols[18]                         # (p has been kept, c has not)
+        y = _near_tie(k, seed, supp, p, c, gap, rng)
+        st, w = sgc.Sgc(d, k, s, seed, 1e-3, 0.5, 0.999, 1e-8), torch.zeros(d, device="cuda")
+        st.set_mode(sgc.MODE_SPECULATIVE)
+        g = np.zeros(d, dtype=np.float32)
+        g[cols[:18]] = rng.choice([-1, 1], 18) * (1 + rng.random(18))
+        st.step(cuda(g), w)
+        st.set_state(y, st.get("V"), 0)                                    # beta1 = 1/2 and t = 0: M^ is y to the last bit
+        st.step(cuda(g * np.float32(1e-30)), w)
+        lam = st.get("lamM")
+        assert set(lam[:16]) == set(supp.astype(np.uint32)) and lam[16] == (c if gap > 0 else p) and lam[17] == (p if gap > 0 else c)
+        assert int(st.get("fallback")) == 0
+        st.close()
