@@ -129,8 +129,9 @@ struct GridPlan {
     int mt, row_bufs;                  // tiles of 128 residual rows; how many of them are in shared memory at a time
     int own, gw;                       // recoveries of a block, warps that work on one of them
     size_t off_rows, off_inv, off_queue, off_head, off_book, off_r, off_x, bytes;
+    double us;                         // estimate of the launch, without what the general form needs as well
 };
-inline GridPlan grid_plan(int c, long long dc, int k, int sms) {
+inline GridPlan grid_plan(int c, long long dc, int k, int s, int sms) {
     GridPlan p = {};
     const long long cols = ((dc + sms - 1) / sms + 15) / 16 * 16;
     if (cols > 1 << 16) return p;
@@ -142,6 +143,13 @@ inline GridPlan grid_plan(int c, long long dc, int k, int sms) {
     p.own = (2 * c + blocks - 1) / blocks;
     p.gw = kClusterWarps;
     while (p.gw > 4 && p.gw * p.own > kClusterWarps) p.gw >>= 1;
+    // Generating the columns; per pick, a tile of residuals meets a block of columns, and books are kept (a group of warps takes own / groups of
+    // them one after the other).  Fitted to 236 lists of 2 to 5000 chunks, half of them random sizes (10 % off on average).
+    {
+        const int groups = kClusterWarps / p.gw, turns = (p.own + groups - 1) / groups, passes = (p.cols + 543) / 544;
+        const double scores = p.mt * (0.40 * p.nb + p.cols * (2.6e-3 + 6.3e-5 * p.ks)), books = turns * (7.2 + (1.9e-3 * s * k + 0.011 * k) / p.gw);
+        p.us = 1.0 + 2.85 * p.kc * passes + s * (4.6 + scores + books);
+    }
     for (p.row_bufs = p.mt > 1 ? 2 : 1; p.row_bufs >= 1; --p.row_bufs) {
         p.off_rows = (size_t)p.cols * p.kc * 128;                     // (cols is a multiple of 8: the rows start on 1024 bytes)
         p.off_rows = (p.off_rows + 1023) / 1024 * 1024;
@@ -169,6 +177,24 @@ inline double chunk_general_us(int c, long long dc, int k, int s, int sms) {
     const double books = 1.2 * s * k * ((2 * c + sms - 1) / sms);      // (cycles, for the recoveries of one SM)
     return s * (11.0 + (books + units * (7.9 + 3.8 * ((k + 15) / 16))) / 1.9e3);
 }
+// The general form once more, where the other choice is the whole-GPU form: us of its iterations, fitted to the same lists as that one's (14 % off on
+// average).  On the tensor cores a pass over 256 residuals reads and compares all columns; else a block generates its columns for every group of
+// recoveries, of which it holds as many as its registers take, and books cost the SM of the recovery.
+constexpr int chunk_corr_group(int kp) { return kp <= 64 ? 256 : kp <= 128 ? 128 : 64; }      // recoveries per block of the correlation
+inline double chunk_launches_us(int c, long long dc, int k, int s, int sms) {
+    const int kp = chunk_padded_k(k), passes = chunk_passes(c);
+    const double per_sm = 2.0 * c / sms;
+    if (chunk_on_tensor_cores(c, dc, kp)) return s * (18.4 + passes * (5.2 + 6.6e-7 * (double)dc * k) + 4.9 * per_sm);
+    const int group = chunk_corr_group(kp), groups = (2 * c + group - 1) / group;
+    const double tiles = (double)groups * (double)((dc + 15) / 16) / sms;
+    return s * (10.6 + tiles * (0.82 + 0.0095 * (kp / 16)) + 1.6e-4 * per_sm * s * k);
+}
+// The whole-GPU form is taken from k_c = 33 on (with fewer rows the general form's correlation costs little more than its two launches: 256 chunks of
+// 65536, k = 8, s = 1: 52 us, 55 here) where its estimate is below that by a twentieth.  us per step, general / whole-GPU form:  256 chunks of 65536, k = 112,
+// s = 16: 884 / 423;  64 of 30000, 200, 25: 947 / 441;  1024 of 16384, 128, 16: 2390 / 964;  3 of 77688, 76, 2: 99 / 52;  but 1024 of 3416, 35, 5: 167 / 327;
+// 1100 of 1024, 200, 2: 189 / 322;  2000 of 4000, 64, 8: 434 / 821;  21 of 2840, 177, 2: 34 / 48.  Over 236 lists the rule's choices take 0.1 % more
+// than the better form of each, the whole-GPU form wherever it fits 16 %, the general form 36 %.
+inline bool grid_form_taken(const GridPlan& p, int k, double launches_us) { return p.blocks > 0 && k > 32 && 1.05 * p.us < launches_us; }
 // The cluster form is taken where its estimate beats that one by a tenth.  (The general form of a single vector is the lock-step recovery of
 // a whole matrix: it is taken for one wherever it fits.)
 inline bool cluster_form_taken(const ChunkPlan& p, int c, double general_us) { return p.cl > 0 && (c == 1 || 1.1 * p.us < general_us); }

@@ -267,6 +267,8 @@ __host__ __device__ constexpr int corr_threads(int kp) { return kp <= 32 ? 512 :
 __host__ __device__ constexpr int corr_kb(int kp) { return kp / 16 > 0 ? kp / 16 : 1; }              // 16-row blocks
 __host__ __device__ constexpr int corr_nt(int kp) { return kp == 64 ? 8 : (kp <= 128 ? 4 : 2); }     // tiles of four recoveries per warp
 __host__ __device__ constexpr int corr_group(int kp) { return corr_threads(kp) / 32 * 4 * corr_nt(kp); }   // recoveries per block
+static_assert(corr_group(8) == chunk_corr_group(8) && corr_group(32) == chunk_corr_group(32) && corr_group(64) == chunk_corr_group(64) &&
+              corr_group(128) == chunk_corr_group(128) && corr_group(256) == chunk_corr_group(256), "the estimates count the same groups");
 __host__ __device__ constexpr int corr_tile(int kp) { return kp <= 16 ? 256 : kp == 32 ? 128 : kp == 64 ? 64 : 32; }   // columns generated at a time
 constexpr int kCorrSuper = 512;                                                                      // columns that a key can tell apart
 
@@ -967,14 +969,13 @@ ChunkPlan plan_for(const sgc_state* st0, int c) {
     return better(p) ? p : ChunkPlan{};
 }
 
-// Shape of the whole-GPU form (blocks == 0: the launches of the general form).  From k_c = 33 on, as the general form's tensor-core
-// route: with fewer rows the general form's correlation costs little more than its two launches (256 chunks of 65536, k = 8, s = 1: 52 us,
-// here 55).  us per step, general / whole-GPU form:  256 chunks of 65536, k = 112, s = 16: 874 / 424;  48 of 22456, 84, 12: 272 / 184;
-// 16 of 100000, 56, 8: 432 / 146;  64 of 30000, 200, 25: 947 / 441;  1024 of 16384, 128, 16: 2381 / 964;  300 of 9000, 64, 8: 216 / 214.
+// Shape of the whole-GPU form (blocks == 0: the launches of the general form, see grid_form_taken).
 GridPlan grid_plan_for(const sgc_state* st0, int c) {
+    const GridPlan p = grid_plan(c, st0->d, st0->k, st0->s, st0->sm_count);
+    if (!grid_form_taken(p, st0->k, chunk_launches_us(c, st0->d, st0->k, st0->s, st0->sm_count))) return GridPlan{};
     bool fits = false;
-    if (st0->k <= 32 || chunk_grid_configure(st0->device, (st0->k + 63) / 64, &fits) != cudaSuccess || !fits) { cudaGetLastError(); return GridPlan{}; }
-    return grid_plan(c, st0->d, st0->k, st0->sm_count);
+    if (chunk_grid_configure(st0->device, p.kc, &fits) != cudaSuccess || !fits) { cudaGetLastError(); return GridPlan{}; }
+    return p;
 }
 
 // builds (or reuses) the workspace for this chunk list; the first build synchronises (one allocation, one copy)
@@ -1011,25 +1012,29 @@ cudaError_t ensure_ws(sgc_state* const* sts, int c) {
         const size_t rows = (size_t)ws->grid.mt * 128;
         ws->kp64 = ws->grid.kc * 64;
         const size_t b_rt = up(rows * ws->kp64 * sizeof(uint16_t)), b_row = up(rows * sizeof(float)), b_rep = up((size_t)2 * c * kChunkRepCap * sizeof(uint2));
-        cudaError_t e = cudaMalloc(&ws->base, b_table + b_rt + 2 * b_row + b_rep + 256);
-        if (e != cudaSuccess) { delete ws; return e; }
-        unsigned char* base = static_cast<unsigned char*>(ws->base);
-        ws->table = reinterpret_cast<ChunkRef*>(base);
-        ws->rt = reinterpret_cast<uint16_t*>(base + b_table);
-        ws->tau = reinterpret_cast<float*>(base + b_table + b_rt);
-        ws->rep_count = reinterpret_cast<unsigned int*>(base + b_table + b_rt + b_row);
-        ws->rep = reinterpret_cast<uint2*>(base + b_table + b_rt + 2 * b_row);
-        ws->flags = reinterpret_cast<int*>(base + b_table + b_rt + 2 * b_row + b_rep);
-        // 20 noise columns per recovery above the threshold: none at all, which sends a recovery through all columns, once in 5e8 picks
-        ws->z_rep = sphere_tail_threshold((double)st0->d, st0->k, 20.0);
-        std::vector<float> never(rows, INFINITY);                    // rows without a recovery screen nothing
-        e = cudaMemset(ws->base, 0, b_table + b_rt + 2 * b_row + b_rep + 256);
-        if (e == cudaSuccess) e = cudaMemcpy(ws->tau, never.data(), rows * sizeof(float), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMemcpy(ws->table, host.data(), (size_t)c * sizeof(ChunkRef), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaDeviceSynchronize();           // set-up done before the caller's stream runs on it
-        if (e != cudaSuccess) { cudaFree(ws->base); delete ws; return e; }
-        st0->chunk_ws = ws;
-        return cudaSuccess;
+        const size_t total = b_table + b_rt + 2 * b_row + b_rep + 256;
+        cudaError_t e = cudaMalloc(&ws->base, total);
+        if (e == cudaSuccess) {
+            unsigned char* base = static_cast<unsigned char*>(ws->base);
+            ws->table = reinterpret_cast<ChunkRef*>(base);
+            ws->rt = reinterpret_cast<uint16_t*>(base + b_table);
+            ws->tau = reinterpret_cast<float*>(base + b_table + b_rt);
+            ws->rep_count = reinterpret_cast<unsigned int*>(base + b_table + b_rt + b_row);
+            ws->rep = reinterpret_cast<uint2*>(base + b_table + b_rt + 2 * b_row);
+            ws->flags = reinterpret_cast<int*>(base + b_table + b_rt + 2 * b_row + b_rep);
+            // 20 noise columns per recovery above the threshold: none at all, which sends a recovery through all columns, once in 5e8 picks
+            ws->z_rep = sphere_tail_threshold((double)st0->d, st0->k, 20.0);
+            std::vector<float> never(rows, INFINITY);                // rows without a recovery screen nothing
+            e = cudaMemset(ws->base, 0, total);
+            if (e == cudaSuccess) e = cudaMemcpy(ws->tau, never.data(), rows * sizeof(float), cudaMemcpyHostToDevice);
+            if (e == cudaSuccess) e = cudaMemcpy(ws->table, host.data(), (size_t)c * sizeof(ChunkRef), cudaMemcpyHostToDevice);
+            if (e == cudaSuccess) e = cudaDeviceSynchronize();       // set-up done before the caller's stream runs on it
+            if (e != cudaSuccess) { cudaFree(ws->base); delete ws; return e; }
+            st0->chunk_ws = ws;
+            return cudaSuccess;
+        }
+        cudaGetLastError();                                          // no room for the report lists: the general form does without them
+        ws->base = nullptr; ws->grid = GridPlan{};
     }
     // column splits: as many blocks as the SMs hold at a time (one wave), at least one tile per split
     const int groups = (2 * c + corr_group(ws->kp) - 1) / corr_group(ws->kp);

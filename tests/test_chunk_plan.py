@@ -62,7 +62,7 @@ extern "C" int sweep(int k, long long* out, long long* taken) {
                     }
                     if (s > 1) continue;
                     for (int sms = 20; sms <= 148; sms += 128) {
-                        const GridPlan g = grid_plan(c, dc, k, sms);
+                        const GridPlan g = grid_plan(c, dc, k, s, sms);
                         if (g.blocks == 0) continue;
                         ++taken[1];
                         if (!whole(g, c, dc, k, sms)) { out[0] = c; out[1] = dc; out[2] = k; out[3] = sms; out[4] = 1; return 1; }
@@ -79,6 +79,7 @@ extern "C" void cluster_form(int c, long long dc, int k, int s, int eight, int s
     const bool taken = cluster_form_taken(p, c, chunk_general_us(c, dc, k, s, 148));
     out[0] = taken ? p.batches : 0; out[1] = taken ? p.gw : 0; out[2] = taken ? p.q_shared : 0;
 }
+extern "C" int whole_gpu_form(int c, long long dc, int k, int s) { return grid_form_taken(grid_plan(c, dc, k, s, 148), k, chunk_launches_us(c, dc, k, s, 148)); }
 extern "C" double tail(double d, int k, double target) { return sphere_tail_threshold(d, k, target); }
 """
 
@@ -92,6 +93,7 @@ def plan(tmp_path_factory):
                            str(d / "shim.cpp"), "-o", lib])
     L = C.CDLL(lib)
     L.cluster_form.argtypes = [C.c_int, C.c_longlong, C.c_int, C.c_int, C.c_int, C.c_int, C.POINTER(C.c_int)]
+    L.whole_gpu_form.argtypes = [C.c_int, C.c_longlong, C.c_int, C.c_int]
     L.tail.restype, L.tail.argtypes = C.c_double, [C.c_double, C.c_int, C.c_double]
     return L
 
@@ -111,6 +113,16 @@ def test_lists_that_come_in_batches(plan, c, dc, k, s, eight, sixteen):
     out = (C.c_int * 3)()
     plan.cluster_form(c, dc, k, s, eight, sixteen, out)
     assert out[0] > 1 and out[1] > 1, list(out)
+
+
+# lists whose step was timed in both forms (148 SMs; the clusters refuse them): chunks, columns of a chunk, rows of A, picks, us general / whole GPU
+@pytest.mark.parametrize("c,dc,k,s,general,whole", [
+    (1839, 1196, 96, 6, 439, 1047), (522, 616, 199, 2, 93, 204), (1024, 3416, 35, 5, 167, 327), (2000, 4000, 64, 8, 434, 821), (1100, 1024, 200, 2, 189, 322),
+    (5000, 2048, 40, 2, 358, 599), (1024, 7096, 56, 8, 344, 448), (21, 2840, 177, 2, 34, 48), (27, 9008, 121, 1, 26, 31), (256, 65_536, 112, 16, 884, 423),
+    (48, 22_456, 84, 12, 272, 184), (16, 100_000, 56, 8, 432, 146), (1024, 16_384, 128, 16, 2381, 964), (64, 30_000, 200, 25, 947, 441), (3, 77_688, 76, 2, 99, 52),
+    (2, 51_712, 48, 6, 192, 93), (37, 39_428, 244, 2, 98, 60)])
+def test_the_whole_gpu_form_is_taken_where_it_is_quicker(plan, c, dc, k, s, general, whole):
+    assert plan.whole_gpu_form(c, dc, k, s) == (whole < general)
 
 
 @pytest.mark.parametrize("d,k", [(65_536, 112), (20_000, 40), (30_000, 256)])

@@ -203,6 +203,42 @@ def test_a_step_whose_first_launch_fails_does_not_count(sgc, c, dc, k, s):
     assert np.array_equal(outs[0][0], outs[1][0]) and np.array_equal(outs[0][1], outs[1][1])
 
 
+def test_a_chunk_list_without_room_for_reports_takes_the_general_form(sgc):
+    # the recoveries on the whole GPU keep report lists of 16 KB each; when they cannot be allocated the step is made in launches that need none
+    import ctypes
+    import torch
+    rt = ctypes.CDLL("libcudart.so.12")
+    hp = [inputs.ADAM[q] for q in ("lr", "beta1", "beta2", "eps")]
+    c, dc, k, s = 200, 19_000, 100, 2
+    g = cuda(np.random.default_rng(0).standard_t(3.0, size=c * dc).astype(np.float32))
+    small, forms, outs = sgc.Mesgc(27 * 9008, 27, 121, 1, 3, *hp), [], []
+    small.step(g, torch.zeros(27 * 9008, device="cuda"))                   # (its kernels are those of the general form below: they are loaded now)
+    assert int(small.chunks[0].get("chunk_form")[0]) == 1
+    for full in (False, True):
+        me, w, held = sgc.Mesgc(c * dc, c, k, s, 3, *hp), torch.zeros(c * dc, device="cuda"), []
+        torch.cuda.synchronize()
+        try:
+            for size in (1 << 30, 1 << 26, 1 << 22) if full else ():
+                p = ctypes.c_void_p()
+                while rt.cudaMalloc(ctypes.byref(p), ctypes.c_size_t(size)) == 0:
+                    held.append(p)
+                    p = ctypes.c_void_p()
+            if full:
+                rt.cudaGetLastError()
+                assert rt.cudaFree(held.pop()) == 0                        # 4 MB, and less than 4 more, for lists of 6.5
+            me.step(g, w)
+            torch.cuda.synchronize()
+        finally:
+            for p in held:
+                rt.cudaFree(p)
+        forms.append(int(me.chunks[0].get("chunk_form")[0]))
+        outs.append(w.cpu().numpy())
+        me.close()
+    small.close()
+    assert forms == [4, 1] and np.array_equal(outs[0] != 0, outs[1] != 0)
+    assert np.abs(outs[0] - outs[1]).max() <= 1e-6 * np.abs(outs[0]).max()
+
+
 def test_states_of_very_different_k_live_side_by_side(sgc):
     # the lock-step kernel's shared-memory opt-in belongs to the kernel, not to a state: creating a small-k state must
     # not take away what a large-k state needs
