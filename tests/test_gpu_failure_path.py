@@ -93,11 +93,13 @@ def test_step_survives_an_expired_wait_and_recovers(sgc):
     ref.close()
 
 
-def test_chunked_tensor_route_survives_an_expired_wait(sgc):
-    # MESGC chunks with k_c > 32 and at least 1e9 multiply-adds per OMP iteration screen on the tensor cores (steps 0 and
-    # 2 check that route against the oracles); an expired wait (step 1) sends every recovery of that step through the
-    # fp32 kernels and is reported in the chunks' status words
-    c, dc, k, sc, seed = 64, 65_536, 112, 4, 9
+# form 4: all picks in one launch on the whole GPU; form 2: a screening pass per pick
+@pytest.mark.parametrize("c,dc,k,sc,form", [(64, 65_536, 112, 4, 4), (10, 200_000, 256, 2, 2)])
+def test_chunked_tensor_route_survives_an_expired_wait(sgc, c, dc, k, sc, form):
+    # MESGC chunks with k_c > 32 and many columns screen on the tensor cores (steps 0 and 2 check that route against the oracles); an expired
+    # wait (step 1) sends every recovery of that step through all columns (4) or through the fp32 kernels (2), and is reported in the
+    # chunks' status words
+    seed = 9
     hp = inputs.ADAM
     me = sgc.Mesgc(c * dc, c, k, sc, seed, hp["lr"], hp["beta1"], hp["beta2"], hp["eps"])
     refs = [oracle.Oracle(dc, k, sc, seed, hp["lr"], hp["beta1"], hp["beta2"], hp["eps"]) for _ in range(c)]
@@ -112,6 +114,7 @@ def test_chunked_tensor_route_survives_an_expired_wait(sgc):
             ref.step(g[i * dc:(i + 1) * dc], w_ref[i * dc:(i + 1) * dc])
             assert np.array_equal(me.chunks[i].get("lamM"), ref.get("lamM")), (step, i)
             assert np.array_equal(me.chunks[i].get("lamV"), ref.get("lamV")), (step, i)
+        assert int(me.chunks[0].get("chunk_form")[0]) == form
         timed_out = any(ch.status() & sgc.STATUS_TIMEOUT for ch in me.chunks)
         assert timed_out == (step == 1)
         for ch in me.chunks:

@@ -257,18 +257,44 @@ def test_the_first_speculating_step_leaves_another_streams_capture_alone(sgc):  
     st.close()
 
 
-# chunk recoveries inside clusters: fewer columns than blocks, ragged last block, odd k and the largest, one pick and the most, several
-# recoveries per warp group and per warp, chunks in batches, orthogonal vectors in global memory; then the general form's side of the rule
-@pytest.mark.parametrize("c,dc,k,sc", [(3, 12, 9, 3), (1, 2052, 255, 32), (7, 1300, 256, 32), (40, 508, 3, 1), (200, 640, 33, 2), (700, 260, 17, 2),
-                                       (1000, 52, 250, 2), (33, 2064, 241, 12), (2, 60_000, 15, 4), (260, 20_000, 7, 1)])
+def _chunk_parity(sgc, c, dc, k, sc, form):  # noqa: F811
+    parity.test_mesgc_small_chunks_batched_path_matches_independent_oracles(sgc, c, dc, k, sc, "student", form=form)
+
+
+# chunk recoveries inside clusters (form 3): fewer columns than blocks, ragged last block, odd k and the largest, one pick and the most, several
+# recoveries per group of 4 warps, of 2, and per warp, orthogonal vectors in global memory
+@pytest.mark.parametrize("c,dc,k,sc", [(3, 12, 9, 3), (1, 2052, 255, 32), (7, 1300, 256, 32), (200, 640, 33, 2), (33, 2064, 241, 12), (2, 60_000, 15, 4),
+                                       (300, 64, 20, 3), (1000, 64, 20, 3), (150, 64, 212, 20), (300, 64, 68, 32)])
 def test_chunk_recoveries_in_clusters(sgc, c, dc, k, sc):  # noqa: F811
-    parity.test_mesgc_small_chunks_batched_path_matches_independent_oracles(sgc, c, dc, k, sc, "student")
+    _chunk_parity(sgc, c, dc, k, sc, 3)
 
 
 # the same with more chunks than the clusters have room for: a batch begins while the records of the one before are still being written
 @pytest.mark.parametrize("c,dc,k,sc", BATCHED)
 def test_chunk_recoveries_in_batches(sgc, c, dc, k, sc):  # noqa: F811
-    parity.test_mesgc_small_chunks_batched_path_matches_independent_oracles(sgc, c, dc, k, sc, "student")
+    _chunk_parity(sgc, c, dc, k, sc, 3)
+
+
+def test_records_of_the_chunk_form_name_batches_and_teams(sgc):  # noqa: F811
+    hp = [inputs.ADAM[q] for q in ("lr", "beta1", "beta2", "eps")]
+    g = cuda(np.random.default_rng(0).standard_t(3.0, size=256 * 8064).astype(np.float32))
+    seen = set()
+    for c, dc, k, s in BATCHED + [(300, 64, 20, 3), (1000, 64, 20, 3), (150, 64, 212, 20)]:
+        me = sgc.Mesgc(c * dc, c, k, s, 3, *hp)
+        me.step(g, cuda(np.zeros(c * dc, dtype=np.float32)))
+        form, batches, warps, shared = (int(v) for v in me.chunks[-1].get("chunk_form"))
+        assert form == 3 and ((c, dc, k, s) not in BATCHED or (batches > 1 and warps > 1))
+        seen |= {("warps", warps), ("shared", shared)}
+        me.close()
+    assert {("warps", 1), ("warps", 2), ("warps", 4), ("shared", 0), ("shared", 1)} <= seen
+
+
+# the general form's side of the rules: a correlation and a decision per pick (form 1), the correlations on the tensor cores (form 2: more than
+# 1e9 multiply-adds, too many columns for the whole GPU's shared memory; one pass over the residuals, and two)
+@pytest.mark.parametrize("c,dc,k,sc,form", [(40, 508, 3, 1, 1), (700, 260, 17, 2, 1), (1000, 52, 250, 2, 1), (260, 20_000, 7, 1, 1), (522, 616, 199, 2, 1),
+                                            (10, 200_000, 256, 2, 2), (130, 60_000, 250, 1, 2), (70, 65_540, 130, 2, 2)])
+def test_chunk_lists_in_the_general_form(sgc, c, dc, k, sc, form):  # noqa: F811
+    _chunk_parity(sgc, c, dc, k, sc, form)
 
 
 # the first step of a list builds its table; a stream that does not wait for the default one finds it complete, whichever form the list takes
@@ -291,11 +317,12 @@ def test_first_chunked_step_on_a_side_stream(sgc, c, dc, k, sc):  # noqa: F811
         me.close()
 
 
-# chunk recoveries on the whole GPU (too many columns for a cluster): 64 to 256 rows of A, a ragged last block, tiles of residual rows
-# that are full, nearly empty, and brought in one after the other where there is room for one only
-@pytest.mark.parametrize("c,dc,k,sc", [(65, 60_000, 40, 2), (3, 40_004, 130, 3), (130, 22_004, 250, 1), (70, 30_000, 97, 2), (1, 70_016, 64, 5)])
+# chunk recoveries on the whole GPU (form 4; too many columns for a cluster): 64 to 256 rows of A, a ragged last block, tiles of residual rows
+# that are full, nearly empty, and brought in one after the other where there is room for one only; books in several turns
+@pytest.mark.parametrize("c,dc,k,sc", [(65, 60_000, 40, 2), (3, 40_004, 130, 3), (130, 22_004, 250, 1), (70, 30_000, 97, 2), (1, 70_016, 64, 5),
+                                       (400, 14_000, 40, 2)])
 def test_chunk_recoveries_on_the_whole_gpu(sgc, c, dc, k, sc):  # noqa: F811
-    parity.test_mesgc_small_chunks_batched_path_matches_independent_oracles(sgc, c, dc, k, sc, "student")
+    _chunk_parity(sgc, c, dc, k, sc, 4)
 
 
 # single vectors small enough for one cluster: every remainder of four, several blocks in the first kernel, kept entries in the tail
@@ -314,7 +341,7 @@ def test_small_states_recover_in_one_cluster(sgc, d, k, s, n):  # noqa: F811
             sgc.step_group(sts, [cuda(g) for g in gs], ws)
         for st, ref, g, w in zip(sts, refs, gs, wr):
             ref.step(g, w)
-            assert st.last_launches() == 3 and int(st.get("fallback")) == 1
+            assert st.last_launches() == 3 and int(st.get("fallback")) == 1 and int(st.get("chunk_form")[0]) == 3
             for name in ("sel_idx", "sel_val", "lamM", "lamV", "doneM", "doneV", "upd_idx"):
                 assert np.array_equal(st.get(name), ref.get(name)), (step, name)
     for w, r in zip(ws, wr):
