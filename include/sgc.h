@@ -276,7 +276,9 @@ SGC_API int sgc_sparsify_static(const float* grad, int64_t d, int32_t s, uint32_
  *   ms[0] unused          ms[1] top-s, the pass over the gradient           ms[2] top-s pick
  *   ms[3] projection+Adam ms[4] OMP kernels (candidate-list and lock-step)   ms[5] resolve + bookkeeping
  *   ms[6] combine+scatter ms[7] tensor-core screening passes
- *   launches[i] = number of kernel launches behind ms[i].   Both are host arrays of 8 entries. */
+ *   launches[i] = number of kernel launches behind ms[i].   Both are host arrays of 8 entries.
+ * Steps that one launch would make all picks of (small states, chunk lists) run as those of larger ones meanwhile, kernel by
+ * kernel: the same results, but not the launches or the time of an ordinary step of theirs. */
 SGC_API int sgc_set_profile(sgc_state* st, int enable);
 SGC_API int sgc_get_profile(sgc_state* st, float* ms, int32_t* launches);
 

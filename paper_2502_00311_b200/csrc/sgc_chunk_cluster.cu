@@ -10,8 +10,8 @@
 // The recoveries of different clusters have nothing to say to one another, so nothing is grid-wide, and nothing but the records
 // leaves the SMs.  What is sent goes by st.async, which counts its bytes on a barrier in the receiver's shared memory: a
 // block waits for what it needs and for nothing else (a cluster-wide barrier of 16 blocks takes 0.6 us, and an iteration needs two).
-// Latency bounds it: 5.6 us per pick for one vector of 4096 (k = 256; three cluster barriers and L2 trips of the lock-step kernel: 11), 9.2 us for 20 recoveries per
-// cluster over 2048 columns (k = 217; two launches: 17), of which scoring takes a quarter, bound by shared-memory reads of the operands.
+// Latency bounds it: 5.6 us per pick for one vector of 4096 (k = 256; three cluster barriers and L2 trips of the lock-step kernel: 11), 9.0 us for 10 recoveries per
+// cluster of 8 blocks over 2048 columns (k = 217; two launches: 17); scoring takes a quarter to a third, bound by shared-memory reads of the operands.
 // Every wait is bounded; on expiry the block marks its chunks, leaves the loops, gives what is still on its way time to land, meets the
 // others, and makes the picks that its recoveries lack by itself, going through all columns in fp64.
 #include <mutex>

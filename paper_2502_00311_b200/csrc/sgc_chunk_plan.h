@@ -15,7 +15,7 @@ constexpr int kClusterTiles = 63;                     // column tiles of 16 per 
 constexpr int kChunkShapes = 5;                       // clusters of 1, 2, 4, 8 and 16 blocks
 constexpr size_t kClusterSmem = 224 * 1024;           // dynamic shared memory of a block, at most
 constexpr size_t kClusterHead = 32;                   // barriers
-constexpr size_t kClusterBook = 1296;                 // a recovery's small records (ClusterBook)
+constexpr size_t kClusterBook = 1296;                 // a recovery's small records (ChunkBook)
 
 struct ChunkPlan {
     int cl;                            // blocks per cluster; 0: the recoveries do not fit

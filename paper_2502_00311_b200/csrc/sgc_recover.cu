@@ -1018,8 +1018,9 @@ static cudaError_t recover_batches(sgc_state* const* sts, float* const* weights,
 // Which states of a group share passes.  One pass serves a batch of states only while it has room for all their residuals
 // (kPassMaxN rows), and the two-level screening -- what keeps the number of passes over all d columns down when the
 // recovery picks columns outside the kept sets -- is a single-state scheme.  So a state goes alone when a batch could hold
-// nothing beside it, or when its last step needed three or more passes over all columns (the same signal that switches
-// its two-level screening on); the others are batched.  The result does not depend on the split.
+// nothing beside it, or when its last step needed three or more passes over all columns (the signal that switches its two-level
+// screening on, from k d = kTwoLevelWork on; smaller states go by the same rule, and make their rounds alone without it); the others
+// are batched.  The result does not depend on the split.
 cudaError_t launch_recover_group(sgc_state* const* sts, float* const* weights, int n, cudaStream_t stream, int* launches) {
     if (n == 1) return recover_batches(sts, weights, 1, stream, launches);
     std::vector<sgc_state*> together;

@@ -170,8 +170,8 @@ def test_small_state_goes_on_when_a_wait_expires(sgc):
 
 
 # a list in clusters, on the whole GPU and in the general form; a single small state and one that is not small
-@pytest.mark.parametrize("c,dc,k,s", [(6, 512, 100, 8), (3, 40_004, 130, 3), (1000, 512, 8, 1), (0, 4096, 256, 16), (0, 40_000, 300, 4)])
-def test_a_step_whose_first_launch_fails_does_not_count(sgc, c, dc, k, s):
+@pytest.mark.parametrize("c,dc,k,s,form", [(6, 512, 100, 8, 3), (3, 40_004, 130, 3, 4), (1000, 512, 8, 1, 1), (0, 4096, 256, 16, 3), (0, 40_000, 300, 4, 0)])
+def test_a_step_whose_first_launch_fails_does_not_count(sgc, c, dc, k, s, form):
     # launches into a stream whose capture has become invalid are refused by the runtime: M, V and t stay what they were
     import ctypes
     import torch
@@ -185,6 +185,7 @@ def test_a_step_whose_first_launch_fails_does_not_count(sgc, c, dc, k, s):
         st, w = opt.chunks[-1] if c else opt, torch.zeros(max(c, 1) * dc, device="cuda")
         torch.cuda.synchronize()
         opt.step(grads[0], w, stream=side)
+        assert int(st.get("chunk_form")[0]) == form
         if refused:
             before = st.get("M"), st.get("V"), w.cpu().numpy()
             cs = ctypes.c_void_p(side.cuda_stream)

@@ -299,8 +299,8 @@ def test_chunk_lists_in_the_general_form(sgc, c, dc, k, sc, form):  # noqa: F811
 
 # the first step of a list builds its table; a stream that does not wait for the default one finds it complete, whichever form the list takes
 # (cluster, whole GPU, general)
-@pytest.mark.parametrize("c,dc,k,sc", [(600, 64, 20, 4), (3, 40_004, 130, 3), (1000, 512, 8, 1)])
-def test_first_chunked_step_on_a_side_stream(sgc, c, dc, k, sc):  # noqa: F811
+@pytest.mark.parametrize("c,dc,k,sc,form", [(600, 64, 20, 4, 3), (3, 40_004, 130, 3, 4), (1000, 512, 8, 1, 1)])
+def test_first_chunked_step_on_a_side_stream(sgc, c, dc, k, sc, form):  # noqa: F811
     import torch
     hp = [inputs.ADAM[q] for q in ("lr", "beta1", "beta2", "eps")]
     g = cuda(np.random.default_rng(c).standard_t(3.0, size=c * dc).astype(np.float32))
@@ -311,6 +311,7 @@ def test_first_chunked_step_on_a_side_stream(sgc, c, dc, k, sc):  # noqa: F811
         torch.cuda.synchronize()
         me.step(g, w, stream=side if turn else None)
         side.synchronize()
+        assert int(me.chunks[0].get("chunk_form")[0]) == form
         got = w.cpu().numpy()
         want = got if want is None else want
         assert np.array_equal(got, want) and (got != 0).any()
