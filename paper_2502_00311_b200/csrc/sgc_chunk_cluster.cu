@@ -357,9 +357,8 @@ __device__ __forceinline__ double open_books(const ChunkArgs& a, ChunkBook& bk, 
 
 // A wait has expired at pick j0 of the batch that starts with chunk c0: this block goes on without the others.  Its recoveries go through all
 // columns in fp64, which decides as the kernel does (of equal scores the lowest column), from pick j0 on, and those of the batches behind it
-// from their first.
-template <bool SHARED>
-__device__ __noinline__ void finish_alone(const ChunkArgs& a, const ChunkPlan& p, unsigned char* sm, int rank, int c0, int last, int j0, const Team& tm) {
+// from their first.  (Rare: one copy of the code for vectors in shared and in global memory.)
+__device__ __noinline__ void finish_alone(const ChunkArgs& a, const ChunkPlan& p, unsigned char* sm, int rank, int c0, int last, int j0, const Team tm) {
     const int teams = kClusterWarps / p.gw;
     double* xs = reinterpret_cast<double*>(sm + p.off_x) + (size_t)tm.id * p.kq;
     for (bool open = true; c0 < last; c0 += p.batch, j0 = 0, open = false) {
@@ -370,14 +369,15 @@ __device__ __noinline__ void finish_alone(const ChunkArgs& a, const ChunkPlan& p
             double* r = reinterpret_cast<double*>(sm + p.off_r) + (size_t)own * p.kq;
             if (!open) open_books(a, bk, chunk_ref(a, c0 + (rec >> 1)), r, m, tm);
             const ChunkRef& ref = bk.ref;
-            double* qs = SHARED ? reinterpret_cast<double*>(sm + p.off_q) + (size_t)own * a.s * p.kq : ref.qb + (size_t)m * a.s * a.k;
+            double* qs = p.q_shared ? reinterpret_cast<double*>(sm + p.off_q) + (size_t)own * a.s * p.kq : ref.qb + (size_t)m * a.s * a.k;
+            const int qstride = p.q_shared ? p.kq : a.k;
             for (int j = j0; j < a.s && !bk.stopped; ++j) {
                 BestColumn b;
                 scan_columns(a, bk, r, tm, j, 0, a.dc, b);
                 uint32_t col = join_columns(bk, tm, b);
                 double gamma = 0.0, aj = 0.0, rn2 = 0.0;
                 if (col == kNoColumn) { if (tm.t == 0) { ref.cnt->stopped[m] = 1; ref.cnt->done[m] = j; } }
-                else if (!extend_basis<SHARED>(a, bk, ref, r, qs, SHARED ? p.kq : a.k, xs, m, j, col, tm, &gamma, &aj, &rn2)) col = kNoColumn;
+                else if (!extend_basis<false>(a, bk, ref, r, qs, qstride, xs, m, j, col, tm, &gamma, &aj, &rn2)) col = kNoColumn;
                 tm.meet();
                 if (tm.warp == tm.warps - 1) {
                     if (col == kNoColumn) { if (tm.lane == 0) bk.stopped = 1; }
@@ -432,9 +432,9 @@ __global__ void __launch_bounds__(kCT, 1) k_chunk_cluster(const __grid_constant_
             double* r = reinterpret_cast<double*>(sm + p.off_r) + (size_t)own * p.kq;
             send_residual(p, sm, rec, r, open_books(a, bk, ref, r, m, tm), tm);
         }
-        for (int j = 0; j < a.s; ++j) {
+        int j = 0;
+        for (; j < a.s; ++j) {
             if (t == 0 && n_own > 0) mbar_arrive_expect_tx(bar_cand, cand_bytes);
-            c_left = c0; j_left = j;
             if (!(ok = block_wait(bar_res, ph_res & 1u, &head->abort_flag, limit_ns))) break;
             ++ph_res;
             if (t == 0 && j + 1 < a.s) mbar_arrive_expect_tx(bar_res, res_bytes);
@@ -448,8 +448,10 @@ __global__ void __launch_bounds__(kCT, 1) k_chunk_cluster(const __grid_constant_
                 else make_pick<false>(a, p, sm, rec, rec & 1, own, j, tm);
             }
         }
-        if (!ok)
+        if (!ok) {
+            c_left = c0; j_left = j;
             for (int ch = c0 + t; ch < last; ch += kCT) atomicOr(&chunk_ref(a, ch).cnt->status, (unsigned int)SGC_STATUS_TIMEOUT);
+        }
     }
     // after an expired wait: what was sent, by this block and to it, may still be on its way; it lands in microseconds
     auto settle = [] { const unsigned long long t0 = global_ns(); while (global_ns() - t0 < 200000ull) __nanosleep(1000); };
@@ -457,8 +459,7 @@ __global__ void __launch_bounds__(kCT, 1) k_chunk_cluster(const __grid_constant_
     cluster.sync();
     if (!ok) {
         settle();
-        if (p.q_shared) finish_alone<true>(a, p, sm, rank, c_left, last, j_left, tm);
-        else finish_alone<false>(a, p, sm, rank, c_left, last, j_left, tm);
+        finish_alone(a, p, sm, rank, c_left, last, j_left, tm);
     }
 }
 
